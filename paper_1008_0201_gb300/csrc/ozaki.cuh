@@ -69,9 +69,9 @@ __device__ __forceinline__ unsigned oz_h2(__half lo, __half hi) {
   return (unsigned)__half_as_ushort(lo) | ((unsigned)__half_as_ushort(hi) << 16);
 }
 
-// D += A B, m16n8k16, FP16 operands, FP32 accumulate
+// D += A B, m16n8k16, FP16 operands, FP32 accumulate (no side effect: the compiler may move it)
 __device__ __forceinline__ void oz_mma(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm volatile(
+  asm(
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};\n"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -93,15 +93,17 @@ __device__ __forceinline__ void oz_ldsm2(unsigned& r0, unsigned& r1, const __hal
 }
 
 // The digit products of one 16 x 16 (A) by 16 x 8 (B) piece into the level accumulators
-// L = 0..NL-1 (NL = 8: 36 products; NL = 9: 43).
+// L = 0..NL-1 (NL = 8: 36 products; NL = 9: 43).  Digit t of A goes to all its levels before digit
+// t + 1: two products of one level are then up to NL products apart, and the warp does not wait
+// for the mma it has just issued.  (Level by level, every product waited for the one before it.)
+// The sums are exact integers, so the order does not change them.
 template <int NL>
 __device__ __forceinline__ void oz_levels(float (&acc)[NL][4], const unsigned (&fa)[OZ_T][4],
                                           const unsigned (&fb)[OZ_T][2]) {
 #pragma unroll
-  for (int L = 0; L < NL; ++L)
+  for (int t = 0; t < OZ_T; ++t)
 #pragma unroll
-    for (int t = (L >= OZ_T ? L - OZ_T + 1 : 0); t <= (L < OZ_T ? L : OZ_T - 1); ++t)
-      oz_mma(acc[L], fa[t], fb[L - t][0], fb[L - t][1]);
+    for (int L = t; L < (t + OZ_T < NL ? t + OZ_T : NL); ++L) oz_mma(acc[L], fa[t], fb[L - t][0], fb[L - t][1]);
 }
 
 // GB300 issues ~1.6 FP64 operations per clock per SM (FP32: 128), so the recombination avoids
