@@ -64,7 +64,6 @@ __global__ void k_restructure(int h, int n, const double* in, double* out, const
 __global__ void k_fill_uniform(double* x, long long n, unsigned long long seed);
 __global__ void k_fill_gauss(double* x, long long n, unsigned long long seed);
 __global__ void k_gram_oz(const JacProb* probs, int s, int CS);
-__global__ void k_update_oz(const JacProb* probs, int s, int gslabs);
 __global__ void k_gram32_tc(const JacProb* probs, int s, int CS, const __grid_constant__ CUtensorMap tmG);
 __global__ void k_update32_tc(const JacProb* probs, int s, int gtiles, int tpc, const __grid_constant__ CUtensorMap tmG,
                               const __grid_constant__ CUtensorMap tmV);
@@ -75,7 +74,6 @@ size_t tc_gram_oz_smem_bytes();
 size_t tc_gram32_smem_bytes();
 size_t tc_update32_smem_bytes();
 size_t oz_gram_smem_bytes();
-size_t oz_update_smem_bytes();
 int oz_gemm_launch(int Mr, int Nc, int K, const double* A, int lda, int transA, const double* B, int ldb,
                    const int8_t* sb, const int8_t* dsub, double* C, int ldc, int sym, int transB, long long sa,
                    long long sbb, long long sc, int batch, cudaStream_t st);
@@ -171,8 +169,6 @@ int setup_attributes(int dev) {
   ok &= cudaFuncSetAttribute(k_gram_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oz_gram_smem_bytes()) ==
         cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gram_oz, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_update_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oz_update_smem_bytes()) ==
-        cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gram32_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_gram32_smem_bytes()) ==
         cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gram32_tc, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;

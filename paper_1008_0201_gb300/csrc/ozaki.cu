@@ -1,13 +1,10 @@
-// ozaki.cu -- the FP64 Gram (Eq. (3.4)) and update (Algorithm 3.4) of a step, and a batched
-// GEMM (the precision switch's V^T J V and G_in V, the backward's products), from exact FP16
-// tensor-core digit products (ozaki.cuh).  Same grids, work split and results as k_gram /
-// k_update (gram_update.cu) and k_gemm64 (dense.cu), to FP64 accuracy.
+// ozaki.cu -- the FP64 Gram (Eq. (3.4)) of a step, and a batched GEMM (the precision switch's
+// V^T J V and G_in V, the backward's products), from exact FP16 tensor-core digit products
+// (ozaki.cuh).  Same grids, work split and results as k_gram (gram_update.cu) and k_gemm64
+// (dense.cu), to FP64 accuracy.  The digit update (Algorithm 3.4) is in tc_digits.cu.
 //
-// Scale groups.  Gram X^T X: the columns of X over a stage of rows (each column is one row of
-// A = X^T and one column of B = X).  Update Y = X V_P: the columns of X are first brought to a
-// common size, X~ = X D^-1 and V~ = D V_P with D = diag(2^(c_k)) over the slab (exact, and only
-// in the exponent arithmetic), then the rows of X~ and the columns of V~ are the groups.  A
-// small column of G stays accurate relative to itself: its entries of V~ are small too.
+// Scale groups of the Gram X^T X: the columns of X over a stage of rows (each column is one row
+// of A = X^T and one column of B = X).
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -103,12 +100,11 @@ __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ pro
       const int c = 8 * warp + cc;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        __half d0[OZ_T], d1[OZ_T];
-        oz_split(oz_fixed(x[cc][i].x, oz_bexp(x[cc][i].x) - ec[cc]), d0);
-        oz_split(oz_fixed(x[cc][i].y, oz_bexp(x[cc][i].y) - ec[cc]), d1);
+        unsigned w[OZ_T];
+        oz_split2(oz_biased(x[cc][i].x, oz_bexp(x[cc][i].x) - ec[cc]),
+                  oz_biased(x[cc][i].y, oz_bexp(x[cc][i].y) - ec[cc]), w);
 #pragma unroll
-        for (int t = 0; t < OZ_T; ++t)
-          *reinterpret_cast<unsigned*>(&sm.D[t][c][64 * i + 2 * lane]) = oz_h2(d0[t], d1[t]);
+        for (int t = 0; t < OZ_T; ++t) *reinterpret_cast<unsigned*>(&sm.D[t][c][64 * i + 2 * lane]) = w[t];
       }
     }
     __syncthreads();
@@ -141,7 +137,7 @@ __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ pro
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         const int i = 16 * ti + g + 8 * (v >> 1), j = 8 * tj + 2 * t4 + (v & 1);
-        tot[u][v] += oz_value(acc, v, sm.E[i] + sm.E[j] - 2056);
+        tot[u][v] += oz_value<true>(acc, v, sm.E[i] + sm.E[j] - 2056);
       }
     }
   }
@@ -180,186 +176,9 @@ __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ pro
   cluster.sync();  // keep every partial alive until all remote reads are done
 }
 
-// ---------------------------------------------------------------------------------- update
-// Grid (half, nslab, nprob), 256 threads; slab y covers 64 rows of Gw (y < gslabs) or of Vw, as
-// in k_update: Y = X V_P in place.  Warp w loads slab columns 8w..8w+7 (lane: rows lane and
-// lane + 32) and V_P columns 8w..8w+7 (lane: rows lane and lane + 32).
-//   c_k  = bound exponent of slab column k (0: zero column),
-//   Ea_r = max_k (ex(X[r][k]) - c_k)   (row group of X~),
-//   Eb_c = max_k (ex(V[k][c]) + c_k)   (column group of V~, over k with c_k > 0),
-//   Y[r][c] = 2^(Ea_r + Eb_c - 2056) sum_L 2^(-7 L) acc_L.
-#define OZU_ROWS 64
-#define OZU_NL 9  // levels kept: the update's row and column bounds can sit far above a term
-#define OZU_P (JAC_KMAX + 8)  // 144-byte digit rows
-struct OzUpdSmem {
-  __half A[OZ_T][OZU_ROWS][OZU_P];  // digits of X~: [t][row][k]
-  __half B[OZ_T][JAC_KMAX][OZU_P];  // digits of V~: [t][column][k]
-  int cexp[JAC_KMAX];
-  int rexp[OZU_ROWS];
-  int vexp[JAC_KMAX];
-};
-
 #define OZ_NO_EXP (-100000)
 
-__global__ void __launch_bounds__(256) k_update_oz(const JacProb* __restrict__ probs, int s, int gslabs) {
-  extern __shared__ __align__(16) unsigned char oz_raw[];
-  OzUpdSmem& sm = *reinterpret_cast<OzUpdSmem*>(oz_raw);
-  const JacProb& a = probs[blockIdx.z];
-  const int pair = blockIdx.x;
-  if (!a.active || s >= a.nsteps || pair >= a.counts[s] || a.skip[pair]) return;
-  const int* sp = a.pairs + (size_t)s * a.half * 2;
-  const int p = sp[2 * pair], q = sp[2 * pair + 1];
-  const int op = a.boff[p], wp = a.boff[p + 1] - op, oq = a.boff[q], wq = a.boff[q + 1] - oq;
-  const int k = wp + wq, KP = (k + 15) & ~15;
-  double* base;
-  int ld, r0, rs;
-  if ((int)blockIdx.y < gslabs) {
-    base = a.Gw;
-    ld = a.mp;
-    r0 = blockIdx.y * OZU_ROWS;
-    rs = min(OZU_ROWS, a.mp - r0);
-  } else {
-    if (!a.Vw) return;
-    base = a.Vw;
-    ld = a.np;
-    r0 = (blockIdx.y - gslabs) * OZU_ROWS;
-    rs = min(OZU_ROWS, a.np - r0);
-  }
-  if (rs <= 0) return;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
-  const double* Vp = a.vp + (size_t)pair * a.apld * a.apld;
-  if (tid < OZU_ROWS) sm.rexp[tid] = OZ_NO_EXP;
-  // ---- loads (all issued before use)
-  double x[8][2], v[8][2];
-#pragma unroll
-  for (int cc = 0; cc < 8; ++cc) {
-    const int c = 8 * warp + cc;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int r = lane + 32 * i;
-      x[cc][i] = (c < k && r < rs) ? base[(size_t)oz_pair_col(c, wp, op, oq) * ld + r0 + r] : 0.0;
-      v[cc][i] = (c < k && r < k) ? __ldg(Vp + (size_t)c * a.apld + r) : 0.0;
-    }
-  }
-  // ---- column bounds of the slab (warp-local)
-  int ce[8];
-#pragma unroll
-  for (int cc = 0; cc < 8; ++cc) ce[cc] = warp_max_i(max(oz_bexp(x[cc][0]), oz_bexp(x[cc][1])));
-  if (lane == 0) {
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) sm.cexp[8 * warp + cc] = ce[cc];
-  }
-  __syncthreads();  // cexp and the rexp initialization visible
-  // ---- row groups of X~
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    int m = OZ_NO_EXP;
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
-      const int ex = oz_bexp(x[cc][i]);
-      if (ex != 0) m = max(m, ex - ce[cc]);
-    }
-    if (m != OZ_NO_EXP) atomicMax(&sm.rexp[lane + 32 * i], m);
-  }
-  // ---- column groups of V~ (warp-local); the row index of V_P is a slab column
-  const int ck0 = sm.cexp[lane], ck1 = sm.cexp[lane + 32];
-  int eb[8];
-#pragma unroll
-  for (int cc = 0; cc < 8; ++cc) {
-    const int e0 = oz_bexp(v[cc][0]), e1 = oz_bexp(v[cc][1]);
-    int m = OZ_NO_EXP;
-    if (e0 != 0 && ck0 != 0) m = e0 + ck0;
-    if (e1 != 0 && ck1 != 0) m = max(m, e1 + ck1);
-    eb[cc] = warp_max_i(m);
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) sm.vexp[8 * warp + cc] = eb[cc];
-  }
-  __syncthreads();  // rexp complete
-  // ---- digits of X~: row r, columns 8w..8w+7 as one 16-byte store per digit
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int r = lane + 32 * i, ea = sm.rexp[r];
-    unsigned w[OZ_T][4];
-#pragma unroll
-    for (int cc = 0; cc < 8; cc += 2) {
-      __half d0[OZ_T], d1[OZ_T];
-      const int ex0 = oz_bexp(x[cc][i]), ex1 = oz_bexp(x[cc + 1][i]);
-      oz_split(oz_fixed(x[cc][i], ex0 - ce[cc] - ea), d0);
-      oz_split(oz_fixed(x[cc + 1][i], ex1 - ce[cc + 1] - ea), d1);
-#pragma unroll
-      for (int t = 0; t < OZ_T; ++t) w[t][cc >> 1] = oz_h2(d0[t], d1[t]);
-    }
-#pragma unroll
-    for (int t = 0; t < OZ_T; ++t)
-      *reinterpret_cast<uint4*>(&sm.A[t][r][8 * warp]) = make_uint4(w[t][0], w[t][1], w[t][2], w[t][3]);
-  }
-  // ---- digits of V~: column c, rows lane and lane + 32 (zero where the slab column is zero)
-#pragma unroll
-  for (int cc = 0; cc < 8; ++cc) {
-    const int c = 8 * warp + cc;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int kr = lane + 32 * i, ck = i ? ck1 : ck0;
-      __half d[OZ_T];
-      const long long V = (ck != 0) ? oz_fixed(v[cc][i], oz_bexp(v[cc][i]) + ck - eb[cc]) : 0ll;
-      oz_split(V, d);
-#pragma unroll
-      for (int t = 0; t < OZ_T; ++t) sm.B[t][c][kr] = d[t];
-    }
-  }
-  __syncthreads();
-  // ---- products: warp w takes row tile ti = w & 3 and column tiles 4 (w >> 2) .. + 3, two at a
-  // time (one ldmatrix.x4 of B per digit covers both)
-  const int ti = warp & 3;
-  if (16 * ti >= rs) return;
-  const int arow = 16 * ti + (lane & 7) + 8 * ((lane >> 3) & 1), akof = 8 * (lane >> 4);
-#pragma unroll 1
-  for (int h = 0; h < 2; ++h) {
-    const int tj0 = 4 * (warp >> 2) + 2 * h;
-    if (8 * tj0 >= KP) break;
-    float acc0[OZU_NL][4], acc1[OZU_NL][4];
-#pragma unroll
-    for (int L = 0; L < OZU_NL; ++L)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        acc0[L][e] = 0.0f;
-        acc1[L][e] = 0.0f;
-      }
-    const int bcol = 8 * tj0 + (lane & 7) + 8 * (lane >> 4), bkof = 8 * ((lane >> 3) & 1);
-#pragma unroll 1
-    for (int kk = 0; kk < KP; kk += 16) {
-      unsigned fa[OZ_T][4], fb0[OZ_T][2], fb1[OZ_T][2];
-#pragma unroll
-      for (int t = 0; t < OZ_T; ++t) {
-        unsigned r4[4];
-        oz_ldsm4(fa[t], &sm.A[t][arow][kk + akof]);
-        oz_ldsm4(r4, &sm.B[t][bcol][kk + bkof]);
-        fb0[t][0] = r4[0];
-        fb0[t][1] = r4[1];
-        fb1[t][0] = r4[2];
-        fb1[t][1] = r4[3];
-      }
-      oz_levels(acc0, fa, fb0);
-      oz_levels(acc1, fa, fb1);
-    }
-#pragma unroll
-    for (int hh = 0; hh < 2; ++hh) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int r = 16 * ti + g + 8 * (e >> 1), c = 8 * (tj0 + hh) + 2 * t4 + (e & 1);
-        if (r < rs && c < k) {
-          const int E = sm.rexp[r] + sm.vexp[c] - 2056;
-          base[(size_t)oz_pair_col(c, wp, op, oq) * ld + r0 + r] = hh ? oz_value(acc1, e, E) : oz_value(acc0, e, E);
-        }
-      }
-    }
-  }
-}
-
 size_t oz_gram_smem_bytes() { return sizeof(OzGramSmem); }
-size_t oz_update_smem_bytes() { return sizeof(OzUpdSmem); }
 
 // ------------------------------------------------------------------------------- GEMM
 // C = op(A) diag(sb) op(B) - diag(dsub), the contract of k_gemm64 (dense.cu), from FP16 digit
@@ -369,7 +188,7 @@ size_t oz_update_smem_bytes() { return sizeof(OzUpdSmem); }
 //   sb: optional +-1 per r; dsub: optional, its sign subtracted on the diagonal;
 //   sym = 1: C symmetric (Mr == Nc), entries j >= i computed and mirrored.
 // K runs in segments of 256 (4 chunks of 64), each an exact FP32 level sum recombined into FP64.
-// Per segment the scales are those of k_update_oz: c_r = bound exponent of column r of the CTA's
+// Per segment the scales are those of the digit update (tc_digits.cu): c_r = bound exponent of column r of the CTA's
 // op(A) rows, then the rows of op(A) D^-1 and the columns of D op(B) (D = diag(2^c_r)) are the
 // scale groups, so a term is exact to 2^-53 of its own row and column sizes even when the columns
 // of A (or rows of B) are graded.  Grid (ceil(Mr/64), ceil(Nc/32), batch), 256 threads: warp w
@@ -471,33 +290,34 @@ __global__ void __launch_bounds__(256) k_gemm_oz(int Mr, int Nc, int K, const do
       // ---- chunk values (all loads first), digits
       double xa[16], xb[8];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const int r = kc + ar + 4 * u;
+      for (int u = 0; u < 16; ++u) {  // pairs of neighbours: one 32-bit store per digit
+        const int r = kc + 2 * ar + 8 * (u >> 1) + (u & 1);
         xa[u] = (rowok && r < slen) ? a_at(ai, s0 + r) : 0.0;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int r = kc + br + 8 * u;
+        const int r = kc + 2 * br + 16 * (u >> 1) + (u & 1);
         xb[u] = (colok && r < slen) ? b_at(bj, s0 + r) : 0.0;
       }
       __syncthreads();  // the previous chunk's digits are consumed
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const int r = kc + ar + 4 * u;
-        __half d[OZ_T];
-        const int c = (r < slen) ? sm.ck[r] : 0;
-        oz_split(oz_fixed(xa[u], oz_bexp(xa[u]) - c - my_ea), d);
+      for (int u = 0; u < 16; u += 2) {
+        const int rl = 2 * ar + 8 * (u >> 1), r = kc + rl;
+        unsigned w[OZ_T];
+        const int c0 = (r < slen) ? sm.ck[r] : 0, c1 = (r + 1 < slen) ? sm.ck[r + 1] : 0;
+        oz_split2(oz_biased(xa[u], oz_bexp(xa[u]) - c0 - my_ea), oz_biased(xa[u + 1], oz_bexp(xa[u + 1]) - c1 - my_ea), w);
 #pragma unroll
-        for (int t = 0; t < OZ_T; ++t) sm.A[t][ai][ar + 4 * u] = d[t];
+        for (int t = 0; t < OZ_T; ++t) *reinterpret_cast<unsigned*>(&sm.A[t][ai][rl]) = w[t];
       }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int r = kc + br + 8 * u;
-        __half d[OZ_T];
-        const int c = (r < slen) ? sm.ck[r] : 0;
-        oz_split(c != 0 ? oz_fixed(xb[u], oz_bexp(xb[u]) + c - my_eb) : 0ll, d);
+      for (int u = 0; u < 8; u += 2) {
+        const int rl = 2 * br + 16 * (u >> 1), r = kc + rl;
+        unsigned w[OZ_T];
+        const int c0 = (r < slen) ? sm.ck[r] : 0, c1 = (r + 1 < slen) ? sm.ck[r + 1] : 0;
+        oz_split2(c0 != 0 ? oz_biased(xb[u], oz_bexp(xb[u]) + c0 - my_eb) : OZ_BIAS,
+                  c1 != 0 ? oz_biased(xb[u + 1], oz_bexp(xb[u + 1]) + c1 - my_eb) : OZ_BIAS, w);
 #pragma unroll
-        for (int t = 0; t < OZ_T; ++t) sm.B[t][bj][br + 8 * u] = d[t];
+        for (int t = 0; t < OZ_T; ++t) *reinterpret_cast<unsigned*>(&sm.B[t][bj][rl]) = w[t];
       }
       __syncthreads();
 #pragma unroll 1
@@ -522,8 +342,8 @@ __global__ void __launch_bounds__(256) k_gemm_oz(int Mr, int Nc, int K, const do
     for (int e = 0; e < 4; ++e) {
       const int il = 16 * ti + g + 8 * (e >> 1);
       const int jl0 = 8 * tj0 + 2 * t4 + (e & 1), jl1 = jl0 + 8;
-      res[0][e] += oz_value(acc0, e, sm.rexp[il] + sm.cexp[jl0] - 2056);
-      res[1][e] += oz_value(acc1, e, sm.rexp[il] + sm.cexp[jl1] - 2056);
+      res[0][e] += oz_value<false>(acc0, e, sm.rexp[il] + sm.cexp[jl0] - 2056);
+      res[1][e] += oz_value<false>(acc1, e, sm.rexp[il] + sm.cexp[jl1] - 2056);
     }
   }
 #pragma unroll

@@ -155,10 +155,10 @@ __device__ float oz_residual(PivotSmem<KM, LPP>& sm, const double* Vs, int k, in
   for (int cc = 0; cc < 8; ++cc) {
 #pragma unroll
     for (int i = 0; i < RI; ++i) {
-      __half d[OZ_T];
-      oz_split(oz_fixed(w[cc][i], oz_bexp(w[cc][i]) - ec[cc]), d);
+      unsigned d[OZ_T];
+      oz_split2(oz_biased(w[cc][i], oz_bexp(w[cc][i]) - ec[cc]), OZ_BIAS, d);
 #pragma unroll
-      for (int t = 0; t < OZ_T; ++t) sm.D[t][8 * warp + cc][lane + 32 * i] = d[t];
+      for (int t = 0; t < OZ_T; ++t) sm.D[t][8 * warp + cc][lane + 32 * i] = __ushort_as_half((unsigned short)d[t]);
     }
   }
   __syncthreads();
@@ -198,7 +198,7 @@ __device__ float oz_residual(PivotSmem<KM, LPP>& sm, const double* Vs, int k, in
       float sxj = 0.0f, sjx = 0.0f;
       if (x < k && j < k) {  // FP64 work kept to ~7 operations per entry (J by sign bits)
         const bool nx = sm.jphys[x] < 0, nj = sm.jphys[j] < 0;
-        double m = oz_value(acc, v, sm.dexp[x] + sm.dexp[j] - 2056);
+        double m = oz_value<true>(acc, v, sm.dexp[x] + sm.dexp[j] - 2056);
         if (x == j) {
           const double wxx = Vs[x * LDV + x] - 1.0, l = sm.dlo[x];
           m += oz_neg_if(wxx + wxx, nx);

@@ -1,7 +1,7 @@
 // tc_digits.cu -- the FP64-accurate block update (Algorithm 3.4: [G_p G_q] <- [G_p G_q] V_P, and
 // the same for V) from exact FP16 digit products on the fifth-generation tensor cores.
 //
-// Same arithmetic as k_update_oz (ozaki.cu), rebuilt around tcgen05:
+// Arithmetic and layout:
 //   - a CTA takes 128-row tiles of Gw (then Vw) of one pair; per tile the columns are brought to
 //     a common size (X~ = X D^-1, V~ = D V_P, D = diag(2^c_k), c_k the bound exponent of tile
 //     column k), the rows of X~ and the columns of V~ are the scale groups, and every value
@@ -34,9 +34,6 @@ namespace {
 __device__ __forceinline__ unsigned char* align1k_d(unsigned char* p) {
   return reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~(uintptr_t)1023);
 }
-// an FP32 value that holds an integer of magnitude <= 2^22, as that integer (one FP32 add: the
-// integer lands in the low mantissa bits of 1.5 * 2^23 + x)
-__device__ __forceinline__ int f32_small_int(float x) { return __float_as_int(x + 12582912.0f) - 0x4B400000; }
 __device__ __forceinline__ int warp_max_int(int v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -155,12 +152,12 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
         unsigned w[OZ_T][4];
 #pragma unroll
         for (int jj = 0; jj < 8; jj += 2) {
-          __half d0[OZ_T], d1[OZ_T];
+          unsigned d[OZ_T];
           const int c0 = 16 * cq + j0 + jj;
-          oz_split(oz_fixed(x[j0 + jj], oz_bexp(x[j0 + jj]) - cexp[c0] - ea), d0);
-          oz_split(oz_fixed(x[j0 + jj + 1], oz_bexp(x[j0 + jj + 1]) - cexp[c0 + 1] - ea), d1);
+          oz_split2(oz_biased(x[j0 + jj], oz_bexp(x[j0 + jj]) - cexp[c0] - ea),
+                    oz_biased(x[j0 + jj + 1], oz_bexp(x[j0 + jj + 1]) - cexp[c0 + 1] - ea), d);
 #pragma unroll
-          for (int tt = 0; tt < OZ_T; ++tt) w[tt][jj >> 1] = oz_h2(d0[tt], d1[tt]);
+          for (int tt = 0; tt < OZ_T; ++tt) w[tt][jj >> 1] = d[tt];
         }
         const uint32_t off = tc::sw128_offset(r, 16 * cq + j0, 2);
 #pragma unroll
@@ -172,12 +169,12 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
       unsigned w[OZ_T][4];
 #pragma unroll
       for (int jj = 0; jj < 8; jj += 2) {
-        __half d0[OZ_T], d1[OZ_T];
+        unsigned d[OZ_T];
         const int ck0 = cexp[vk0 + jj], ck1 = cexp[vk0 + jj + 1];
-        oz_split((ck0 != 0 && ev != TD_NO_EXP) ? oz_fixed(v[jj], oz_bexp(v[jj]) + ck0 - ev) : 0ll, d0);
-        oz_split((ck1 != 0 && ev != TD_NO_EXP) ? oz_fixed(v[jj + 1], oz_bexp(v[jj + 1]) + ck1 - ev) : 0ll, d1);
+        oz_split2((ck0 != 0 && ev != TD_NO_EXP) ? oz_biased(v[jj], oz_bexp(v[jj]) + ck0 - ev) : OZ_BIAS,
+                  (ck1 != 0 && ev != TD_NO_EXP) ? oz_biased(v[jj + 1], oz_bexp(v[jj + 1]) + ck1 - ev) : OZ_BIAS, d);
 #pragma unroll
-        for (int tt = 0; tt < OZ_T; ++tt) w[tt][jj >> 1] = oz_h2(d0[tt], d1[tt]);
+        for (int tt = 0; tt < OZ_T; ++tt) w[tt][jj >> 1] = d[tt];
       }
       const uint32_t off = tc::sw128_offset(vc, vk0, 2);
 #pragma unroll
@@ -220,22 +217,28 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
                       (kk > 0 || tt > 1) ? 1u : 0u);
       tc::mma_commit(&bar[1]);
     }
+    // levels 1, then 2 and 3, 4 and 5, 6 and 7: two levels are joined in 32 bits
     long long hi[16], lo[16];
+    {
+      uint32_t lv[16];
+      tc::tmem_ld16(lrow + 64, lv);
+      tc::tmem_wait_ld();
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      hi[j] = f32_small_int(__uint_as_float(l0[j]));
-      lo[j] = 0;
+      for (int j = 0; j < 16; ++j)
+        hi[j] = f32_small_int(__uint_as_float(l0[j])) * 128 + f32_small_int(__uint_as_float(lv[j]));
     }
 #pragma unroll
-    for (int L = 1; L < OZ_T; ++L) {
-      uint32_t lv[16];
-      tc::tmem_ld16(lrow + 64 * L, lv);
+    for (int L = 2; L < OZ_T; L += 2) {
+      uint32_t la[16], lb[16];
+      tc::tmem_ld16(lrow + 64 * L, la);
+      tc::tmem_ld16(lrow + 64 * L + 64, lb);
       tc::tmem_wait_ld();
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const long long iv = f32_small_int(__uint_as_float(lv[j]));
-        if (L < 4) hi[j] = hi[j] * 128 + iv;
-        else lo[j] = lo[j] * 128 + iv;
+        const int q = f32_small_int(__uint_as_float(la[j])) * 128 + f32_small_int(__uint_as_float(lb[j]));
+        if (L == 2) hi[j] = (long long)(int)hi[j] * 16384 + q;
+        else if (L == 4) lo[j] = q;
+        else lo[j] = (long long)(int)lo[j] * 16384 + q;
       }
     }
     if (__syncthreads_or(!tc::mbar_wait(&bar[1], it & 1))) {
@@ -363,13 +366,16 @@ __global__ void __launch_bounds__(512, 1) k_gram_oz_tc(const JacProb* __restrict
       unsigned char* base = sm + (lane >> 4) * TGD_CHUNK;
 #pragma unroll
       for (int cc = 0; cc < 4; ++cc) {
-        __half d[4][OZ_T];
+        unsigned long long b[4];
+        unsigned w0[OZ_T], w1[OZ_T];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) oz_split(oz_fixed(x[cc][i], oz_bexp(x[cc][i]) - ec[cc]), d[i]);
+        for (int i = 0; i < 4; ++i) b[i] = oz_biased(x[cc][i], oz_bexp(x[cc][i]) - ec[cc]);
+        oz_split2(b[0], b[1], w0);
+        oz_split2(b[2], b[3], w1);
         const uint32_t off = tc::sw128_offset(4 * warp + cc, (4 * lane) & 63, 2);
 #pragma unroll
         for (int tt = 0; tt < OZ_T; ++tt)
-          *reinterpret_cast<uint2*>(base + tt * 8192 + off) = make_uint2(oz_h2(d[0][tt], d[1][tt]), oz_h2(d[2][tt], d[3][tt]));
+          *reinterpret_cast<uint2*>(base + tt * 8192 + off) = make_uint2(w0[tt], w1[tt]);
       }
     }
     tc::fence_proxy_async_smem();
