@@ -30,10 +30,13 @@ __global__ void k_update(const JacProb* probs, int s, int gslabs);
 __global__ void k_gram32(const JacProb* probs, int s, int CS);
 __global__ void k_update32(const JacProb* probs, int s, int gslabs);
 int pivot_set_attributes();
-void pivot_launch(int km, int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s, const PivotParams& pp);
+int pivot_launch(int km, int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s, const PivotParams& pp);
 void fused_step_launch(int km, int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s,
-                       const PivotParams& pp);
+                       const PivotParams& pp, int mmax);
 int fused_step_max_rows(int km);
+int pivot_shifted_set_attributes();
+void pivot_shifted_launch(int km, int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s,
+                          const PivotParams& pp);
 int pivot64_set_attributes();
 void pivot64_launch(int km, int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s,
                     const PivotParams& pp);
@@ -180,6 +183,7 @@ int setup_attributes(int dev) {
                              (int)tc_gram_oz_smem_bytes()) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gram_oz_tc, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
   ok &= pivot_set_attributes() == 0;
+  ok &= pivot_shifted_set_attributes() == 0;
   ok &= pivot64_set_attributes() == 0;
   ok &= cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess;
   if (!ok) {
@@ -394,16 +398,16 @@ struct TcSplit {
 int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, int tslabs, int CS, int CS32, int s,
                 bool lowp, bool fallback, const PivotParams& pp, cudaStream_t st, ProfRun& prof,
                 long long& launches, const TcMaps* maps = nullptr, const TcSplit* tsp = nullptr,
-                bool fused = false) {
+                int fused_rows = 0) {
   // the pair cache: record step s - 1, then mark the pairs of step s whose outcome is known
   k_cache_step<<<count, 256, 0, st>>>(dprobs, s - 1, s);
   int r = 0;
-  if (lowp && fused) {
+  if (lowp && fused_rows > 0) {
     // FP32 sweep step of small problems: Gram, pivot and update of each pair in one CTA (pivot.cu,
     // k_step_fused); a block it hands over takes the FP64 pivot, then the plain FP32 update,
     // which acts only on those blocks (the fused kernel marks its own pairs done)
     size_t pm = prof.pre(JAC_KERNEL_STEP_FUSED, st);
-    fused_step_launch(km, max_half, count, st, dprobs, s, pp);
+    fused_step_launch(km, max_half, count, st, dprobs, s, pp, fused_rows);
     if (fallback) pivot64_launch(km, max_half, count, st, dprobs, s, pp);
     prof.post(pm, st);
     if (fallback) {
@@ -431,7 +435,12 @@ int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, in
   prof.post(pm, st);
   if (r) return r;
   pm = prof.pre(JAC_KERNEL_PIVOT, st);
-  pivot_launch(km, max_half, count, st, dprobs, s, pp);
+  if (pp.shifted) {
+    pivot_shifted_launch(km, max_half, count, st, dprobs, s, pp);
+    ++launches;
+  } else {
+    launches += pivot_launch(km, max_half, count, st, dprobs, s, pp);
+  }
   if (fallback) pivot64_launch(km, max_half, count, st, dprobs, s, pp);  // blocks the FP32 kernel handed over
   prof.post(pm, st);
   pm = prof.pre(lowp ? JAC_KERNEL_UPDATE_LOWP : JAC_KERNEL_UPDATE, st);
@@ -450,7 +459,7 @@ int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, in
   else
     k_update<<<dim3(max_half, tslabs, count), 128, kUpdSmem, st>>>(dprobs, s, gslabs);
   prof.post(pm, st);
-  launches += fallback ? 5 : 4;
+  launches += fallback ? 4 : 3;  // and the pivot's
   return cudaGetLastError() == cudaSuccess ? 0 : JAC_ECUDA;
 }
 
@@ -526,7 +535,7 @@ struct Single {
 // ------------------------------------------------------------------ single solve
 int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, const jac_opts* opts_in, double* lambda,
                void* Uv, int ldu, void* Vv, int ldv, jac_info* info, cudaStream_t st, const ArgPos& ap,
-               const double* Vinit = nullptr, bool strict_stop = false) {
+               const double* Vinit = nullptr, bool strict_stop = false, bool shifted = false) {
   jac_opts o;
   jacobi_default_opts(&o);
   if (opts_in) o = *opts_in;
@@ -679,7 +688,7 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   // entries carry errors ~ eps_32 sqrt(m) relative to ||g_i|| ||g_j||)
   const double tau_lo = std::max(o.tol, 8.0 * 5.9604644775390625e-08 * std::sqrt((double)m));
   // FP32 sweeps of small problems: one fused kernel per step
-  const bool fused = o.fused_step == 1 && P.mp <= fused_step_max_rows(P.km);
+  const int fused = (o.fused_step == 1 && !shifted && P.mp <= fused_step_max_rows(P.km)) ? P.mp : 0;
   int phase = mixed ? 1 : (fp32_only ? 4 : 3);  // 1: FP32 sweeps of the mixed mode, 3: FP64, 4: FP32 only
   if (lowp && status == JAC_OK) {
     k_lowp_copy<<<dim3(ew_blocks, 1), 256, 0, st>>>(L.probs, 0);  // FP64 layout -> FP32 copies
@@ -714,6 +723,7 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
     pp.factor = o.factor;
     pp.ns_mode = low ? 0 : 1;
     pp.oriented = (o.block_mode == JAC_BLOCK_ORIENTED) ? 1 : 0;
+    pp.shifted = shifted ? 1 : 0;
     pp.oz = (o.f64_products == JAC_F64_SPLIT16) ? 1 : (o.f64_products == JAC_F64_SPLIT16_TC ? 2 : 0);
     if (weights) {
       const int npairs = P.nb * (P.nb - 1) / 2;
@@ -978,9 +988,14 @@ int solve_complex(int m, int n, void* Gv, int ldg, const int8_t* Jdev, const jac
   const int eb = (int)std::min<size_t>(4096, ((size_t)m * n + 255) / 256);
   k_realify<<<eb, 256, 0, st>>>(m, n, static_cast<const double2*>(Gv), ldg, Jdev, Gr, Jr);
   if (cudaGetLastError() != cudaSuccess) status = JAC_ECUDA;
+  // large orders keep the pivot in shifted representation: the pairing below carries the rounding
+  // of pass 1 into the eigenvectors (pivot_shifted.cu); at 2 m >= 512 rows the FP32 sweeps never
+  // take the fused step
+  const bool shifted = n >= 256;
   // pass 1: the sweep as requested
   if (status == JAC_OK)
-    status = solve_real((int)m2, (int)n2, JAC_R64, Gr, (int)m2, Jr, &o, lam_r, nullptr, 0, Vr, (int)n2, info, st, ap);
+    status = solve_real((int)m2, (int)n2, JAC_R64, Gr, (int)m2, Jr, &o, lam_r, nullptr, 0, Vr, (int)n2, info, st, ap,
+                        nullptr, false, shifted);
   jac_info info1 = {};
   if (info) info1 = *info;
   double* Gres = Gr;
@@ -996,7 +1011,7 @@ int solve_complex(int m, int n, void* Gv, int ldg, const int8_t* Jdev, const jac
     if (o2.precision == JAC_PREC_FP32) o2.precision = JAC_PREC_FP64;
     if (status == JAC_OK)
       status = solve_real((int)m2, (int)n2, JAC_R64, Gr2, (int)m2, Jr2, &o2, lam_r, nullptr, 0, Vr, (int)n2, info, st, ap,
-                          want_v ? Vr2 : nullptr, /*strict_stop=*/true);
+                          want_v ? Vr2 : nullptr, /*strict_stop=*/true, shifted);
     if (info) {  // totals over both passes; the per-sweep maxima of pass 1, then of pass 2
       double merged[64], merged_ms[64];
       int t = 0;
@@ -1252,6 +1267,7 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
   pp.factor = o.factor;
   pp.ns_mode = fp32_only ? 0 : 1;
   pp.oriented = (o.block_mode == JAC_BLOCK_ORIENTED) ? 1 : 0;
+  pp.shifted = 0;
   pp.oz = (o.f64_products == JAC_F64_SPLIT16) ? 1 : (o.f64_products == JAC_F64_SPLIT16_TC ? 2 : 0);
   ProfRun prof;
   prof.begin();
@@ -1266,7 +1282,7 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
         for (int s = 0; s < c.max_steps; ++s)
           if (int r = launch_step(c.probs, c.count, c.km, c.max_half, c.gslabs, c.tslabs, 1, 1, s, fp32_only, true, pp,
                                   ss, pr, nl, nullptr, nullptr,
-                                  o.fused_step == 1 && c.max_mp <= fused_step_max_rows(c.km)))
+                                  (o.fused_step == 1 && c.max_mp <= fused_step_max_rows(c.km)) ? c.max_mp : 0))
             return r;
         k_cache_step<<<c.count, 256, 0, ss>>>(c.probs, -2, -1);  // record the last step of the sweep
         k_sweep_reduce<<<c.count, 256, 0, ss>>>(c.probs, c.io, c.rec, 1, d_remaining);

@@ -14,77 +14,123 @@
 //  4. V_P = P W Pi (rows permuted back as Algorithm 3.4 states; Pi = the reversed order of the
 //     J = -1 columns of Algorithm 3.3), J_P-unitary to FP64 accuracy when requested.
 //
-// GB300 placement.  The inner rotations run in FP32, LPP lanes per column pair and every pair of
-// an inner step at once, the columns held in registers (see phase 3).  To keep relative precision when A_P is nearly diagonal, the factor is carried as
-//     A_P = D (I + E) D,   R = Dp + F,   W = I + Wd,
-// where D = diag(fp32(sqrt(a_ii))) is fixed and only the deviations F, Wd are stored in FP32:
-// every rotation Q is applied as F <- F Q + Dp (Q - I) and Wd <- Wd Q + (Q - I), so small
-// entries keep their own relative precision and the angles need FP32 only.  The transform that
-// is applied to G in FP64 must be J-unitary in FP64; it is corrected by Newton-Schulz,
+// GB300 placement.  Phases 1-3 (pivot_core) are a dependent chain of FP32 work: 2 KM threads, one
+// block barrier per Cholesky step and per inner step.  Every FP32 pass runs on pairs of values
+// (fma.rn.f32x2: two FMAs per issued instruction), since with at most one or two warps per
+// scheduler the chain is bound by issue slots and latency, not by arithmetic.
+//
+// Precision of phases 2 and 3.  A_P is scaled, A_P = D (I + E) D with D = diag(fp32(sqrt(a_ii))),
+// and only deviations from the identity enter the Cholesky step in FP32, so small off-diagonal
+// entries keep their own relative precision.  The inner rotations act on the columns of R and of
+// V as they stand; what a near-diagonal block needs beyond FP32 is carried beside the columns:
+//   - the squared column norms as ||r_c||^2 = d_c^2 + cn_c, the deviation cn_c taken from the FP64
+//     diagonal and moved by every rotation, so that the gap a_jj - a_ii of two nearly equal
+//     columns keeps its relative precision;
+//   - the diagonal of V - I, which the rounding of V_cc near 1 would lose, from the J-norm of the
+//     column's other entries when the inner sweeps are done.
+// The off-diagonal entries of R and V are FP32 numbers of their own size throughout.
+//
+// The transform that is applied to G in FP64 must be J-unitary in FP64 (phase 4, pivot_orth); it
+// is corrected by Newton-Schulz,
 //     V <- V - V J (V^T J V - J) / 2   (quadratic),
-// whose residual M = V^T J V - J is formed in FP32 from the small Wd when max|Wd| <= 2^-20 and
-// otherwise from FP16 digit products of Wd (oz_residual) or on the FP64 mma path (symmetric
-// tiles only); the correction product itself is small and is formed in FP32.
+// on W = V - I: the residual M = W^T J + J W + W^T J W is formed in FP32 when max|W| <= 2^-20 and
+// otherwise from FP16 digit products of W (oz_residual) or on the FP64 mma path (symmetric tiles
+// only); the correction product itself is small and is formed in FP32.
 #include "jacobi_common.cuh"
 #include "ozaki.cuh"
 
 namespace jac {
 
-// Pivot capacity KM (largest k = w_p + w_q of the class); KM / 2 pair slots of LPP lanes each.
-template <int KM, int LPP>
-struct PivotSmem {
-  static constexpr int LDF = KM;       // F, W column stride (floats)
-  static constexpr int LDS = KM + 1;   // Cholesky matrix / FP32 scratch stride (floats)
-  static constexpr int LDV = KM + 1;   // FP64 V / M stride
-  static constexpr int NT = (KM / 2) * LPP;
-  static constexpr int NW = NT / 32;
-  static constexpr int P2 = KM / 2;    // pair slots
-  static constexpr int MBS = 2 * KM + 8;  // mailbox slot: F and W column; +8 floats spreads banks
-  static constexpr int LDD = KM + 8;   // digit rows of W (halves): 16-byte aligned, ldmatrix conflict-free
-  static constexpr int LDC = KM + 8;   // Cholesky rows (floats, in the mailboxes): 8 mod 32
-  double V[KM * LDV];   // A_P first, then V (physical coordinates), FP64
-  union {
-    double M[KM * LDV];           // FP64 residual (FP64 mma products)
-    __half D[OZ_T][KM][LDD];      // digits of W = V - I by column (digit products)
-  };
-  double dlo[KM];       // V_ii - 1 - fl(V_ii - 1) (digit products)
-  int dexp[KM];         // bound exponent of column c of W (digit products)
-  float S[KM * LDS];    // Cholesky working matrix (upper triangle), later FP32 J M
-  float F[KM * LDF];
-  float W[KM * LDF];
-  float Vf[KM * LDS];   // FP32 copy of V for the correction product
-  float mb[2][P2 * MBS];  // column mailboxes of the inner sweep (double-buffered)
-  int mphys[2][P2];
-  float mcn[2][P2];
-  float dd[KM];
-  float fid[KM];        // fp32(1 / d_i)
-  int perm[KM];
-  int lpos[KM];
-  int jphys[KM];
-  int jloc[KM];
-  float dg[2][KM];       // shifted Schur diagonal of the Cholesky steps (double-buffered)
-  unsigned pkey[2][KM];  // pivot search keys of the Cholesky steps (double-buffered)
-  int pres[KM / 2];      // block-oriented cross step: columns of block p (pivot order) per slot
-  int ptrav[KM / 2];     // ... and of block q
-  float red_f[NW][4];
-  int red_i[NW][2];
-  double trs[2];
-  int piv;
-  int bad;
+// ---- pairs of FP32 values in one 64-bit register ----------------------------------------------
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_make(float lo, float hi) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float f2_lo(f2 v) {
+  return __uint_as_float((unsigned)v);
+}
+__device__ __forceinline__ float f2_hi(f2 v) {
+  return __uint_as_float((unsigned)(v >> 32));
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// (float)x by integer operations (round to nearest, ties away from zero) for x of FP32 normal
+// size or zero; `slow` is set for any other x (an FP64 conversion per entry costs ~0.6 clocks of
+// the SM's FP64 pipe: 2.5k clocks for a 64 x 64 block)
+__device__ __forceinline__ float d2f_fast(double x, bool& slow) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), m = hi & 0x7fffffffu;
+  slow |= (m - (897u << 20)) >= (253u << 20) && (m | lo) != 0;
+  const unsigned b = (((m - (896u << 20)) << 3) | (lo >> 29)) + ((lo >> 28) & 1u);
+  return __uint_as_float(m < (897u << 20) ? 0u : (b | (hi & 0x80000000u)));
+}
+
+// ---- the core: statistics, Cholesky, inner Jacobi ---------------------------------------------
+// Pivot capacity KM (largest k = w_p + w_q of the class); KM / 2 pair slots of LPP lanes each, R
+// rows of both columns per lane.
+template <int KM>
+struct PivotDim {
+  static constexpr int LPP = 4;
+  static constexpr int R = KM / LPP;
+  static constexpr int H = R / 2;        // row pairs per lane
+  static constexpr int P2 = KM / 2;      // pair slots
+  static constexpr int NTC = P2 * LPP;   // threads of the core
+  static constexpr int NWC = NTC / 32;
+  static constexpr int LDT = KM + 4;     // rows of R~ - I by column (floats; 16-byte aligned)
+  static constexpr int LDW = KM + 4;     // columns of W = V - I (floats; 16-byte aligned)
+  static constexpr int TX = KM / 4;      // Cholesky tile of a thread: RU rows x 4 columns
+  static constexpr int RU = KM / 8;
+  static constexpr int MB = 2 * KM * P2; // floats of one mailbox: F and V column of every slot
+  static_assert(TX * 8 == NTC && R % 4 == 0, "tile and lane layout");
 };
 
-template <int KM, int LPP>
-__device__ __forceinline__ float block_max_f(float v, PivotSmem<KM, LPP>& sm, int slot) {
-  constexpr int NW = PivotSmem<KM, LPP>::NW;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (lane == 0) sm.red_f[warp][slot] = v;
-  __syncthreads();
-  float r = 0.0f;
-  for (int w = 0; w < NW; ++w) r = fmaxf(r, sm.red_f[w][slot]);
-  __syncthreads();
-  return r;
+template <int KM>
+struct alignas(16) PivotState {
+  using D = PivotDim<KM>;
+  int4 mst[2][D::P2];   // traveling column of each slot: index, cn, d, sign
+  float colb[2][KM];    // pivot column of a Cholesky step (double-buffered)
+  float dd[KM];         // d_c
+  float fid[KM];        // fp32(1 / d_c), 0 beyond k
+  float ed[KM];         // e_cc
+  float cn0[KM];        // a_cc - d_c^2
+  double adiag[KM];
+  int perm[KM];
+  int lpos[KM];         // column at logical position l
+  int linv[KM];         // logical position of column c
+  int jphys[KM];        // signs in pivot order
+  int jloc[KM];         // signs in local order
+  int pres[D::P2];      // block-oriented cross step: columns of block p (pivot order) per slot
+  int ptrav[D::P2];     // ... and of block q
+  float red_f[D::NWC][4];
+  int red_i[D::NWC][2];
+  double trs[2];
+  int k, bad, code;
+  long long t_core;     // clock at the end of the core
+  PairStat st;          // kept by thread 0
+};
+
+template <int KM>
+struct alignas(16) PivotWork {  // dead outside the core
+  using D = PivotDim<KM>;
+  union {
+    float frt[KM * D::LDT];  // frt[c LDT + i]: row i of R~ - I at column c
+    float mb[2][D::MB];      // column mailboxes of the inner sweep (double-buffered)
+  };
+};
+
+template <int KM>
+__device__ __forceinline__ void core_sync() {  // barrier of the core's threads only
+  asm volatile("bar.sync 1, %0;" ::"n"(PivotDim<KM>::NTC) : "memory");
 }
 
 // sum over the LPP lanes of a pair slot (aligned lane groups)
@@ -95,169 +141,43 @@ __device__ __forceinline__ float group_sum(float v) {
   return v;
 }
 
-// entry r of a register-held column (row l R + u in lane l of the group), broadcast to the group;
-// a select chain instead of a dynamic register index
-template <int R>
-__device__ __forceinline__ float col_entry(const float (&f)[R], int r, int group_lane0) {
-  float v = f[0];
-#pragma unroll
-  for (int u = 1; u < R; ++u) v = ((r & (R - 1)) == u) ? f[u] : v;
-  return __shfl_sync(0xffffffffu, v, group_lane0 + r / R);
-}
-
-// J-orthogonality residual M = V^T J V - J from digit products (ozaki.cuh).  With W = fl(V - I)
-// column by column and l_i = (V_ii - 1) - W_ii exactly (TwoSum), V = I + W + diag(l) and
-//   M = W^T J + J W + W^T J W + diag(2 J l) + diag(l) J W + W^T J diag(l)   (+ l^2 terms, dropped)
-// The linear and diag(l) terms are elementwise FP64; W^T J W, of size |W|^2, runs on the digit
-// path with the columns of W (over the k rows) as scale groups and J_r applied to the A digits
-// by their sign bit.  So M is accurate to ~2^-53 |W|^2 + 2^-53 |W|, where the FP64 product
-// V^T J V carries ~2^-53 |V|^2.  Writes S = fp32(J M) (zero outside k x k) and returns this
-// thread's max |M_ij|.  Warp w prepares columns 8w..8w+7 (lane: rows lane, lane + 32).
-template <int KM, int LPP>
-__device__ float oz_residual(PivotSmem<KM, LPP>& sm, const double* Vs, int k, int KP) {
-  using SM = PivotSmem<KM, LPP>;
-  constexpr int NW = SM::NW, LDV = SM::LDV, LDS = SM::LDS;
-  constexpr int RI = KM / 32;
-  static_assert(NW * 8 == KM, "one warp per 8 columns");
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
-  // ---- W, its column bounds and digits
-  double w[8][RI];
-#pragma unroll
-  for (int cc = 0; cc < 8; ++cc) {
-    const int c = 8 * warp + cc;
-#pragma unroll
-    for (int i = 0; i < RI; ++i) {
-      const int r = lane + 32 * i;
-      double x = (r < k && c < k) ? Vs[c * LDV + r] : 0.0;
-      if (r == c && r < k) {  // TwoSum(V_cc, -1)
-        const double hi = x - 1.0, bv = hi - x, av = hi - bv;
-        sm.dlo[c] = (x - av) + (-1.0 - bv);
-        x = hi;
-      }
-      w[cc][i] = x;
-    }
-  }
-  int ec[8];
-#pragma unroll
-  for (int cc = 0; cc < 8; ++cc) {
-    int e = 0;
-#pragma unroll
-    for (int i = 0; i < RI; ++i) e = max(e, oz_bexp(w[cc][i]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-    ec[cc] = e;
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) sm.dexp[8 * warp + cc] = ec[cc];
-  }
-#pragma unroll
-  for (int cc = 0; cc < 8; ++cc) {
-#pragma unroll
-    for (int i = 0; i < RI; ++i) {
-      unsigned d[OZ_T];
-      oz_split2(oz_biased(w[cc][i], oz_bexp(w[cc][i]) - ec[cc]), OZ_BIAS, d);
-#pragma unroll
-      for (int t = 0; t < OZ_T; ++t) sm.D[t][8 * warp + cc][lane + 32 * i] = __ushort_as_half((unsigned short)d[t]);
-    }
-  }
-  __syncthreads();
-  // ---- upper 16 x 8 tiles of W^T J W, then M and S
-  float mloc = 0.0f;
-  const int ntj = KP / 8, ntiles = (KP / 16) * ntj;
-  for (int tile = warp; tile < ntiles; tile += NW) {
-    const int ti = tile / ntj, tj = tile % ntj;
-    if (8 * tj + 7 < 16 * ti) continue;
-    float acc[OZ_T][4];
-#pragma unroll
-    for (int L = 0; L < OZ_T; ++L)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) acc[L][v] = 0.0f;
-    const int arow = 16 * ti + (lane & 7) + 8 * ((lane >> 3) & 1), akof = 8 * (lane >> 4);
-    const int brow = 8 * tj + (lane & 7), bkof = 8 * ((lane >> 3) & 1);
-    for (int kk = 0; kk < KP; kk += 16) {
-      const int r0 = kk + 2 * t4;
-      const unsigned slo = (sm.jphys[r0] < 0 ? 0x8000u : 0u) | (sm.jphys[r0 + 1] < 0 ? 0x80000000u : 0u);
-      const unsigned shi = (sm.jphys[r0 + 8] < 0 ? 0x8000u : 0u) | (sm.jphys[r0 + 9] < 0 ? 0x80000000u : 0u);
-      unsigned fa[OZ_T][4], fb[OZ_T][2];
-#pragma unroll
-      for (int t = 0; t < OZ_T; ++t) {
-        oz_ldsm4(fa[t], &sm.D[t][arow][kk + akof]);
-        fa[t][0] ^= slo;
-        fa[t][1] ^= slo;
-        fa[t][2] ^= shi;
-        fa[t][3] ^= shi;
-        oz_ldsm2(fb[t][0], fb[t][1], &sm.D[t][brow][kk + bkof]);
-      }
-      oz_levels(acc, fa, fb);
-    }
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int x = 16 * ti + g + 8 * (v >> 1), j = 8 * tj + 2 * t4 + (v & 1);
-      if (j < x) continue;  // (x, j), j >= x, covers the block; (j, x) is its mirror
-      float sxj = 0.0f, sjx = 0.0f;
-      if (x < k && j < k) {  // FP64 work kept to ~7 operations per entry (J by sign bits)
-        const bool nx = sm.jphys[x] < 0, nj = sm.jphys[j] < 0;
-        double m = oz_value<true>(acc, v, sm.dexp[x] + sm.dexp[j] - 2056);
-        if (x == j) {
-          const double wxx = Vs[x * LDV + x] - 1.0, l = sm.dlo[x];
-          m += oz_neg_if(wxx + wxx, nx);
-          if (__double_as_longlong(l) << 1) m += oz_neg_if(2.0 * l * (1.0 + wxx), nx);
-        } else {
-          const double wxj = Vs[j * LDV + x], wjx = Vs[x * LDV + j];  // W[x][j], W[j][x]
-          const double lx = sm.dlo[x], lj = sm.dlo[j];
-          m += oz_neg_if(wjx, nj) + oz_neg_if(wxj, nx);
-          if ((__double_as_longlong(lx) << 1) | (__double_as_longlong(lj) << 1))
-            m += oz_neg_if(lx * wxj, nx) + oz_neg_if(lj * wjx, nj);
-        }
-        const float f = (float)m;
-        mloc = fmaxf(mloc, fabsf(f));
-        sxj = nx ? -f : f;  // (J M)[x][j]
-        sjx = nj ? -f : f;  // (J M)[j][x]
-      }
-      sm.S[j * LDS + x] = sxj;
-      sm.S[x * LDS + j] = sjx;
-    }
-  }
-  return mloc;
-}
-
-// The pivot of one pair in one CTA.  Returns 0 when V_P was formed and the pair is to be updated,
-// 2 when the block was handed over to the FP64 pivot kernel (A_P still in sm.V), 1 otherwise (no
-// rotation, or a reported error); uniform over the CTA.  FUSED = false: A_P is read from the Gram kernel's output and
-// V_P written for the update kernel.  FUSED = true (the fused step kernel): A_P is already in
-// sm.V and V = I + W stays in shared memory (sm.Vf, sm.perm, sm.lpos) for the caller's update.
-template <int KM, int LPP, bool FUSED>
-__device__ __forceinline__ int pivot_block(PivotSmem<KM, LPP>& sm, const JacProb& a, int s, int pair,
-                                           const PivotParams& pp) {
-  using SM = PivotSmem<KM, LPP>;
-  constexpr int NT = SM::NT, NW = SM::NW;
-  constexpr int LDF = SM::LDF, LDS = SM::LDS, LDV = SM::LDV;
+// Phases 1-3 of one pair, run by threads 0..NTC-1 of a CTA.  Returns (uniformly) 0 when V_P was
+// formed: W = V - I in Wf (column c at c LDW, pivot order), the orders in sm; 2 when the block was
+// handed over to the FP64 pivot kernel; 1 otherwise (no rotation, or a reported error).  A32: A_P is
+// read from shared memory (FP32, column c at c LDW), else from the Gram kernel's output.  `skip` and
+// the statistics of the pair are written here unless the result is 0.
+template <int KM, bool A32>
+__device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk, const float* As, float* Wf,
+                                          const JacProb& a, int s, int pair, const PivotParams& pp) {
+  using D = PivotDim<KM>;
+  constexpr int NW = D::NWC, TX = D::TX, RU = D::RU, LDT = D::LDT, LDW = D::LDW, P2 = D::P2;
+  constexpr int LPP = D::LPP, R = D::R, H = D::H;
   unsigned* err = a.pflags;
   PairStat* stats = a.stats + (size_t)s * a.half;
   const long long t_start = clock64();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tx = tid % TX, ty = tid / TX, c0 = 4 * tx, r0 = RU * ty;
+
   // ---- 1. load A_P, scaled matrix E, statistics ----------------------------------------------
-  // The A_P tile's address depends on the pair slot only: its loads (the whole KM x KM tile,
-  // entries beyond k unused) are issued first, so that their latency overlaps the dependent
-  // lookups of the pair's blocks below (pair table, block offsets: ~10k clocks per pivot when
-  // they ran in sequence on GB300)
-  constexpr int NLD = KM * KM / NT;
-  static_assert(NLD * NT == KM * KM, "whole tile per thread set");
-  double av[NLD];
-  if constexpr (!FUSED) {
-    const double* A = a.Ap + (size_t)pair * a.apld * a.apld;
+  // The addresses depend on the pair slot only: these loads (the whole tile, entries beyond k
+  // unused) are issued before the dependent lookups of the pair's blocks
+  const double* A = a.Ap + (size_t)pair * a.apld * a.apld;
+  float e[RU][4];
+  double adg = 1.0;
+  bool slow = false;
+  double2 av[4][RU / 2];
+  if constexpr (!A32) {
 #pragma unroll
-    for (int u = 0; u < NLD; ++u) {
-      const int e = tid + u * NT;
-      av[u] = __ldg(A + (e / KM) * a.apld + e % KM);
-    }
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int u = 0; u < RU / 2; ++u)
+        av[j][u] = __ldg(reinterpret_cast<const double2*>(A + (size_t)(c0 + j) * a.apld + r0 + 2 * u));
+    if (tid < KM) adg = __ldg(A + (size_t)tid * a.apld + tid);
   }
   const int* sp = a.pairs + (size_t)s * a.half * 2;
-  const int p = sp[2 * pair], q = sp[2 * pair + 1];
-  const int op = a.boff[p], wp = a.boff[p + 1] - op, oq = a.boff[q], wq = a.boff[q + 1] - oq;
-  const int k = wp + wq, KP = (k + 15) & ~15;
-  double* Vs = sm.V;
+  const int p_ = sp[2 * pair], q_ = sp[2 * pair + 1];
+  const int op = a.boff[p_], wp = a.boff[p_ + 1] - op, oq = a.boff[q_], wq = a.boff[q_ + 1] - oq;
+  const int k = wp + wq;
   if (k > KM) {  // the driver assigns classes by k; reported, never trapped
     if (tid == 0) {
       atomicOr(err, JAC_DEVERR_INNER_LIMIT);
@@ -265,38 +185,62 @@ __device__ __forceinline__ int pivot_block(PivotSmem<KM, LPP>& sm, const JacProb
     }
     return 1;
   }
-  // the sign of this thread's column, needed after the first barrier
-  const int jcol = (tid < k) ? a.Js[tid < wp ? op + tid : oq + (tid - wp)] : 0;
-  if constexpr (!FUSED) {
+  if (tid == 0) {
+    sm.bad = 0;
+    sm.k = k;
+  }
+  if (tid < P2) {
+    sm.pres[tid] = -1;
+    sm.ptrav[tid] = -1;
+  }
+  core_sync<KM>();  // bad cleared
+  if constexpr (!A32) {
 #pragma unroll
-    for (int u = 0; u < NLD; ++u) {
-      const int e = tid + u * NT, r = e % KM, c = e / KM;
-      if (r < k && c < k) Vs[c * LDV + r] = av[u];
-    }
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int u = 0; u < RU; ++u) {
+        bool sl = false;
+        const float x = d2f_fast((u & 1) ? av[j][u / 2].y : av[j][u / 2].x, sl);
+        const bool in = r0 + u < k && c0 + j < k;
+        e[u][j] = in ? x : 0.0f;
+        slow |= in && sl;
+      }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int u = 0; u < RU; u += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(As + (c0 + j) * LDW + r0 + u);
+        e[u][j] = v.x;
+        e[u + 1][j] = v.y;
+        e[u + 2][j] = v.z;
+        e[u + 3][j] = v.w;
+      }
+    if (tid < k) adg = (double)As[tid * LDW + tid];
   }
-  if (tid == 0) sm.bad = 0;
-  __syncthreads();
   double tr = 0.0;
-  if (tid < k) {
-    sm.jloc[tid] = jcol;
-    const double aii = Vs[tid * LDV + tid];
-    if (!(aii > 0.0) || !(aii < 1.0e300)) atomicOr(&sm.bad, 1);
-    const float d = sqrtf((float)aii);
-    const double d2 = (double)d * (double)d;  // exact
+  if (tid < KM) {
+    float d = 1.0f, fid = 0.0f, ed = 0.0f, cn = 0.0f;
+    int j = 1;
+    if (tid < k) {
+      j = a.Js[tid < wp ? op + tid : oq + (tid - wp)];
+      if (!(adg > 0.0) || !(adg < 1.0e300)) atomicOr(&sm.bad, 1);
+      d = sqrtf((float)adg);
+      fid = 1.0f / d;
+      // a_ii - d_i^2 is exact in FP64 (both agree to FP32 accuracy), rounded once
+      const double d2 = (double)d * (double)d;
+      cn = (float)(adg - d2);
+      ed = cn / (float)d2;
+      tr = adg;
+    }
     sm.dd[tid] = d;
-    sm.fid[tid] = 1.0f / d;
-    sm.perm[tid] = tid;
-    // e_ii = a_ii / d_i^2 - 1 = (a_ii - d_i^2) / d_i^2: the difference is exact in FP64 (both
-    // agree to FP32 accuracy), so one FP32 division rounds the result (no FP64 division, whose
-    // latency is ~650 clocks on GB300)
-    sm.S[tid * LDS + tid] = (float)(aii - d2) / (float)d2;
-    tr = aii;
+    sm.fid[tid] = fid;
+    sm.ed[tid] = ed;
+    sm.cn0[tid] = cn;
+    sm.adiag[tid] = adg;
+    sm.jloc[tid] = j;
   }
-  for (int e = tid; e < KM * LDF; e += NT) {
-    sm.F[e] = 0.0f;
-    sm.W[e] = 0.0f;
-  }
-  __syncthreads();
+  core_sync<KM>();
   if (sm.bad) {
     if (tid == 0) {
       atomicOr(err, JAC_DEVERR_NOTPD);
@@ -307,706 +251,984 @@ __device__ __forceinline__ int pivot_block(PivotSmem<KM, LPP>& sm, const JacProb
     }
     return 1;
   }
+  if constexpr (!A32) {
+    if (slow) {  // some entry outside the FP32 normal range
+#pragma unroll 1
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int u = 0; u < RU; ++u) {
+          const float x = (r0 + u < k && c0 + j < k) ? (float)__ldg(A + (size_t)(c0 + j) * a.apld + r0 + u) : 0.0f;
+          if (j == 0) e[u][0] = x;
+          else if (j == 1) e[u][1] = x;
+          else if (j == 2) e[u][2] = x;
+          else e[u][3] = x;
+        }
+    }
+  }
   // off-diagonal e_ij = a_ij / (d_i d_j) in FP32: it is the scaled off-diagonal entry
   // |a_ij| / sqrt(a_ii a_jj) to FP32 accuracy, so it drives the statistics; only entries within
-  // 2^-12 of the threshold are re-decided in FP64.
+  // 2^-12 of the threshold are re-decided in FP64.  Both triangles are counted (sums halved).
   const double tol = pp.tol > 0.0 ? pp.tol : fmax((double)a.n, pp.tol_m * sqrt((double)a.mp)) * pp.tol_eps;
   const float tolf = (float)tol;
   float mx = 0.0f, oc = 0.0f, od = 0.0f;
-  int cnt = 0;
-  // the whole KM x KM tile in a fixed, unrolled pattern (no division by k; the loads of the
-  // iterations issue together), entries beyond k skipped
+  bool hit = false;
+  unsigned near = 0;
+  {
+    float fr[RU];
 #pragma unroll
-  for (int u = 0; u < NLD; ++u) {
-    const int e = tid + u * NT, i = e % KM, j = e / KM;
-    if (i >= k || j >= k || i == j) continue;
-    const float aij = (float)Vs[j * LDV + i];
-    const float eij = aij * sm.fid[i] * sm.fid[j];
-    sm.S[j * LDS + i] = eij;
-    if (i < j) {
-      const float r = fabsf(eij);
-      mx = fmaxf(mx, r);
-      bool hit = r > tolf;
-      if (fabsf(r - tolf) <= tolf * 2.44140625e-4f) {
-        const double ad = Vs[j * LDV + i];
-        hit = ad * ad > tol * tol * Vs[i * LDV + i] * Vs[j * LDV + j];
+    for (int u = 0; u < RU; u += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(&sm.fid[r0 + u]);
+      fr[u] = v.x;
+      fr[u + 1] = v.y;
+      fr[u + 2] = v.z;
+      fr[u + 3] = v.w;
+    }
+    const float4 fc4 = *reinterpret_cast<const float4*>(&sm.fid[c0]);
+    const float fc[4] = {fc4.x, fc4.y, fc4.z, fc4.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int u = 0; u < RU; ++u) {
+        const int i_ = r0 + u, j_ = c0 + j;
+        const float x = (i_ < k && j_ < k && i_ != j_) ? e[u][j] : 0.0f;
+        const float x2 = x * x, v = x * fr[u] * fc[j], r = fabsf(v);
+        e[u][j] = v;
+        mx = fmaxf(mx, r);
+        hit |= r > tolf;
+        near |= (fabsf(r - tolf) <= tolf * 2.44140625e-4f) ? 1u << (RU * j + u) : 0u;
+        if ((i_ < wp) != (j_ < wp)) oc += x2;
+        else od += x2;
       }
-      cnt += hit ? 1 : 0;
-      const float a2 = aij * aij;
-      if ((i < wp) != (j < wp)) oc += a2; else od += a2;
+    if (near) {
+      hit = false;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int u = 0; u < RU; ++u)
+          if (!((near >> (RU * j + u)) & 1u)) hit |= fabsf(e[u][j]) > tolf;
+      for (unsigned m = near; m; m &= m - 1) {
+        const int b = __ffs((int)m) - 1, i_ = r0 + b % RU, j_ = c0 + b / RU;
+        const double ad = A32 ? (double)As[j_ * LDW + i_] : __ldg(A + (size_t)j_ * a.apld + i_);
+        hit |= ad * ad > tol * tol * sm.adiag[i_] * sm.adiag[j_];
+      }
     }
   }
+  // npos: the J = +1 columns come first
+  int npos = __popc(__ballot_sync(0xffffffffu, lane < k && sm.jloc[lane] > 0));
+  if constexpr (KM == 64) npos += __popc(__ballot_sync(0xffffffffu, lane + 32 < k && sm.jloc[lane + 32] > 0));
+  mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+  hit = __any_sync(0xffffffffu, hit);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     oc += __shfl_xor_sync(0xffffffffu, oc, o);
     od += __shfl_xor_sync(0xffffffffu, od, o);
-    cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
   }
-  if (warp < 2) tr = warp_sum_d(tr);  // k <= 64 diagonal entries live in warps 0 and 1
+  if (warp < KM / 32) tr = warp_sum_d(tr);
   if (lane == 0) {
     sm.red_f[warp][0] = mx;
     sm.red_f[warp][1] = oc;
     sm.red_f[warp][2] = od;
-    sm.red_i[warp][0] = cnt;
-    if (warp < 2) sm.trs[warp] = tr;
+    sm.red_i[warp][0] = hit;
+    if (warp < KM / 32) sm.trs[warp] = tr;
   }
-  __syncthreads();
+  core_sync<KM>();
   mx = oc = od = 0.0f;
-  cnt = 0;
+  hit = false;
+#pragma unroll
   for (int w = 0; w < NW; ++w) {
     mx = fmaxf(mx, sm.red_f[w][0]);
     oc += sm.red_f[w][1];
     od += sm.red_f[w][2];
-    cnt += sm.red_i[w][0];
+    hit |= sm.red_i[w][0] != 0;
   }
-  PairStat st;
-  st.max_scaled = (double)mx;
-  st.off2_cross = (double)oc;
-  st.off2_diag = (double)od;
-  st.trace = sm.trs[0] + ((NW > 1 && k > 32) ? sm.trs[1] : 0.0);
-  st.rotations = 0;
-  st.inner_sweeps = 0;
-  st.ns_steps = 0;
-  st.active = (cnt > 0) ? 1 : 0;
-  st.evaluated = 1;
   const long long t_stats = clock64();
-  if (cnt == 0) {
-    if (tid == 0) {
+  if (tid == 0) {
+    PairStat& st = sm.st;
+    st.max_scaled = (double)mx;
+    st.off2_cross = 0.5 * (double)oc;
+    st.off2_diag = 0.5 * (double)od;
+    st.trace = sm.trs[0] + (KM == 64 ? sm.trs[1] : 0.0);
+    st.rotations = 0;
+    st.inner_sweeps = 0;
+    st.ns_steps = 0;
+    st.active = hit ? 1 : 0;
+    st.evaluated = 1;
+    st.cyc[0] = t_stats - t_start;
+    st.cyc[1] = st.cyc[2] = st.cyc[3] = 0;
+    if (!hit) {
       a.skip[pair] = 1;
-      st.cyc[0] = t_stats - t_start;
-      st.cyc[1] = st.cyc[2] = st.cyc[3] = 0;
       stats[pair] = st;
     }
-    return 1;
   }
-  __syncthreads();  // red_* and the trace slots are reused below
+  if (!hit) return 1;
 
   // ---- 2. scaled, optionally sign-pivoted Cholesky in FP32 -----------------------------------
-  int npos = 0;
-  for (int c = 0; c < k; ++c) npos += (sm.jloc[c] > 0) ? 1 : 0;  // J sorted: + block first
-  __syncthreads();
-  const bool signpiv = (pp.factor == 2), diagpiv = (pp.factor == 1);
-  // Left-looking Cholesky of I + E with diagonal pivoting inside the sign groups, on unpermuted
-  // storage: the pivot of step i is perm[i]; row i of R~ - I is kept by column index in Fr (the
-  // scaled entries e_ab stay untouched in S).  Step i forms row i only: for every column c not
-  // yet pivoted, (e_pc - sum_{l<i} R~_lp R~_lc) / r_ii, the sum split over TPC lanes of one warp
-  // (rows l = t mod TPC) and combined by shuffles; the shifted Schur diagonal s_cc (dg) and the
-  // search key of the next step are updated by the column's own thread, both double-buffered,
-  // so one block barrier per step suffices.  Every step is a short dependent chain: the loads
-  // that do not depend on the pivot are issued before the key reduction, and the sum runs over
-  // all rows without predicates (rows >= i of Fr are zero; row i is written in step i only after
-  // the shuffles of the warp that reads it, so its products are 0).
-  constexpr int TPC = NT / KM, CPW = 32 / TPC, NU = KM / TPC, LDC = SM::LDC;
-  static_assert(TPC * KM == NT && CPW * TPC == 32 && NU % 4 == 0, "TPC lanes of one warp per column");
-  static_assert(2 * SM::P2 * SM::MBS >= KM * LDC, "Cholesky rows fit in the mailboxes");
-  float* Fr = &sm.mb[0][0];  // row i at Fr[i * LDC + c]; LDC = 8 mod 32: a warp's loads hit 32 banks
-  const int ct = lane / CPW, cc = warp * CPW + lane % CPW;  // share of the sum, column
-  const bool pivsel = signpiv || diagpiv;
-  // the key of column c for step i: the largest unscaled Schur diagonal d_c^2 (1 + s_cc) in the
-  // sign group of step i (sign pivoting, Algorithm 3.3) or among all remaining columns (diagonal
-  // pivoting, HFC), as the value's bits above the low 6 (order-preserving for v >= 0) and 63 - c,
-  // so that one warp max-reduction yields the largest value, ties to the smaller index
-  auto in_group = [&](int i, int c) { return c < k && (!signpiv || ((i < npos) ? (c < npos) : (c >= npos))); };
-  auto key_of = [&](float d2, float s, int c) {
-    const float v = fmaxf(d2 * (1.0f + s), 0.0f);
-    return (__float_as_uint(v) & 0xFFFFFFC0u) | (unsigned)(63 - c);
-  };
-  for (int e = tid; e < KM * LDC; e += NT) Fr[e] = 0.0f;
-  if (tid < KM) {
-    const float s0 = (tid < k) ? sm.S[tid * LDS + tid] : 0.0f;
-    sm.dg[0][tid] = s0;
-    sm.dg[1][tid] = s0;
-    sm.pkey[0][tid] = in_group(0, tid) ? key_of(sm.dd[tid] * sm.dd[tid], s0, tid) : 0u;
-  }
-  const bool colk = cc < k;
-  const float ddc2 = colk ? sm.dd[cc] * sm.dd[cc] : 0.0f;
-  bool pivd = !colk;  // this thread's column pivoted already (or absent)
-  const float* fcol = Fr + ct * LDC + cc;
-  const float* frow = Fr + ct * LDC;
-  __syncthreads();
-  for (int i = 0; i < k; ++i) {
-    // independent of the pivot
-    const int b = i & 1;
-    const float dgc = sm.dg[b][cc];
-    float fc[NU];
+  // Right-looking on unpermuted storage, the whole symmetric matrix E (both triangles) in
+  // registers: thread (ty, tx) holds rows r0.. and columns c0.. .  Step i with pivot column p: the
+  // threads of column p publish it (double-buffered, one barrier), every thread scales it to
+  // t = s_p / sqrt(s_pp) and subtracts t_r t_c from its tile.  Every warp carries the shifted Schur
+  // diagonal s_cc of all columns (lane: c = lane, lane + 32) with the same operations, so the pivot
+  // search of the next step needs no barrier: a warp max-reduction of keys, the value's bits above
+  // the low 6 (order-preserving for v >= 0) and 63 - c, the largest unscaled Schur diagonal
+  // d_c^2 (1 + s_cc) in the sign group of the step (sign pivoting, Algorithm 3.3) or among all
+  // remaining columns (diagonal pivoting, HFC), ties to the smaller index.
+  // A step is one chain (barrier, column, rsqrt, key, search, publish): 540 clocks; left-looking with
+  // the rows in shared memory it took 940 (64-column block of the 512 x 512 workload: 34.5k clocks per
+  // factorization against 60.6k).
+  const bool signpiv = (pp.factor == 2), diagpiv = (pp.factor == 1), pivsel = signpiv || diagpiv;
+  f2 S[RU / 2][4];
 #pragma unroll
-    for (int u = 0; u < NU; ++u) fc[u] = fcol[TPC * u * LDC];
-    int p = i;
-    if (pivsel) {
-      const unsigned key = __reduce_max_sync(0xffffffffu, max(sm.pkey[b][lane], sm.pkey[b][lane + 32 < KM ? lane + 32 : lane]));
-      p = 63 - (int)(key & 63u);
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int u = 0; u < RU / 2; ++u) {
+      const int i_ = r0 + 2 * u, j_ = c0 + j;
+      S[u][j] = f2_make(i_ == j_ ? sm.ed[j_] : e[2 * u][j], i_ + 1 == j_ ? sm.ed[j_] : e[2 * u + 1][j]);
     }
-    // dependent on the pivot
-    const float sii = sm.dg[b][p];
-    const float scp = sm.S[max(p, cc) * LDS + min(p, cc)];
-    float fp[NU];
+  float dv0 = sm.ed[lane], dq0 = sm.dd[lane] * sm.dd[lane], dv1 = 0.0f, dq1 = 0.0f;
+  bool al0 = lane < k, al1 = false;
+  if constexpr (KM == 64) {
+    dv1 = sm.ed[lane + 32];
+    dq1 = sm.dd[lane + 32] * sm.dd[lane + 32];
+    al1 = lane + 32 < k;
+  }
+  auto next_pivot = [&](int i) -> int {
+    if (!pivsel) return i;
+    auto key_of = [&](bool alive, float dq, float dv, int c) {
+      const bool in = alive && (!signpiv || ((i < npos) == (c < npos)));
+      const float v = fmaxf(dq * (1.0f + dv), 0.0f);
+      return in ? (__float_as_uint(v) & 0xFFFFFFC0u) | (unsigned)(63 - c) : 0u;
+    };
+    unsigned key = key_of(al0, dq0, dv0, lane);
+    if constexpr (KM == 64) key = max(key, key_of(al1, dq1, dv1, lane + 32));
+    return 63 - (int)(__reduce_max_sync(0xffffffffu, key) & 63u);
+  };
+  int p = next_pivot(0);
+  for (int i = 0; i < k; ++i) {
+    const int b = i & 1;
+    if (tx == (p >> 2)) {
+      f2* dst = reinterpret_cast<f2*>(&sm.colb[b][r0]);
+      auto put = [&](int j) {
 #pragma unroll
-    for (int u = 0; u < NU; ++u) fp[u] = frow[TPC * u * LDC + p];
-    const float piv1 = 1.0f + sii;
+        for (int u = 0; u < RU / 2; ++u) dst[u] = S[u][j];
+      };
+      switch (p & 3) {  // uniform
+        case 0: put(0); break;
+        case 1: put(1); break;
+        case 2: put(2); break;
+        default: put(3);
+      }
+    }
+    core_sync<KM>();
+    const float spp = sm.colb[b][p];
+    const float v0 = sm.colb[b][lane];
+    const float v1 = (KM == 64) ? sm.colb[b][lane + (KM - 32)] : 0.0f;
+    const float4 vc = *reinterpret_cast<const float4*>(&sm.colb[b][c0]);
+    f2 vr[RU / 2];
+#pragma unroll
+    for (int u = 0; u < RU / 2; ++u) vr[u] = reinterpret_cast<const f2*>(&sm.colb[b][r0])[u];
     // The scaled Schur pivot is 1 / (A~^-1)_pp >= 1 / kappa(A~).  Below 64 eps_32 the column is
     // in the span of the previous ones at the precision of this factorization: the block goes
     // to the FP64 pivot kernel (which tells an ill-conditioned block from a singular one).
+    const float piv1 = 1.0f + spp;
     if (!(piv1 > 3.8146973e-6f)) {
       if (tid == 0) sm.bad = 1;
       break;  // uniform: every thread read the same pivot
     }
-    pivd = pivd || (p == cc);
     const float rinv = rsqrtf(piv1);  // 1 / r
-    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
-#pragma unroll
-    for (int u = 0; u < NU; u += 4) {
-      a0 = fmaf(fp[u], fc[u], a0);
-      a1 = fmaf(fp[u + 1], fc[u + 1], a1);
-      a2 = fmaf(fp[u + 2], fc[u + 2], a2);
-      a3 = fmaf(fp[u + 3], fc[u + 3], a3);
+    const float t0 = v0 * rinv, t1 = v1 * rinv;
+    dv0 = fmaf(-t0, t0, dv0);
+    dv1 = fmaf(-t1, t1, dv1);
+    al0 = al0 && lane != p;
+    al1 = al1 && lane + 32 != p;
+    const int pn = (i + 1 < k) ? next_pivot(i + 1) : 0;
+    if (warp == i % NW) {  // row i of R~ - I by column
+      const float rp = __fdividef(spp, 1.0f + piv1 * rinv);  // r - 1 without cancellation
+      wk.frt[lane * LDT + i] = (lane == p) ? rp : t0;
+      if constexpr (KM == 64) wk.frt[(lane + 32) * LDT + i] = (lane + 32 == p) ? rp : t1;
+      if (lane == 0) sm.perm[i] = p;
     }
-    float dot = (a0 + a1) + (a2 + a3);
+    const f2 rinv2 = f2_make(rinv, rinv);
 #pragma unroll
-    for (int o = CPW; o < 32; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    // row i of R~ - I (by column index), the Schur diagonal and the next step's key
-    const float v = (scp - dot) * rinv;
-    const float dn = fmaf(-v, v, dgc);
-    const unsigned nk = (!pivd && in_group(i + 1, cc)) ? key_of(ddc2, dn, cc) : 0u;
-    if (ct == 0) {
-      if (!pivd) {
-        Fr[i * LDC + cc] = v;
-        sm.dg[b ^ 1][cc] = dn;
-      }
-      sm.pkey[b ^ 1][cc] = nk;
-    } else if (ct == 1 && cc == 0) {
-      const float r = piv1 * rinv;
-      Fr[i * LDC + p] = __fdividef(sii, 1.0f + r);  // r - 1 without cancellation
-      sm.perm[i] = p;
+    for (int u = 0; u < RU / 2; ++u) vr[u] = f2_mul(vr[u], rinv2);
+    const float tc[4] = {-vc.x * rinv, -vc.y * rinv, -vc.z * rinv, -vc.w * rinv};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const f2 t2 = f2_make(tc[j], tc[j]);
+#pragma unroll
+      for (int u = 0; u < RU / 2; ++u) S[u][j] = f2_fma(vr[u], t2, S[u][j]);
     }
-    __syncthreads();
+    p = pn;
   }
-  __syncthreads();
+  core_sync<KM>();
   if (sm.bad) {  // handed over to the FP64 pivot kernel, which decides on rank deficiency
     if (tid == 0) {
       a.skip[pair] = 2;
       atomicOr(err, JAC_DEVERR_HANDOVER);
-      st.cyc[0] = t_stats - t_start;
-      st.cyc[1] = clock64() - t_stats;
-      st.cyc[2] = st.cyc[3] = 0;
-      stats[pair] = st;
+      sm.st.cyc[1] = clock64() - t_stats;
+      stats[pair] = sm.st;
     }
     return 2;
   }
-  // R = Dp + F in pivot order: F[c][r] = (R~ - I)[r][c] d_c, r <= c; then d and the signs in
-  // pivot order, and the logical order of the inner sweep
-  for (int e = tid; e < k * k; e += NT) {
-    const int r = e % k, c = e / k;
-    if (r <= c) {
-      const int pc = sm.perm[c];
-      sm.F[c * LDF + r] = Fr[r * LDC + pc] * sm.dd[pc];
-    }
-  }
-  float d_new = 0.0f;
-  int j_new = 0;
-  if (tid < k) {
-    d_new = sm.dd[sm.perm[tid]];
-    j_new = sm.jloc[sm.perm[tid]];
-  }
-  __syncthreads();
-  // block-oriented steps after the first of a sweep rotate only the cross pairs (one column of
-  // block p, one of block q): block p's columns become the residents of the ring, block q's the
-  // travelers, each in pivot order
+  // Orders.  Block-oriented steps after the first of a sweep rotate only the cross pairs (one
+  // column of block p, one of block q): block p's columns become the residents of the ring, block
+  // q's the travelers, each in pivot order.  Diagonal pivoting mixes the signs: the output order
+  // puts the pivot-order columns back on positions of their own sign (positives, then negatives,
+  // each in pivot order), so that V_P^* J_P V_P = J_P in the block's local order (the reordering of
+  // HFC).  Sign pivoting takes the J = -1 columns in reverse.
   const bool cross_only = pp.oriented && s > 0;
-  if (tid < SM::P2) {
-    sm.pres[tid] = -1;
-    sm.ptrav[tid] = -1;
-  }
-  __syncthreads();
-  if (tid < k) {
-    sm.dd[tid] = d_new;
-    sm.jphys[tid] = j_new;
-    if (diagpiv) {
-      // diagonal pivoting mixes the signs: the output order puts the pivot-order columns back
-      // on positions of their own sign (positives, then negatives, each in pivot order), so
-      // that V_P^* J_P V_P = J_P in the block's local order (the reordering of HFC)
-      const bool pos = j_new > 0;
-      int rank = 0;
-      for (int c = 0; c < tid; ++c) rank += ((sm.jloc[sm.perm[c]] > 0) == pos) ? 1 : 0;
-      sm.lpos[pos ? rank : npos + rank] = tid;
-    } else {
-      sm.lpos[tid] = (signpiv && tid >= npos) ? (k - 1 - (tid - npos)) : tid;
+  {
+    auto mask64 = [&](auto f) -> unsigned long long {  // f(position) over the k positions
+      unsigned long long m = __ballot_sync(0xffffffffu, lane < k && f(lane < k ? lane : 0));
+      if constexpr (KM == 64)
+        m |= (unsigned long long)__ballot_sync(0xffffffffu, lane + 32 < k && f(lane + 32 < k ? lane + 32 : 0)) << 32;
+      return m;
+    };
+    const unsigned long long mpos = mask64([&](int c) { return sm.jloc[sm.perm[c]] > 0; });
+    const unsigned long long mp = mask64([&](int c) { return sm.perm[c] < wp; });
+    if (tid < k) {
+      const unsigned long long below = (1ull << tid) - 1;
+      const bool pos = (mpos >> tid) & 1;
+      int l = tid;
+      if (diagpiv) l = pos ? __popcll(mpos & below) : npos + __popcll(~mpos & below);
+      else if (signpiv && tid >= npos) l = k - 1 - (tid - npos);
+      sm.lpos[l] = tid;
+      sm.linv[tid] = l;
+      sm.jphys[tid] = pos ? 1 : -1;
+      if (cross_only) {
+        if ((mp >> tid) & 1) sm.pres[__popcll(mp & below)] = tid;
+        else sm.ptrav[__popcll(~mp & below)] = tid;
+      }
+    } else if (tid < KM) {
+      sm.jphys[tid] = 1;
     }
-    if (cross_only) {
-      const bool in_p = sm.perm[tid] < wp;
-      int rank = 0;
-      for (int c = 0; c < tid; ++c) rank += ((sm.perm[c] < wp) == in_p) ? 1 : 0;
-      if (in_p) sm.pres[rank] = tid;
-      else sm.ptrav[rank] = tid;
-    }
   }
-  __syncthreads();
+  core_sync<KM>();
   const long long t_chol = clock64();
 
-  // ---- 3. inner one-sided Jacobi (FP32, shifted representation) -----------------------------
+  // ---- 3. inner one-sided Jacobi (FP32) -------------------------------------------------------
   // inner threshold: at most half the outer one (so that a pair flagged in FP64 is rotated in
-  // FP32), at least the FP32 noise level of the shifted dot products
+  // FP32), at least the FP32 noise level of the dot products
   const float tol_in = fmaxf(0.5f * tolf, 64.0f * 5.9604645e-8f * mx);
   // The columns live in registers: pair slot q (LPP lanes of a warp) holds a resident and a
-  // traveler column, R rows per lane (row l R + u in lane l).  An inner sweep is a recursive
-  // cross ordering of the KM positions: at group size g (KM/2, KM/4, ..., 1 slots) the
-  // travelers of each group go round its ring of g slots, so every resident meets every
+  // traveler column of R and of V, R rows per lane (row l R + u in lane l), as row pairs.  An inner
+  // sweep is a recursive cross ordering of the KM positions: at group size g (KM/2, KM/4, ..., 1
+  // slots) the travelers of each group go round its ring of g slots, so every resident meets every
   // traveler of the group in g steps; then each group splits in two, its residents pairing among
   // themselves in the first half and its travelers in the second.  Every pair of positions
   // meets once in KM - 1 steps, and between steps each slot passes exactly one column to one
-  // other slot through a shared-memory mailbox: one block barrier per step.  Positions >= k are
+  // other slot through a shared-memory mailbox: one barrier per step.  Positions >= k are
   // empty.  The logical order of Algorithm 3.3 (reversed J = -1 part) gives the initial
   // placement: position p is the resident of slot p (p < KM/2) or the traveler of slot p - KM/2.
-  constexpr int R = KM / LPP, GP = 32 / LPP, P2 = SM::P2, MBS = SM::MBS;
-  const int grp = lane / LPP, l = lane % LPP, slot = warp * GP + grp, lane0 = grp * LPP;
+  // Four lanes per slot, one warp per scheduler: the parameter chain (~90 instructions per warp
+  // and step) is issued half as often as with eight, and the reduction is one shuffle shorter.  Full
+  // inner sweep of a 64-column block (63 steps): 61k clocks; with eight lanes, scalar FMAs and
+  // predicated diagonal terms 78k.
+  const int slot = tid / LPP, l = tid % LPP;
   int ci = cross_only ? sm.pres[slot] : ((slot < k) ? sm.lpos[slot] : -1);
   int cj = cross_only ? sm.ptrav[slot] : ((slot + P2 < k) ? sm.lpos[slot + P2] : -1);
   // block-oriented: one inner sweep; after the first step of an outer sweep only the ring of
   // its first level (every column of block p meets every column of block q once)
   const int g_last = cross_only ? P2 : 1;
   const int max_inner = pp.oriented ? 1 : JAC_INNER_MAX_SWEEPS;
-  float fi[R], fj[R], wi[R], wj[R];
+  f2 fi[H], fj[H], wi[H], wj[H];
+  float cni, cnj, si, sj;  // ||r||^2 = s^2 + cn
+  int ji, jj;
+  auto load_col = [&](int c, f2(&f)[H], f2(&w)[H], float& cn, float& d, int& sg) {
+    const int pc = c >= 0 ? sm.perm[c] : 0;
+    cn = c >= 0 ? sm.cn0[pc] : 0.0f;
+    d = c >= 0 ? sm.dd[pc] : 1.0f;
+    sg = c >= 0 ? sm.jphys[c] : 1;
 #pragma unroll
-  for (int u = 0; u < R; ++u) {
-    fi[u] = (ci >= 0) ? sm.F[ci * LDF + l * R + u] : 0.0f;
-    fj[u] = (cj >= 0) ? sm.F[cj * LDF + l * R + u] : 0.0f;
-    wi[u] = 0.0f;
-    wj[u] = 0.0f;
-  }
-  int total_rot = 0, inner = 0, buf = 0;
-  for (inner = 0; inner < max_inner; ++inner) {
-    // c = ||r||^2 - s^2 = 2 s F_cc + ||f||^2 of both columns, recomputed every inner sweep and
-    // tracked through the rotations
-    float cni, cnj;
-    {
-      float qi = 0.0f, qj = 0.0f;
+    for (int u = 0; u < H; u += 2) {
+      const float4 x4 = *reinterpret_cast<const float4*>(&wk.frt[pc * LDT + l * R + 2 * u]);
+      const float x[4] = {x4.x, x4.y, x4.z, x4.w};
+      float r[4], v[4];
 #pragma unroll
-      for (int u = 0; u < R; ++u) {
-        qi = fmaf(fi[u], fi[u], qi);
-        qj = fmaf(fj[u], fj[u], qj);
+      for (int t = 0; t < 4; ++t) {
+        const int row = l * R + 2 * u + t;
+        r[t] = (row < c) ? x[t] * d : (row == c) ? fmaf(x[t], d, d) : 0.0f;
+        v[t] = (row == c) ? 1.0f : 0.0f;
       }
-      qi = group_sum<LPP>(qi);
-      qj = group_sum<LPP>(qj);
-      const float di = col_entry<R>(fi, ci >= 0 ? ci : 0, lane0);
-      const float dj = col_entry<R>(fj, cj >= 0 ? cj : 0, lane0);
-      cni = (ci >= 0) ? 2.0f * sm.dd[ci] * di + qi : 0.0f;
-      cnj = (cj >= 0) ? 2.0f * sm.dd[cj] * dj + qj : 0.0f;
+      f[u] = f2_make(r[0], r[1]);
+      f[u + 1] = f2_make(r[2], r[3]);
+      w[u] = f2_make(v[0], v[1]);
+      w[u + 1] = f2_make(v[2], v[3]);
     }
+  };
+  load_col(ci, fi, wi, cni, si, ji);
+  load_col(cj, fj, wj, cnj, sj, jj);
+  core_sync<KM>();  // the Cholesky rows are read; the mailboxes take their place
+  int total_rot = 0, inner = 0, buf = 0;
+  // a column's mailbox: 16-byte chunk q of lane l at ((q P2 + slot) LPP + l): a quarter warp writes
+  // and reads 128 consecutive bytes
+  auto box = [&](int b, int q, int sl) { return reinterpret_cast<ulonglong2*>(wk.mb[b]) + ((q * P2 + sl) * LPP + l); };
+  auto send = [&](int dst, const f2(&f)[H], const f2(&w)[H], int c, float cn, float d, int sg) {
+#pragma unroll
+    for (int u = 0; u < H; u += 2) {
+      *box(buf, u / 2, dst) = make_ulonglong2(f[u], f[u + 1]);
+      *box(buf, H / 2 + u / 2, dst) = make_ulonglong2(w[u], w[u + 1]);
+    }
+    if (l == 0) sm.mst[buf][dst] = make_int4(c, __float_as_int(cn), __float_as_int(d), sg);
+  };
+  auto receive = [&](f2(&f)[H], f2(&w)[H], int& c, float& cn, float& d, int& sg) {
+    const int4 m = sm.mst[buf][slot];
+#pragma unroll
+    for (int u = 0; u < H; u += 2) {
+      const ulonglong2 x = *box(buf, u / 2, slot);
+      f[u] = x.x;
+      f[u + 1] = x.y;
+    }
+#pragma unroll
+    for (int u = 0; u < H; u += 2) {
+      const ulonglong2 x = *box(buf, H / 2 + u / 2, slot);
+      w[u] = x.x;
+      w[u + 1] = x.y;
+    }
+    c = m.x;
+    cn = __int_as_float(m.y);
+    d = __int_as_float(m.z);
+    sg = m.w;
+  };
+  for (inner = 0; inner < max_inner; ++inner) {
     int my_rot = 0;       // per slot (uniform over its lanes)
     float my_max = 0.0f;  // largest scaled |a_ij| rotated
     for (int g = P2; g >= g_last; g >>= 1) {
       const int base = slot & ~(g - 1), pos = slot - base;
       for (int st_ = 0; st_ < g; ++st_) {
         // ---- rotate the pair (ci, cj) of this slot
-        const bool act = (ci >= 0) && (cj >= 0);
-        const int ii = act ? ci : 0, jj = act ? cj : 0;
+        const bool act = (ci | cj) >= 0;
         // what does not depend on the dot product first
-        const float si = sm.dd[ii], sj = sm.dd[jj];
-        const bool trig = sm.jphys[ii] == sm.jphys[jj];
+        const bool trig = ji == jj;
         const float aii = fmaf(si, si, cni), ajj = fmaf(sj, sj, cnj);
         const float rs = rsqrtf(aii) * rsqrtf(ajj);
-        // a_ij = (d_i e_i + f_i) . (d_j e_j + f_j) = s_i F_ij + s_j F_ji + f_i . f_j in one group
-        // reduction: the cross terms enter the partial sums of the lanes that hold rows i and j
-        // (predicated FMAs; fetching F_ij and F_ji from the owner lanes first costs a dependent
-        // select chain and a shuffle per entry, ~11% of the step)
-        float sij = 0.0f, xc = 0.0f;
+        const float x = trig ? (sj - si) * (sj + si) + (cnj - cni) : aii + ajj;
+        f2 d0 = f2_mul(fi[0], fj[0]), d1 = f2_mul(fi[1], fj[1]);
 #pragma unroll
-        for (int u = 0; u < R; ++u) {
-          const int row = l * R + u;
-          sij = fmaf(fi[u], fj[u], sij);
-          if (row == ii) xc = fmaf(si, fj[u], xc);
-          if (row == jj) xc = fmaf(sj, fi[u], xc);
+        for (int u = 2; u < H; u += 2) {
+          d0 = f2_fma(fi[u], fj[u], d0);
+          d1 = f2_fma(fi[u + 1], fj[u + 1], d1);
         }
-        const float aij_all = group_sum<LPP>(sij + xc);
-        if (act) {
-          const float aij = aij_all;
-          const float beta = fabsf(aij);
-          const float scaled = beta * rs;
-          if (scaled > tol_in) {
-            ++my_rot;
-            my_max = fmaxf(my_max, scaled);
-            const float e = (aij < 0.0f) ? -1.0f : 1.0f;
-            // One branch-free path for both kinds (sg = +1 trigonometric, -1 hyperbolic), so
-            // that the slots of a warp never split on the sign pattern:
-            //  trigonometric, Eq. (2.1): cot(2 phi) = (a_jj - a_ii) / (2 |a_ij|), i.e.
-            //    t = sign(x) 2|a_ij| / (|x| + sqrt(x^2 + 4|a_ij|^2)),  x = a_jj - a_ii;
-            //  hyperbolic: coth(2 phi) = -(a_ii + a_jj) / (2 |a_ij|), i.e.
-            //    t = -2|a_ij| / (x + sqrt((x - 2|a_ij|)(x + 2|a_ij|))),  x = a_ii + a_jj,
-            //    with the |tanh| < 1 guard of Sec. 3.2;
-            // both evaluated after an exact power-of-two scaling of x and 2|a_ij| into [1, 4).
-            // The square roots are x rsqrt(x): the angle needs FP32 accuracy only, the
-            // rotation built from it is orthogonal (J-orthogonal) whatever t is.
-            const float sg = trig ? 1.0f : -1.0f;
-            const float x = trig ? (sj - si) * (sj + si) + (cnj - cni) : aii + ajj;
-            const float mxv = fmaxf(fabsf(x), 2.0f * beta);
-            const float sc = __int_as_float(0x7f000000 - (__float_as_int(mxv) & 0x7f800000));
-            const float nu = x * sc, b2 = 2.0f * beta * sc;
-            const float rr = trig ? fmaf(nu, nu, b2 * b2) : (nu - b2) * (nu + b2);
-            const bool ok = rr > 0.0f;
-            const float root = ok ? rr * rsqrtf(rr) : 0.0f;
-            const float tm = __fdividef(b2, fabsf(nu) + root);
-            float t = trig ? copysignf(tm, x) : (ok ? -tm : -1.0f);
-            if (!trig && (!(fabsf(t) < 1.0f) || !((1.0f - t) * (1.0f + t) > 0.0f))) t = copysignf(0.9f, t);
-            const float c = rsqrtf(fmaf(sg * t, t, 1.0f));  // cos or cosh
-            const float s_ = t * c;                          // sin or sinh
-            const float q11 = c, q12 = e * s_, q21 = -sg * e * s_;
-            const float cm1 = -sg * __fdividef(s_ * s_, 1.0f + c);  // c - 1 without cancellation
-            // a_ii' = a_ii - t |a_ij|, a_jj' = a_jj + t |a_ij| (trigonometric); both move by
-            // t |a_ij| (hyperbolic: the J-trace is invariant)
-            const float dci = -sg * t * beta, dcj = t * beta;
-            // F <- F Q + Dp (Q - I), Wd <- Wd Q + (Q - I): the Dp (Q - I) / (Q - I) terms touch
-            // rows i and j only
+        const float aij = group_sum<LPP>((f2_lo(d0) + f2_lo(d1)) + (f2_hi(d0) + f2_hi(d1)));
+        const float beta = fabsf(aij), scaled = beta * rs;
+        if (act && scaled > tol_in) {
+          ++my_rot;
+          my_max = fmaxf(my_max, scaled);
+          // One branch-free path for both kinds (sg = +1 trigonometric, -1 hyperbolic), so
+          // that the slots of a warp never split on the sign pattern:
+          //  trigonometric, Eq. (2.1): cot(2 phi) = (a_jj - a_ii) / (2 |a_ij|), i.e.
+          //    t = sign(x) 2|a_ij| / (|x| + sqrt(x^2 + 4|a_ij|^2)),  x = a_jj - a_ii;
+          //  hyperbolic: coth(2 phi) = -(a_ii + a_jj) / (2 |a_ij|), i.e.
+          //    t = -2|a_ij| / (x + sqrt((x - 2|a_ij|)(x + 2|a_ij|))),  x = a_ii + a_jj,
+          //    with the |tanh| < 1 guard of Sec. 3.2;
+          // both evaluated after an exact power-of-two scaling of x and 2|a_ij| into [1, 4).
+          // The square roots are x rsqrt(x): the angle needs FP32 accuracy only, the
+          // rotation built from it is orthogonal (J-orthogonal) whatever t is.
+          const float sg = trig ? 1.0f : -1.0f;
+          const float mxv = fmaxf(fabsf(x), 2.0f * beta);
+          const float sc = __int_as_float(0x7f000000 - (__float_as_int(mxv) & 0x7f800000));
+          const float nu = x * sc, b2 = 2.0f * beta * sc;
+          const float rr = trig ? fmaf(nu, nu, b2 * b2) : (nu - b2) * (nu + b2);
+          const bool ok = rr > 0.0f;
+          const float root = ok ? rr * rsqrtf(rr) : 0.0f;
+          const float tm = __fdividef(b2, fabsf(nu) + root);
+          float t = trig ? copysignf(tm, x) : (ok ? -tm : -1.0f);
+          const bool guard = !trig && (!(fabsf(t) < 1.0f) || !((1.0f - t) * (1.0f + t) > 0.0f));
+          if (guard) t = copysignf(0.9f, t);
+          // cos or cosh; of a small angle as 1 - y / 2 rounded once (rsqrtf returns the value below
+          // 1 too often there, and thousands of tiny rotations would shrink V: with it alone the
+          // FP32-only eigenvalues of order 128 came out 5e-5 small, with this rule 2e-5)
+          const float y = sg * t * t, c0 = rsqrtf(1.0f + y);
+          const float c = fabsf(y) < 1.52587890625e-5f ? fmaf(-0.5f, y, 1.0f) : c0;
+          const float es = copysignf(t * c, aij < 0.0f ? -t : t);  // +- sin or sinh
+          const f2 q11 = f2_make(c, c), q12 = f2_make(es, es), q21 = f2_make(-sg * es, -sg * es);
+          // a_ii' = a_ii - t |a_ij|, a_jj' = a_jj + t |a_ij| (trigonometric); both move by
+          // t |a_ij| (hyperbolic: the J-trace is invariant)
+          cni = fmaf(-sg * t, beta, cni);
+          cnj = fmaf(t, beta, cnj);
+          if (guard) {  // a_ij not annihilated: the norms from their definition
+            const float cc = c * c, ss = t * t * cc, cs = 2.0f * t * cc * beta;
+            cni = fmaf(cc, aii, fmaf(ss, ajj, cs)) - si * si;
+            cnj = fmaf(cc, ajj, fmaf(ss, aii, cs)) - sj * sj;
+          }
 #pragma unroll
-            for (int u = 0; u < R; ++u) {
-              const int row = l * R + u;
-              const float a_i = fi[u], a_j = fj[u], b_i = wi[u], b_j = wj[u];
-              float nfi = fmaf(q11, a_i, q21 * a_j), nfj = fmaf(q11, a_j, q12 * a_i);
-              float nwi = fmaf(q11, b_i, q21 * b_j), nwj = fmaf(q11, b_j, q12 * b_i);
-              if (row == ii) {
-                nfi += si * cm1;
-                nfj += si * q12;
-                nwi += cm1;
-                nwj += q12;
-              }
-              if (row == jj) {
-                nfi += sj * q21;
-                nfj += sj * cm1;
-                nwi += q21;
-                nwj += cm1;
-              }
-              fi[u] = nfi;
-              fj[u] = nfj;
-              wi[u] = nwi;
-              wj[u] = nwj;
-            }
-            cni += dci;
-            cnj += dcj;
+          for (int u = 0; u < H; ++u) {
+            const f2 a_i = fi[u], a_j = fj[u];
+            fi[u] = f2_fma(q11, a_i, f2_mul(q21, a_j));
+            fj[u] = f2_fma(q11, a_j, f2_mul(q12, a_i));
+          }
+#pragma unroll
+          for (int u = 0; u < H; ++u) {
+            const f2 a_i = wi[u], a_j = wj[u];
+            wi[u] = f2_fma(q11, a_i, f2_mul(q21, a_j));
+            wj[u] = f2_fma(q11, a_j, f2_mul(q12, a_i));
           }
         }
         // ---- pass one column on: the traveler round the ring, or at the end of the group's
         // ring its split (first half: traveler to slot + g/2, which sends back its resident)
         if (st_ < g - 1) {
-          // ring step (uniform over the block): the traveler goes to the next slot of the group.
-          // Row l * R + u of a column sits at u * LPP + l of its mailbox slot: the 8 lanes of a
-          // slot write 32 consecutive bytes per u, and the 4 slots of a warp land on distinct
-          // banks (lane-contiguous rows l * R + u put lanes l and l + 4 on the same banks)
-          const int dst = base + ((pos + 1) & (g - 1));
-          float* box = sm.mb[buf] + dst * MBS + l;
-#pragma unroll
-          for (int u = 0; u < R; ++u) {
-            box[u * LPP] = fj[u];
-            box[KM + u * LPP] = wj[u];
-          }
-          if (l == 0) {
-            sm.mphys[buf][dst] = cj;
-            sm.mcn[buf][dst] = cnj;
-          }
-          __syncthreads();
-          const float* in = sm.mb[buf] + slot * MBS + l;
-#pragma unroll
-          for (int u = 0; u < R; ++u) {
-            fj[u] = in[u * LPP];
-            wj[u] = in[KM + u * LPP];
-          }
-          cj = sm.mphys[buf][slot];
-          cnj = sm.mcn[buf][slot];
+          send(base + ((pos + 1) & (g - 1)), fj, wj, cj, cnj, sj, jj);
+          core_sync<KM>();
+          receive(fj, wj, cj, cnj, sj, jj);
           buf ^= 1;
         } else if (g > g_last) {
-          // end of the group's ring: its split (first half: traveler to slot + g/2, which sends
-          // back its resident)
           const bool give_res = pos >= g / 2;
           const int dst = pos < g / 2 ? slot + g / 2 : slot - g / 2;
-          float* box = sm.mb[buf] + dst * MBS + l;
-#pragma unroll
-          for (int u = 0; u < R; ++u) {
-            box[u * LPP] = give_res ? fi[u] : fj[u];
-            box[KM + u * LPP] = give_res ? wi[u] : wj[u];
-          }
-          if (l == 0) {
-            sm.mphys[buf][dst] = give_res ? ci : cj;
-            sm.mcn[buf][dst] = give_res ? cni : cnj;
-          }
-          __syncthreads();
-          const float* in = sm.mb[buf] + slot * MBS + l;
-          const int cin = sm.mphys[buf][slot];
-          const float cnin = sm.mcn[buf][slot];
-          if (give_res) {
-#pragma unroll
-            for (int u = 0; u < R; ++u) {
-              fi[u] = in[u * LPP];
-              wi[u] = in[KM + u * LPP];
-            }
-            ci = cin;
-            cni = cnin;
-          } else {
-#pragma unroll
-            for (int u = 0; u < R; ++u) {
-              fj[u] = in[u * LPP];
-              wj[u] = in[KM + u * LPP];
-            }
-            cj = cin;
-            cnj = cnin;
-          }
+          if (give_res) send(dst, fi, wi, ci, cni, si, ji);
+          else send(dst, fj, wj, cj, cnj, sj, jj);
+          core_sync<KM>();
+          if (give_res) receive(fi, wi, ci, cni, si, ji);
+          else receive(fj, wj, cj, cnj, sj, jj);
           buf ^= 1;
         }
       }
     }
     // sweep totals: one count per slot (its lane 0)
-    int cnt = (l == 0) ? my_rot : 0;
-    cnt = warp_sum_i(cnt);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) my_max = fmaxf(my_max, __shfl_xor_sync(0xffffffffu, my_max, o));
+    const int cnt = (int)__reduce_add_sync(0xffffffffu, (l == 0) ? (unsigned)my_rot : 0u);
+    my_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(my_max)));
     if (lane == 0) {
       sm.red_i[warp][1] = cnt;
-      sm.red_f[warp][2] = my_max;
+      sm.red_f[warp][3] = my_max;
     }
-    __syncthreads();
+    core_sync<KM>();
     int tot = 0;
     float dmax = 0.0f;
+#pragma unroll
     for (int w = 0; w < NW; ++w) {
       tot += sm.red_i[w][1];
-      dmax = fmaxf(dmax, sm.red_f[w][2]);
+      dmax = fmaxf(dmax, sm.red_f[w][3]);
     }
-    __syncthreads();
+    core_sync<KM>();
     total_rot += tot;
     // done when nothing was rotated, or when every rotated pair was already so small that the
     // next sweep (quadratic convergence: off-diagonals ~ k delta^2) would find nothing above tol_in
     if (tot == 0 || (float)k * dmax * dmax <= tol_in) break;
   }
   if (!pp.oriented && inner >= JAC_INNER_MAX_SWEEPS && tid == 0) atomicOr(err, JAC_DEVERR_INNER_LIMIT);
-  // W columns back to shared memory, physical coordinates
+  // W = V - I.  The diagonal from the J-norm of the column, J_c sum_r J_r v_rc^2 = 1:
+  // v_cc - 1 = -S / (1 + sqrt(1 - S)), S = J_c sum_{r != c} J_r v_rc^2, where S is small; the
+  // rounded v_cc itself would lose W_cc ~ S / 2 below 2^-24
+  auto finish = [&](int c, int sg, const f2(&w)[H]) {
+    float S1 = 0.0f;
+    float v[R];
 #pragma unroll
-  for (int u = 0; u < R; ++u) {
-    if (ci >= 0) sm.W[ci * LDF + l * R + u] = wi[u];
-    if (cj >= 0) sm.W[cj * LDF + l * R + u] = wj[u];
-  }
-  __syncthreads();
+    for (int u = 0; u < H; ++u) {
+      v[2 * u] = f2_lo(w[u]);
+      v[2 * u + 1] = f2_hi(w[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      const int row = l * R + u;
+      const float q = (row == c) ? 0.0f : v[u] * v[u];
+      S1 += (sm.jphys[row] < 0) ? -q : q;
+    }
+    S1 = group_sum<LPP>(S1) * (float)sg;
+    const float wd = -__fdividef(S1, 1.0f + sqrtf(1.0f - fminf(S1, 0.5f)));
+    if (c < 0) return;
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      if (l * R + u == c) v[u] = (v[u] > 0.0f && fabsf(S1) < 0.5f) ? wd : v[u] - 1.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < R; u += 4)
+      *reinterpret_cast<float4*>(&Wf[c * LDW + l * R + u]) = make_float4(v[u], v[u + 1], v[u + 2], v[u + 3]);
+  };
+  finish(ci, ji, wi);
+  finish(cj, jj, wj);
   const long long t_inner = clock64();
-
-  // ---- 4. V = I + Wd (physical coordinates), J-orthogonalized in FP64 if requested ----------
-  float wm = 0.0f;
-  for (int e = tid; e < KP * KP; e += NT) {
-    const int r = e % KP, c = e / KP;
-    const float w = (r < k && c < k) ? sm.W[c * LDF + r] : 0.0f;
-    const bool diag = (r == c && r < k);
-    const double v = oz_f2d(w);  // integer conversion: FP64 instructions are scarce on GB300
-    Vs[c * LDV + r] = diag ? v + 1.0 : v;
-    sm.Vf[c * LDS + r] = diag ? w + 1.0f : w;
-    wm = fmaxf(wm, fabsf(w));
-  }
-  int ns = 0;
-  bool ns_ok = true;
-  if (pp.ns_mode) {
-    ns_ok = false;
-    wm = block_max_f<KM, LPP>(wm, sm, 3);  // includes the barrier after the V build
-    const bool small_w = wm <= 9.5367431640625e-7f;  // 2^-20
-    for (int it = 0; it < 3; ++it) {
-      // residual M = V^T J V - J, J = diag(jphys) on rows and columns
-      float mloc = 0.0f;
-      if (it == 0 && small_w) {
-        // V = I + Wd: M = Wd^T J + J Wd + Wd^T J Wd.  The linear part is exact in FP32 when it
-        // cancels (Sterbenz) and rounds relative to itself otherwise; the quadratic part is at
-        // most k 2^-40 and carries FP32 relative error.  Stored as fp32(J M) directly.
-        for (int e = tid; e < KP * KP; e += NT) {
-          const int x = e % KP, j = e / KP;
-          float mv = 0.0f;
-          if (x < k && j < k) {
-            const float jx = (float)sm.jphys[x], jj = (float)sm.jphys[j];
-            float quad = 0.0f;
-            for (int r = 0; r < k; ++r) quad = fmaf(sm.W[x * LDF + r] * (float)sm.jphys[r], sm.W[j * LDF + r], quad);
-            mv = (sm.W[x * LDF + j] * jj + jx * sm.W[j * LDF + x]) + quad;
-          }
-          mloc = fmaxf(mloc, fabsf(mv));
-          sm.S[j * LDS + x] = (x < k) ? (float)sm.jphys[x] * mv : 0.0f;  // (J M)[x][j]
-        }
-      } else if (pp.oz) {
-        mloc = oz_residual<KM, LPP>(sm, Vs, k, KP);
-      } else {
-        // FP64 mma, upper tiles (8 tj + 7 >= 16 ti) and the mirror of the strict lower part
-        const int g = lane >> 2, t = lane & 3;
-        const int ntj = KP / 8, ntiles = (KP / 16) * ntj;
-        for (int tile = warp; tile < ntiles; tile += NW) {
-          const int ti = tile / ntj, tj = tile % ntj;
-          if (8 * tj + 7 < 16 * ti) continue;
-          double c4[4] = {0.0, 0.0, 0.0, 0.0};
-          for (int kq = 0; kq < KP; kq += 16) {
-            double av[8], bv[4];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) av[u] = Vs[(16 * ti + g + 8 * (u & 1)) * LDV + kq + 4 * t + (u >> 1)];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int r = kq + 4 * t + u;
-              const double v = Vs[(8 * tj + g) * LDV + r];
-              bv[u] = (r < k && sm.jphys[r] < 0) ? -v : v;
-            }
-            dmma16816(c4, av, bv);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int i = 16 * ti + g + 8 * (u >> 1), j = 8 * tj + 2 * t + (u & 1);
-            if (j < i) continue;  // written once, from the tile holding (j, i) ... (i, j), j >= i
-            double v = c4[u];
-            if (i == j && i < k) v -= (sm.jphys[i] < 0) ? -1.0 : 1.0;
-            sm.M[j * LDV + i] = v;
-            sm.M[i * LDV + j] = v;
-          }
-        }
-        __syncthreads();
-        for (int e = tid; e < KP * KP; e += NT) {
-          const int x = e % KP, j = e / KP;
-          const double mv = sm.M[j * LDV + x];
-          mloc = fmaxf(mloc, (float)fabs(mv));
-          sm.S[j * LDS + x] = (x < k) ? (float)((sm.jphys[x] < 0) ? -mv : mv) : 0.0f;
-        }
-      }
-      const float mm = block_max_f<KM, LPP>(mloc, sm, 0);
-      if (mm <= 4.0e-16f) {
-        ns_ok = true;
-        break;
-      }
-      // V <- V - V (J M) / 2: the correction is O(|M|), formed in FP32 from the FP32 copy of V;
-      // each thread a 4 x CB block (rows rg + RG i, columns cg + CGN c) of the product, so a
-      // shared-memory load feeds 4 or CB FMAs; the FP32 copy follows V in FP32
-      {
-        constexpr int RG = KM / 4, CGN = NT / RG, CB = KM / CGN;
-        static_assert(RG * CGN == NT && CGN * CB == KM, "correction blocking");
-        const int rg = tid % RG, cg = tid / RG;
-        float sum[4][CB];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int c = 0; c < CB; ++c) sum[i][c] = 0.0f;
-        for (int x = 0; x < k; ++x) {
-          float vf[4], sv[CB];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) vf[i] = sm.Vf[x * LDS + rg + RG * i];
-#pragma unroll
-          for (int c = 0; c < CB; ++c) sv[c] = sm.S[(cg + CGN * c) * LDS + x];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int c = 0; c < CB; ++c) sum[i][c] = fmaf(vf[i], sv[c], sum[i][c]);
-        }
-        __syncthreads();  // every read of Vf done
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int c = 0; c < CB; ++c) {
-            const int r = rg + RG * i, j = cg + CGN * c;
-            if (r < KP && j < KP) {
-              Vs[j * LDV + r] -= oz_f2d(0.5f * sum[i][c]);
-              sm.Vf[j * LDS + r] -= 0.5f * sum[i][c];
-            }
-          }
-      }
-      ++ns;
-      __syncthreads();
-      // predicted residual after this step: quadratic term + FP32 rounding of the correction
-      if (mm * mm + 1.0e-6f * mm <= 2.0e-16f) {
-        ns_ok = true;
-        break;
-      }
-    }
-  } else {
-    __syncthreads();
-  }
-  const long long t_ns = clock64();
-  if (!ns_ok) {  // V is not J-unitary to FP64 accuracy after the step budget: FP64 pivot kernel
-    if (tid == 0) {
-      a.skip[pair] = 2;
-      atomicOr(err, JAC_DEVERR_HANDOVER);
-      st.rotations = total_rot;
-      st.inner_sweeps = (inner < max_inner) ? inner + 1 : max_inner;
-      st.ns_steps = ns;
-      st.cyc[0] = t_stats - t_start;
-      st.cyc[1] = t_chol - t_stats;
-      st.cyc[2] = t_inner - t_chol;
-      st.cyc[3] = t_ns - t_inner;
-      stats[pair] = st;
-    }
-    return 2;
-  }
-  // V_P = P V Pi: V_P[perm[r]][l] = V[r][lpos[l]]
-  if constexpr (!FUSED) {
-    double* out = a.vp + (size_t)pair * a.apld * a.apld;
-    for (int e = tid; e < KP * KP; e += NT) {
-      const int r = e % KP, l = e / KP;
-      double v = 0.0;
-      int row = r;
-      if (r < k && l < k) {
-        v = Vs[sm.lpos[l] * LDV + r];
-        row = sm.perm[r];
-      }
-      out[l * a.apld + row] = v;
-    }
-  }
   if (tid == 0) {
-    a.skip[pair] = FUSED ? 3 : 0;  // 3: updated by the fused step kernel itself
-    st.rotations = total_rot;
-    st.inner_sweeps = (inner < max_inner) ? inner + 1 : max_inner;
-    st.ns_steps = ns;
-    st.cyc[0] = t_stats - t_start;
-    st.cyc[1] = t_chol - t_stats;
-    st.cyc[2] = t_inner - t_chol;
-    st.cyc[3] = t_ns - t_inner;
-    stats[pair] = st;
+    sm.st.rotations = total_rot;
+    sm.st.inner_sweeps = (inner < max_inner) ? inner + 1 : max_inner;
+    sm.st.cyc[1] = t_chol - t_stats;
+    sm.st.cyc[2] = t_inner - t_chol;
+    sm.t_core = t_inner;
   }
   return 0;
 }
 
-// KM = 32: four CTAs per SM (shared memory allows four; the register cap keeps them resident, no
-// spills), which the batched solves of many small pivots need; KM = 64: one CTA per SM
-template <int KM, int LPP>
-__global__ void __launch_bounds__((KM / 2) * LPP, KM == 32 ? 4 : 1)
+// ---- phase 4: V = I + W, J-orthogonalized in FP64 ---------------------------------------------
+template <int KM>
+struct alignas(16) PivotOrth {
+  static constexpr int LDV = KM + 1;   // FP64 W stride
+  static constexpr int LDD = KM + 8;   // digit rows of W (halves): 16-byte aligned, ldmatrix conflict-free
+  static constexpr int LDS = KM + 4;   // rows of S = fp32(J M) (floats; 16-byte aligned)
+  static constexpr int NT = 4 * KM;    // threads: one warp per 8 columns
+  double V[KM * LDV];                  // W = V - I, FP64, column-major
+  float S[KM * LDS];                   // S[x LDS + j] = fp32((J M)[x][j])
+  int dexp[KM];                        // bound exponent of column c of W (digit products)
+  float red_f[NT / 32][2];
+  union {
+    __half D[OZ_T][KM][LDD];           // digits of W by column (digit products)
+    double M[KM * LDV];                // FP64 residual (FP64 mma products)
+  };
+};
+
+template <int KM>
+__device__ __forceinline__ float block_max_f(float v, PivotOrth<KM>& so, int slot) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  v = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));  // v >= 0
+  if (lane == 0) so.red_f[warp][slot] = v;
+  __syncthreads();
+  float r = 0.0f;
+#pragma unroll
+  for (int w = 0; w < PivotOrth<KM>::NT / 32; ++w) r = fmaxf(r, so.red_f[w][slot]);
+  __syncthreads();
+  return r;
+}
+
+// (float)(2^E (hi 2^28 + lo) + x + y) by integer operations, for digit products of at most 64 terms
+// (|hi| < 2^40, |lo| < 2^43): the terms are aligned to a common unit of 2^-53 of the largest possible
+// digit product or 2^-58 of x and y, so the result is as accurate as an FP64 sum of them.  (GB300
+// issues ~1.6 FP64 operations per clock per SM; the FP64 form took 7 per entry, ~9k clocks per
+// residual of a 64-column block.)
+__device__ __forceinline__ long long align_bits(double x, int ub) {  // x in units of 2^(ub - 1075), truncated
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((u >> 52) & 0x7ff);
+  unsigned long long m = ((u & ((1ull << 52) - 1)) | (e ? 1ull << 52 : 0ull)) << 6;
+  m >>= min((unsigned)(ub + 6 - max(e, 1)), 63u);
+  return (u >> 63) ? -(long long)m : (long long)m;
+}
+__device__ __forceinline__ float residual_sum(long long hi, long long lo, int E, double x, double y) {
+  const int ex = max(oz_bexp(x), 1), ey = max(oz_bexp(y), 1);
+  // units of 2^(ub - 1075): hi 2^28 + lo = (hi 2^20 + (lo >> 8)) 2^8, so its unit is 2^(E + 8)
+  const int ub = max(max(ex, ey) - 6, E + 8 + 1075);
+  const long long q = ((hi << 20) + (lo >> 8)) >> min((unsigned)(ub - (E + 8 + 1075)), 63u);
+  const long long s = q + align_bits(x, ub) + align_bits(y, ub);
+  const int sh = ub - 1075;  // s 2^sh, in two exact steps (FP32 range)
+  const int h = max(min(sh / 2, 120), -120), h2 = max(min(sh - h, 120), -120);
+  return ((float)s * __int_as_float((h + 127) << 23)) * __int_as_float((h2 + 127) << 23);
+}
+
+// J-orthogonality residual M = V^T J V - J = W^T J + J W + W^T J W from digit products (ozaki.cuh).
+// The linear terms are exact; W^T J W, of size |W|^2, runs on the digit path with the columns of W
+// (over the k rows) as scale groups and J_r applied to the A digits by their sign bit.  So M is
+// accurate to ~2^-53 |W|^2 + 2^-53 |W|, where the FP64 product V^T J V carries ~2^-53 |V|^2.
+// Writes S = fp32(J M) (zero outside k x k) and returns this thread's max |M_ij|.  Warp w prepares
+// columns 8w..8w+7.
+template <int KM>
+__device__ float oz_residual(PivotOrth<KM>& so, const int* jphys, int k, int KP) {
+  constexpr int NW = PivotOrth<KM>::NT / 32, LDV = PivotOrth<KM>::LDV, LDS = PivotOrth<KM>::LDS;
+  static_assert(NW * 8 == KM, "one warp per 8 columns");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
+  // ---- column bounds and digits; lane: rows 2 lane, 2 lane + 1 (KM = 32: the row lane)
+#pragma unroll
+  for (int cc = 0; cc < 8; ++cc) {
+    const int c = 8 * warp + cc;
+    if constexpr (KM == 64) {
+      const double x0 = so.V[c * LDV + 2 * lane], x1 = so.V[c * LDV + 2 * lane + 1];
+      const int ec = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(oz_bexp(x0), oz_bexp(x1)));
+      unsigned d[OZ_T];
+      oz_split2(oz_biased(x0, oz_bexp(x0) - ec), oz_biased(x1, oz_bexp(x1) - ec), d);
+#pragma unroll
+      for (int t = 0; t < OZ_T; ++t) *reinterpret_cast<unsigned*>(&so.D[t][c][2 * lane]) = d[t];
+      if (lane == 0) so.dexp[c] = ec;
+    } else {
+      const double x0 = so.V[c * LDV + lane];
+      const int ec = (int)__reduce_max_sync(0xffffffffu, (unsigned)oz_bexp(x0));
+      unsigned d[OZ_T];
+      oz_split2(oz_biased(x0, oz_bexp(x0) - ec), OZ_BIAS, d);
+#pragma unroll
+      for (int t = 0; t < OZ_T; ++t) so.D[t][c][lane] = __ushort_as_half((unsigned short)d[t]);
+      if (lane == 0) so.dexp[c] = ec;
+    }
+  }
+  __syncthreads();
+  // ---- upper 16 x 8 tiles of W^T J W, then M and S
+  float mloc = 0.0f;
+  const int ntj = KP / 8, ntiles = (KP / 16) * ntj;
+  int nth = 0;  // tiles on or above the diagonal, dealt to the warps in turn
+  for (int tile = 0; tile < ntiles; ++tile) {
+    const int ti = tile / ntj, tj = tile - ti * ntj;
+    if (8 * tj + 7 < 16 * ti) continue;
+    if (nth++ % NW != warp) continue;
+    float acc[OZ_T][4];
+#pragma unroll
+    for (int L = 0; L < OZ_T; ++L)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) acc[L][v] = 0.0f;
+    const int arow = 16 * ti + (lane & 7) + 8 * ((lane >> 3) & 1), akof = 8 * (lane >> 4);
+    const int brow = 8 * tj + (lane & 7), bkof = 8 * ((lane >> 3) & 1);
+    for (int kk = 0; kk < KP; kk += 16) {
+      const int r0 = kk + 2 * t4;
+      const unsigned slo = (jphys[r0] < 0 ? 0x8000u : 0u) | (jphys[r0 + 1] < 0 ? 0x80000000u : 0u);
+      const unsigned shi = (jphys[r0 + 8] < 0 ? 0x8000u : 0u) | (jphys[r0 + 9] < 0 ? 0x80000000u : 0u);
+      unsigned fa[OZ_T][4], fb[OZ_T][2];
+#pragma unroll
+      for (int t = 0; t < OZ_T; ++t) {
+        oz_ldsm4(fa[t], &so.D[t][arow][kk + akof]);
+        fa[t][0] ^= slo;
+        fa[t][1] ^= slo;
+        fa[t][2] ^= shi;
+        fa[t][3] ^= shi;
+        oz_ldsm2(fb[t][0], fb[t][1], &so.D[t][brow][kk + bkof]);
+      }
+      oz_levels(acc, fa, fb);
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int x = 16 * ti + g + 8 * (v >> 1), j = 8 * tj + 2 * t4 + (v & 1);
+      if (j < x) continue;  // (x, j), j >= x, covers the block; (j, x) is its mirror
+      float sxj = 0.0f, sjx = 0.0f;
+      if (x < k && j < k) {
+        const bool nx = jphys[x] < 0, nj = jphys[j] < 0;
+        int q[OZ_T];
+#pragma unroll
+        for (int L = 0; L < OZ_T; ++L) q[L] = f32_small_int(acc[L][v]);
+        const long long hi = (long long)(q[0] * 128 + q[1]) * 16384 + (q[2] * 128 + q[3]);
+        const long long lo = (long long)(q[4] * 128 + q[5]) * 16384 + (q[6] * 128 + q[7]);
+        // M_xj = (W^T J W)_xj + j_j W[j][x] + j_x W[x][j]
+        const float f = residual_sum(hi, lo, so.dexp[x] + so.dexp[j] - 2056 - 49, oz_neg_if(so.V[x * LDV + j], nj),
+                                     oz_neg_if(so.V[j * LDV + x], nx));
+        mloc = fmaxf(mloc, fabsf(f));
+        sxj = nx ? -f : f;  // (J M)[x][j]
+        sjx = nj ? -f : f;  // (J M)[j][x]
+      }
+      so.S[x * LDS + j] = sxj;
+      so.S[j * LDS + x] = sjx;
+    }
+  }
+  return mloc;
+}
+
+// Phase 4 of one pair, run by all 4 KM threads of a CTA on W (Wf, column c at c LDW, k valid columns):
+// true (uniform) when V is J-unitary to FP64 accuracy, with W in so.V.
+template <int KM>
+__device__ __forceinline__ bool pivot_orth(PivotOrth<KM>& so, float* Wf, const int* jphys, int k, int oz, int& ns) {
+  using SO = PivotOrth<KM>;
+  constexpr int NT = SO::NT, NW = NT / 32, LDV = SO::LDV, LDS = SO::LDS, LDW = PivotDim<KM>::LDW;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int KP = (k + 15) & ~15;
+  float wm = 0.0f;
+#pragma unroll
+  for (int u = 0; u < KM * KM / NT; ++u) {
+    const int e = tid + u * NT, r = e % KM, c = e / KM;
+    const bool in = r < k && c < k;
+    const float w = in ? Wf[c * LDW + r] : 0.0f;
+    so.V[c * LDV + r] = oz_f2d(w);  // integer conversion: FP64 instructions are scarce on GB300
+    if (!in) Wf[c * LDW + r] = 0.0f;
+    wm = fmaxf(wm, fabsf(w));
+  }
+  wm = block_max_f<KM>(wm, so, 1);  // includes the barrier after the loop
+  const bool small_w = wm <= 9.5367431640625e-7f;  // 2^-20
+  // products of the FP32 columns: thread (rg, cg) takes a 4 x CB block, rows 4 rg.. , columns cg + CGN c
+  constexpr int RG = KM / 4, CGN = NT / RG, CB = KM / CGN;
+  static_assert(RG * CGN == NT && CGN * CB == KM, "correction blocking");
+  const int rg = tid % RG, cg = tid / RG;
+  ns = 0;
+  for (int it = 0; it < 3; ++it) {
+    // residual M = V^T J V - J, J = diag(jphys) on rows and columns
+    float mloc = 0.0f;
+    if (it == 0 && small_w) {
+      // M = W^T J + J W + W^T J W.  The linear part is exact in FP32 when it cancels (Sterbenz)
+      // and rounds relative to itself otherwise; the quadratic part is at most k 2^-40 and
+      // carries FP32 relative error.  Stored as fp32(J M) directly.
+      float quad[4][CB];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < CB; ++c) quad[i][c] = 0.0f;
+      for (int r = 0; r < k; ++r) {
+        float xv[4], jv[CB];
+        const float sg = (float)jphys[r];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) xv[i] = Wf[(4 * rg + i) * LDW + r] * sg;
+#pragma unroll
+        for (int c = 0; c < CB; ++c) jv[c] = Wf[(cg + CGN * c) * LDW + r];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int c = 0; c < CB; ++c) quad[i][c] = fmaf(xv[i], jv[c], quad[i][c]);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < CB; ++c) {
+          const int x = 4 * rg + i, j = cg + CGN * c;
+          float mv = 0.0f;
+          if (x < k && j < k) {
+            const float jx = (float)jphys[x], jj = (float)jphys[j];
+            mv = (Wf[x * LDW + j] * jj + jx * Wf[j * LDW + x]) + quad[i][c];
+            so.S[x * LDS + j] = jx * mv;  // (J M)[x][j]
+          } else {
+            so.S[x * LDS + j] = 0.0f;
+          }
+          mloc = fmaxf(mloc, fabsf(mv));
+        }
+    } else if (oz) {
+      mloc = oz_residual<KM>(so, jphys, k, KP);
+    } else {
+      // FP64 mma, upper tiles (8 tj + 7 >= 16 ti) and the mirror of the strict lower part
+      const int g = lane >> 2, t = lane & 3;
+      const int ntj = KP / 8, ntiles = (KP / 16) * ntj;
+      for (int tile = warp; tile < ntiles; tile += NW) {
+        const int ti = tile / ntj, tj = tile % ntj;
+        if (8 * tj + 7 < 16 * ti) continue;
+        double c4[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int kq = 0; kq < KP; kq += 16) {
+          double av[8], bv[4];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) av[u] = so.V[(16 * ti + g + 8 * (u & 1)) * LDV + kq + 4 * t + (u >> 1)];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int r = kq + 4 * t + u;
+            bv[u] = oz_neg_if(so.V[(8 * tj + g) * LDV + r], jphys[r] < 0);
+          }
+          dmma16816(c4, av, bv);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = 16 * ti + g + 8 * (u >> 1), j = 8 * tj + 2 * t + (u & 1);
+          if (j < i) continue;  // written once, from the tile holding (j, i) ... (i, j), j >= i
+          const double v = c4[u] + (oz_neg_if(so.V[i * LDV + j], jphys[j] < 0) + oz_neg_if(so.V[j * LDV + i], jphys[i] < 0));
+          so.M[j * LDV + i] = v;
+          so.M[i * LDV + j] = v;
+        }
+      }
+      __syncthreads();
+      for (int e = tid; e < KP * KP; e += NT) {
+        const int x = e % KP, j = e / KP;
+        const double mv = (x < k && j < k) ? so.M[j * LDV + x] : 0.0;
+        mloc = fmaxf(mloc, (float)fabs(mv));
+        so.S[x * LDS + j] = (float)oz_neg_if(mv, jphys[x] < 0);
+      }
+    }
+    const float mm = block_max_f<KM>(mloc, so, 0);
+    if (mm <= 4.0e-16f) return true;
+    // V <- V - V (J M) / 2 = V - (S + W S) / 2: the correction is O(|M|), formed in FP32 from the
+    // FP32 columns; the FP32 columns follow in FP32
+    f2 sum[2][CB];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int c = 0; c < CB; ++c) {
+        const int r = 4 * rg + 2 * i, j = cg + CGN * c;
+        sum[i][c] = f2_make(so.S[r * LDS + j], so.S[(r + 1) * LDS + j]);
+      }
+    for (int x = 0; x < k; ++x) {
+      const ulonglong2 wv = *reinterpret_cast<const ulonglong2*>(&Wf[x * LDW + 4 * rg]);
+#pragma unroll
+      for (int c = 0; c < CB; ++c) {
+        const float sv = so.S[x * LDS + cg + CGN * c];
+        const f2 s2 = f2_make(sv, sv);
+        sum[0][c] = f2_fma(wv.x, s2, sum[0][c]);
+        sum[1][c] = f2_fma(wv.y, s2, sum[1][c]);
+      }
+    }
+    __syncthreads();  // every read of Wf done
+#pragma unroll
+    for (int c = 0; c < CB; ++c) {
+      const int j = cg + CGN * c;
+      if (j >= k) continue;
+      const float h[4] = {f2_lo(sum[0][c]), f2_hi(sum[0][c]), f2_lo(sum[1][c]), f2_hi(sum[1][c])};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = 4 * rg + i;
+        if (r < k) {
+          so.V[j * LDV + r] -= oz_f2d(0.5f * h[i]);
+          Wf[j * LDW + r] -= 0.5f * h[i];
+        }
+      }
+    }
+    ++ns;
+    __syncthreads();
+    // predicted residual after this step: quadratic term + FP32 rounding of the correction
+    if (mm * mm + 1.0e-6f * mm <= 2.0e-16f) return true;
+  }
+  return false;
+}
+
+// What the core leaves for the other kernels of the step when the pivot's phases run apart: in the
+// pair's V_P buffer (KM x KM doubles), W in FP32, then the orders and signs.
+template <int KM>
+struct PivotHandoff {
+  float W[KM * PivotDim<KM>::LDW];
+  int perm[KM], linv[KM], jphys[KM];
+  static_assert((KM * PivotDim<KM>::LDW + 3 * KM) * 4 <= KM * KM * 8, "fits the V_P buffer");
+};
+
+// V_P = P V Pi: V_P[perm[r]][linv[c]] = V[r][c], FP64
+template <int KM, class F>
+__device__ __forceinline__ void write_vp(const JacProb& a, int pair, int k, const int* perm, const int* linv, int nt, F v) {
+  double* out = a.vp + (size_t)pair * a.apld * a.apld;
+  for (int e = threadIdx.x; e < KM * KM; e += nt) {
+    const int r = e % KM, c = e / KM;
+    if (r < k && c < k) out[(size_t)linv[c] * a.apld + perm[r]] = v(r, c);
+  }
+}
+
+template <int KM>
+struct PivotSmem {  // ORTH kernels; the core alone needs st, work and Wf
+  PivotState<KM> st;
+  float Wf[KM * PivotDim<KM>::LDW];
+  union {
+    PivotWork<KM> work;
+    PivotOrth<KM> orth;
+  };
+};
+template <int KM>
+constexpr size_t core_smem_bytes() {
+  return offsetof(PivotSmem<KM>, work) + sizeof(PivotWork<KM>);
+}
+
+template <int KM>
+__device__ __forceinline__ bool pivot_guard(const JacProb& a, int s, int pair) {
+  if (!a.active || s >= a.nsteps || pair >= a.counts[s]) return false;
+  return !(a.cached && a.cached[pair]);  // cached: skip set, statistics kept (pair_cache.cu)
+}
+
+// Modes of the pivot kernel.  PV_FULL: phases 1-4 in one CTA (FP64 sweeps).  PV_CORE: phases 1-3,
+// V_P in FP64 storage from the FP32 transform (FP32 sweeps).  PV_SPLIT: phases 1-3, W handed to
+// k_pivot_orth: the core needs a quarter of the shared memory of phase 4, so four pivots run on an
+// SM while phase 4 takes the SM for a short time only (many pivots per step).  4000 problems of
+// orders 8..128, all pivots of a sweep step: 2.1 ms, against 4.1 ms with one 212 KB CTA per SM.
+enum { PV_FULL = 0, PV_CORE = 1, PV_SPLIT = 2 };
+
+template <int KM, int MODE>
+__global__ void __launch_bounds__(MODE == PV_FULL ? 4 * KM : 2 * KM, MODE == PV_FULL ? (KM == 32 ? 4 : 1) : (KM == 32 ? 8 : 4))
     k_pivot(const JacProb* __restrict__ probs, int s, PivotParams pp) {
   extern __shared__ __align__(16) unsigned char pv_raw[];
-  PivotSmem<KM, LPP>& sm = *reinterpret_cast<PivotSmem<KM, LPP>*>(pv_raw);
+  PivotSmem<KM>& sm = *reinterpret_cast<PivotSmem<KM>*>(pv_raw);
   const JacProb& a = probs[blockIdx.y];
-  const int pair = blockIdx.x;
-  if (!a.active || s >= a.nsteps || pair >= a.counts[s]) return;
-  if (a.cached && a.cached[pair]) return;  // skip set, statistics kept (pair_cache.cu)
-  pivot_block<KM, LPP, false>(sm, a, s, pair, pp);
+  const int pair = blockIdx.x, tid = threadIdx.x;
+  if (!pivot_guard<KM>(a, s, pair)) return;
+  PairStat* stats = a.stats + (size_t)s * a.half;
+  if constexpr (MODE != PV_FULL) {
+    if (pivot_core<KM, false>(sm.st, sm.work, nullptr, sm.Wf, a, s, pair, pp) != 0) return;
+    __syncthreads();
+    const int k = sm.st.k;
+    if constexpr (MODE == PV_CORE) {
+      write_vp<KM>(a, pair, k, sm.st.perm, sm.st.linv, 2 * KM, [&](int r, int c) {
+        const float w = sm.Wf[c * PivotDim<KM>::LDW + r];
+        return r == c ? oz_f2d(w) + 1.0 : oz_f2d(w);
+      });
+    } else {
+      PivotHandoff<KM>& h = *reinterpret_cast<PivotHandoff<KM>*>(a.vp + (size_t)pair * a.apld * a.apld);
+      for (int e = tid; e < k * PivotDim<KM>::LDW / 4; e += 2 * KM)
+        reinterpret_cast<float4*>(h.W)[e] = reinterpret_cast<const float4*>(sm.Wf)[e];
+      if (tid < KM) {
+        h.perm[tid] = sm.st.perm[tid];
+        h.linv[tid] = sm.st.linv[tid];
+        h.jphys[tid] = sm.st.jphys[tid];
+      }
+    }
+    if (tid == 0) {
+      a.skip[pair] = 0;
+      stats[pair] = sm.st.st;
+    }
+  } else {
+    if (tid < PivotDim<KM>::NTC) {
+      const int code = pivot_core<KM, false>(sm.st, sm.work, nullptr, sm.Wf, a, s, pair, pp);
+      if (tid == 0) sm.st.code = code;
+    }
+    __syncthreads();
+    if (sm.st.code != 0) return;
+    const int k = sm.st.k;
+    int ns = 0;
+    const bool ok = pivot_orth<KM>(sm.orth, sm.Wf, sm.st.jphys, k, pp.oz, ns);
+    if (ok)
+      write_vp<KM>(a, pair, k, sm.st.perm, sm.st.linv, 4 * KM, [&](int r, int c) {
+        const double w = sm.orth.V[c * PivotOrth<KM>::LDV + r];
+        return r == c ? w + 1.0 : w;
+      });
+    if (tid == 0) {
+      // not J-unitary to FP64 accuracy after the step budget: FP64 pivot kernel
+      a.skip[pair] = ok ? 0 : 2;
+      if (!ok) atomicOr(a.pflags, JAC_DEVERR_HANDOVER);
+      sm.st.st.ns_steps = ns;
+      sm.st.st.cyc[3] = clock64() - sm.st.t_core;
+      stats[pair] = sm.st.st;
+    }
+  }
+}
+
+// Phase 4 of the pairs whose core ran in k_pivot<KM, PV_SPLIT>.  Grid and guards as the core.
+template <int KM>
+struct OrthSmem {
+  float Wf[KM * PivotDim<KM>::LDW];
+  int perm[KM], linv[KM], jphys[KM];
+  PivotOrth<KM> orth;
+};
+template <int KM>
+__global__ void __launch_bounds__(4 * KM, KM == 32 ? 4 : 1)
+    k_pivot_orth(const JacProb* __restrict__ probs, int s, PivotParams pp) {
+  extern __shared__ __align__(16) unsigned char pv_raw[];
+  OrthSmem<KM>& sm = *reinterpret_cast<OrthSmem<KM>*>(pv_raw);
+  const JacProb& a = probs[blockIdx.y];
+  const int pair = blockIdx.x, tid = threadIdx.x;
+  if (!pivot_guard<KM>(a, s, pair) || a.skip[pair] != 0) return;
+  const long long t0 = clock64();
+  const int* sp = a.pairs + (size_t)s * a.half * 2;
+  const int p = sp[2 * pair], q = sp[2 * pair + 1];
+  const int k = a.boff[p + 1] - a.boff[p] + a.boff[q + 1] - a.boff[q];
+  const PivotHandoff<KM>& h = *reinterpret_cast<const PivotHandoff<KM>*>(a.vp + (size_t)pair * a.apld * a.apld);
+  for (int e = tid; e < k * PivotDim<KM>::LDW / 4; e += 4 * KM)
+    reinterpret_cast<float4*>(sm.Wf)[e] = reinterpret_cast<const float4*>(h.W)[e];
+  if (tid < KM) {
+    sm.perm[tid] = h.perm[tid];
+    sm.linv[tid] = h.linv[tid];
+    sm.jphys[tid] = h.jphys[tid];
+  }
+  __syncthreads();  // the hand-over is read: V_P may take its place
+  int ns = 0;
+  const bool ok = pivot_orth<KM>(sm.orth, sm.Wf, sm.jphys, k, pp.oz, ns);
+  if (ok)
+    write_vp<KM>(a, pair, k, sm.perm, sm.linv, 4 * KM, [&](int r, int c) {
+      const double w = sm.orth.V[c * PivotOrth<KM>::LDV + r];
+      return r == c ? w + 1.0 : w;
+    });
+  if (tid == 0) {
+    if (!ok) {
+      a.skip[pair] = 2;
+      atomicOr(a.pflags, JAC_DEVERR_HANDOVER);
+    }
+    PairStat& st = a.stats[(size_t)s * a.half + pair];
+    st.ns_steps = ns;
+    st.cyc[3] = clock64() - t0;
+  }
 }
 
 // ---- the fused step kernel ---------------------------------------------------------------------
 // One step of the FP32 sweeps for one pair in one CTA: the Gram block, the pivot and the block
 // update, with X_P = [G_p G_q] read from global memory once and written once.  The m rows of X_P
-// stay in shared memory from the Gram to the update, in the pivot's digit-product region (the
-// FP32 sweeps never form the FP64 J-orthogonality residual); the rows of V go through the column
-// mailboxes in chunks of 64.  Used when every problem of the launch has m <= FusedLayout::MF.
-template <int KM, int LPP>
+// stay in shared memory from the Gram to the update; the rows of V go through the pivot's work area
+// in chunks of 64.  Used when every problem of the launch has m <= fused_step_max_rows(KM).  The
+// launch asks for the shared memory of its largest m, so several CTAs share an SM.
+template <int KM>
 struct FusedLayout {
-  using SM = PivotSmem<KM, LPP>;
   static constexpr int LDX = KM + 4;  // staged rows of X_P (floats; 16-byte aligned rows)
   static constexpr int LDB = KM + 4;  // V_P in FP32, row c = input column
-  static constexpr int REGION = (int)((sizeof(SM::M) > sizeof(SM::D) ? sizeof(SM::M) : sizeof(SM::D)) / 4);
-  static constexpr int MF = ((REGION - KM * LDB) / LDX) / 32 * 32;  // largest m
-  static_assert(MF >= 32, "staging region");
-  static_assert(2 * SM::P2 * SM::MBS >= 64 * LDX, "a 64-row chunk of V fits in the mailboxes");
+  static constexpr int MF = KM == 32 ? 96 : 192;  // largest m
+  // Bs, then the chunk of V, over the pivot's work area
+  static constexpr int WORK = (int)sizeof(PivotWork<KM>) / 4 > KM * LDB + 64 * LDX ? (int)sizeof(PivotWork<KM>) / 4
+                                                                                   : KM * LDB + 64 * LDX;
+  struct Smem {
+    PivotState<KM> st;
+    float Wf[KM * PivotDim<KM>::LDW];  // A_P in FP32, then W
+    alignas(16) float work[WORK];
+    alignas(16) float X[1];            // [r][c], m rows
+  };
+  static constexpr size_t bytes(int m) { return offsetof(Smem, X) + (size_t)m * LDX * 4; }
 };
 
-template <int KM, int LPP>
-__global__ void __launch_bounds__((KM / 2) * LPP, KM == 32 ? 3 : 1)  // KM = 32: no spills at 3 per SM
-    k_step_fused(const JacProb* __restrict__ probs, int s, PivotParams pp) {
-  using SM = PivotSmem<KM, LPP>;
-  using FL = FusedLayout<KM, LPP>;
-  constexpr int NT = SM::NT, LDS = SM::LDS, LDV = SM::LDV, LDX = FL::LDX, LDB = FL::LDB, MF = FL::MF;
+template <int KM>
+__global__ void __launch_bounds__(4 * KM, KM == 32 ? 4 : 2)
+    k_step_fused(const JacProb* __restrict__ probs, int s, PivotParams pp, int mmax) {
+  using FL = FusedLayout<KM>;
+  constexpr int NT = 4 * KM, LDX = FL::LDX, LDB = FL::LDB, LDW = PivotDim<KM>::LDW;
   constexpr int CT = KM / 4;  // 4-column groups
-  static_assert(NT % CT == 0 && NT / CT == 16, "16 row groups");
+  static_assert(NT / CT == 16, "16 row groups");
   extern __shared__ __align__(16) unsigned char pv_raw[];
-  SM& sm = *reinterpret_cast<SM*>(pv_raw);
+  typename FL::Smem& sm = *reinterpret_cast<typename FL::Smem*>(pv_raw);
   const JacProb& a = probs[blockIdx.y];
   const int pair = blockIdx.x;
-  if (!a.active || s >= a.nsteps || pair >= a.counts[s]) return;
-  if (a.cached && a.cached[pair]) return;  // skip set, statistics kept (pair_cache.cu)
+  if (!pivot_guard<KM>(a, s, pair)) return;
   const int tid = threadIdx.x, tx = tid % CT, ty = tid / CT;
   const int* sp = a.pairs + (size_t)s * a.half * 2;
   const int p = sp[2 * pair], q = sp[2 * pair + 1];
   const int op = a.boff[p], wp = a.boff[p + 1] - op, oq = a.boff[q], wq = a.boff[q + 1] - oq;
   const int k = wp + wq, m = a.mp;
-  // the driver launches this kernel for the FP32 sweeps (no FP64 residual: the staging region is
-  // free) within these bounds; anything else is reported, never trapped
-  if (k > KM || m > MF || pp.ns_mode) {
+  // the driver launches this kernel for the FP32 sweeps within these bounds; anything else is
+  // reported, never trapped
+  if (k > KM || m > mmax || pp.ns_mode) {
     if (tid == 0) {
       atomicOr(a.pflags, JAC_DEVERR_INNER_LIMIT);
       a.skip[pair] = 1;
@@ -1014,24 +1236,27 @@ __global__ void __launch_bounds__((KM / 2) * LPP, KM == 32 ? 3 : 1)  // KM = 32:
     return;
   }
   auto pcol = [&](int c) { return c < wp ? op + c : oq + (c - wp); };
-  float* Xs = reinterpret_cast<float*>(&sm.M[0]);  // [r][c], m rows
-  float* Bs = Xs + MF * LDX;                       // [c][j]
-  float* Vst = &sm.mb[0][0];                       // 64-row chunk of V, [r][c]
+  float* Xs = sm.X;                  // [r][c], m rows
+  float* Bs = sm.work;               // [c][j]
+  float* Vst = sm.work + KM * LDB;   // 64-row chunk of V, [r][c]
 
-  // ---- 0. X_P into shared memory; A_P = X_P^T X_P in FP32 (FP64 storage for the pivot)
+  // ---- 0. X_P into shared memory (zero columns beyond k); A_P = X_P^T X_P in FP32
   {
-    constexpr int NB = 16;  // loads in flight per thread
-    for (int e0 = 0; e0 < k * m; e0 += NT * NB) {
-      float v[NB];
+    const int nw = NT / 32, warp = tid >> 5, lane = tid & 31;
+    for (int c = warp; c < KM; c += nw) {  // a warp per column, consecutive lanes consecutive rows
+      const float* col = a.G32 + (size_t)pcol(c < k ? c : 0) * a.mp;
+      for (int rr = 0; rr < m; rr += 32 * 6) {
+        float v[6];
 #pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        const int e = e0 + u * NT + tid;  // consecutive threads: consecutive rows of a column
-        v[u] = (e < k * m) ? __ldg(a.G32 + (size_t)pcol(e / m) * a.mp + e % m) : 0.0f;
-      }
+        for (int u = 0; u < 6; ++u) {
+          const int r = rr + lane + 32 * u;
+          v[u] = (c < k && r < m) ? __ldg(col + r) : 0.0f;
+        }
 #pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        const int e = e0 + u * NT + tid;
-        if (e < k * m) Xs[(e % m) * LDX + e / m] = v[u];
+        for (int u = 0; u < 6; ++u) {
+          const int r = rr + lane + 32 * u;
+          if (r < m) Xs[r * LDX + c] = v[u];
+        }
       }
     }
   }
@@ -1040,73 +1265,83 @@ __global__ void __launch_bounds__((KM / 2) * LPP, KM == 32 ? 3 : 1)  // KM = 32:
     // thread (ty, tx): rows RPT ty .. RPT ty + RPT - 1 and columns 4 tx .. 4 tx + 3 of A_P; the
     // entries (i, j) and (j, i) take the same products in the same order (exactly symmetric)
     constexpr int RPT = KM / 16;
-    float acc[RPT][4];
+    f2 acc[RPT][2];
 #pragma unroll
-    for (int u = 0; u < RPT; ++u)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) acc[u][v] = 0.0f;
+    for (int u = 0; u < RPT; ++u) acc[u][0] = acc[u][1] = f2_make(0.0f, 0.0f);
+#pragma unroll 4
     for (int r = 0; r < m; ++r) {
       const float* xr = Xs + r * LDX;
-      const float4 xj = *reinterpret_cast<const float4*>(xr + 4 * tx);
-      const float vj[4] = {xj.x, xj.y, xj.z, xj.w};
+      const ulonglong2 xj = *reinterpret_cast<const ulonglong2*>(xr + 4 * tx);
 #pragma unroll
       for (int u = 0; u < RPT; ++u) {
         const float xi = xr[RPT * ty + u];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(xi, vj[v], acc[u][v]);
+        const f2 x2 = f2_make(xi, xi);
+        acc[u][0] = f2_fma(x2, xj.x, acc[u][0]);
+        acc[u][1] = f2_fma(x2, xj.y, acc[u][1]);
       }
     }
 #pragma unroll
-    for (int u = 0; u < RPT; ++u)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const int i = RPT * ty + u, j = 4 * tx + v;
-        if (i < k && j < k) sm.V[j * LDV + i] = oz_f2d(acc[u][v]);
-      }
+    for (int u = 0; u < RPT; ++u) {
+      const int i = RPT * ty + u;
+      sm.Wf[(4 * tx) * LDW + i] = f2_lo(acc[u][0]);
+      sm.Wf[(4 * tx + 1) * LDW + i] = f2_hi(acc[u][0]);
+      sm.Wf[(4 * tx + 2) * LDW + i] = f2_lo(acc[u][1]);
+      sm.Wf[(4 * tx + 3) * LDW + i] = f2_hi(acc[u][1]);
+    }
   }
-  // (pivot_block's first barrier publishes A_P)
+  __syncthreads();
 
-  // ---- 1.-4. the pivot
-  const int pr = pivot_block<KM, LPP, true>(sm, a, s, pair, pp);  // uniform
+  // ---- 1.-3. the pivot
+  if (tid < PivotDim<KM>::NTC) {
+    const int code = pivot_core<KM, true>(sm.st, *reinterpret_cast<PivotWork<KM>*>(sm.work), sm.Wf, sm.Wf, a, s, pair, pp);
+    if (tid == 0) sm.st.code = code;
+  }
+  __syncthreads();
+  const int pr = sm.st.code;  // uniform
   if (pr == 2) {
     // handed over: the FP64 pivot kernel reads A_P from the Gram output, as after the Gram kernel
     double* A = a.Ap + (size_t)pair * a.apld * a.apld;
-    for (int e = tid; e < k * k; e += NT) A[(e / k) * a.apld + e % k] = sm.V[(e / k) * LDV + e % k];
+    for (int e = tid; e < k * k; e += NT) A[(e / k) * a.apld + e % k] = oz_f2d(sm.Wf[(e / k) * LDW + e % k]);
   }
   if (pr != 0) return;
 
-  // ---- 5. [X_P; V rows] <- [X_P; V rows] V_P in FP32, V_P[perm[r]][l] = V[r][lpos[l]]
-  __syncthreads();
-  for (int e = tid; e < k * k; e += NT) {
-    const int r = e % k, l = e / k;
-    Bs[sm.perm[r] * LDB + l] = sm.Vf[sm.lpos[l] * LDS + r];
+  // ---- 4. [X_P; V rows] <- [X_P; V rows] V_P in FP32, V_P[perm[r]][linv[c]] = V[r][c]
+  for (int e = tid; e < KM * KM; e += NT) {
+    const int r = e % KM, c = e / KM;
+    if (r < k && c < k) Bs[sm.st.perm[r] * LDB + sm.st.linv[c]] = sm.Wf[c * LDW + r] + (r == c ? 1.0f : 0.0f);
+  }
+  if (tid == 0) {
+    a.skip[pair] = 3;  // updated by this kernel itself
+    a.stats[(size_t)s * a.half + pair] = sm.st.st;
   }
   __syncthreads();
   // thread (ty, tx): rows 4 ty .. 4 ty + 3 of a 64-row chunk, columns 4 tx .. 4 tx + 3
   auto update_chunk = [&](const float* X, int rows, float* dst, int ld, int r0) {
-    float acc[4][4];
+    f2 acc[4][2];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < 4; ++u) acc[u][0] = acc[u][1] = f2_make(0.0f, 0.0f);
+    if (4 * ty < rows) {
+#pragma unroll 4
+      for (int c = 0; c < k; ++c) {
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(Bs + c * LDB + 4 * tx);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) acc[u][v] = 0.0f;
-    for (int c = 0; c < k; ++c) {
-      const float4 b = *reinterpret_cast<const float4*>(Bs + c * LDB + 4 * tx);
-      const float bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float x = X[(4 * ty + u) * LDX + c];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(x, bv[v], acc[u][v]);
+        for (int u = 0; u < 4; ++u) {
+          const float x = X[(4 * ty + u) * LDX + c];
+          const f2 x2 = f2_make(x, x);
+          acc[u][0] = f2_fma(x2, b.x, acc[u][0]);
+          acc[u][1] = f2_fma(x2, b.y, acc[u][1]);
+        }
       }
-    }
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int j = 4 * tx + v;
-      if (j >= k) continue;
-      float* col = dst + (size_t)pcol(j) * ld + r0;
+      for (int v = 0; v < 4; ++v) {
+        const int j = 4 * tx + v;
+        if (j >= k) continue;
+        float* col = dst + (size_t)pcol(j) * ld + r0 + 4 * ty;  // rows are a multiple of 16
+        float o[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (4 * ty + u < rows) col[4 * ty + u] = acc[u][v];
+        for (int u = 0; u < 4; ++u) o[u] = (v & 1) ? f2_hi(acc[u][v >> 1]) : f2_lo(acc[u][v >> 1]);
+        *reinterpret_cast<float4*>(col) = make_float4(o[0], o[1], o[2], o[3]);
+      }
     }
   };
   for (int r0 = 0; r0 < m; r0 += 64) update_chunk(Xs + r0 * LDX, min(64, m - r0), a.G32, a.mp, r0);
@@ -1132,52 +1367,57 @@ __global__ void __launch_bounds__((KM / 2) * LPP, KM == 32 ? 3 : 1)  // KM = 32:
   }
 }
 
-// Lanes per pair slot of each pivot capacity: KM = 64 -> 8 lanes x 8 rows, 256 threads;
-// KM = 32 -> 8 lanes x 4 rows, 128 threads.
-constexpr int kLpp64 = 8, kLpp32 = 8;
-static_assert(sizeof(PivotSmem<64, kLpp64>) <= 232448, "pivot shared memory above the 227 KB per-CTA limit");
+int fused_step_max_rows(int km) { return km == 32 ? FusedLayout<32>::MF : FusedLayout<64>::MF; }
 
-int fused_step_max_rows(int km) {
-  return km == 32 ? FusedLayout<32, kLpp32>::MF : FusedLayout<64, kLpp64>::MF;
+static_assert(sizeof(PivotSmem<64>) <= 232448, "pivot shared memory above the 227 KB per-CTA limit");
+
+// Host side of the instantiations (a kernel template is launched from its own translation unit).
+template <int KM>
+static bool set_attributes() {
+  auto set = [](auto kern, size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+  };
+  bool ok = set(k_pivot<KM, PV_FULL>, sizeof(PivotSmem<KM>));
+  ok &= set(k_pivot<KM, PV_CORE>, core_smem_bytes<KM>());
+  ok &= set(k_pivot<KM, PV_SPLIT>, core_smem_bytes<KM>());
+  ok &= set(k_pivot_orth<KM>, sizeof(OrthSmem<KM>));
+  ok &= set(k_step_fused<KM>, FusedLayout<KM>::bytes(FusedLayout<KM>::MF));
+  return ok;
+}
+int pivot_set_attributes() { return set_attributes<32>() && set_attributes<64>() ? 0 : 1; }
+
+// Grid (max_half, nprob): one CTA per pivot block.  Returns the number of kernels launched.
+// FP64 sweeps with more pivots in the step than SMs run the core and phase 4 as two kernels.
+constexpr int kSplitPivots = 152;
+
+template <int KM>
+static int launch_pivot(int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s, const PivotParams& pp) {
+  const dim3 grid(max_half, nprob);
+  if (!pp.ns_mode) {
+    k_pivot<KM, PV_CORE><<<grid, 2 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
+    return 1;
+  }
+  if ((long long)max_half * nprob <= kSplitPivots) {
+    k_pivot<KM, PV_FULL><<<grid, 4 * KM, sizeof(PivotSmem<KM>), st>>>(probs, s, pp);
+    return 1;
+  }
+  k_pivot<KM, PV_SPLIT><<<grid, 2 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
+  k_pivot_orth<KM><<<grid, 4 * KM, sizeof(OrthSmem<KM>), st>>>(probs, s, pp);
+  return 2;
+}
+int pivot_launch(int km, int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s, const PivotParams& pp) {
+  return km == 32 ? launch_pivot<32>(max_half, nprob, st, probs, s, pp)
+                  : launch_pivot<64>(max_half, nprob, st, probs, s, pp);
 }
 
-size_t pivot_smem_bytes(int km) {
-  return km == 32 ? sizeof(PivotSmem<32, kLpp32>) : sizeof(PivotSmem<64, kLpp64>);
-}
-
-// Host side of the two instantiations (a kernel template is launched from its own translation unit).
-int pivot_set_attributes() {
-  bool ok = cudaFuncSetAttribute(k_pivot<32, kLpp32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(PivotSmem<32, kLpp32>)) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_pivot<64, kLpp64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(PivotSmem<64, kLpp64>)) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_step_fused<32, kLpp32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(PivotSmem<32, kLpp32>)) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_step_fused<64, kLpp64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(PivotSmem<64, kLpp64>)) == cudaSuccess;
-  return ok ? 0 : 1;
-}
-
-// Grid (max_half, nprob): one CTA per pivot block.
-void pivot_launch(int km, int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s,
-                  const PivotParams& pp) {
-  if (km == 32)
-    k_pivot<32, kLpp32><<<dim3(max_half, nprob), PivotSmem<32, kLpp32>::NT, sizeof(PivotSmem<32, kLpp32>), st>>>(
-        probs, s, pp);
-  else
-    k_pivot<64, kLpp64><<<dim3(max_half, nprob), PivotSmem<64, kLpp64>::NT, sizeof(PivotSmem<64, kLpp64>), st>>>(
-        probs, s, pp);
-}
-
-// Grid (max_half, nprob): one CTA per pair, the whole FP32 step (fused_step_max_rows bounds m).
+// Grid (max_half, nprob): one CTA per pair, the whole FP32 step; every problem has m <= mmax <=
+// fused_step_max_rows(km) padded rows.
 void fused_step_launch(int km, int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s,
-                       const PivotParams& pp) {
+                       const PivotParams& pp, int mmax) {
   if (km == 32)
-    k_step_fused<32, kLpp32><<<dim3(max_half, nprob), PivotSmem<32, kLpp32>::NT, sizeof(PivotSmem<32, kLpp32>),
-                               st>>>(probs, s, pp);
+    k_step_fused<32><<<dim3(max_half, nprob), 4 * 32, FusedLayout<32>::bytes(mmax), st>>>(probs, s, pp, mmax);
   else
-    k_step_fused<64, kLpp64><<<dim3(max_half, nprob), PivotSmem<64, kLpp64>::NT, sizeof(PivotSmem<64, kLpp64>),
-                               st>>>(probs, s, pp);
+    k_step_fused<64><<<dim3(max_half, nprob), 4 * 64, FusedLayout<64>::bytes(mmax), st>>>(probs, s, pp, mmax);
 }
 
 }  // namespace jac
