@@ -99,6 +99,7 @@ struct alignas(16) PivotState {
   using D = PivotDim<KM>;
   int4 mst[2][D::P2];   // traveling column of each slot: index, cn, d, sign
   float colb[2][KM];    // pivot column of a Cholesky step (double-buffered)
+  float cold[2][KM];    // ... its low parts (two-float factorization)
   float dd[KM];         // d_c
   float fid[KM];        // fp32(1 / d_c), 0 beyond k
   float ed[KM];         // e_cc
@@ -139,6 +140,157 @@ __device__ __forceinline__ float group_sum(float v) {
 #pragma unroll
   for (int o = LPP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// ---- two-float numbers (hi + lo, |lo| <= ulp(hi) / 2: about 48 bits) ---------------------------
+__device__ __forceinline__ void ff_renorm(float& h, float& l) {
+  const float s = h + l;
+  l = l - (s - h);
+  h = s;
+}
+__device__ __forceinline__ void ff_mul(float ah, float al, float bh, float bl, float& h, float& l) {
+  h = ah * bh;
+  l = fmaf(ah, bh, -h);
+  l = fmaf(ah, bl, fmaf(al, bh, l));
+  ff_renorm(h, l);
+}
+__device__ __forceinline__ void ff_sub(float& sh, float& sl, float ph, float pl) {  // s -= p
+  const float d = sh - ph, bb = d - sh;
+  const float e = (sh - (d - bb)) - (ph + bb);
+  sh = d;
+  sl = (sl + e) - pl;
+  ff_renorm(sh, sl);
+}
+// 1 / sqrt(s): one Newton step on the FP32 seed, the residual formed in two floats
+__device__ __forceinline__ void ff_rsqrt(float sh, float sl, float& h, float& l) {
+  const float y = rsqrtf(sh);
+  const float ph = y * y, pl = fmaf(y, y, -ph);
+  const float qh = sh * ph, ql = fmaf(sh, ph, -qh);
+  const float e = ((1.0f - qh) - ql) - fmaf(sh, pl, sl * ph);
+  h = y;
+  l = 0.5f * y * e;
+  ff_renorm(h, l);
+}
+
+// The Cholesky factor of a block that FP32 cannot factor (a Schur pivot below 64 eps_32 of its
+// diagonal entry), in two-float arithmetic: as the FP32 factorization of pivot_core (same tiles, same
+// orders), on A_P scaled by powers of two.  Leaves row i of R~ in frt (FP32, R = R~ D with D =
+// diag(dd), r_ii itself on the diagonal) and the order in perm; false (uniform) when a Schur pivot
+// falls below 2^-36 of its diagonal entry: the FP64 pivot kernel then decides.
+// Square Gaussian factors of order 33..64 are often beyond FP32 in their first sweep (kappa(A~) above
+// 2.6e5), and there the FP64 pivot took 1 to 3 ms per block (704 FP64 operations per pair of
+// columns and step at ~1.6 per clock): 1000 problems of orders 8..128 spent 42% of their time in
+// it.  This factorization costs ~60k clocks, and the FP32 rotations that follow bring the block
+// within FP32's reach for the next sweep.
+template <int KM>
+__device__ __noinline__ bool chol_two_float(PivotState<KM>& sm, float* frt, const double* A, int apld, int k, int npos,
+                                            int factor) {
+  using D = PivotDim<KM>;
+  constexpr int NW = D::NWC, TX = D::TX, RU = D::RU, LDT = D::LDT;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tx = tid % TX, ty = tid / TX, c0 = 4 * tx, r0 = RU * ty;
+  const bool signpiv = (factor == 2), pivsel = factor != 0;
+  // power-of-two scale near d_c: 2^-e_c
+  auto pscale = [&](int c) { return __int_as_float(0x7f000000 - (__float_as_int(sm.dd[c]) & 0x7f800000)); };
+  float H[RU][4], L[RU][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int u = 0; u < RU; ++u) {
+      const int i_ = r0 + u, j_ = c0 + j;
+      const bool in = i_ < k && j_ < k;
+      const double a = in ? __ldg(A + (size_t)j_ * apld + i_) : 0.0;
+      const double b = a * (double)pscale(in ? i_ : 0) * (double)pscale(in ? j_ : 0);  // exact
+      H[u][j] = (float)b;
+      L[u][j] = (float)(b - (double)H[u][j]);
+    }
+  float dh[2], dl[2], dq[2], d0[2];
+  bool al[2];
+#pragma unroll
+  for (int w = 0; w < KM / 32; ++w) {
+    const int c = lane + 32 * w;
+    const float ps = pscale(c < k ? c : 0);
+    const double b = c < k ? sm.adiag[c] * (double)ps * (double)ps : 1.0;
+    dh[w] = (float)b;
+    dl[w] = (float)(b - (double)dh[w]);
+    d0[w] = dh[w];
+    dq[w] = 1.0f / (ps * ps);
+    al[w] = c < k;
+  }
+  auto next_pivot = [&](int i) -> int {
+    if (!pivsel) return i;
+    unsigned key = 0;
+#pragma unroll
+    for (int w = 0; w < KM / 32; ++w) {
+      const int c = lane + 32 * w;
+      const bool in = al[w] && (!signpiv || ((i < npos) == (c < npos)));
+      if (in) key = max(key, (__float_as_uint(fmaxf(dq[w] * dh[w], 0.0f)) & 0xFFFFFFC0u) | (unsigned)(63 - c));
+    }
+    return 63 - (int)(__reduce_max_sync(0xffffffffu, key) & 63u);
+  };
+  core_sync<KM>();  // the failed factorization's columns and rows are no longer read
+  if (tid == 0) sm.bad = 0;
+  int p = next_pivot(0);
+  for (int i = 0; i < k; ++i) {
+    const int b = i & 1;
+    if (tx == (p >> 2)) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if ((p & 3) == j) {
+#pragma unroll
+          for (int u = 0; u < RU; ++u) {
+            sm.colb[b][r0 + u] = H[u][j];
+            sm.cold[b][r0 + u] = L[u][j];
+          }
+        }
+    }
+    // the smallest acceptable pivot, from the lane that carries column p
+    const float dp = __shfl_sync(0xffffffffu, (KM == 64 && p >= 32) ? d0[KM / 32 - 1] : d0[0], p & 31);
+    core_sync<KM>();
+    const float ph = sm.colb[b][p], pl = sm.cold[b][p];
+    if (!(ph > 1.4551915e-11f * dp)) {
+      if (tid == 0) sm.bad = 1;
+      break;  // uniform
+    }
+    float yh, yl;
+    ff_rsqrt(ph, pl, yh, yl);
+    float th[2], tl[2];
+#pragma unroll
+    for (int w = 0; w < KM / 32; ++w) {
+      const int c = lane + 32 * w;
+      ff_mul(sm.colb[b][c], sm.cold[b][c], yh, yl, th[w], tl[w]);
+      float qh, ql;
+      ff_mul(th[w], tl[w], th[w], tl[w], qh, ql);
+      ff_sub(dh[w], dl[w], qh, ql);
+      al[w] = al[w] && c != p;
+    }
+    const int pn = (i + 1 < k) ? next_pivot(i + 1) : 0;
+    if (warp == i % NW) {
+#pragma unroll
+      for (int w = 0; w < KM / 32; ++w) {
+        const int c = lane + 32 * w;
+        // R column c is t 2^e_c; frt holds it relative to d_c
+        if (c < k) frt[c * LDT + i] = th[w] / (pscale(c) * sm.dd[c]);
+      }
+      if (lane == 0) sm.perm[i] = p;
+    }
+    float ch[4], cl[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ff_mul(sm.colb[b][c0 + j], sm.cold[b][c0 + j], yh, yl, ch[j], cl[j]);
+#pragma unroll
+    for (int u = 0; u < RU; ++u) {
+      float rh, rl;
+      ff_mul(sm.colb[b][r0 + u], sm.cold[b][r0 + u], yh, yl, rh, rl);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float q = rh * ch[j], e = fmaf(rh, cl[j], fmaf(rl, ch[j], fmaf(rh, ch[j], -q)));
+        ff_sub(H[u][j], L[u][j], q, e);
+      }
+    }
+    p = pn;
+  }
+  core_sync<KM>();
+  return sm.bad == 0;
 }
 
 // Phases 1-3 of one pair, run by threads 0..NTC-1 of a CTA.  Returns (uniformly) 0 when V_P was
@@ -460,6 +612,10 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
     p = pn;
   }
   core_sync<KM>();
+  bool raw = false;  // frt holds r_ii itself on the diagonal
+  if constexpr (!A32) {
+    if (sm.bad && pp.ns_mode) raw = chol_two_float<KM>(sm, wk.frt, A, a.apld, k, npos, pp.factor);
+  }
   if (sm.bad) {  // handed over to the FP64 pivot kernel, which decides on rank deficiency
     if (tid == 0) {
       a.skip[pair] = 2;
@@ -546,7 +702,7 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         const int row = l * R + 2 * u + t;
-        r[t] = (row < c) ? x[t] * d : (row == c) ? fmaf(x[t], d, d) : 0.0f;
+        r[t] = (row < c) ? x[t] * d : (row == c) ? fmaf(x[t], d, raw ? 0.0f : d) : 0.0f;
         v[t] = (row == c) ? 1.0f : 0.0f;
       }
       f[u] = f2_make(r[0], r[1]);
@@ -590,6 +746,25 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
     sg = m.w;
   };
   for (inner = 0; inner < max_inner; ++inner) {
+    if (inner > 0) {
+      // a norm that has moved far from its reference d^2 (nearly dependent columns) is no longer
+      // resolved by d^2 + cn: take it from the column, with a new reference
+      auto fresh = [&](const f2(&f)[H], float& cn, float& d) {
+        f2 q0 = f2_mul(f[0], f[0]), q1 = f2_mul(f[1], f[1]);
+#pragma unroll
+        for (int u = 2; u < H; u += 2) {
+          q0 = f2_fma(f[u], f[u], q0);
+          q1 = f2_fma(f[u + 1], f[u + 1], q1);
+        }
+        const float q = group_sum<LPP>((f2_lo(q0) + f2_lo(q1)) + (f2_hi(q0) + f2_hi(q1)));
+        if (!(fabsf(cn) < 0.75f * d * d) && q > 0.0f) {
+          d = sqrtf(q);
+          cn = fmaf(-d, d, q);
+        }
+      };
+      fresh(fi, cni, si);
+      fresh(fj, cnj, sj);
+    }
     int my_rot = 0;       // per slot (uniform over its lanes)
     float my_max = 0.0f;  // largest scaled |a_ij| rotated
     for (int g = P2; g >= g_last; g >>= 1) {
