@@ -14,7 +14,7 @@
 //  4. V_P = P W Pi (rows permuted back as Algorithm 3.4 states; Pi = the reversed order of the
 //     J = -1 columns of Algorithm 3.3), J_P-unitary to FP64 accuracy when requested.
 //
-// GB300 placement.  Phases 1-3 (pivot_core) are a dependent chain of FP32 work: 2 KM threads, one
+// GB300 placement.  Phases 1-3 (pivot_core) are a dependent chain of FP32 work: 4 KM threads, one
 // block barrier per Cholesky step and per inner step.  Every FP32 pass runs on pairs of values
 // (fma.rn.f32x2: two FMAs per issued instruction), since with at most one or two warps per
 // scheduler the chain is bound by issue slots and latency, not by arithmetic.
@@ -76,30 +76,55 @@ __device__ __forceinline__ float d2f_fast(double x, bool& slow) {
 }
 
 // ---- the core: statistics, Cholesky, inner Jacobi ---------------------------------------------
-// Pivot capacity KM (largest k = w_p + w_q of the class); KM / 2 pair slots of LPP lanes each, R
-// rows of both columns per lane.
+// Pivot capacity KM (largest k = w_p + w_q of the class): 4 KM threads; KM / 2 pair slots of LPP lanes
+// each, R rows of both columns per lane, once for the columns of R (the first 2 KM threads) and once
+// for those of V.
 template <int KM>
 struct PivotDim {
   static constexpr int LPP = 4;
   static constexpr int R = KM / LPP;
   static constexpr int H = R / 2;        // row pairs per lane
   static constexpr int P2 = KM / 2;      // pair slots
-  static constexpr int NTC = P2 * LPP;   // threads of the core
-  static constexpr int NWC = NTC / 32;
-  static constexpr int LDT = KM + 4;     // rows of R~ - I by column (floats; 16-byte aligned)
+  static constexpr int NT = 4 * KM;      // threads
+  static constexpr int NF = P2 * LPP;    // threads of the columns of R
+  static constexpr int NW = NT / 32;
+  static constexpr int LDT = KM + 4;     // Schur columns of the pivots (floats; 16-byte aligned)
   static constexpr int LDW = KM + 4;     // columns of W = V - I (floats; 16-byte aligned)
   static constexpr int TX = KM / 4;      // Cholesky tile of a thread: RU rows x 4 columns
-  static constexpr int RU = KM / 8;
-  static constexpr int MB = 2 * KM * P2; // floats of one mailbox: F and V column of every slot
-  static_assert(TX * 8 == NTC && R % 4 == 0, "tile and lane layout");
+  static constexpr int RU = KM / 16;
+  static constexpr int MB = KM * P2;     // floats of one mailbox: a column of every slot
+  static_assert(TX * 16 == NT && 2 * NF == NT && R % 4 == 0, "tile and lane layout");
 };
+
+// Block barrier of the inner sweep, where the two halves of the threads wait in code of their own.
+template <int KM>
+__device__ __forceinline__ void half_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(PivotDim<KM>::NT) : "memory");
+}
+
+// N floats (2 or 4) from shared memory
+template <int N>
+__device__ __forceinline__ void load_n(float (&v)[N], const float* p) {
+  if constexpr (N == 4) {
+    const float4 x = *reinterpret_cast<const float4*>(p);
+    v[0] = x.x;
+    v[1] = x.y;
+    v[2] = x.z;
+    v[3] = x.w;
+  } else {
+    const float2 x = *reinterpret_cast<const float2*>(p);
+    v[0] = x.x;
+    v[1] = x.y;
+  }
+}
 
 template <int KM>
 struct alignas(16) PivotState {
   using D = PivotDim<KM>;
   int4 mst[2][D::P2];   // traveling column of each slot: index, cn, d, sign
-  float colb[2][KM];    // pivot column of a Cholesky step (double-buffered)
-  float cold[2][KM];    // ... its low parts (two-float factorization)
+  float colb[2][KM];    // two-float factorization: pivot column of a step (double-buffered)
+  float cold[2][KM];    // ... its low parts
+  int4 piv[KM];         // Cholesky step i: pivot column, 1 / r, r (floats)
   float dd[KM];         // d_c
   float fid[KM];        // fp32(1 / d_c), 0 beyond k
   float ed[KM];         // e_cc
@@ -112,10 +137,11 @@ struct alignas(16) PivotState {
   int jloc[KM];         // signs in local order
   int pres[D::P2];      // block-oriented cross step: columns of block p (pivot order) per slot
   int ptrav[D::P2];     // ... and of block q
-  float red_f[D::NWC][4];
-  int red_i[D::NWC][2];
+  float4 prm[2][D::P2]; // rotation of each slot's pair: c, q12, q21 (double-buffered)
+  float red_f[D::NW][4];
+  int red_i[D::NW][2];
   double trs[2];
-  int k, bad, code;
+  int k, bad;
   long long t_core;     // clock at the end of the core
   PairStat st;          // kept by thread 0
 };
@@ -124,14 +150,15 @@ template <int KM>
 struct alignas(16) PivotWork {  // dead outside the core
   using D = PivotDim<KM>;
   union {
-    float frt[KM * D::LDT];  // frt[c LDT + i]: row i of R~ - I at column c
-    float mb[2][D::MB];      // column mailboxes of the inner sweep (double-buffered)
+    float colh[KM * D::LDT];  // colh[i LDT + c]: Schur column of pivot i; times 1 / r, row i of R~
+    float mb[2][2][D::MB];   // column mailboxes of the inner sweep: R, V (double-buffered)
   };
 };
 
-template <int KM>
-__device__ __forceinline__ void core_sync() {  // barrier of the core's threads only
-  asm volatile("bar.sync 1, %0;" ::"n"(PivotDim<KM>::NTC) : "memory");
+__device__ __forceinline__ float rsqrt_ftz(float x) {  // arguments of FP32 normal size
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 // sum over the LPP lanes of a pair slot (aligned lane groups)
@@ -174,19 +201,19 @@ __device__ __forceinline__ void ff_rsqrt(float sh, float sl, float& h, float& l)
 
 // The Cholesky factor of a block that FP32 cannot factor (a Schur pivot below 64 eps_32 of its
 // diagonal entry), in two-float arithmetic: as the FP32 factorization of pivot_core (same tiles, same
-// orders), on A_P scaled by powers of two.  Leaves row i of R~ in frt (FP32, R = R~ D with D =
-// diag(dd), r_ii itself on the diagonal) and the order in perm; false (uniform) when a Schur pivot
-// falls below 2^-36 of its diagonal entry: the FP64 pivot kernel then decides.
+// orders), on A_P scaled by powers of two.  Leaves row i of R~ in colh (FP32, R = R~ D with D =
+// diag(dd), its 1 / r taken as 1) and the order in piv; sm.bad is set when a Schur pivot falls below 2^-36 of its diagonal
+// entry (the FP64 pivot kernel then decides) and cleared otherwise.
 // Square Gaussian factors of order 33..64 are often beyond FP32 in their first sweep (kappa(A~) above
 // 2.6e5), and there the FP64 pivot took 1 to 3 ms per block (704 FP64 operations per pair of
 // columns and step at ~1.6 per clock): 1000 problems of orders 8..128 spent 42% of their time in
 // it.  This factorization costs ~60k clocks, and the FP32 rotations that follow bring the block
 // within FP32's reach for the next sweep.
 template <int KM>
-__device__ __noinline__ bool chol_two_float(PivotState<KM>& sm, float* frt, const double* A, int apld, int k, int npos,
+__device__ __noinline__ void chol_two_float(PivotState<KM>& sm, float* colh, const double* A, int apld, int k, int npos,
                                             int factor) {
   using D = PivotDim<KM>;
-  constexpr int NW = D::NWC, TX = D::TX, RU = D::RU, LDT = D::LDT;
+  constexpr int NW = D::NW, TX = D::TX, RU = D::RU, LDT = D::LDT;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tx = tid % TX, ty = tid / TX, c0 = 4 * tx, r0 = RU * ty;
   const bool signpiv = (factor == 2), pivsel = factor != 0;
@@ -228,7 +255,7 @@ __device__ __noinline__ bool chol_two_float(PivotState<KM>& sm, float* frt, cons
     }
     return 63 - (int)(__reduce_max_sync(0xffffffffu, key) & 63u);
   };
-  core_sync<KM>();  // the failed factorization's columns and rows are no longer read
+  __syncthreads();  // the failed factorization's columns and rows are no longer read
   if (tid == 0) sm.bad = 0;
   int p = next_pivot(0);
   for (int i = 0; i < k; ++i) {
@@ -246,7 +273,7 @@ __device__ __noinline__ bool chol_two_float(PivotState<KM>& sm, float* frt, cons
     }
     // the smallest acceptable pivot, from the lane that carries column p
     const float dp = __shfl_sync(0xffffffffu, (KM == 64 && p >= 32) ? d0[KM / 32 - 1] : d0[0], p & 31);
-    core_sync<KM>();
+    __syncthreads();
     const float ph = sm.colb[b][p], pl = sm.cold[b][p];
     if (!(ph > 1.4551915e-11f * dp)) {
       if (tid == 0) sm.bad = 1;
@@ -269,10 +296,11 @@ __device__ __noinline__ bool chol_two_float(PivotState<KM>& sm, float* frt, cons
 #pragma unroll
       for (int w = 0; w < KM / 32; ++w) {
         const int c = lane + 32 * w;
-        // R column c is t 2^e_c; frt holds it relative to d_c
-        if (c < k) frt[c * LDT + i] = th[w] / (pscale(c) * sm.dd[c]);
+        // R column c is t 2^e_c; colh holds it relative to d_c
+        const float t = c < k ? th[w] / (pscale(c) * sm.dd[c]) : 0.0f;
+        colh[i * LDT + c] = t;
+        if (c == p) sm.piv[i] = make_int4(p, __float_as_int(1.0f), __float_as_int(t), 0);
       }
-      if (lane == 0) sm.perm[i] = p;
     }
     float ch[4], cl[4];
 #pragma unroll
@@ -289,11 +317,10 @@ __device__ __noinline__ bool chol_two_float(PivotState<KM>& sm, float* frt, cons
     }
     p = pn;
   }
-  core_sync<KM>();
-  return sm.bad == 0;
+  __syncthreads();
 }
 
-// Phases 1-3 of one pair, run by threads 0..NTC-1 of a CTA.  Returns (uniformly) 0 when V_P was
+// Phases 1-3 of one pair, run by all 4 KM threads of a CTA.  Returns (uniformly) 0 when V_P was
 // formed: W = V - I in Wf (column c at c LDW, pivot order), the orders in sm; 2 when the block was
 // handed over to the FP64 pivot kernel; 1 otherwise (no rotation, or a reported error).  A32: A_P is
 // read from shared memory (FP32, column c at c LDW), else from the Gram kernel's output.  `skip` and
@@ -302,7 +329,7 @@ template <int KM, bool A32>
 __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk, const float* As, float* Wf,
                                           const JacProb& a, int s, int pair, const PivotParams& pp) {
   using D = PivotDim<KM>;
-  constexpr int NW = D::NWC, TX = D::TX, RU = D::RU, LDT = D::LDT, LDW = D::LDW, P2 = D::P2;
+  constexpr int NW = D::NW, TX = D::TX, RU = D::RU, LDT = D::LDT, LDW = D::LDW, P2 = D::P2;
   constexpr int LPP = D::LPP, R = D::R, H = D::H;
   unsigned* err = a.pflags;
   PairStat* stats = a.stats + (size_t)s * a.half;
@@ -345,7 +372,7 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
     sm.pres[tid] = -1;
     sm.ptrav[tid] = -1;
   }
-  core_sync<KM>();  // bad cleared
+  __syncthreads();  // bad cleared
   if constexpr (!A32) {
 #pragma unroll
     for (int j = 0; j < 4; ++j)
@@ -359,15 +386,12 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
       }
   } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < 4; ++j) {
+      float v[RU];
+      load_n<RU>(v, As + (c0 + j) * LDW + r0);
 #pragma unroll
-      for (int u = 0; u < RU; u += 4) {
-        const float4 v = *reinterpret_cast<const float4*>(As + (c0 + j) * LDW + r0 + u);
-        e[u][j] = v.x;
-        e[u + 1][j] = v.y;
-        e[u + 2][j] = v.z;
-        e[u + 3][j] = v.w;
-      }
+      for (int u = 0; u < RU; ++u) e[u][j] = v[u];
+    }
     if (tid < k) adg = (double)As[tid * LDW + tid];
   }
   double tr = 0.0;
@@ -392,7 +416,7 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
     sm.adiag[tid] = adg;
     sm.jloc[tid] = j;
   }
-  core_sync<KM>();
+  __syncthreads();
   if (sm.bad) {
     if (tid == 0) {
       atomicOr(err, JAC_DEVERR_NOTPD);
@@ -427,14 +451,7 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
   unsigned near = 0;
   {
     float fr[RU];
-#pragma unroll
-    for (int u = 0; u < RU; u += 4) {
-      const float4 v = *reinterpret_cast<const float4*>(&sm.fid[r0 + u]);
-      fr[u] = v.x;
-      fr[u + 1] = v.y;
-      fr[u + 2] = v.z;
-      fr[u + 3] = v.w;
-    }
+    load_n<RU>(fr, &sm.fid[r0]);
     const float4 fc4 = *reinterpret_cast<const float4*>(&sm.fid[c0]);
     const float fc[4] = {fc4.x, fc4.y, fc4.z, fc4.w};
 #pragma unroll
@@ -483,7 +500,7 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
     sm.red_i[warp][0] = hit;
     if (warp < KM / 32) sm.trs[warp] = tr;
   }
-  core_sync<KM>();
+  __syncthreads();
   mx = oc = od = 0.0f;
   hit = false;
 #pragma unroll
@@ -517,25 +534,24 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
   // ---- 2. scaled, optionally sign-pivoted Cholesky in FP32 -----------------------------------
   // Right-looking on unpermuted storage, the whole symmetric matrix E (both triangles) in
   // registers: thread (ty, tx) holds rows r0.. and columns c0.. .  Step i with pivot column p: the
-  // threads of column p publish it (double-buffered, one barrier), every thread scales it to
-  // t = s_p / sqrt(s_pp) and subtracts t_r t_c from its tile.  Every warp carries the shifted Schur
-  // diagonal s_cc of all columns (lane: c = lane, lane + 32) with the same operations, so the pivot
-  // search of the next step needs no barrier: a warp max-reduction of keys, the value's bits above
-  // the low 6 (order-preserving for v >= 0) and 63 - c, the largest unscaled Schur diagonal
-  // d_c^2 (1 + s_cc) in the sign group of the step (sign pivoting, Algorithm 3.3) or among all
-  // remaining columns (diagonal pivoting, HFC), ties to the smaller index.
-  // A step is one chain (barrier, column, rsqrt, key, search, publish): 540 clocks; left-looking with
-  // the rows in shared memory it took 940 (64-column block of the 512 x 512 workload: 34.5k clocks per
-  // factorization against 60.6k).
+  // threads of column p have published it (as row i of colh, one barrier per step), every thread
+  // scales it to t = s_p / sqrt(s_pp), and t_r t_c comes off its tile.  Every warp carries the shifted
+  // Schur diagonal s_cc of all columns (lane: c = lane, lane + 32) with the same operations, so the
+  // pivot search of the next step needs no barrier: a warp max-reduction of keys, the value's bits
+  // above the low 6 (order-preserving for v >= 0, negative for v < 0) and 63 - c, the largest unscaled
+  // Schur diagonal d_c^2 (1 + s_cc) in the sign group of the step (sign pivoting, Algorithm 3.3) or
+  // among all remaining columns (diagonal pivoting, HFC), ties to the smaller index.
+  // A step is one chain: barrier, column, rsqrt, key, search, publish.  What is not on it stays out
+  // of its way: the next column is published with its own update first and the tile's update
+  // follows after the loads of the next step, the rows of R~ need no stores of their own, no branch
+  // but the loop's.  ~410 clocks per step; left-looking with the rows in shared memory it took 940.
   const bool signpiv = (pp.factor == 2), diagpiv = (pp.factor == 1), pivsel = signpiv || diagpiv;
-  f2 S[RU / 2][4];
+  // the tile of E: its shifted diagonal into e
 #pragma unroll
   for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int u = 0; u < RU / 2; ++u) {
-      const int i_ = r0 + 2 * u, j_ = c0 + j;
-      S[u][j] = f2_make(i_ == j_ ? sm.ed[j_] : e[2 * u][j], i_ + 1 == j_ ? sm.ed[j_] : e[2 * u + 1][j]);
-    }
+    for (int u = 0; u < RU; ++u)
+      if (r0 + u == c0 + j) e[u][j] = sm.ed[c0 + j];
   float dv0 = sm.ed[lane], dq0 = sm.dd[lane] * sm.dd[lane], dv1 = 0.0f, dq1 = 0.0f;
   bool al0 = lane < k, al1 = false;
   if constexpr (KM == 64) {
@@ -545,76 +561,76 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
   }
   auto next_pivot = [&](int i) -> int {
     if (!pivsel) return i;
+    const bool first = i < npos;
     auto key_of = [&](bool alive, float dq, float dv, int c) {
-      const bool in = alive && (!signpiv || ((i < npos) == (c < npos)));
-      const float v = fmaxf(dq * (1.0f + dv), 0.0f);
-      return in ? (__float_as_uint(v) & 0xFFFFFFC0u) | (unsigned)(63 - c) : 0u;
+      const bool in = alive && (!signpiv || first == (c < npos));
+      return in ? (int)((__float_as_uint(fmaf(dq, dv, dq)) & 0xFFFFFFC0u) | (unsigned)(63 - c)) : (int)0x80000000;
     };
-    unsigned key = key_of(al0, dq0, dv0, lane);
+    int key = key_of(al0, dq0, dv0, lane);
     if constexpr (KM == 64) key = max(key, key_of(al1, dq1, dv1, lane + 32));
-    return 63 - (int)(__reduce_max_sync(0xffffffffu, key) & 63u);
+    return 63 - (__reduce_max_sync(0xffffffffu, key) & 63);  // signed: a negative value never wins
+  };
+  auto pick = [](int p, const float(&x)[4]) {  // x[p & 3] by selects: a jump on it costs ~50 clocks
+    const float lo = (p & 1) ? x[1] : x[0], hi = (p & 1) ? x[3] : x[2];
+    return (p & 2) ? hi : lo;
+  };
+  auto publish = [&](int i, int p, const float(&x)[RU]) {
+    if (tx == (p >> 2)) {
+      if constexpr (RU == 4) *reinterpret_cast<float4*>(&wk.colh[i * LDT + r0]) = make_float4(x[0], x[1], x[2], x[3]);
+      else *reinterpret_cast<float2*>(&wk.colh[i * LDT + r0]) = make_float2(x[0], x[1]);
+    }
   };
   int p = next_pivot(0);
+  float tu[RU], tc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  bool bad = false;
+  {
+    float x[RU];
+#pragma unroll
+    for (int u = 0; u < RU; ++u) {
+      x[u] = pick(p, e[u]);
+      tu[u] = 0.0f;
+    }
+    publish(0, p, x);
+  }
   for (int i = 0; i < k; ++i) {
-    const int b = i & 1;
-    if (tx == (p >> 2)) {
-      f2* dst = reinterpret_cast<f2*>(&sm.colb[b][r0]);
-      auto put = [&](int j) {
+    __syncthreads();
+    const float* col = wk.colh + i * LDT;
+    const float spp = col[p], v0 = col[lane], v1 = (KM == 64) ? col[lane + (KM - 32)] : 0.0f;
+    float vc[4], vr[RU];
+    load_n<4>(vc, &col[c0]);
+    load_n<RU>(vr, &col[r0]);
 #pragma unroll
-        for (int u = 0; u < RU / 2; ++u) dst[u] = S[u][j];
-      };
-      switch (p & 3) {  // uniform
-        case 0: put(0); break;
-        case 1: put(1); break;
-        case 2: put(2); break;
-        default: put(3);
-      }
-    }
-    core_sync<KM>();
-    const float spp = sm.colb[b][p];
-    const float v0 = sm.colb[b][lane];
-    const float v1 = (KM == 64) ? sm.colb[b][lane + (KM - 32)] : 0.0f;
-    const float4 vc = *reinterpret_cast<const float4*>(&sm.colb[b][c0]);
-    f2 vr[RU / 2];
+    for (int j = 0; j < 4; ++j)  // the previous step's update of the tile
 #pragma unroll
-    for (int u = 0; u < RU / 2; ++u) vr[u] = reinterpret_cast<const f2*>(&sm.colb[b][r0])[u];
+      for (int u = 0; u < RU; ++u) e[u][j] = fmaf(tu[u], tc[j], e[u][j]);
     // The scaled Schur pivot is 1 / (A~^-1)_pp >= 1 / kappa(A~).  Below 64 eps_32 the column is
-    // in the span of the previous ones at the precision of this factorization: the block goes
-    // to the FP64 pivot kernel (which tells an ill-conditioned block from a singular one).
+    // in the span of the previous ones at the precision of this factorization: a more precise one
+    // takes the block (below).
     const float piv1 = 1.0f + spp;
-    if (!(piv1 > 3.8146973e-6f)) {
-      if (tid == 0) sm.bad = 1;
-      break;  // uniform: every thread read the same pivot
-    }
-    const float rinv = rsqrtf(piv1);  // 1 / r
+    bad |= !(piv1 > 3.8146973e-6f);
+    const float rinv = rsqrt_ftz(fmaxf(piv1, 3.8146973e-6f));  // 1 / r
     const float t0 = v0 * rinv, t1 = v1 * rinv;
     dv0 = fmaf(-t0, t0, dv0);
     dv1 = fmaf(-t1, t1, dv1);
     al0 = al0 && lane != p;
     al1 = al1 && lane + 32 != p;
-    const int pn = (i + 1 < k) ? next_pivot(i + 1) : 0;
-    if (warp == i % NW) {  // row i of R~ - I by column
-      const float rp = __fdividef(spp, 1.0f + piv1 * rinv);  // r - 1 without cancellation
-      wk.frt[lane * LDT + i] = (lane == p) ? rp : t0;
-      if constexpr (KM == 64) wk.frt[(lane + 32) * LDT + i] = (lane + 32 == p) ? rp : t1;
-      if (lane == 0) sm.perm[i] = p;
-    }
-    const f2 rinv2 = f2_make(rinv, rinv);
+    if (tid == 0) sm.piv[i] = make_int4(p, __float_as_int(rinv), __float_as_int(piv1 * rinv), 0);
+    const int pn = next_pivot(i + 1) & (KM - 1);
 #pragma unroll
-    for (int u = 0; u < RU / 2; ++u) vr[u] = f2_mul(vr[u], rinv2);
-    const float tc[4] = {-vc.x * rinv, -vc.y * rinv, -vc.z * rinv, -vc.w * rinv};
+    for (int j = 0; j < 4; ++j) tc[j] = -vc[j] * rinv;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const f2 t2 = f2_make(tc[j], tc[j]);
-#pragma unroll
-      for (int u = 0; u < RU / 2; ++u) S[u][j] = f2_fma(vr[u], t2, S[u][j]);
-    }
+    for (int u = 0; u < RU; ++u) tu[u] = vr[u] * rinv;
     p = pn;
+    const float tp = pick(p, tc);
+    float x[RU];
+#pragma unroll
+    for (int u = 0; u < RU; ++u) x[u] = fmaf(tu[u], tp, pick(p, e[u]));
+    if (i + 1 < k) publish(i + 1, p, x);
   }
-  core_sync<KM>();
-  bool raw = false;  // frt holds r_ii itself on the diagonal
+  if (tid == 0) sm.bad = bad ? 1 : 0;  // the same in every thread
+  __syncthreads();
   if constexpr (!A32) {
-    if (sm.bad && pp.ns_mode) raw = chol_two_float<KM>(sm, wk.frt, A, a.apld, k, npos, pp.factor);
+    if (sm.bad && pp.ns_mode) chol_two_float<KM>(sm, wk.colh, A, a.apld, k, npos, pp.factor);
   }
   if (sm.bad) {  // handed over to the FP64 pivot kernel, which decides on rank deficiency
     if (tid == 0) {
@@ -632,6 +648,8 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
   // each in pivot order), so that V_P^* J_P V_P = J_P in the block's local order (the reordering of
   // HFC).  Sign pivoting takes the J = -1 columns in reverse.
   const bool cross_only = pp.oriented && s > 0;
+  if (tid < k) sm.perm[tid] = sm.piv[tid].x;
+  __syncthreads();
   {
     auto mask64 = [&](auto f) -> unsigned long long {  // f(position) over the k positions
       unsigned long long m = __ballot_sync(0xffffffffu, lane < k && f(lane < k ? lane : 0));
@@ -658,7 +676,7 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
       sm.jphys[tid] = 1;
     }
   }
-  core_sync<KM>();
+  __syncthreads();
   const long long t_chol = clock64();
 
   // ---- 3. inner one-sided Jacobi (FP32) -------------------------------------------------------
@@ -675,184 +693,228 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
   // other slot through a shared-memory mailbox: one barrier per step.  Positions >= k are
   // empty.  The logical order of Algorithm 3.3 (reversed J = -1 part) gives the initial
   // placement: position p is the resident of slot p (p < KM/2) or the traveler of slot p - KM/2.
-  // Four lanes per slot, one warp per scheduler: the parameter chain (~90 instructions per warp
-  // and step) is issued half as often as with eight, and the reduction is one shuffle shorter.  Full
-  // inner sweep of a 64-column block (63 steps): 61k clocks; with eight lanes, scalar FMAs and
-  // predicated diagonal terms 78k.
-  const int slot = tid / LPP, l = tid % LPP;
-  int ci = cross_only ? sm.pres[slot] : ((slot < k) ? sm.lpos[slot] : -1);
-  int cj = cross_only ? sm.ptrav[slot] : ((slot + P2 < k) ? sm.lpos[slot + P2] : -1);
+  // What bounds a step is its chain: mailbox, dot product and its reduction, the parameters, the
+  // rotation, mailbox, barrier.  The columns of V are not on it: they belong to the second half of
+  // the threads, which rotate them one barrier later, with the parameters the first half left in
+  // shared memory, in the shadow of the first half's next step.  ~700 clocks per step for a 64-column
+  // block; rotating both in the same threads, with the parameters by way of the tangent, took 965 (and
+  // spreading the columns over 32 lanes, to keep the ring in registers, 1235: five shuffle rounds
+  // and the exchange of the parameters cost more than the mailboxes).
+  const bool is_f = tid < D::NF;
+  const int slot = (is_f ? tid : tid - D::NF) / LPP, l = tid % LPP;
+  const int ci0 = cross_only ? sm.pres[slot] : ((slot < k) ? sm.lpos[slot] : -1);
+  const int cj0 = cross_only ? sm.ptrav[slot] : ((slot + P2 < k) ? sm.lpos[slot + P2] : -1);
   // block-oriented: one inner sweep; after the first step of an outer sweep only the ring of
   // its first level (every column of block p meets every column of block q once)
   const int g_last = cross_only ? P2 : 1;
   const int max_inner = pp.oriented ? 1 : JAC_INNER_MAX_SWEEPS;
-  f2 fi[H], fj[H], wi[H], wj[H];
-  float cni, cnj, si, sj;  // ||r||^2 = s^2 + cn
-  int ji, jj;
-  auto load_col = [&](int c, f2(&f)[H], f2(&w)[H], float& cn, float& d, int& sg) {
-    const int pc = c >= 0 ? sm.perm[c] : 0;
-    cn = c >= 0 ? sm.cn0[pc] : 0.0f;
-    d = c >= 0 ? sm.dd[pc] : 1.0f;
-    sg = c >= 0 ? sm.jphys[c] : 1;
+  f2 xi[H], xj[H];  // resident and traveler of this half's columns
+  float cni = 0.0f, cnj = 0.0f, si = 1.0f, sj = 1.0f;  // ||r||^2 = s^2 + cn
+  int ci = ci0, cj = cj0, ji = 1, jj = 1;
+  if (is_f) {
+    auto load_col = [&](int c, f2(&f)[H], float& cn, float& d, int& sg) {
+      const int pc = c >= 0 ? sm.perm[c] : 0;
+      cn = c >= 0 ? sm.cn0[pc] : 0.0f;
+      d = c >= 0 ? sm.dd[pc] : 1.0f;
+      sg = c >= 0 ? sm.jphys[c] : 1;
 #pragma unroll
-    for (int u = 0; u < H; u += 2) {
-      const float4 x4 = *reinterpret_cast<const float4*>(&wk.frt[pc * LDT + l * R + 2 * u]);
-      const float x[4] = {x4.x, x4.y, x4.z, x4.w};
-      float r[4], v[4];
+      for (int u = 0; u < H; ++u) {
+        float r[2];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int row = l * R + 2 * u + t;
-        r[t] = (row < c) ? x[t] * d : (row == c) ? fmaf(x[t], d, raw ? 0.0f : d) : 0.0f;
-        v[t] = (row == c) ? 1.0f : 0.0f;
+        for (int t = 0; t < 2; ++t) {  // R[row][c] = R~[row][c] d_c, upper triangular in pivot order
+          const int row = l * R + 2 * u + t;
+          const int4 pv = sm.piv[row];
+          const float v = (row == c) ? __int_as_float(pv.z) : wk.colh[row * LDT + pc] * __int_as_float(pv.y);
+          r[t] = (row <= c) ? v * d : 0.0f;
+        }
+        f[u] = f2_make(r[0], r[1]);
       }
-      f[u] = f2_make(r[0], r[1]);
-      f[u + 1] = f2_make(r[2], r[3]);
-      w[u] = f2_make(v[0], v[1]);
-      w[u + 1] = f2_make(v[2], v[3]);
+    };
+    load_col(ci, xi, cni, si, ji);
+    load_col(cj, xj, cnj, sj, jj);
+  } else {
+#pragma unroll
+    for (int u = 0; u < H; ++u) {
+      const int row = l * R + 2 * u;
+      xi[u] = f2_make(row == ci ? 1.0f : 0.0f, row + 1 == ci ? 1.0f : 0.0f);
+      xj[u] = f2_make(row == cj ? 1.0f : 0.0f, row + 1 == cj ? 1.0f : 0.0f);
     }
-  };
-  load_col(ci, fi, wi, cni, si, ji);
-  load_col(cj, fj, wj, cnj, sj, jj);
-  core_sync<KM>();  // the Cholesky rows are read; the mailboxes take their place
+  }
+  __syncthreads();  // the Cholesky rows are read; the mailboxes take their place
   int total_rot = 0, inner = 0, buf = 0;
   // a column's mailbox: 16-byte chunk q of lane l at ((q P2 + slot) LPP + l): a quarter warp writes
   // and reads 128 consecutive bytes
-  auto box = [&](int b, int q, int sl) { return reinterpret_cast<ulonglong2*>(wk.mb[b]) + ((q * P2 + sl) * LPP + l); };
-  auto send = [&](int dst, const f2(&f)[H], const f2(&w)[H], int c, float cn, float d, int sg) {
-#pragma unroll
-    for (int u = 0; u < H; u += 2) {
-      *box(buf, u / 2, dst) = make_ulonglong2(f[u], f[u + 1]);
-      *box(buf, H / 2 + u / 2, dst) = make_ulonglong2(w[u], w[u + 1]);
-    }
-    if (l == 0) sm.mst[buf][dst] = make_int4(c, __float_as_int(cn), __float_as_int(d), sg);
+  auto box = [&](int b, int q, int sl) {
+    return reinterpret_cast<ulonglong2*>(wk.mb[b][is_f ? 0 : 1]) + ((q * P2 + sl) * LPP + l);
   };
-  auto receive = [&](f2(&f)[H], f2(&w)[H], int& c, float& cn, float& d, int& sg) {
-    const int4 m = sm.mst[buf][slot];
+  auto put = [&](int b, int dst, const f2(&f)[H]) {
+#pragma unroll
+    for (int u = 0; u < H; u += 2) *box(b, u / 2, dst) = make_ulonglong2(f[u], f[u + 1]);
+  };
+  auto get = [&](int b, f2(&f)[H]) {
 #pragma unroll
     for (int u = 0; u < H; u += 2) {
-      const ulonglong2 x = *box(buf, u / 2, slot);
+      const ulonglong2 x = *box(b, u / 2, slot);
       f[u] = x.x;
       f[u + 1] = x.y;
     }
+  };
+  auto rotate = [&](float c, float s12, float s21) {
+    const f2 q11 = f2_make(c, c), q12 = f2_make(s12, s12), q21 = f2_make(s21, s21);
 #pragma unroll
-    for (int u = 0; u < H; u += 2) {
-      const ulonglong2 x = *box(buf, H / 2 + u / 2, slot);
-      w[u] = x.x;
-      w[u + 1] = x.y;
+    for (int u = 0; u < H; ++u) {
+      const f2 a_i = xi[u], a_j = xj[u];
+      xi[u] = f2_fma(q11, a_i, f2_mul(q21, a_j));
+      xj[u] = f2_fma(q11, a_j, f2_mul(q12, a_i));
     }
-    c = m.x;
-    cn = __int_as_float(m.y);
-    d = __int_as_float(m.z);
-    sg = m.w;
   };
   for (inner = 0; inner < max_inner; ++inner) {
-    if (inner > 0) {
-      // a norm that has moved far from its reference d^2 (nearly dependent columns) is no longer
-      // resolved by d^2 + cn: take it from the column, with a new reference
-      auto fresh = [&](const f2(&f)[H], float& cn, float& d) {
-        f2 q0 = f2_mul(f[0], f[0]), q1 = f2_mul(f[1], f[1]);
-#pragma unroll
-        for (int u = 2; u < H; u += 2) {
-          q0 = f2_fma(f[u], f[u], q0);
-          q1 = f2_fma(f[u + 1], f[u + 1], q1);
-        }
-        const float q = group_sum<LPP>((f2_lo(q0) + f2_lo(q1)) + (f2_hi(q0) + f2_hi(q1)));
-        if (!(fabsf(cn) < 0.75f * d * d) && q > 0.0f) {
-          d = sqrtf(q);
-          cn = fmaf(-d, d, q);
-        }
-      };
-      fresh(fi, cni, si);
-      fresh(fj, cnj, sj);
-    }
     int my_rot = 0;       // per slot (uniform over its lanes)
     float my_max = 0.0f;  // largest scaled |a_ij| rotated
-    for (int g = P2; g >= g_last; g >>= 1) {
-      const int base = slot & ~(g - 1), pos = slot - base;
-      for (int st_ = 0; st_ < g; ++st_) {
-        // ---- rotate the pair (ci, cj) of this slot
-        const bool act = (ci | cj) >= 0;
-        // what does not depend on the dot product first
-        const bool trig = ji == jj;
-        const float aii = fmaf(si, si, cni), ajj = fmaf(sj, sj, cnj);
-        const float rs = rsqrtf(aii) * rsqrtf(ajj);
-        const float x = trig ? (sj - si) * (sj + si) + (cnj - cni) : aii + ajj;
-        f2 d0 = f2_mul(fi[0], fj[0]), d1 = f2_mul(fi[1], fj[1]);
+    if (is_f) {
+      if (inner > 0) {
+        // a norm that has moved far from its reference d^2 (nearly dependent columns) is no longer
+        // resolved by d^2 + cn: take it from the column, with a new reference
+        auto fresh = [&](const f2(&f)[H], float& cn, float& d) {
+          f2 q0 = f2_mul(f[0], f[0]), q1 = f2_mul(f[1], f[1]);
 #pragma unroll
-        for (int u = 2; u < H; u += 2) {
-          d0 = f2_fma(fi[u], fj[u], d0);
-          d1 = f2_fma(fi[u + 1], fj[u + 1], d1);
-        }
-        const float aij = group_sum<LPP>((f2_lo(d0) + f2_lo(d1)) + (f2_hi(d0) + f2_hi(d1)));
-        const float beta = fabsf(aij), scaled = beta * rs;
-        if (act && scaled > tol_in) {
-          ++my_rot;
-          my_max = fmaxf(my_max, scaled);
-          // One branch-free path for both kinds (sg = +1 trigonometric, -1 hyperbolic), so
-          // that the slots of a warp never split on the sign pattern:
-          //  trigonometric, Eq. (2.1): cot(2 phi) = (a_jj - a_ii) / (2 |a_ij|), i.e.
-          //    t = sign(x) 2|a_ij| / (|x| + sqrt(x^2 + 4|a_ij|^2)),  x = a_jj - a_ii;
-          //  hyperbolic: coth(2 phi) = -(a_ii + a_jj) / (2 |a_ij|), i.e.
-          //    t = -2|a_ij| / (x + sqrt((x - 2|a_ij|)(x + 2|a_ij|))),  x = a_ii + a_jj,
-          //    with the |tanh| < 1 guard of Sec. 3.2;
-          // both evaluated after an exact power-of-two scaling of x and 2|a_ij| into [1, 4).
-          // The square roots are x rsqrt(x): the angle needs FP32 accuracy only, the
-          // rotation built from it is orthogonal (J-orthogonal) whatever t is.
-          const float sg = trig ? 1.0f : -1.0f;
-          const float mxv = fmaxf(fabsf(x), 2.0f * beta);
-          const float sc = __int_as_float(0x7f000000 - (__float_as_int(mxv) & 0x7f800000));
-          const float nu = x * sc, b2 = 2.0f * beta * sc;
-          const float rr = trig ? fmaf(nu, nu, b2 * b2) : (nu - b2) * (nu + b2);
-          const bool ok = rr > 0.0f;
-          const float root = ok ? rr * rsqrtf(rr) : 0.0f;
-          const float tm = __fdividef(b2, fabsf(nu) + root);
-          float t = trig ? copysignf(tm, x) : (ok ? -tm : -1.0f);
-          const bool guard = !trig && (!(fabsf(t) < 1.0f) || !((1.0f - t) * (1.0f + t) > 0.0f));
-          if (guard) t = copysignf(0.9f, t);
-          // cos or cosh; of a small angle as 1 - y / 2 rounded once (rsqrtf returns the value below
-          // 1 too often there, and thousands of tiny rotations would shrink V: with it alone the
+          for (int u = 2; u < H; u += 2) {
+            q0 = f2_fma(f[u], f[u], q0);
+            q1 = f2_fma(f[u + 1], f[u + 1], q1);
+          }
+          const float q = group_sum<LPP>((f2_lo(q0) + f2_lo(q1)) + (f2_hi(q0) + f2_hi(q1)));
+          if (!(fabsf(cn) < 0.75f * d * d) && q > 0.0f) {
+            d = sqrtf(q);
+            cn = fmaf(-d, d, q);
+          }
+        };
+        fresh(xi, cni, si);
+        fresh(xj, cnj, sj);
+      }
+      for (int g = P2; g >= g_last; g >>= 1) {
+        const int base = slot & ~(g - 1), pos = slot - base;
+        for (int st_ = 0; st_ < g; ++st_) {
+          // ---- rotate the pair (ci, cj) of this slot; what does not depend on the dot product first.
+          // One branch-free path for both kinds, the slots of a warp never split on the sign
+          // pattern.  With x = a_jj - a_ii (trigonometric, Eq. (2.1): cot(2 phi) = x / (2 |a_ij|)) or
+          // x = a_ii + a_jj (hyperbolic: coth(2 phi) = -x / (2 |a_ij|)), everything scaled by
+          // rs = 1 / sqrt(a_ii a_jj) (nu = |x| rs, scaled = |a_ij| rs):
+          //   h = 1 / sqrt(nu^2 +- 4 scaled^2),  cos(h)^2 phi = 1/2 + nu h / 2,
+          //   |sin(h) phi| = scaled h / cos(h) phi.
+          // The roots need FP32 accuracy only: the rotation is orthogonal (J-orthogonal) to their
+          // rounding whatever the angle.  Two MUFU operations deep, ~90 clocks; by way of the
+          // tangent, with x and a_ij scaled by powers of two, it took 330.
+          const bool trig = ji == jj;
+          const float sg = trig ? 1.0f : -1.0f, sg4 = 4.0f * sg;
+          const float aii = fmaf(si, si, cni), ajj = fmaf(sj, sj, cnj);
+          const float rs = rsqrtf(aii) * rsqrtf(ajj);
+          const float x = trig ? (sj - si) * (sj + si) + (cnj - cni) : aii + ajj;
+          const float nu = fminf(fabsf(x) * rs, 1.0e18f), nu2 = nu * nu;
+          // sign of the tangent: that of x (trigonometric), negative (hyperbolic)
+          const unsigned tsign = trig ? __float_as_uint(x) & 0x80000000u : 0x80000000u;
+          f2 d0 = f2_mul(xi[0], xj[0]), d1 = f2_mul(xi[1], xj[1]);
+#pragma unroll
+          for (int u = 2; u < H; u += 2) {
+            d0 = f2_fma(xi[u], xj[u], d0);
+            d1 = f2_fma(xi[u + 1], xj[u + 1], d1);
+          }
+          const float aij = group_sum<LPP>((f2_lo(d0) + f2_lo(d1)) + (f2_hi(d0) + f2_hi(d1)));
+          const float scaled = fabsf(aij) * rs;
+          const bool rot = (ci | cj) >= 0 && scaled > tol_in;
+          const float rr = fmaf(sg4, scaled * scaled, nu2);
+          const float h = rsqrt_ftz(rr), w = scaled * h;
+          const float c2 = fmaf(0.5f * nu, h, 0.5f), cinv = rsqrt_ftz(c2);
+          float sa = w * cinv, ca = c2 * cinv;
+          // the cosine of a small angle as 1 -+ s^2 / 2 rounded once (rsqrt returns the value below 1
+          // too often there, and thousands of tiny rotations would shrink V: with it alone the
           // FP32-only eigenvalues of order 128 came out 5e-5 small, with this rule 2e-5)
-          const float y = sg * t * t, c0 = rsqrtf(1.0f + y);
-          const float c = fabsf(y) < 1.52587890625e-5f ? fmaf(-0.5f, y, 1.0f) : c0;
-          const float es = copysignf(t * c, aij < 0.0f ? -t : t);  // +- sin or sinh
-          const f2 q11 = f2_make(c, c), q12 = f2_make(es, es), q21 = f2_make(-sg * es, -sg * es);
+          const float y = sa * sa;
+          if (y < 3.8146973e-6f) ca = fmaf(-0.5f * sg, y, 1.0f);
+          // no hyperbolic angle annihilates a_ij (2 |a_ij| >= a_ii + a_jj by rounding): tanh = 0.9, the
+          // guard of Sec. 3.2
+          const bool guard = !(rr > 0.0f);
+          if (guard) {
+            ca = 2.2941573f;
+            sa = 2.0647416f;
+          }
+          const float c = rot ? ca : 1.0f;
+          const float es = rot ? __uint_as_float(__float_as_uint(sa) ^ ((__float_as_uint(aij) & 0x80000000u) ^ tsign)) : 0.0f;
+          const float q21 = -sg * es;
+          if (l == 0) sm.prm[buf][slot] = make_float4(c, es, q21, 0.0f);
+          rotate(c, es, q21);
+          my_rot += rot ? 1 : 0;
+          my_max = fmaxf(my_max, rot ? scaled : 0.0f);
           // a_ii' = a_ii - t |a_ij|, a_jj' = a_jj + t |a_ij| (trigonometric); both move by
-          // t |a_ij| (hyperbolic: the J-trace is invariant)
-          cni = fmaf(-sg * t, beta, cni);
-          cnj = fmaf(t, beta, cnj);
-          if (guard) {  // a_ij not annihilated: the norms from their definition
-            const float cc = c * c, ss = t * t * cc, cs = 2.0f * t * cc * beta;
-            cni = fmaf(cc, aii, fmaf(ss, ajj, cs)) - si * si;
-            cnj = fmaf(cc, ajj, fmaf(ss, aii, cs)) - sj * sj;
+          // t |a_ij| (hyperbolic: the J-trace is invariant); t = s / c, 1 / c = cinv.  Where the
+          // guard acted a_ij is not annihilated: both norms are put out of range, so that the columns
+          // rest until the next inner sweep takes them afresh
+          const float ta = rot ? __uint_as_float(__float_as_uint(sa * cinv * fabsf(aij)) ^ tsign) : 0.0f;
+          const bool far = rot && guard;
+          cni = far ? 1.0e8f * si * si : fmaf(-sg, ta, cni);
+          cnj = far ? 1.0e8f * sj * sj : cnj + ta;
+          // ---- pass one column on: the traveler round the ring, or at the end of the group's
+          // ring its split (first half: traveler to slot + g/2, which sends back its resident).  The
+          // two cases are uniform over the block and keep code of their own: with one code for both,
+          // the choice of the column split every warp
+          if (st_ < g - 1) {
+            const int dst = base + ((pos + 1) & (g - 1));
+            put(buf, dst, xj);
+            if (l == 0) sm.mst[buf][dst] = make_int4(cj, __float_as_int(cnj), __float_as_int(sj), jj);
+            half_sync<KM>();
+            const int4 m = sm.mst[buf][slot];
+            get(buf, xj);
+            cj = m.x;
+            cnj = __int_as_float(m.y);
+            sj = __int_as_float(m.z);
+            jj = m.w;
+          } else if (g > g_last) {
+            const bool res = pos >= g / 2;
+            const int dst = res ? slot - g / 2 : slot + g / 2;
+            if (res) put(buf, dst, xi);
+            else put(buf, dst, xj);
+            if (l == 0)
+              sm.mst[buf][dst] = res ? make_int4(ci, __float_as_int(cni), __float_as_int(si), ji)
+                                     : make_int4(cj, __float_as_int(cnj), __float_as_int(sj), jj);
+            half_sync<KM>();
+            const int4 m = sm.mst[buf][slot];
+            if (res) {
+              get(buf, xi);
+              ci = m.x;
+              cni = __int_as_float(m.y);
+              si = __int_as_float(m.z);
+              ji = m.w;
+            } else {
+              get(buf, xj);
+              cj = m.x;
+              cnj = __int_as_float(m.y);
+              sj = __int_as_float(m.z);
+              jj = m.w;
+            }
+          } else {
+            half_sync<KM>();
           }
-#pragma unroll
-          for (int u = 0; u < H; ++u) {
-            const f2 a_i = fi[u], a_j = fj[u];
-            fi[u] = f2_fma(q11, a_i, f2_mul(q21, a_j));
-            fj[u] = f2_fma(q11, a_j, f2_mul(q12, a_i));
-          }
-#pragma unroll
-          for (int u = 0; u < H; ++u) {
-            const f2 a_i = wi[u], a_j = wj[u];
-            wi[u] = f2_fma(q11, a_i, f2_mul(q21, a_j));
-            wj[u] = f2_fma(q11, a_j, f2_mul(q12, a_i));
-          }
-        }
-        // ---- pass one column on: the traveler round the ring, or at the end of the group's
-        // ring its split (first half: traveler to slot + g/2, which sends back its resident)
-        if (st_ < g - 1) {
-          send(base + ((pos + 1) & (g - 1)), fj, wj, cj, cnj, sj, jj);
-          core_sync<KM>();
-          receive(fj, wj, cj, cnj, sj, jj);
           buf ^= 1;
-        } else if (g > g_last) {
-          const bool give_res = pos >= g / 2;
-          const int dst = pos < g / 2 ? slot + g / 2 : slot - g / 2;
-          if (give_res) send(dst, fi, wi, ci, cni, si, ji);
-          else send(dst, fj, wj, cj, cnj, sj, jj);
-          core_sync<KM>();
-          if (give_res) receive(fi, wi, ci, cni, si, ji);
-          else receive(fj, wj, cj, cnj, sj, jj);
+        }
+      }
+    } else {
+      for (int g = P2; g >= g_last; g >>= 1) {
+        const int base = slot & ~(g - 1), pos = slot - base;
+        for (int st_ = 0; st_ < g; ++st_) {
+          half_sync<KM>();  // the parameters of this step, the columns passed on in the previous one
+          const float4 q = sm.prm[buf][slot];
+          if (st_ > 0) {
+            get(buf ^ 1, xj);
+          } else if (g < P2) {  // the split that ended the ring of 2 g slots
+            if (slot & g) get(buf ^ 1, xi);
+            else get(buf ^ 1, xj);
+          }
+          rotate(q.x, q.y, q.z);
+          if (st_ < g - 1) {
+            put(buf, base + ((pos + 1) & (g - 1)), xj);
+          } else if (g > g_last) {
+            if (pos >= g / 2) put(buf, slot - g / 2, xi);
+            else put(buf, slot + g / 2, xj);
+          }
           buf ^= 1;
         }
       }
@@ -864,21 +926,24 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
       sm.red_i[warp][1] = cnt;
       sm.red_f[warp][3] = my_max;
     }
-    core_sync<KM>();
+    __syncthreads();
     int tot = 0;
     float dmax = 0.0f;
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
+    for (int w = 0; w < NW / 2; ++w) {
       tot += sm.red_i[w][1];
       dmax = fmaxf(dmax, sm.red_f[w][3]);
     }
-    core_sync<KM>();
+    __syncthreads();
     total_rot += tot;
     // done when nothing was rotated, or when every rotated pair was already so small that the
     // next sweep (quadratic convergence: off-diagonals ~ k delta^2) would find nothing above tol_in
     if (tot == 0 || (float)k * dmax * dmax <= tol_in) break;
   }
   if (!pp.oriented && inner >= JAC_INNER_MAX_SWEEPS && tid == 0) atomicOr(err, JAC_DEVERR_INNER_LIMIT);
+  // which columns the slots of V hold now
+  if (is_f && l == 0) sm.mst[0][slot] = make_int4(ci, cj, ji, jj);
+  __syncthreads();
   // W = V - I.  The diagonal from the J-norm of the column, J_c sum_r J_r v_rc^2 = 1:
   // v_cc - 1 = -S / (1 + sqrt(1 - S)), S = J_c sum_{r != c} J_r v_rc^2, where S is small; the
   // rounded v_cc itself would lose W_cc ~ S / 2 below 2^-24
@@ -907,8 +972,11 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
     for (int u = 0; u < R; u += 4)
       *reinterpret_cast<float4*>(&Wf[c * LDW + l * R + u]) = make_float4(v[u], v[u + 1], v[u + 2], v[u + 3]);
   };
-  finish(ci, ji, wi);
-  finish(cj, jj, wj);
+  if (!is_f) {
+    const int4 m = sm.mst[0][slot];
+    finish(m.x, m.z, xi);
+    finish(m.y, m.w, xj);
+  }
   const long long t_inner = clock64();
   if (tid == 0) {
     sm.st.rotations = total_rot;
@@ -1252,13 +1320,13 @@ __device__ __forceinline__ bool pivot_guard(const JacProb& a, int s, int pair) {
 
 // Modes of the pivot kernel.  PV_FULL: phases 1-4 in one CTA (FP64 sweeps).  PV_CORE: phases 1-3,
 // V_P in FP64 storage from the FP32 transform (FP32 sweeps).  PV_SPLIT: phases 1-3, W handed to
-// k_pivot_orth: the core needs a quarter of the shared memory of phase 4, so four pivots run on an
+// k_pivot_orth: the core needs less than half the shared memory of phase 4, so three pivots run on an
 // SM while phase 4 takes the SM for a short time only (many pivots per step).  4000 problems of
-// orders 8..128, all pivots of a sweep step: 2.1 ms, against 4.1 ms with one 212 KB CTA per SM.
+// orders 8..128, all pivots of a sweep step: 1.4 ms, against 4.1 ms with one 212 KB CTA per SM.
 enum { PV_FULL = 0, PV_CORE = 1, PV_SPLIT = 2 };
 
 template <int KM, int MODE>
-__global__ void __launch_bounds__(MODE == PV_FULL ? 4 * KM : 2 * KM, MODE == PV_FULL ? (KM == 32 ? 4 : 1) : (KM == 32 ? 8 : 4))
+__global__ void __launch_bounds__(4 * KM, MODE == PV_FULL ? (KM == 32 ? 4 : 1) : (KM == 32 ? 6 : 3))
     k_pivot(const JacProb* __restrict__ probs, int s, PivotParams pp) {
   extern __shared__ __align__(16) unsigned char pv_raw[];
   PivotSmem<KM>& sm = *reinterpret_cast<PivotSmem<KM>*>(pv_raw);
@@ -1271,13 +1339,13 @@ __global__ void __launch_bounds__(MODE == PV_FULL ? 4 * KM : 2 * KM, MODE == PV_
     __syncthreads();
     const int k = sm.st.k;
     if constexpr (MODE == PV_CORE) {
-      write_vp<KM>(a, pair, k, sm.st.perm, sm.st.linv, 2 * KM, [&](int r, int c) {
+      write_vp<KM>(a, pair, k, sm.st.perm, sm.st.linv, 4 * KM, [&](int r, int c) {
         const float w = sm.Wf[c * PivotDim<KM>::LDW + r];
         return r == c ? oz_f2d(w) + 1.0 : oz_f2d(w);
       });
     } else {
       PivotHandoff<KM>& h = *reinterpret_cast<PivotHandoff<KM>*>(a.vp + (size_t)pair * a.apld * a.apld);
-      for (int e = tid; e < k * PivotDim<KM>::LDW / 4; e += 2 * KM)
+      for (int e = tid; e < k * PivotDim<KM>::LDW / 4; e += 4 * KM)
         reinterpret_cast<float4*>(h.W)[e] = reinterpret_cast<const float4*>(sm.Wf)[e];
       if (tid < KM) {
         h.perm[tid] = sm.st.perm[tid];
@@ -1290,12 +1358,8 @@ __global__ void __launch_bounds__(MODE == PV_FULL ? 4 * KM : 2 * KM, MODE == PV_
       stats[pair] = sm.st.st;
     }
   } else {
-    if (tid < PivotDim<KM>::NTC) {
-      const int code = pivot_core<KM, false>(sm.st, sm.work, nullptr, sm.Wf, a, s, pair, pp);
-      if (tid == 0) sm.st.code = code;
-    }
+    if (pivot_core<KM, false>(sm.st, sm.work, nullptr, sm.Wf, a, s, pair, pp) != 0) return;
     __syncthreads();
-    if (sm.st.code != 0) return;
     const int k = sm.st.k;
     int ns = 0;
     const bool ok = pivot_orth<KM>(sm.orth, sm.Wf, sm.st.jphys, k, pp.oz, ns);
@@ -1467,12 +1531,8 @@ __global__ void __launch_bounds__(4 * KM, KM == 32 ? 4 : 2)
   __syncthreads();
 
   // ---- 1.-3. the pivot
-  if (tid < PivotDim<KM>::NTC) {
-    const int code = pivot_core<KM, true>(sm.st, *reinterpret_cast<PivotWork<KM>*>(sm.work), sm.Wf, sm.Wf, a, s, pair, pp);
-    if (tid == 0) sm.st.code = code;
-  }
+  const int pr = pivot_core<KM, true>(sm.st, *reinterpret_cast<PivotWork<KM>*>(sm.work), sm.Wf, sm.Wf, a, s, pair, pp);
   __syncthreads();
-  const int pr = sm.st.code;  // uniform
   if (pr == 2) {
     // handed over: the FP64 pivot kernel reads A_P from the Gram output, as after the Gram kernel
     double* A = a.Ap + (size_t)pair * a.apld * a.apld;
@@ -1569,14 +1629,14 @@ template <int KM>
 static int launch_pivot(int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s, const PivotParams& pp) {
   const dim3 grid(max_half, nprob);
   if (!pp.ns_mode) {
-    k_pivot<KM, PV_CORE><<<grid, 2 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
+    k_pivot<KM, PV_CORE><<<grid, 4 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
     return 1;
   }
   if ((long long)max_half * nprob <= kSplitPivots) {
     k_pivot<KM, PV_FULL><<<grid, 4 * KM, sizeof(PivotSmem<KM>), st>>>(probs, s, pp);
     return 1;
   }
-  k_pivot<KM, PV_SPLIT><<<grid, 2 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
+  k_pivot<KM, PV_SPLIT><<<grid, 4 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
   k_pivot_orth<KM><<<grid, 4 * KM, sizeof(OrthSmem<KM>), st>>>(probs, s, pp);
   return 2;
 }
