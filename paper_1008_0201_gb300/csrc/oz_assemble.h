@@ -101,4 +101,32 @@ OZ_HD double oz_assemble(long long hi, long long lo, int sh, int e) {
   return oz_ldexp(m, p - 52 + e);
 }
 
+// The same for |hi| 2^sh + |lo| < 2^102 without a branch on the size: the sum is shifted so that its
+// leading bit is bit 127, the top 53 bits are rounded with the 75 below them, and the carry of the
+// rounding runs into the exponent field by itself.  ~45 instructions and no divergence, against ~75 with
+// three cases in oz_assemble; normal results, zero, and the rest by ldexp as there.
+OZ_HD double oz_assemble_small(long long hi, long long lo, int sh, int e) {
+  unsigned long long L = (unsigned long long)hi << sh;
+  long long H = hi >> (64 - sh);
+  const unsigned long long L2 = L + (unsigned long long)lo;
+  H += (lo >> 63) + (L2 < L ? 1 : 0);
+  const unsigned long long sg = (unsigned long long)(H >> 63);  // all ones when negative
+  unsigned long long uL = L2 ^ sg, uH = (unsigned long long)H ^ sg;
+  uL -= sg;
+  uH += (sg != 0 && uL == 0) ? 1ull : 0ull;
+  const bool wide = uH != 0;
+  const int lz = (wide ? 0 : 64) + oz_clz64(wide ? uH : uL);  // 128 for zero
+  const unsigned long long a = wide ? uH : uL, b = wide ? uL : 0ull;
+  const int s = lz & 63;
+  const unsigned long long hi64 = (a << s) | ((b >> 1) >> (63 - s)), lo64 = b << s;
+  const unsigned rem = (unsigned)hi64 & 0x7ffu;
+  unsigned long long mant = hi64 >> 11;
+  mant += (rem > 0x400u || (rem == 0x400u && (lo64 != 0 || (mant & 1ull)))) ? 1ull : 0ull;
+  const int be = 127 - lz + e + 1023;  // biased exponent of the leading bit
+  if (lz >= 128) return 0.0;
+  if (be >= 1 && be <= 2045) return oz_bits_to_double((sg << 63) + ((unsigned long long)(be - 1) << 52) + mant);
+  const double m = sg ? -(double)mant : (double)mant;  // exact: 53 bits
+  return oz_ldexp(m, 75 - lz + e);
+}
+
 }  // namespace jac

@@ -18,18 +18,16 @@ namespace jac {
 
 __device__ __forceinline__ int oz_pair_col(int c, int wp, int op, int oq) { return c < wp ? op + c : oq + (c - wp); }
 
-__device__ __forceinline__ int warp_max_i(int v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
 // ------------------------------------------------------------------------------------ Gram
 // Grid (half * CS, nprob), cluster (CS, 1, 1), 256 threads; the CS CTAs of a cluster split the
 // rows of one pair as in k_gram.  A CTA takes its rows in stages of 128: warp w loads columns
-// 8w..8w+7 (lane: rows 2 lane, 2 lane + 1, 64 + 2 lane, 65 + 2 lane), sets each column's bound
-// exponent E_c over the stage, and stores the digits D[t][c][row].  The 20 upper 16 x 8 tiles of
-// the 64 x 64 block go to the warps (at most 3 each) and are summed in FP64 across stages.
+// w, w + 8, .. (lane: rows 2 lane, 2 lane + 1, 64 + 2 lane, 65 + 2 lane), sets each column's bound
+// exponent E_c over the stage, and stores the digits D[t][c][row].  The upper 16 x 8 tiles of the
+// k x k block (20 at k = 64) go to the warps (at most 3 each) and are summed in FP64 across stages.
+// Columns, rows and tiles past k and past the rows are not formed, a level sum is rounded without an
+// FP64 instruction, and the cluster's sum adds only what is there: one block of 64 rows and 16
+// columns 21.5 -> 10.4 us, 4000 problems of orders 8..128 572 -> 265 us, 32 pairs of 2304 rows
+// 112 -> 94 us (mma.sync is then ~half of a stage).
 #define OZG_ROWS 128
 #define OZG_NL 8  // levels kept: the Gram's groups are its own columns, bounds within ~4x of the terms
 #define OZG_P (OZG_ROWS + 8)  // 272-byte digit rows: 16-byte aligned, ldmatrix conflict-free
@@ -39,12 +37,17 @@ struct OzGramSmem {
   int E[JAC_KMAX];
 };
 
-// idx-th upper tile (8 tj + 7 >= 16 ti) of the 4 x 8 tile grid: ti = 0: tj 0..7, 1: 2..7,
-// 2: 4..7, 3: 6..7
-__device__ __forceinline__ void oz_upper_tile(int idx, int& ti, int& tj) {
-  ti = (idx >= 18) ? 3 : (idx >= 14) ? 2 : (idx >= 8) ? 1 : 0;
-  const int start = (ti == 0) ? 0 : (ti == 1) ? 8 : (ti == 2) ? 14 : 18;
-  tj = 2 * ti + (idx - start);
+// idx-th upper tile (8 tj + 7 >= 16 ti) of a block of ntj 8-column tiles, row by row; false past the last
+__device__ __forceinline__ bool oz_upper_tile(int idx, int ntj, int& ti, int& tj) {
+  for (ti = 0; 2 * ti < ntj; ++ti) {
+    const int len = ntj - 2 * ti;
+    if (idx < len) {
+      tj = 2 * ti + idx;
+      return true;
+    }
+    idx -= len;
+  }
+  return false;
 }
 
 __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ probs, int s, int CS) {
@@ -58,10 +61,12 @@ __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ pro
   const int* sp = a.pairs + (size_t)s * a.half * 2;
   const int p = sp[2 * pair], q = sp[2 * pair + 1];
   const int op = a.boff[p], wp = a.boff[p + 1] - op, oq = a.boff[q], wq = a.boff[q + 1] - oq;
-  const int k = wp + wq;
+  const int k = wp + wq, ntj = (k + 7) >> 3;  // 8-column tiles
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
   const int rpc = ((a.mp / CS + 15) & ~15);
   const int r_begin = min(a.mp, crank * rpc), r_end = min(a.mp, r_begin + rpc);
+  // columns warp, warp + 8, ... below the last 16-column tile's end; columns >= k have zero digits
+  const int ncc = (((k + 15) & ~15) - warp + 7) >> 3;
 
   double tot[3][4];
 #pragma unroll
@@ -71,11 +76,12 @@ __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ pro
 
   for (int r0 = r_begin; r0 < r_end; r0 += OZG_ROWS) {
     const int rs = min(OZG_ROWS, r_end - r0);  // multiple of 16
+    const bool two = rs > 64;                  // rows 64.. of the stage
     // ---- load the stage (all loads first), bound exponents, digits
     double2 x[8][2];
 #pragma unroll
     for (int cc = 0; cc < 8; ++cc) {
-      const int c = 8 * warp + cc;
+      const int c = warp + 8 * cc;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const int r = 64 * i + 2 * lane;
@@ -84,25 +90,19 @@ __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ pro
                        : make_double2(0.0, 0.0);
       }
     }
-    int ec[8];
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
-      int e = max(max(oz_bexp(x[cc][0].x), oz_bexp(x[cc][0].y)), max(oz_bexp(x[cc][1].x), oz_bexp(x[cc][1].y)));
-      ec[cc] = warp_max_i(e);
-    }
     __syncthreads();  // the previous stage's digits and exponents are no longer read
-    if (lane == 0) {
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) sm.E[8 * warp + cc] = ec[cc];
-    }
 #pragma unroll
     for (int cc = 0; cc < 8; ++cc) {
-      const int c = 8 * warp + cc;
+      if (cc >= ncc) break;
+      const int c = warp + 8 * cc;
+      const int e = max(max(oz_bexp(x[cc][0].x), oz_bexp(x[cc][0].y)), max(oz_bexp(x[cc][1].x), oz_bexp(x[cc][1].y)));
+      const int ec = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+      if (lane == 0) sm.E[c] = ec;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
+        if (i == 1 && !two) break;
         unsigned w[OZ_T];
-        oz_split2(oz_biased(x[cc][i].x, oz_bexp(x[cc][i].x) - ec[cc]),
-                  oz_biased(x[cc][i].y, oz_bexp(x[cc][i].y) - ec[cc]), w);
+        oz_split2(oz_biased(x[cc][i].x, oz_bexp(x[cc][i].x) - ec), oz_biased(x[cc][i].y, oz_bexp(x[cc][i].y) - ec), w);
 #pragma unroll
         for (int t = 0; t < OZ_T; ++t) *reinterpret_cast<unsigned*>(&sm.D[t][c][64 * i + 2 * lane]) = w[t];
       }
@@ -112,10 +112,8 @@ __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ pro
     const int kend = (rs + 15) & ~15;
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
-      const int idx = warp + 8 * u;
-      if (idx >= 20) break;
       int ti, tj;
-      oz_upper_tile(idx, ti, tj);
+      if (!oz_upper_tile(warp + 8 * u, ntj, ti, tj)) break;
       float acc[OZG_NL][4];
 #pragma unroll
       for (int L = 0; L < OZG_NL; ++L)
@@ -137,41 +135,60 @@ __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ pro
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         const int i = 16 * ti + g + 8 * (v >> 1), j = 8 * tj + 2 * t4 + (v & 1);
-        tot[u][v] += oz_value<true>(acc, v, sm.E[i] + sm.E[j] - 2056);
+        const double y = oz_value_int(acc, v, sm.E[i] + sm.E[j] - 2056);
+        tot[u][v] = (r0 == r_begin) ? y : tot[u][v] + y;
       }
     }
   }
-  // ---- partial -> own shared memory: (i, j), j >= i, and its mirror
+  double* out = a.Ap + (size_t)pair * a.apld * a.apld;
+  if (CS == 1) {  // nothing to add up: (i, j), j >= i, and its mirror
 #pragma unroll
-  for (int u = 0; u < 3; ++u) {
-    const int idx = warp + 8 * u;
-    if (idx < 20) {
+    for (int u = 0; u < 3; ++u) {
       int ti, tj;
-      oz_upper_tile(idx, ti, tj);
+      if (!oz_upper_tile(warp + 8 * u, ntj, ti, tj)) break;
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         const int i = 16 * ti + g + 8 * (v >> 1), j = 8 * tj + 2 * t4 + (v & 1);
-        if (j >= i) {
-          sm.C[i][j] = tot[u][v];
-          sm.C[j][i] = tot[u][v];
+        if (j >= i && j < k) {
+          out[j * a.apld + i] = tot[u][v];
+          out[i * a.apld + j] = tot[u][v];
         }
       }
     }
+    return;
+  }
+  // ---- partial -> own shared memory: (i, j), j >= i
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    int ti, tj;
+    if (!oz_upper_tile(warp + 8 * u, ntj, ti, tj)) break;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) sm.C[16 * ti + g + 8 * (v >> 1)][8 * tj + 2 * t4 + (v & 1)] = tot[u][v];
   }
   cluster.sync();
-  const int totn = k * k, per = (totn + CS - 1) / CS;
+  // the upper triangle, rows n and k - 1 - n together as one row of k + 1 entries; only the CS - 1
+  // additions that are needed (an FP64 addition costs the SM 20 clocks per warp: sixteen for every
+  // entry of the full block, most of them of zeros, were a third of a single-stage Gram)
+  const int totn = ((k + 1) >> 1) * (k + 1), per = (totn + CS - 1) / CS;
   const int e0 = crank * per, e1 = min(totn, e0 + per);
-  double* out = a.Ap + (size_t)pair * a.apld * a.apld;
   for (int e = e0 + tid; e < e1; e += 256) {
-    const int i = e % k, j = e / k;
+    const int n = e / (k + 1), o = e - n * (k + 1);
+    int i = n, j = n + o;
+    if (j >= k) {
+      i = k - 1 - n;
+      j = i + (o - (k - n));
+      if (i == n) continue;  // the middle row of an odd block
+    }
     double part[16];  // all remote loads issued before the fixed-order sum
 #pragma unroll
     for (int rk = 0; rk < 16; ++rk)
       part[rk] = (rk < CS) ? cluster.map_shared_rank(&sm.C[0][0], rk)[i * (JAC_KMAX + 1) + j] : 0.0;
-    double sum = 0.0;
+    double sum = part[0];
 #pragma unroll
-    for (int rk = 0; rk < 16; ++rk) sum += part[rk];
+    for (int rk = 1; rk < 16; ++rk)
+      if (rk < CS) sum += part[rk];
     out[j * a.apld + i] = sum;
+    out[i * a.apld + j] = sum;
   }
   cluster.sync();  // keep every partial alive until all remote reads are done
 }

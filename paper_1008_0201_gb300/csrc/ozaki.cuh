@@ -21,6 +21,8 @@
 #pragma once
 #include <cuda_fp16.h>
 
+#include "oz_assemble.h"
+
 namespace jac {
 
 #define OZ_T 8  // digits per value
@@ -133,6 +135,16 @@ __device__ __forceinline__ double oz_value(const float (&acc)[NL][4], int v, int
   const double s = fma(oz_i2d(hi), (double)(1ll << (7 * (NL - 4))), oz_i2d(lo));
   const int e = E - 7 * (NL - 1);
   return (e >= -1022 && e <= 1023) ? s * __longlong_as_double((long long)(e + 1023) << 52) : ldexp(s, e);
+}
+
+// The same value without an FP64 instruction (NL = 8, |acc_L| <= 2^22): both round the exact sum once
+__device__ __forceinline__ double oz_value_int(const float (&acc)[8][4], int v, int E) {
+  int q[8];
+#pragma unroll
+  for (int L = 0; L < 8; ++L) q[L] = f32_small_int(acc[L][v]);
+  const long long hi = (long long)(q[0] * 128 + q[1]) * 16384 + (q[2] * 128 + q[3]);
+  const long long lo = (long long)(q[4] * 128 + q[5]) * 16384 + (q[6] * 128 + q[7]);
+  return oz_assemble_small(hi, lo, 28, E - 49);
 }
 
 // (double)f by integer operations (FP32 subnormals flush to zero)

@@ -51,8 +51,8 @@ __device__ __forceinline__ int warp_max_int(int v) {
 
 size_t tc_update_oz_smem_bytes() { return TD_SMEM; }
 
-// the integer rounding, called rather than inlined: it runs once per output and keeping it out of
-// line keeps the unrolled kernels within the instruction cache
+// the integer rounding of k_gram_oz_tc, called rather than inlined: keeping it out of line keeps the
+// unrolled kernel within the instruction cache
 __device__ __noinline__ double oz_assemble_call(long long hi, long long lo, int sh, int e) {
   return oz_assemble(hi, lo, sh, e);
 }
@@ -82,7 +82,6 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tb = *tslot;
-  constexpr uint32_t idesc = tc::idesc_f32acc(tc::FMT_F16, 128, 64, 0, 0);
   const uint32_t xs = tc::smem_u32(sm + TD_XOFF), vs = tc::smem_u32(sm + TD_VOFF);
   // tile row r and output columns 16 cq .. + 15 of this thread, for the loads and digits of X~
   // and for the epilogue (warp w reads TMEM lanes 32 (w & 3) .. + 31: tid & 127 = r)
@@ -104,6 +103,14 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     const int ld = isg ? a.mp : a.np;
     const int r0 = (isg ? t : t - gtiles) << 7;
     const int rows = min(128, (isg ? a.mp : a.np) - r0);
+    // What lies past the tile's rows or the pair's columns is not formed: a warp whose 32 rows or 16
+    // columns lie past them rests, the contraction takes ceil(k / 16) steps of 16 and the product
+    // N = 16 ceil(k / 16) columns.  (Operand rows left unwritten reach only their own, unread, rows or
+    // columns of the product.)  One pair of 64 rows and 16 columns 25.6 -> 17.9 us, 4000 problems of
+    // orders 8..128 819 -> 756 us.
+    const int k16 = (k + 15) >> 4;
+    const bool works = 32 * (warp & 3) < rows && cq < k16;  // uniform per warp: its part of X~ and of Y
+    const bool vworks = vc < 16 * k16 && vk0 < 16 * k16;    // its part of V~
     // ---- loads (all issued before use)
     double x[16], v[8];
 #pragma unroll
@@ -117,14 +124,16 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     if (tid < 128) rexp[tid] = TD_NO_EXP;
     __syncthreads();
     // ---- column bounds c_k of the tile (a warp holds 32 rows of 16 columns)
+    if (works) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int e = warp_max_int(oz_bexp(x[j]));
-      if (lane == 0 && e > 0) atomicMax(&cexp[16 * cq + j], e);
+      for (int j = 0; j < 16; ++j) {
+        const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)oz_bexp(x[j]));
+        if (lane == 0 && e > 0) atomicMax(&cexp[16 * cq + j], e);
+      }
     }
     __syncthreads();
     // ---- row groups of X~ and column groups of V~
-    {
+    if (works) {
       int m = TD_NO_EXP;
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
@@ -132,6 +141,8 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
         if (ex != 0) m = max(m, ex - cexp[16 * cq + j]);
       }
       if (m != TD_NO_EXP) atomicMax(&rexp[r], m);
+    }
+    {
       int mv = TD_NO_EXP;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
@@ -145,7 +156,7 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     // the previous tile's MMAs were waited for before its epilogue: the planes are free
     __syncthreads();
     // ---- digits of X~ (row r) and of V~ (operand row vc): 16-byte stores, 8 K entries each
-    {
+    if (works) {
       const int ea = rexp[r];
 #pragma unroll
       for (int j0 = 0; j0 < 16; j0 += 8) {
@@ -165,6 +176,8 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
           *reinterpret_cast<uint4*>(sm + TD_XOFF + tt * TD_XPLANE + off) = make_uint4(w[tt][0], w[tt][1], w[tt][2],
                                                                                       w[tt][3]);
       }
+    }
+    if (vworks) {
       const int ev = vexp[vc];
       unsigned w[OZ_T][4];
 #pragma unroll
@@ -185,10 +198,11 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     tc::fence_proxy_async_smem();
     __syncthreads();
     // ---- levels 0..7: block L (TMEM columns 64 L ..) accumulates sum_{t+u=L} X_t V_u
+    const uint32_t idesc = tc::idesc_f32acc(tc::FMT_F16, 128, 16 * k16, 0, 0);
     if (tid == 0) {
       tc::fence_after_sync();
 #pragma unroll 1
-      for (int kk = 0; kk < 4; ++kk)
+      for (int kk = 0; kk < k16; ++kk)
 #pragma unroll 1
         for (int L = 0; L < OZ_T; ++L)
           for (int tt = 0; tt <= L; ++tt)
@@ -203,63 +217,78 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     }
     tc::fence_after_sync();
     uint32_t l0[16];
-    tc::tmem_ld16(lrow, l0);
-    tc::tmem_wait_ld();
+    if (works) {
+      tc::tmem_ld16(lrow, l0);
+      tc::tmem_wait_ld();
+    }
     tc::fence_before_sync();
     __syncthreads();  // level 0 read everywhere: block 0 is free for level 8
     if (tid == 0) {
       tc::fence_after_sync();
 #pragma unroll 1
-      for (int kk = 0; kk < 4; ++kk)
+      for (int kk = 0; kk < k16; ++kk)
         for (int tt = 1; tt < OZ_T; ++tt)
           tc::mma_f16(tb, tc::desc_sw128(xs + tt * TD_XPLANE + kk * 32, 16, 1024),
                       tc::desc_sw128(vs + (8 - tt) * TD_VPLANE + kk * 32, 16, 1024), idesc,
                       (kk > 0 || tt > 1) ? 1u : 0u);
       tc::mma_commit(&bar[1]);
     }
-    // levels 1, then 2 and 3, 4 and 5, 6 and 7: two levels are joined in 32 bits
-    long long hi[16], lo[16];
-    {
-      uint32_t lv[16];
-      tc::tmem_ld16(lrow + 64, lv);
-      tc::tmem_wait_ld();
+    // eight output columns at a time (sixteen at once need all the registers and spill): levels 1..7,
+    // two levels joined in 32 bits, then level 8
+    const int ea = rexp[r];
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      int q01[8], q23[8], q45[8], q67[8];
+      if (works) {
+        uint32_t la[8], lb[8], lc[8];
+        tc::tmem_ld8(lrow + 64 + 8 * h, la);
+        tc::tmem_ld8(lrow + 128 + 8 * h, lb);
+        tc::tmem_ld8(lrow + 192 + 8 * h, lc);
+        tc::tmem_wait_ld();
 #pragma unroll
-      for (int j = 0; j < 16; ++j)
-        hi[j] = f32_small_int(__uint_as_float(l0[j])) * 128 + f32_small_int(__uint_as_float(lv[j]));
-    }
+        for (int j = 0; j < 8; ++j) {
+          q01[j] = f32_small_int(__uint_as_float(h ? l0[8 + j] : l0[j])) * 128 + f32_small_int(__uint_as_float(la[j]));
+          q23[j] = f32_small_int(__uint_as_float(lb[j])) * 128 + f32_small_int(__uint_as_float(lc[j]));
+        }
+        tc::tmem_ld8(lrow + 256 + 8 * h, la);
+        tc::tmem_ld8(lrow + 320 + 8 * h, lb);
+        tc::tmem_wait_ld();
 #pragma unroll
-    for (int L = 2; L < OZ_T; L += 2) {
-      uint32_t la[16], lb[16];
-      tc::tmem_ld16(lrow + 64 * L, la);
-      tc::tmem_ld16(lrow + 64 * L + 64, lb);
-      tc::tmem_wait_ld();
+        for (int j = 0; j < 8; ++j)
+          q45[j] = f32_small_int(__uint_as_float(la[j])) * 128 + f32_small_int(__uint_as_float(lb[j]));
+        tc::tmem_ld8(lrow + 384 + 8 * h, la);
+        tc::tmem_ld8(lrow + 448 + 8 * h, lb);
+        tc::tmem_wait_ld();
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int q = f32_small_int(__uint_as_float(la[j])) * 128 + f32_small_int(__uint_as_float(lb[j]));
-        if (L == 2) hi[j] = (long long)(int)hi[j] * 16384 + q;
-        else if (L == 4) lo[j] = q;
-        else lo[j] = (long long)(int)lo[j] * 16384 + q;
+        for (int j = 0; j < 8; ++j)
+          q67[j] = f32_small_int(__uint_as_float(la[j])) * 128 + f32_small_int(__uint_as_float(lb[j]));
       }
-    }
-    if (__syncthreads_or(!tc::mbar_wait(&bar[1], it & 1))) {
-      bad = true;
-      break;
-    }
-    tc::fence_after_sync();
-    tc::tmem_ld16(lrow, l0);
-    tc::tmem_wait_ld();
-    if (r < rows) {
-      const int ea = rexp[r];
+      if (h == 0) {
+        if (__syncthreads_or(!tc::mbar_wait(&bar[1], it & 1))) {
+          bad = true;
+          break;
+        }
+        tc::fence_after_sync();
+      }
+      if (works) {
+        uint32_t l8[8];
+        tc::tmem_ld8(lrow + 8 * h, l8);
+        tc::tmem_wait_ld();
+        if (r < rows) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int c = 16 * cq + j;
-        if (c < k) {
-          const long long lf = lo[j] * 128 + f32_small_int(__uint_as_float(l0[j]));
-          base[(size_t)(c < wp ? op + c : oq + c - wp) * ld + r0 + r] =
-              oz_assemble_call(hi[j], lf, 35, ea + vexp[c] - 2056 - 56);
+          for (int j = 0; j < 8; ++j) {
+            const int c = 16 * cq + 8 * h + j;
+            if (c < k) {
+              const long long hi = (long long)q01[j] * 16384 + q23[j];
+              const long long lo = ((long long)q45[j] * 16384 + q67[j]) * 128 + f32_small_int(__uint_as_float(l8[j]));
+              base[(size_t)(c < wp ? op + c : oq + c - wp) * ld + r0 + r] =
+                  oz_assemble_small(hi, lo, 35, ea + vexp[c] - 2056 - 56);
+            }
+          }
         }
       }
     }
+    if (bad) break;
     tc::fence_before_sync();
     __syncthreads();  // TMEM and the exponent arrays read before the next tile reuses them
     ++it;
