@@ -685,14 +685,14 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
   const float tol_in = fmaxf(0.5f * tolf, 64.0f * 5.9604645e-8f * mx);
   // The columns live in registers: pair slot q (LPP lanes of a warp) holds a resident and a
   // traveler column of R and of V, R rows per lane (row l R + u in lane l), as row pairs.  An inner
-  // sweep is a recursive cross ordering of the KM positions: at group size g (KM/2, KM/4, ..., 1
+  // sweep is a recursive cross ordering of 2 p2 >= k positions: at group size g (p2, p2/2, ..., 1
   // slots) the travelers of each group go round its ring of g slots, so every resident meets every
   // traveler of the group in g steps; then each group splits in two, its residents pairing among
   // themselves in the first half and its travelers in the second.  Every pair of positions
-  // meets once in KM - 1 steps, and between steps each slot passes exactly one column to one
+  // meets once in 2 p2 - 1 steps, and between steps each slot passes exactly one column to one
   // other slot through a shared-memory mailbox: one barrier per step.  Positions >= k are
   // empty.  The logical order of Algorithm 3.3 (reversed J = -1 part) gives the initial
-  // placement: position p is the resident of slot p (p < KM/2) or the traveler of slot p - KM/2.
+  // placement: position p is the resident of slot p (p < p2) or the traveler of slot p - p2.
   // What bounds a step is its chain: mailbox, dot product and its reduction, the parameters, the
   // rotation, mailbox, barrier.  The columns of V are not on it: they belong to the second half of
   // the threads, which rotate them one barrier later, with the parameters the first half left in
@@ -702,11 +702,14 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
   // and the exchange of the parameters cost more than the mailboxes).
   const bool is_f = tid < D::NF;
   const int slot = (is_f ? tid : tid - D::NF) / LPP, l = tid % LPP;
-  const int ci0 = cross_only ? sm.pres[slot] : ((slot < k) ? sm.lpos[slot] : -1);
-  const int cj0 = cross_only ? sm.ptrav[slot] : ((slot + P2 < k) ? sm.lpos[slot + P2] : -1);
+  // only as many slots as k needs (a power of two): a block of 16 columns takes 15 steps per sweep, not
+  // the 31 of 32 columns (64 x 64 problem of width 8: 46k clocks of inner sweeps per pivot, now 24k)
+  const int p2 = 1 << (32 - __clz((k + 1) / 2 - 1));
+  const int ci0 = cross_only ? sm.pres[slot] : ((slot < p2 && slot < k) ? sm.lpos[slot] : -1);
+  const int cj0 = cross_only ? sm.ptrav[slot] : ((slot < p2 && slot + p2 < k) ? sm.lpos[slot + p2] : -1);
   // block-oriented: one inner sweep; after the first step of an outer sweep only the ring of
   // its first level (every column of block p meets every column of block q once)
-  const int g_last = cross_only ? P2 : 1;
+  const int g_last = cross_only ? p2 : 1;
   const int max_inner = pp.oriented ? 1 : JAC_INNER_MAX_SWEEPS;
   f2 xi[H], xj[H];  // resident and traveler of this half's columns
   float cni = 0.0f, cnj = 0.0f, si = 1.0f, sj = 1.0f;  // ||r||^2 = s^2 + cn
@@ -791,7 +794,7 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
         fresh(xi, cni, si);
         fresh(xj, cnj, sj);
       }
-      for (int g = P2; g >= g_last; g >>= 1) {
+      for (int g = p2; g >= g_last; g >>= 1) {
         const int base = slot & ~(g - 1), pos = slot - base;
         for (int st_ = 0; st_ < g; ++st_) {
           // ---- rotate the pair (ci, cj) of this slot; what does not depend on the dot product first.
@@ -897,14 +900,14 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
         }
       }
     } else {
-      for (int g = P2; g >= g_last; g >>= 1) {
+      for (int g = p2; g >= g_last; g >>= 1) {
         const int base = slot & ~(g - 1), pos = slot - base;
         for (int st_ = 0; st_ < g; ++st_) {
           half_sync<KM>();  // the parameters of this step, the columns passed on in the previous one
           const float4 q = sm.prm[buf][slot];
           if (st_ > 0) {
             get(buf ^ 1, xj);
-          } else if (g < P2) {  // the split that ended the ring of 2 g slots
+          } else if (g < p2) {  // the split that ended the ring of 2 g slots
             if (slot & g) get(buf ^ 1, xi);
             else get(buf ^ 1, xj);
           }
