@@ -450,10 +450,20 @@ int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, in
   else if (lowp)
     k_update32<<<dim3(max_half, tslabs, count), 256, 0, st>>>(dprobs, s, gslabs);
   else if (pp.oz) {
-    // tensor-core digit update: persistent CTAs (one per SM) over the (pair, 128-row tile) items
-    // of each problem (tslabs counts 64-row slabs)
-    const int items = max_half * ((tslabs + 1) / 2 + 1);
-    const int nx = std::max(1, std::min(items, (152 + count - 1) / count));
+    // tensor-core digit update: one CTA per SM walks (pair, 128-row tile) items of its problem
+    // (tslabs counts 64-row slabs, gslabs those of G).  nx CTAs per problem: the count whose last
+    // wave leaves the fewest SMs idle, the larger number of items per CTA on ties (256 x 256 problems,
+    // 96 at once: 8 items each, 166 us with 2 CTAs per problem, 129 us with this rule).
+    const int items = max_half * ((gslabs + 1) / 2 + (tslabs - gslabs + 1) / 2);
+    int nx = 1;
+    long long best = -1;
+    for (int c = 1; c <= std::min(items, 152); ++c) {
+      const long long t = (((long long)count * c + 151) / 152) * ((items + c - 1) / c);
+      if (best < 0 || t < best) {
+        best = t;
+        nx = c;
+      }
+    }
     k_update_oz_tc<<<dim3(nx, 1, count), 512, tc_update_oz_smem_bytes(), st>>>(dprobs, s);
   }
   else
