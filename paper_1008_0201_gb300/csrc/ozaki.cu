@@ -208,7 +208,9 @@ size_t oz_gram_smem_bytes() { return sizeof(OzGramSmem); }
 // Per segment the scales are those of the digit update (tc_digits.cu): c_r = bound exponent of column r of the CTA's
 // op(A) rows, then the rows of op(A) D^-1 and the columns of D op(B) (D = diag(2^c_r)) are the
 // scale groups, so a term is exact to 2^-53 of its own row and column sizes even when the columns
-// of A (or rows of B) are graded.  Grid (ceil(Mr/64), ceil(Nc/32), batch), 256 threads: warp w
+// of A (or rows of B) are graded.  Two CTAs per SM (112 KB each): the digits of one are made while
+// the other multiplies; with integer rounding and coalesced column bounds the adjoint of 256 problems
+// of order 256 takes 4.71 ms instead of 6.62.  Grid (ceil(Mr/64), ceil(Nc/32), batch), 256 threads: warp w
 // computes row tile w & 3 (16 rows) and column tiles 2 (w >> 2) + {0, 1}.
 #define OZM_TI 64
 #define OZM_TJ 32
@@ -224,7 +226,7 @@ struct OzGemmSmem {
   int cexp[OZM_TJ];
 };
 
-__global__ void __launch_bounds__(256) k_gemm_oz(int Mr, int Nc, int K, const double* __restrict__ A, int lda,
+__global__ void __launch_bounds__(256, 2) k_gemm_oz(int Mr, int Nc, int K, const double* __restrict__ A, int lda,
                                                 int transA, const double* __restrict__ B, int ldb,
                                                 const int8_t* __restrict__ sb, const int8_t* __restrict__ dsub,
                                                 double* __restrict__ C, int ldc, int sym, int transB, long long sa,
@@ -241,7 +243,7 @@ __global__ void __launch_bounds__(256) k_gemm_oz(int Mr, int Nc, int K, const do
   const bool rowok = i0 + ai < Mr, colok = j0 + bj < Nc;
   const int ti = warp & 3, tj0 = 2 * (warp >> 2);
   const int arow = 16 * ti + (lane & 7) + 8 * ((lane >> 3) & 1), akof = 8 * (lane >> 4);
-  const int bcol = 8 * tj0 + (lane & 7) + 8 * (lane >> 4), bkof = 8 * ((lane >> 3) & 1);
+  const int bcol = 8 * tj0 + (lane & 7), bkof = 8 * ((lane >> 3) & 1);
   auto a_at = [&](int i, int r) -> double {  // op(A)[i0 + i][r], in range
     return transA ? A[(size_t)(i0 + i) * lda + r] : A[(size_t)r * lda + i0 + i];
   };
@@ -257,16 +259,25 @@ __global__ void __launch_bounds__(256) k_gemm_oz(int Mr, int Nc, int K, const do
     for (int e = 0; e < 4; ++e) res[h][e] = 0.0;
   for (int s0 = 0; s0 < K; s0 += OZM_SEG) {
     const int slen = min(OZM_SEG, K - s0);
-    // ---- c_r: thread tid takes column r = s0 + tid of the CTA's op(A) rows
-    {
+    // ---- c_r of the CTA's op(A) rows, the lanes along the contiguous index: thread tid takes column
+    // s0 + tid (rows of A contiguous in r), or warp w columns w, w + 8, ..
+    __syncthreads();  // the previous segment's exponents are no longer read
+    if (transA) {
       int c = 0;
       if (tid < slen) {
         const int imax = min(OZM_TI, Mr - i0);
 #pragma unroll 16
         for (int i = 0; i < imax; ++i) c = max(c, oz_bexp(a_at(i, s0 + tid)));
       }
-      __syncthreads();  // the previous segment's exponents are no longer read
       sm.ck[tid] = c;
+    } else {
+#pragma unroll 8
+      for (int r = warp; r < slen; r += 8) {
+        const int e0 = (i0 + lane < Mr) ? oz_bexp(a_at(lane, s0 + r)) : 0;
+        const int e1 = (i0 + lane + 32 < Mr) ? oz_bexp(a_at(lane + 32, s0 + r)) : 0;
+        const unsigned c = __reduce_max_sync(0xffffffffu, (unsigned)max(e0, e1));
+        if (lane == 0) sm.ck[r] = (int)c;
+      }
     }
     __syncthreads();
     // ---- row groups of op(A) D^-1 and column groups of D op(B)
@@ -304,54 +315,57 @@ __global__ void __launch_bounds__(256) k_gemm_oz(int Mr, int Nc, int K, const do
         acc1[L][e] = 0.0f;
       }
     for (int kc = 0; kc < slen; kc += OZM_KC) {
-      // ---- chunk values (all loads first), digits
-      double xa[16], xb[8];
+      // ---- digits of the chunk, A then B (the other CTA of the SM hides the loads)
+      {
+        double xa[16];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {  // pairs of neighbours: one 32-bit store per digit
-        const int r = kc + 2 * ar + 8 * (u >> 1) + (u & 1);
-        xa[u] = (rowok && r < slen) ? a_at(ai, s0 + r) : 0.0;
+        for (int u = 0; u < 16; ++u) {  // pairs of neighbours: one 32-bit store per digit
+          const int r = kc + 2 * ar + 8 * (u >> 1) + (u & 1);
+          xa[u] = (rowok && r < slen) ? a_at(ai, s0 + r) : 0.0;
+        }
+        __syncthreads();  // the previous chunk's digits are consumed
+#pragma unroll
+        for (int u = 0; u < 16; u += 2) {
+          const int rl = 2 * ar + 8 * (u >> 1), r = kc + rl;
+          unsigned w[OZ_T];
+          const int c0 = (r < slen) ? sm.ck[r] : 0, c1 = (r + 1 < slen) ? sm.ck[r + 1] : 0;
+          oz_split2(oz_biased(xa[u], oz_bexp(xa[u]) - c0 - my_ea), oz_biased(xa[u + 1], oz_bexp(xa[u + 1]) - c1 - my_ea), w);
+#pragma unroll
+          for (int t = 0; t < OZ_T; ++t) *reinterpret_cast<unsigned*>(&sm.A[t][ai][rl]) = w[t];
+        }
       }
+      {
+        double xb[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int r = kc + 2 * br + 16 * (u >> 1) + (u & 1);
-        xb[u] = (colok && r < slen) ? b_at(bj, s0 + r) : 0.0;
-      }
-      __syncthreads();  // the previous chunk's digits are consumed
+        for (int u = 0; u < 8; ++u) {
+          const int r = kc + 2 * br + 16 * (u >> 1) + (u & 1);
+          xb[u] = (colok && r < slen) ? b_at(bj, s0 + r) : 0.0;
+        }
 #pragma unroll
-      for (int u = 0; u < 16; u += 2) {
-        const int rl = 2 * ar + 8 * (u >> 1), r = kc + rl;
-        unsigned w[OZ_T];
-        const int c0 = (r < slen) ? sm.ck[r] : 0, c1 = (r + 1 < slen) ? sm.ck[r + 1] : 0;
-        oz_split2(oz_biased(xa[u], oz_bexp(xa[u]) - c0 - my_ea), oz_biased(xa[u + 1], oz_bexp(xa[u + 1]) - c1 - my_ea), w);
+        for (int u = 0; u < 8; u += 2) {
+          const int rl = 2 * br + 16 * (u >> 1), r = kc + rl;
+          unsigned w[OZ_T];
+          const int c0 = (r < slen) ? sm.ck[r] : 0, c1 = (r + 1 < slen) ? sm.ck[r + 1] : 0;
+          oz_split2(c0 != 0 ? oz_biased(xb[u], oz_bexp(xb[u]) + c0 - my_eb) : OZ_BIAS,
+                    c1 != 0 ? oz_biased(xb[u + 1], oz_bexp(xb[u + 1]) + c1 - my_eb) : OZ_BIAS, w);
 #pragma unroll
-        for (int t = 0; t < OZ_T; ++t) *reinterpret_cast<unsigned*>(&sm.A[t][ai][rl]) = w[t];
-      }
-#pragma unroll
-      for (int u = 0; u < 8; u += 2) {
-        const int rl = 2 * br + 16 * (u >> 1), r = kc + rl;
-        unsigned w[OZ_T];
-        const int c0 = (r < slen) ? sm.ck[r] : 0, c1 = (r + 1 < slen) ? sm.ck[r + 1] : 0;
-        oz_split2(c0 != 0 ? oz_biased(xb[u], oz_bexp(xb[u]) + c0 - my_eb) : OZ_BIAS,
-                  c1 != 0 ? oz_biased(xb[u + 1], oz_bexp(xb[u + 1]) + c1 - my_eb) : OZ_BIAS, w);
-#pragma unroll
-        for (int t = 0; t < OZ_T; ++t) *reinterpret_cast<unsigned*>(&sm.B[t][bj][rl]) = w[t];
+          for (int t = 0; t < OZ_T; ++t) *reinterpret_cast<unsigned*>(&sm.B[t][bj][rl]) = w[t];
+        }
       }
       __syncthreads();
+      const int kend = min(OZM_KC, (slen - kc + 15) & ~15);
 #pragma unroll 1
-      for (int kk = 0; kk < OZM_KC; kk += 16) {
-        unsigned fa[OZ_T][4], fb0[OZ_T][2], fb1[OZ_T][2];
+      for (int kk = 0; kk < kend; kk += 16) {
+        unsigned fa[OZ_T][4], fb[OZ_T][2];
 #pragma unroll
         for (int t = 0; t < OZ_T; ++t) {
-          unsigned r4[4];
           oz_ldsm4(fa[t], &sm.A[t][arow][kk + akof]);
-          oz_ldsm4(r4, &sm.B[t][bcol][kk + bkof]);
-          fb0[t][0] = r4[0];
-          fb0[t][1] = r4[1];
-          fb1[t][0] = r4[2];
-          fb1[t][1] = r4[3];
+          oz_ldsm2(fb[t][0], fb[t][1], &sm.B[t][bcol][kk + bkof]);
         }
-        oz_levels(acc0, fa, fb0);
-        oz_levels(acc1, fa, fb1);
+        oz_levels(acc0, fa, fb);
+#pragma unroll
+        for (int t = 0; t < OZ_T; ++t) oz_ldsm2(fb[t][0], fb[t][1], &sm.B[t][bcol + 8][kk + bkof]);
+        oz_levels(acc1, fa, fb);
       }
     }
     // ---- the segment's exact level sums into FP64
@@ -359,8 +373,10 @@ __global__ void __launch_bounds__(256) k_gemm_oz(int Mr, int Nc, int K, const do
     for (int e = 0; e < 4; ++e) {
       const int il = 16 * ti + g + 8 * (e >> 1);
       const int jl0 = 8 * tj0 + 2 * t4 + (e & 1), jl1 = jl0 + 8;
-      res[0][e] += oz_value<false>(acc0, e, sm.rexp[il] + sm.cexp[jl0] - 2056);
-      res[1][e] += oz_value<false>(acc1, e, sm.rexp[il] + sm.cexp[jl1] - 2056);
+      const double y0 = oz_value9(acc0, e, sm.rexp[il] + sm.cexp[jl0] - 2056);
+      const double y1 = oz_value9(acc1, e, sm.rexp[il] + sm.cexp[jl1] - 2056);
+      res[0][e] = s0 == 0 ? y0 : res[0][e] + y0;
+      res[1][e] = s0 == 0 ? y1 : res[1][e] + y1;
     }
   }
 #pragma unroll

@@ -105,39 +105,17 @@ __device__ __forceinline__ void oz_levels(float (&acc)[NL][4], const unsigned (&
     for (int L = t; L < (t + OZ_T < NL ? t + OZ_T : NL); ++L) oz_mma(acc[L], fa[t], fb[L - t][0], fb[L - t][1]);
 }
 
-// GB300 issues ~1.6 FP64 operations per clock per SM (FP32: 128), so the recombination avoids
-// FP64 work: the integer level sums are gathered exactly in two int64 (hi: L = 0..3 in units of
-// level 3, lo: L = 4..NL-1 in units of level NL-1, both below 2^51 for level sums below 2^23),
-// turned into doubles by the exponent-bias trick and joined with one rounding: 4 FP64
-// operations per value, against ~25 for a per-level sum and ldexp.
-
-// exact double of an integer |x| < 2^51: the bits of 1.5 * 2^52 + x are those of 1.5 * 2^52
-// plus x
-__device__ __forceinline__ double oz_i2d(long long x) {
-  return __longlong_as_double(0x4338000000000000ll + x) - 6755399441055744.0;
-}
+// GB300 issues ~1.6 FP64 operations per clock per SM (FP32: 128), so the recombination takes none:
+// the integer level sums are gathered exactly in two int64 (hi: L = 0..3 in units of level 3, lo: L =
+// 4..NL-1 in units of level NL-1, both below 2^52 for level sums below 2^23) and rounded once to
+// double by integer instructions (oz_assemble_small).
 
 // an FP32 value that holds an integer of magnitude <= 2^22, as that integer (one FP32 add: the
 // integer lands in the low mantissa bits of 1.5 * 2^23 + x)
 __device__ __forceinline__ int f32_small_int(float x) { return __float_as_int(x + 12582912.0f) - 0x4B400000; }
 
-// 2^E sum_L acc_L 2^(-7 L), the acc_L exact integers held in FP32; SMALL: |acc_L| <= 2^22 (up to
-// 128 terms), which spares the conversion instructions.  Two levels are joined in 32 bits.
-template <bool SMALL, int NL>
-__device__ __forceinline__ double oz_value(const float (&acc)[NL][4], int v, int E) {
-  static_assert(NL == 8 || NL == 9, "two int64 accumulators");
-  int q[NL];
-#pragma unroll
-  for (int L = 0; L < NL; ++L) q[L] = SMALL ? f32_small_int(acc[L][v]) : __float2int_rn(acc[L][v]);
-  const long long hi = (long long)(q[0] * 128 + q[1]) * 16384 + (q[2] * 128 + q[3]);
-  long long lo = (long long)(q[4] * 128 + q[5]) * 16384 + (q[6] * 128 + q[7]);
-  if constexpr (NL == 9) lo = lo * 128 + q[8];
-  const double s = fma(oz_i2d(hi), (double)(1ll << (7 * (NL - 4))), oz_i2d(lo));
-  const int e = E - 7 * (NL - 1);
-  return (e >= -1022 && e <= 1023) ? s * __longlong_as_double((long long)(e + 1023) << 52) : ldexp(s, e);
-}
-
-// The same value without an FP64 instruction (NL = 8, |acc_L| <= 2^22): both round the exact sum once
+// 2^E sum_L acc_L 2^(-7 L), the acc_L exact integers held in FP32, |acc_L| <= 2^22 (up to 128 terms);
+// two levels are joined in 32 bits, and the exact sum is rounded once
 __device__ __forceinline__ double oz_value_int(const float (&acc)[8][4], int v, int E) {
   int q[8];
 #pragma unroll
@@ -145,6 +123,16 @@ __device__ __forceinline__ double oz_value_int(const float (&acc)[8][4], int v, 
   const long long hi = (long long)(q[0] * 128 + q[1]) * 16384 + (q[2] * 128 + q[3]);
   const long long lo = (long long)(q[4] * 128 + q[5]) * 16384 + (q[6] * 128 + q[7]);
   return oz_assemble_small(hi, lo, 28, E - 49);
+}
+
+// The same for nine levels and |acc_L| <= 2^23 (256 terms)
+__device__ __forceinline__ double oz_value9(const float (&acc)[9][4], int v, int E) {
+  int q[9];
+#pragma unroll
+  for (int L = 0; L < 9; ++L) q[L] = __float2int_rn(acc[L][v]);
+  const long long hi = (long long)(q[0] * 128 + q[1]) * 16384 + (q[2] * 128 + q[3]);
+  const long long lo = ((long long)(q[4] * 128 + q[5]) * 16384 + (q[6] * 128 + q[7])) * 128 + q[8];
+  return oz_assemble_small(hi, lo, 35, E - 56);
 }
 
 // (double)f by integer operations (FP32 subnormals flush to zero)

@@ -187,7 +187,7 @@ __device__ float oz_residual(ShiftedSmem<KM, LPP>& sm, const double* Vs, int k, 
       float sxj = 0.0f, sjx = 0.0f;
       if (x < k && j < k) {  // FP64 work kept to ~7 operations per entry (J by sign bits)
         const bool nx = sm.jphys[x] < 0, nj = sm.jphys[j] < 0;
-        double m = oz_value<true>(acc, v, sm.dexp[x] + sm.dexp[j] - 2056);
+        double m = oz_value_int(acc, v, sm.dexp[x] + sm.dexp[j] - 2056);
         if (x == j) {
           const double wxx = Vs[x * LDV + x] - 1.0, l = sm.dlo[x];
           m += oz_neg_if(wxx + wxx, nx);
