@@ -20,8 +20,11 @@
  *     device, owned by the caller.  opts and info are HOST pointers.
  *   - All work is ordered on `stream` (NULL = the legacy default stream).  Each call returns
  *     after the solve has finished: the sweep loop reads one small convergence record back
- *     per sweep.  Internal scratch is taken from the stream-ordered allocator
- *     (cudaMallocAsync) and returned before the call returns.
+ *     per sweep.  Internal scratch is taken from the stream-ordered allocator, from a pool
+ *     of the library's own that keeps at most 64 MB per device mapped between calls
+ *     (jacobi_release_scratch), and returned to it before the call returns.  A program that
+ *     gave the device a memory pool, or its default pool a release threshold, gets the
+ *     scratch from there instead (cudaMallocAsync).
  *   - Errors are reported by the return value and never by abort or trap.  A negative value
  *     -k means argument k (1-based) is invalid; nothing has been written then.  Positive
  *     values are the jac_status codes below; outputs are then unspecified except for info.
@@ -170,6 +173,10 @@ const char* jacobi_status_string(int status);
 #define JAC_VERSION 500
 int jacobi_version(void);
 
+/* Gives the scratch memory that the library keeps mapped on the current device back to the system
+ * (what a running solve uses stays).  Returns 0 or JAC_ECUDA. */
+int jacobi_release_scratch(void);
+
 /*
  * jacobi_hsvd -- hyperbolic (or, for J = I, trigonometric) one-sided block Jacobi on G.
  * Sec. 3.2, Algorithm 3.4 (full block; Cholesky per opts->factor, Algorithm 3.3).
@@ -267,7 +274,7 @@ int jacobi_eig_batched(int batch, const int* m, const int* n, int dtype, void* c
  * 22 G_bar, 23 ldgb, 24 s_gb    output dL/dG, or NULL (then G may be NULL)
  * 25 stream
  * Returns 0, a negative argument position, JAC_ENOMEM or JAC_ECUDA.  Asynchronous on stream
- * (its n x n x batch scratch comes from cudaMallocAsync on that stream).
+ * (its n x n x batch scratch is stream-ordered on that stream).
  */
 int jacobi_eig_backward(int batch, int n, const double* lambda, long long s_lam, const double* U,
                         int ldu, long long s_u, const double* lambda_bar, long long s_lbar,

@@ -61,7 +61,8 @@ _lib = None
 
 EXPORTS = ("jacobi_default_opts", "jacobi_status_string", "jacobi_version", "jacobi_hsvd", "jacobi_eig_pd",
            "jacobi_sched_pairs", "jacobi_profile_begin", "jacobi_profile_read", "jacobi_profile_end",
-           "jacobi_sched_pairs_noalloc", "jacobi_eig_batched", "jacobi_eig_backward", "jacobi_autotune_batched")
+           "jacobi_sched_pairs_noalloc", "jacobi_eig_batched", "jacobi_eig_backward", "jacobi_autotune_batched",
+           "jacobi_release_scratch")
 KERNEL = {"gram": 0, "pivot": 1, "update": 2, "gram_lowp": 3, "update_lowp": 4, "step_fused": 5}
 
 

@@ -18,6 +18,7 @@
 #include "jacobi_gb300.h"
 
 namespace jac {
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st);  // capi.cu
 int oz_gemm_launch(int Mr, int Nc, int K, const double* A, int lda, int transA, const double* B, int ldb,
                    const int8_t* sb, const int8_t* dsub, double* C, int ldc, int sym, int transB, long long sa,
                    long long sbb, long long sc, int batch, cudaStream_t st);
@@ -107,7 +108,7 @@ extern "C" int jacobi_eig_backward(int batch, int n, const double* lambda, long 
   if (batch == 0) return JAC_OK;
   const long long nn = (long long)n * n;
   void* scratch = nullptr;
-  if (cudaMallocAsync(&scratch, sizeof(double) * 2 * nn * batch, st) != cudaSuccess) {
+  if (scratch_alloc(&scratch, sizeof(double) * 2 * nn * batch, st) != cudaSuccess) {
     cudaGetLastError();
     return JAC_ENOMEM;
   }

@@ -77,6 +77,7 @@ size_t tc_gram_oz_smem_bytes();
 size_t tc_gram32_smem_bytes();
 size_t tc_update32_smem_bytes();
 size_t oz_gram_smem_bytes();
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st);
 int oz_gemm_launch(int Mr, int Nc, int K, const double* A, int lda, int transA, const double* B, int ldb,
                    const int8_t* sb, const int8_t* dsub, double* C, int ldc, int sym, int transB, long long sa,
                    long long sbb, long long sc, int batch, cudaStream_t st);
@@ -123,14 +124,19 @@ struct ProfRun {
     if (!a || !b) return (size_t)-1;
     evs.push_back(a);
     evs.push_back(b);
-    // external: inside a stream capture the record becomes a graph node that records the event
-    // at every replay (a plain record would only order the capture)
-    cudaEventRecordWithFlags(a, st, cudaEventRecordExternal);
+    cudaEventRecordWithFlags(a, st, flags(st));
     marks.emplace_back(k, evs.size() - 2);
     return evs.size() - 2;
   }
   void post(size_t idx, cudaStream_t st) {
-    if (idx != (size_t)-1) cudaEventRecordWithFlags(evs[idx + 1], st, cudaEventRecordExternal);
+    if (idx != (size_t)-1) cudaEventRecordWithFlags(evs[idx + 1], st, flags(st));
+  }
+  // external inside a stream capture: the record becomes a graph node that records the event at
+  // every replay (a plain record would only order the capture)
+  static unsigned flags(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+    return cs == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : cudaEventRecordDefault;
   }
   void accumulate() {  // after the stream has been synchronized; the events stay with this run
     if (evs.empty()) return;
@@ -156,6 +162,106 @@ struct ProfRun {
     release();
   }
 };
+
+// Set-up calls that a capture running in another thread must not see as its own.
+struct RelaxedCapture {
+  cudaStreamCaptureMode m = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&m); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&m); }
+};
+
+// Scratch of the solves and of the backward comes from a pool of the library's own, one per device.
+// The default pool gives every block back to the system at the next synchronization; mapping it again
+// cost a 24-column solve 175 of its 755 us.  Stream-ordered like cudaMallocAsync, so safe across threads
+// and streams.  At most kPoolKeep bytes stay mapped (the scratch of real solves up to n ~ 1000; larger
+// ones run for 50 ms and more), and jacobi_release_scratch gives those back.  A program that set the
+// device's pool, or a release threshold on its default pool, gets its scratch from that one.
+constexpr unsigned long long kPoolKeep = 64ull << 20;
+constexpr int kMaxDev = 64;
+std::mutex g_pool_mutex;
+cudaMemPool_t g_pool[kMaxDev] = {};
+bool g_pool_failed[kMaxDev] = {};
+
+cudaMemPool_t own_pool(bool create) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return nullptr;
+  std::lock_guard<std::mutex> lk(g_pool_mutex);
+  if (create && !g_pool[dev] && !g_pool_failed[dev]) {
+    RelaxedCapture relaxed;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    unsigned long long keep = kPoolKeep;
+    cudaMemPool_t pool = nullptr;
+    if (cudaMemPoolCreate(&pool, &props) == cudaSuccess &&
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) {
+      g_pool[dev] = pool;
+    } else {
+      cudaGetLastError();
+      if (pool) cudaMemPoolDestroy(pool);
+      g_pool_failed[dev] = true;
+    }
+  }
+  return g_pool[dev];
+}
+
+bool program_chose_pool() {
+  int dev = 0;
+  cudaMemPool_t cur = nullptr, def = nullptr;
+  unsigned long long keep = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetMemPool(&cur, dev) != cudaSuccess ||
+      cudaDeviceGetDefaultMemPool(&def, dev) != cudaSuccess)
+    return true;
+  return cur != def ||
+         cudaMemPoolGetAttribute(def, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess || keep != 0;
+}
+
+// Pinned host memory for the small records a solve reads back (a copy into pageable memory costs
+// the sweep loop ~8 us, into pinned memory ~3 us): 64 slots of 512 bytes for the process, one per
+// running solve, given back when it ends.  A solve that finds none uses its own pageable memory.
+constexpr size_t kSlotBytes = 512;
+constexpr int kSlots = 64;
+std::mutex g_slot_mutex;
+char* g_slot_base = nullptr;
+bool g_slot_failed = false;
+bool g_slot_used[kSlots] = {};
+
+struct HostSlot {
+  alignas(16) char own[kSlotBytes];
+  int idx = -1;
+  char* p = own;
+  HostSlot() {
+    std::lock_guard<std::mutex> lk(g_slot_mutex);
+    if (!g_slot_base && !g_slot_failed) {
+      RelaxedCapture relaxed;
+      void* b = nullptr;
+      g_slot_failed = cudaHostAlloc(&b, kSlotBytes * kSlots, cudaHostAllocPortable) != cudaSuccess;
+      if (g_slot_failed) cudaGetLastError();
+      else g_slot_base = static_cast<char*>(b);
+    }
+    if (!g_slot_base) return;
+    for (int i = 0; i < kSlots; ++i)
+      if (!g_slot_used[i]) {
+        g_slot_used[i] = true;
+        idx = i;
+        p = g_slot_base + kSlotBytes * i;
+        return;
+      }
+  }
+  ~HostSlot() {  // every copy into the slot has been synchronized
+    if (idx < 0) return;
+    std::lock_guard<std::mutex> lk(g_slot_mutex);
+    g_slot_used[idx] = false;
+  }
+  HostSlot(const HostSlot&) = delete;
+  HostSlot& operator=(const HostSlot&) = delete;
+};
+
+// A sweep of at most this many steps is launched directly: capturing and instantiating its graph costs
+// more than the launches it saves over the sweeps of a solve.  One step (24 columns): 799 us with a
+// graph, 755 direct; eight steps (64 columns): 3.20 ms with a graph, 3.62 direct.
+constexpr int kGraphSteps = 2;
 
 std::mutex g_attr_mutex;
 bool g_attr_done[64] = {};
@@ -589,15 +695,24 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   JacIO hio = {};
   int* boff_dev = nullptr;
   Single L;
+  struct Head {  // what the host fills in, copied at once; the block offsets follow
+    JacProb prob;
+    JacIO io;
+    long long jsoff;
+    unsigned flags;
+  };
+  std::vector<char> head(sizeof(Head) + sizeof(int) * (P.nb + 1));
   auto carve_all = [&](Arena& A) {
     carve_problem(A, P, hp, hio, weights);
-    boff_dev = A.take<int>(P.nb + 1);
-    L.probs = A.take<JacProb>(1);
-    L.io = A.take<JacIO>(1);
+    char* h = A.take<char>(head.size());
+    Head* hd = reinterpret_cast<Head*>(h);
+    L.probs = &hd->prob;
+    L.io = &hd->io;
+    L.jsoff = &hd->jsoff;
+    L.flags = &hd->flags;
+    boff_dev = reinterpret_cast<int*>(h + sizeof(Head));
     L.rec = A.take<SweepRecord>(1);
-    L.flags = A.take<unsigned>(1);
     L.Js = A.take<int8_t>(n);
-    L.jsoff = A.take<long long>(1);
     L.pairs = A.take<int>((size_t)P.nsteps * P.half * 2);
     L.counts = A.take<int>(P.nsteps);
     L.weights = weights ? A.take<double>((size_t)P.nb * P.nb) : nullptr;
@@ -610,7 +725,7 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   Arena ar;
   carve_all(ar);
   void* base = nullptr;
-  if (cudaMallocAsync(&base, ar.off, st) != cudaSuccess) {
+  if (scratch_alloc(&base, ar.off, st) != cudaSuccess) {
     cudaGetLastError();
     return JAC_ENOMEM;
   }
@@ -638,12 +753,14 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   auto ck = [&](cudaError_t e) {
     if (e != cudaSuccess && status == JAC_OK) status = JAC_ECUDA;
   };
-  const long long zero = 0;
-  ck(cudaMemcpyAsync(boff_dev, P.boff.data(), sizeof(int) * (P.nb + 1), cudaMemcpyHostToDevice, st));
-  ck(cudaMemcpyAsync(L.probs, &hp, sizeof(JacProb), cudaMemcpyHostToDevice, st));
-  ck(cudaMemcpyAsync(L.io, &hio, sizeof(JacIO), cudaMemcpyHostToDevice, st));
-  ck(cudaMemcpyAsync(L.jsoff, &zero, sizeof(long long), cudaMemcpyHostToDevice, st));
-  ck(cudaMemsetAsync(L.flags, 0, sizeof(unsigned), st));
+  {
+    Head h = {};
+    h.prob = hp;
+    h.io = hio;
+    std::memcpy(head.data(), &h, sizeof(Head));
+    std::memcpy(head.data() + sizeof(Head), P.boff.data(), sizeof(int) * (P.nb + 1));
+    ck(cudaMemcpyAsync(L.probs, head.data(), head.size(), cudaMemcpyHostToDevice, st));
+  }
 
   // FP32 sweeps of a single solve run on the tensor cores (TMA tensor maps of the FP32 copies)
   TcMaps tmaps;
@@ -664,19 +781,21 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   k_sort_signs<<<1, 32, 0, st>>>(L.probs, L.io, L.Js, L.jsoff);
   k_check_finite<<<dim3(std::min(1024, (int)(((size_t)m * n + 255) / 256)), 1), 256, 0, st>>>(L.probs, L.io);
   launches += 2;
-  JacIO hio_back;
-  ck(cudaMemcpyAsync(&hio_back, L.io, sizeof(JacIO), cudaMemcpyDeviceToHost, st));
-  ck(cudaStreamSynchronize(st));
-  if (status == JAC_OK && (hio_back.flags & 2)) {
-    cudaFreeAsync(base, st);
-    cudaStreamSynchronize(st);
-    return fail_arg(ap.J);
-  }
-  if (status == JAC_OK && (hio_back.flags & 1)) status = JAC_ENONFINITE;
+  // The verdict on the input is read with the record of the first sweep (its own round trip costs a
+  // small solve ~15 us): an invalid input is inactive by then, so the sweep's kernels skip it.  A
+  // schedule by weights is planned from the entries, so there the verdict comes first.
+  HostSlot slot;
+  static_assert(sizeof(SweepRecord) + sizeof(int) <= kSlotBytes, "a sweep's record fits a slot");
+  int* in_flags = reinterpret_cast<int*>(slot.p + sizeof(SweepRecord));
+  bool judged = false;
+  auto fetch_verdict = [&]() {
+    ck(cudaMemcpyAsync(in_flags, &L.io->flags, sizeof(int), cudaMemcpyDeviceToHost, st));
+  };
   k_gather_in<<<dim3((P.mp + 255) / 256, n, 1), 256, 0, st>>>(L.probs, L.io);
   if (have_vw) k_init_v<<<dim3((P.np + 255) / 256, n, 1), 256, 0, st>>>(L.probs, L.io);
   k_cache_init<<<1, 256, 0, st>>>(L.probs);
-  launches += have_vw ? 3 : 2;
+  k_apply_flags<<<1, 32, 0, st>>>(L.probs, L.io, 1);
+  launches += have_vw ? 4 : 3;
   ck(cudaGetLastError());
 
   int nsteps = P.nsteps;
@@ -711,12 +830,24 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   long long ev_total = 0, ev_lowp = 0;
   double prev_max = 1e300;
   SweepRecord hrec = {};
+  bool bad_sign = false;
+  auto judge = [&]() {  // after a synchronization behind fetch_verdict
+    if (judged || status != JAC_OK) return;
+    judged = true;
+    bad_sign = (*in_flags & 2) != 0;
+    if (bad_sign || (*in_flags & 1)) status = JAC_ENONFINITE;
+  };
+  if (n == 1 || weights) {  // no sweep; no plan from an invalid input
+    fetch_verdict();
+    ck(cudaStreamSynchronize(st));
+    judge();
+  }
   int last_steps = 0;
   ProfRun prof;
   prof.begin();
   double sweep_ms_h[64] = {};
   SweepGraph graphs[5];
-  bool use_graphs = !weights;
+  bool use_graphs = !weights && P.nsteps > kGraphSteps;
   int phase_sweeps = 0;  // sweeps of the current (FP64 or FP32-only) phase
   for (int sw = 0; status == JAC_OK && n > 1 && sw < o.max_sweeps; ++sw) {
     const auto t_sweep = std::chrono::steady_clock::now();
@@ -783,9 +914,12 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
     } else if (int r = record(st, launches, prof)) {
       status = r;
     }
-    ck(cudaMemcpyAsync(&hrec, L.rec, sizeof(SweepRecord), cudaMemcpyDeviceToHost, st));
+    ck(cudaMemcpyAsync(slot.p, L.rec, sizeof(SweepRecord), cudaMemcpyDeviceToHost, st));
+    if (!judged) fetch_verdict();
     ck(cudaStreamSynchronize(st));
+    std::memcpy(&hrec, slot.p, sizeof(SweepRecord));
     if (replayed) replayed->prof.accumulate();
+    judge();
     if (status != JAC_OK) break;
     if (info && sweeps < 64) info->sweep_max_scaled[sweeps] = hrec.max_scaled;
     ++sweeps;
@@ -909,6 +1043,7 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   cudaFreeAsync(base, st);
   if (cudaStreamSynchronize(st) != cudaSuccess && status == JAC_OK) status = JAC_ECUDA;
   prof.finish();
+  if (bad_sign) return fail_arg(ap.J);
   if (info) {
     for (int u = sweeps; u < 64; ++u) info->sweep_max_scaled[u] = 0.0;
     for (int u = 0; u < 64; ++u) info->sweep_ms[u] = (u < sweeps) ? sweep_ms_h[u] : 0.0;
@@ -985,7 +1120,7 @@ int solve_complex(int m, int n, void* Gv, int ldg, const int8_t* Jdev, const jac
   Arena ar;
   carve(ar);
   void* base = nullptr;
-  if (cudaMallocAsync(&base, ar.off, st) != cudaSuccess) {
+  if (scratch_alloc(&base, ar.off, st) != cudaSuccess) {
     cudaGetLastError();
     if (info) info->status = JAC_ENOMEM;
     return JAC_ENOMEM;
@@ -1170,27 +1305,33 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
   int8_t* d_Js = nullptr;
   long long* d_jsoff = nullptr;
   int* d_remaining = nullptr;
+  // what the host fills in, copied at once: problems, buffers, sign offsets, flags (these four are read
+  // back at the end), block offsets
+  const size_t at_io = sizeof(JacProb) * batch, at_jsoff = at_io + sizeof(JacIO) * batch,
+               at_flags = at_jsoff + sizeof(long long) * batch, at_boff = at_flags + sizeof(unsigned) * batch,
+               head_bytes = at_boff + sizeof(int) * boff_host.size();
   auto carve_all = [&](Arena& A) {
     for (int i = 0; i < batch; ++i) carve_problem(A, plans[order[i]], hp[i], hio[i], false);
-    d_boff = A.take<int>(boff_host.size());
     for (auto& kv : tables) {
       const int nb = kv.first;
       const int steps = (o.ordering == JAC_ORDER_ROUND_ROBIN) ? nb - 1 : nb;
       kv.second.first = A.take<int>((size_t)steps * (nb / 2) * 2);
       kv.second.second = A.take<int>(steps);
     }
-    d_probs = A.take<JacProb>(batch);
-    d_io = A.take<JacIO>(batch);
+    char* h = A.take<char>(head_bytes);
+    d_probs = reinterpret_cast<JacProb*>(h);
+    d_io = reinterpret_cast<JacIO*>(h + at_io);
+    d_jsoff = reinterpret_cast<long long*>(h + at_jsoff);
+    d_flags = reinterpret_cast<unsigned*>(h + at_flags);
+    d_boff = reinterpret_cast<int*>(h + at_boff);
     d_rec = A.take<SweepRecord>(batch);
-    d_flags = A.take<unsigned>(batch);
     d_Js = A.take<int8_t>(nsum);
-    d_jsoff = A.take<long long>(batch);
     d_remaining = A.take<int>(1);
   };
   Arena ar;
   carve_all(ar);
   void* base = nullptr;
-  if (cudaMallocAsync(&base, ar.off, st) != cudaSuccess) {
+  if (scratch_alloc(&base, ar.off, st) != cudaSuccess) {
     cudaGetLastError();
     return JAC_ENOMEM;
   }
@@ -1223,11 +1364,12 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
   auto ck = [&](cudaError_t e) {
     if (e != cudaSuccess && status == JAC_OK) status = JAC_ECUDA;
   };
-  ck(cudaMemcpyAsync(d_boff, boff_host.data(), sizeof(int) * boff_host.size(), cudaMemcpyHostToDevice, st));
-  ck(cudaMemcpyAsync(d_probs, hp.data(), sizeof(JacProb) * batch, cudaMemcpyHostToDevice, st));
-  ck(cudaMemcpyAsync(d_io, hio.data(), sizeof(JacIO) * batch, cudaMemcpyHostToDevice, st));
-  ck(cudaMemcpyAsync(d_jsoff, jsoff.data(), sizeof(long long) * batch, cudaMemcpyHostToDevice, st));
-  ck(cudaMemsetAsync(d_flags, 0, sizeof(unsigned) * batch, st));
+  std::vector<char> head(head_bytes, 0);
+  std::memcpy(head.data(), hp.data(), sizeof(JacProb) * batch);
+  std::memcpy(head.data() + at_io, hio.data(), sizeof(JacIO) * batch);
+  std::memcpy(head.data() + at_jsoff, jsoff.data(), sizeof(long long) * batch);
+  std::memcpy(head.data() + at_boff, boff_host.data(), sizeof(int) * boff_host.size());
+  ck(cudaMemcpyAsync(d_probs, head.data(), head_bytes, cudaMemcpyHostToDevice, st));
   for (auto& kv : tables) {
     const int nb = kv.first;
     const int steps = (o.ordering == JAC_ORDER_ROUND_ROBIN) ? nb - 1 : nb;
@@ -1284,7 +1426,10 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
   long long launches = 0;
   int sweeps = 0;
   SweepGraph graph;  // every sweep of a batch has the same launches
-  bool use_graph = true;
+  int sweep_steps = 0;
+  for (auto& c : cls) sweep_steps += c.max_steps;
+  bool use_graph = sweep_steps > kGraphSteps;
+  HostSlot slot;
   for (int sw = 0; status == JAC_OK && sw < o.max_sweeps; ++sw) {
     auto record = [&](cudaStream_t ss, long long& nl, ProfRun& pr) -> int {
       if (cudaMemsetAsync(d_remaining, 0, sizeof(int), ss) != cudaSuccess) return JAC_ECUDA;
@@ -1315,9 +1460,10 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
     } else if (int r = record(st, launches, prof)) {
       status = r;
     }
-    int remaining = 0;
-    ck(cudaMemcpyAsync(&remaining, d_remaining, sizeof(int), cudaMemcpyDeviceToHost, st));
+    ck(cudaMemcpyAsync(slot.p, d_remaining, sizeof(int), cudaMemcpyDeviceToHost, st));
     ck(cudaStreamSynchronize(st));
+    int remaining = 0;
+    std::memcpy(&remaining, slot.p, sizeof(int));
     if (replayed) graph.prof.accumulate();
     ++sweeps;
     if (remaining == 0) break;
@@ -1333,30 +1479,29 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
     launches += 3;
   }
   ck(cudaGetLastError());
-  std::vector<JacProb> hp_back(batch);
-  std::vector<JacIO> hio_back(batch);
-  std::vector<unsigned> flags_back(batch);
-  ck(cudaMemcpyAsync(hp_back.data(), d_probs, sizeof(JacProb) * batch, cudaMemcpyDeviceToHost, st));
-  ck(cudaMemcpyAsync(hio_back.data(), d_io, sizeof(JacIO) * batch, cudaMemcpyDeviceToHost, st));
-  ck(cudaMemcpyAsync(flags_back.data(), d_flags, sizeof(unsigned) * batch, cudaMemcpyDeviceToHost, st));
+  ck(cudaMemcpyAsync(head.data(), d_probs, at_boff, cudaMemcpyDeviceToHost, st));
   cudaFreeAsync(base, st);
   ck(cudaStreamSynchronize(st));
   prof.finish();
+  std::memcpy(hp.data(), head.data(), sizeof(JacProb) * batch);
+  std::memcpy(hio.data(), head.data() + at_io, sizeof(JacIO) * batch);
+  std::vector<unsigned> flags_back(batch);
+  std::memcpy(flags_back.data(), head.data() + at_flags, sizeof(unsigned) * batch);
   int first_bad = JAC_OK;
   for (int i = 0; i < batch; ++i) {
     const int b = order[i];
     int s = JAC_OK;
-    if (hio_back[i].flags & 2) s = -7;
-    else if (hio_back[i].flags & 1) s = JAC_ENONFINITE;
+    if (hio[i].flags & 2) s = -7;
+    else if (hio[i].flags & 1) s = JAC_ENONFINITE;
     else if (flags_back[i] & JAC_DEVERR_TIMEOUT) s = JAC_EINTERNAL;
     else if (flags_back[i] & JAC_DEVERR_NOTPD) s = JAC_ENOTPD;
-    else if (hp_back[i].active) s = JAC_ENOTCONV;
+    else if (hp[i].active) s = JAC_ENOTCONV;
     if (status != JAC_OK) s = status;
     if (info) {
       info[b].status = s;
       info[b].converged = (s == JAC_OK) ? 1 : 0;
-      info[b].sweeps = hio_back[i].sweeps;
-      info[b].rotations = hio_back[i].rotations;
+      info[b].sweeps = hio[i].sweeps;
+      info[b].rotations = hio[i].rotations;
       info[b].steps_per_sweep = plans[b].nsteps;
       info[b].launches = (b == 0) ? launches : 0;
     }
@@ -1368,7 +1513,30 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
 
 }  // namespace
 
+namespace jac {
+// bytes of stream-ordered scratch, freed with cudaFreeAsync
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
+  if (!program_chose_pool()) {
+    if (cudaMemPool_t pool = own_pool(true)) {
+      if (cudaMallocFromPoolAsync(p, bytes, pool, st) == cudaSuccess) return cudaSuccess;
+      cudaGetLastError();
+      cudaMemPoolTrimTo(pool, 0);
+    }
+  }
+  return cudaMallocAsync(p, bytes, st);
+}
+}  // namespace jac
+
 extern "C" {
+
+int jacobi_release_scratch(void) {
+  cudaMemPool_t pool = own_pool(false);
+  if (pool && cudaMemPoolTrimTo(pool, 0) != cudaSuccess) {
+    cudaGetLastError();
+    return JAC_ECUDA;
+  }
+  return JAC_OK;
+}
 
 void jacobi_default_opts(jac_opts* o) {
   if (!o) return;
