@@ -42,7 +42,6 @@ void pivot64_launch(int km, int max_half, int nprob, cudaStream_t st, const JacP
                     const PivotParams& pp);
 __global__ void k_sweep_reduce(JacProb* probs, JacIO* io, SweepRecord* rec, int deactivate, int* remaining);
 __global__ void k_cache_init(const JacProb* probs);
-__global__ void k_cache_step(const JacProb* probs, int rec, int chk);
 __global__ void k_sort_signs(const JacProb* probs, JacIO* io, int8_t* Js_all, const long long* js_off);
 __global__ void k_apply_flags(JacProb* probs, const JacIO* io, int nprob);
 __global__ void k_gather_in(const JacProb* probs, const JacIO* io);
@@ -480,7 +479,7 @@ void carve_problem(Arena& ar, const Plan& P, JacProb& d, JacIO& io, bool weights
   d.active = 1;
   d.skip = ar.take<int>(P.half);
   d.stats = ar.take<PairStat>((size_t)P.nsteps * P.half);
-  d.cached = weights ? nullptr : ar.take<int>(P.half);  // pair cache: off for the weight ordering
+  // pair cache: off for the weight ordering
   d.pver = weights ? nullptr : ar.take<int4>((size_t)P.nsteps * P.half);
   d.bver = weights ? nullptr : ar.take<int>(P.nb);
   io.perm_in = ar.take<int>(P.n);
@@ -505,8 +504,6 @@ int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, in
                 bool lowp, bool fallback, const PivotParams& pp, cudaStream_t st, ProfRun& prof,
                 long long& launches, const TcMaps* maps = nullptr, const TcSplit* tsp = nullptr,
                 int fused_rows = 0) {
-  // the pair cache: record step s - 1, then mark the pairs of step s whose outcome is known
-  k_cache_step<<<count, 256, 0, st>>>(dprobs, s - 1, s);
   int r = 0;
   if (lowp && fused_rows > 0) {
     // FP32 sweep step of small problems: Gram, pivot and update of each pair in one CTA (pivot.cu,
@@ -521,7 +518,7 @@ int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, in
       k_update32<<<dim3(max_half, tslabs, count), 256, 0, st>>>(dprobs, s, gslabs);
       prof.post(pm, st);
     }
-    launches += fallback ? 4 : 2;
+    launches += fallback ? 3 : 1;
     return cudaGetLastError() == cudaSuccess ? 0 : JAC_ECUDA;
   }
   size_t pm = prof.pre(lowp ? JAC_KERNEL_GRAM_LOWP : JAC_KERNEL_GRAM, st);
@@ -575,7 +572,7 @@ int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, in
   else
     k_update<<<dim3(max_half, tslabs, count), 128, kUpdSmem, st>>>(dprobs, s, gslabs);
   prof.post(pm, st);
-  launches += fallback ? 4 : 3;  // and the pivot's
+  launches += fallback ? 3 : 2;  // and the pivot's
   return cudaGetLastError() == cudaSuccess ? 0 : JAC_ECUDA;
 }
 
@@ -892,9 +889,8 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
         if (int r = launch_step(L.probs, 1, P.km, P.half, gslabs, tslabs, CS, CS32, s, low, phase != 1, pp, ss, pr,
                                 nl, use_tc ? &tmaps : nullptr, use_tc ? &tsplit : nullptr, fused))
           return r;
-      k_cache_step<<<1, 256, 0, ss>>>(L.probs, -2, -1);  // record the last step of the sweep
       k_sweep_reduce<<<1, 256, 0, ss>>>(L.probs, L.io, L.rec, 0, nullptr);
-      nl += 2;
+      nl += 1;
       return cudaGetLastError() == cudaSuccess ? 0 : JAC_ECUDA;
     };
     // graphs: one per precision phase, unless the ordering is re-planned every sweep
@@ -1439,9 +1435,8 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
                                   ss, pr, nl, nullptr, nullptr,
                                   (o.fused_step == 1 && c.max_mp <= fused_step_max_rows(c.km)) ? c.max_mp : 0))
             return r;
-        k_cache_step<<<c.count, 256, 0, ss>>>(c.probs, -2, -1);  // record the last step of the sweep
         k_sweep_reduce<<<c.count, 256, 0, ss>>>(c.probs, c.io, c.rec, 1, d_remaining);
-        nl += 2;
+        nl += 1;
       }
       return cudaGetLastError() == cudaSuccess ? 0 : JAC_ECUDA;
     };

@@ -7,6 +7,7 @@
 #include <cooperative_groups.h>
 
 #include "jacobi_common.cuh"
+#include "pair_cache.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -33,9 +34,10 @@ __global__ void __launch_bounds__(128) k_gram(const JacProb* __restrict__ probs,
   const int pair = blockIdx.x / CS;
   const int crank = (int)cluster.block_rank();
   // uniform over the cluster: no cluster barrier is pending
-  if (!a.active || s >= a.nsteps || pair >= a.counts[s] || (a.cached && a.cached[pair])) return;
+  if (!a.active || s >= a.nsteps || pair >= a.counts[s]) return;
   const int* sp = a.pairs + (size_t)s * a.half * 2;
   const int p = sp[2 * pair], q = sp[2 * pair + 1];
+  if (pair_known(a, s, pair)) return;
   const int op = a.boff[p], wp = a.boff[p + 1] - op, oq = a.boff[q], wq = a.boff[q + 1] - oq;
   const int k = wp + wq, KP = (k + 15) & ~15;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;

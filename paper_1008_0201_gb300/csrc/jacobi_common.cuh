@@ -107,8 +107,7 @@ struct JacProb {
   unsigned* pflags;  // JAC_DEVERR_* bits of this problem
   // Pair cache (NULL: off).  A pair whose two blocks have not changed since it was last
   // evaluated in the same (step, slot), and which did not rotate then, would give bitwise the
-  // same Gram block, decision and statistics: its step kernels return at once.
-  int* cached;       // [half] 1: the pair of this slot is cached in the current step
+  // same Gram block, decision and statistics: its step kernels return at once (pair_cache.cuh).
   int4* pver;        // [nsteps][half] (p, q, version of p, version of q) at the last evaluation;
                      // version of p = -1 if the pair rotated
   int* bver;         // [nb] block versions, bumped when a pair containing the block rotates

@@ -10,6 +10,7 @@
 #include <mutex>
 
 #include "jacobi_common.cuh"
+#include "pair_cache.cuh"
 #include "ozaki.cuh"
 
 namespace cg = cooperative_groups;
@@ -57,9 +58,10 @@ __global__ void __launch_bounds__(256) k_gram_oz(const JacProb* __restrict__ pro
   const JacProb& a = probs[blockIdx.y];
   const int pair = blockIdx.x / CS;
   const int crank = (int)cluster.block_rank();
-  if (!a.active || s >= a.nsteps || pair >= a.counts[s] || (a.cached && a.cached[pair])) return;  // uniform
+  if (!a.active || s >= a.nsteps || pair >= a.counts[s]) return;
   const int* sp = a.pairs + (size_t)s * a.half * 2;
   const int p = sp[2 * pair], q = sp[2 * pair + 1];
+  if (pair_known(a, s, pair)) return;  // uniform
   const int op = a.boff[p], wp = a.boff[p + 1] - op, oq = a.boff[q], wq = a.boff[q + 1] - oq;
   const int k = wp + wq, ntj = (k + 7) >> 3;  // 8-column tiles
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;

@@ -37,6 +37,7 @@
 // otherwise from FP16 digit products of W (oz_residual) or on the FP64 mma path (symmetric tiles
 // only); the correction product itself is small and is formed in FP32.
 #include "jacobi_common.cuh"
+#include "pair_cache.cuh"
 #include "ozaki.cuh"
 
 namespace jac {
@@ -526,6 +527,7 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
     st.cyc[1] = st.cyc[2] = st.cyc[3] = 0;
     if (!hit) {
       a.skip[pair] = 1;
+      pair_record(a, s, pair, false);
       stats[pair] = st;
     }
   }
@@ -1315,10 +1317,8 @@ constexpr size_t core_smem_bytes() {
   return offsetof(PivotSmem<KM>, work) + sizeof(PivotWork<KM>);
 }
 
-template <int KM>
-__device__ __forceinline__ bool pivot_guard(const JacProb& a, int s, int pair) {
-  if (!a.active || s >= a.nsteps || pair >= a.counts[s]) return false;
-  return !(a.cached && a.cached[pair]);  // cached: skip set, statistics kept (pair_cache.cu)
+__device__ __forceinline__ bool in_step(const JacProb& a, int s, int pair) {
+  return a.active && s < a.nsteps && pair < a.counts[s];
 }
 
 // Modes of the pivot kernel.  PV_FULL: phases 1-4 in one CTA (FP64 sweeps).  PV_CORE: phases 1-3,
@@ -1335,7 +1335,7 @@ __global__ void __launch_bounds__(4 * KM, MODE == PV_FULL ? (KM == 32 ? 4 : 1) :
   PivotSmem<KM>& sm = *reinterpret_cast<PivotSmem<KM>*>(pv_raw);
   const JacProb& a = probs[blockIdx.y];
   const int pair = blockIdx.x, tid = threadIdx.x;
-  if (!pivot_guard<KM>(a, s, pair)) return;
+  if (!in_step(a, s, pair) || pair_skip_known(a, s, pair)) return;
   PairStat* stats = a.stats + (size_t)s * a.half;
   if constexpr (MODE != PV_FULL) {
     if (pivot_core<KM, false>(sm.st, sm.work, nullptr, sm.Wf, a, s, pair, pp) != 0) return;
@@ -1358,6 +1358,7 @@ __global__ void __launch_bounds__(4 * KM, MODE == PV_FULL ? (KM == 32 ? 4 : 1) :
     }
     if (tid == 0) {
       a.skip[pair] = 0;
+      if (MODE == PV_CORE) pair_record(a, s, pair, true);
       stats[pair] = sm.st.st;
     }
   } else {
@@ -1375,6 +1376,7 @@ __global__ void __launch_bounds__(4 * KM, MODE == PV_FULL ? (KM == 32 ? 4 : 1) :
       // not J-unitary to FP64 accuracy after the step budget: FP64 pivot kernel
       a.skip[pair] = ok ? 0 : 2;
       if (!ok) atomicOr(a.pflags, JAC_DEVERR_HANDOVER);
+      else pair_record(a, s, pair, true);
       sm.st.st.ns_steps = ns;
       sm.st.st.cyc[3] = clock64() - sm.st.t_core;
       stats[pair] = sm.st.st;
@@ -1396,7 +1398,7 @@ __global__ void __launch_bounds__(4 * KM, KM == 32 ? 4 : 1)
   OrthSmem<KM>& sm = *reinterpret_cast<OrthSmem<KM>*>(pv_raw);
   const JacProb& a = probs[blockIdx.y];
   const int pair = blockIdx.x, tid = threadIdx.x;
-  if (!pivot_guard<KM>(a, s, pair) || a.skip[pair] != 0) return;
+  if (!in_step(a, s, pair) || a.skip[pair] != 0) return;
   const long long t0 = clock64();
   const int* sp = a.pairs + (size_t)s * a.half * 2;
   const int p = sp[2 * pair], q = sp[2 * pair + 1];
@@ -1421,6 +1423,8 @@ __global__ void __launch_bounds__(4 * KM, KM == 32 ? 4 : 1)
     if (!ok) {
       a.skip[pair] = 2;
       atomicOr(a.pflags, JAC_DEVERR_HANDOVER);
+    } else {
+      pair_record(a, s, pair, true);
     }
     PairStat& st = a.stats[(size_t)s * a.half + pair];
     st.ns_steps = ns;
@@ -1462,7 +1466,7 @@ __global__ void __launch_bounds__(4 * KM, KM == 32 ? 4 : 2)
   typename FL::Smem& sm = *reinterpret_cast<typename FL::Smem*>(pv_raw);
   const JacProb& a = probs[blockIdx.y];
   const int pair = blockIdx.x;
-  if (!pivot_guard<KM>(a, s, pair)) return;
+  if (!in_step(a, s, pair) || pair_skip_known(a, s, pair)) return;
   const int tid = threadIdx.x, tx = tid % CT, ty = tid / CT;
   const int* sp = a.pairs + (size_t)s * a.half * 2;
   const int p = sp[2 * pair], q = sp[2 * pair + 1];
@@ -1550,6 +1554,7 @@ __global__ void __launch_bounds__(4 * KM, KM == 32 ? 4 : 2)
   }
   if (tid == 0) {
     a.skip[pair] = 3;  // updated by this kernel itself
+    pair_record(a, s, pair, true);
     a.stats[(size_t)s * a.half + pair] = sm.st.st;
   }
   __syncthreads();

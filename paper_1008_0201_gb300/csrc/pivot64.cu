@@ -16,6 +16,7 @@
 // A Schur pivot at or below 64 eps_64 means the block (so G) is rank deficient: NOTPD.
 // One warp per column pair of an inner step; every lane computes its pair's rotation.
 #include "jacobi_common.cuh"
+#include "pair_cache.cuh"
 
 namespace jac {
 
@@ -285,6 +286,7 @@ __global__ void __launch_bounds__(KM * 16, 1) k_pivot64(const JacProb* __restric
   }
   if (tid == 0) {
     a.skip[pair] = 0;
+    pair_record(a, s, pair, true);
     st.rotations += total_rot;
     st.inner_sweeps += inner + 1;
     st.cyc[1] += t_chol - t_start;

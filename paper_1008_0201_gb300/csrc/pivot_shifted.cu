@@ -15,6 +15,7 @@
 // 1e-4 at order 400 (Gaussian), but by 1e-9 only at order 200.  With this kernel the large ones keep the
 // digits they have always had; the pivots are 7% to 30% of such a solve.
 #include "jacobi_common.cuh"
+#include "pair_cache.cuh"
 #include "ozaki.cuh"
 
 namespace jac {
@@ -362,6 +363,7 @@ __device__ __forceinline__ int pivot_block(ShiftedSmem<KM, LPP>& sm, const JacPr
   if (cnt == 0) {
     if (tid == 0) {
       a.skip[pair] = 1;
+      pair_record(a, s, pair, false);
       st.cyc[0] = t_stats - t_start;
       st.cyc[1] = st.cyc[2] = st.cyc[3] = 0;
       stats[pair] = st;
@@ -930,6 +932,7 @@ __device__ __forceinline__ int pivot_block(ShiftedSmem<KM, LPP>& sm, const JacPr
   }
   if (tid == 0) {
     a.skip[pair] = 0;
+    pair_record(a, s, pair, true);
     st.rotations = total_rot;
     st.inner_sweeps = (inner < max_inner) ? inner + 1 : max_inner;
     st.ns_steps = ns;
@@ -952,7 +955,7 @@ __global__ void __launch_bounds__((KM / 2) * LPP, KM == 32 ? 4 : 1)
   const JacProb& a = probs[blockIdx.y];
   const int pair = blockIdx.x;
   if (!a.active || s >= a.nsteps || pair >= a.counts[s]) return;
-  if (a.cached && a.cached[pair]) return;  // skip set, statistics kept (pair_cache.cu)
+  if (pair_skip_known(a, s, pair)) return;
   pivot_block<KM, LPP>(sm, a, s, pair, pp);
 }
 

@@ -22,6 +22,7 @@
 #include <cooperative_groups.h>
 
 #include "jacobi_common.cuh"
+#include "pair_cache.cuh"
 #include "oz_assemble.h"
 #include "ozaki.cuh"
 #include "tc.cuh"
@@ -341,9 +342,10 @@ __global__ void __launch_bounds__(512, 1) k_gram_oz_tc(const JacProb* __restrict
   const JacProb& a = probs[blockIdx.y];
   const int pair = blockIdx.x / CS;
   const int crank = (int)cluster.block_rank();
-  if (!a.active || s >= a.nsteps || pair >= a.counts[s] || (a.cached && a.cached[pair])) return;  // uniform
+  if (!a.active || s >= a.nsteps || pair >= a.counts[s]) return;
   const int* sp = a.pairs + (size_t)s * a.half * 2;
   const int p = sp[2 * pair], q = sp[2 * pair + 1];
+  if (pair_known(a, s, pair)) return;  // uniform
   const int op = a.boff[p], wp = a.boff[p + 1] - op, oq = a.boff[q], wq = a.boff[q + 1] - oq;
   const int k = wp + wq;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
