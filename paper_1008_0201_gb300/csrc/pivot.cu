@@ -139,6 +139,7 @@ struct alignas(16) PivotState {
   int pres[D::P2];      // block-oriented cross step: columns of block p (pivot order) per slot
   int ptrav[D::P2];     // ... and of block q
   float4 prm[2][D::P2]; // rotation of each slot's pair: c, q12, q21 (double-buffered)
+  int2 back[D::P2];     // places of a slot's columns at the start of an inner sweep
   float red_f[D::NW][4];
   int red_i[D::NW][2];
   double trs[2];
@@ -687,14 +688,21 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
   const float tol_in = fmaxf(0.5f * tolf, 64.0f * 5.9604645e-8f * mx);
   // The columns live in registers: pair slot q (LPP lanes of a warp) holds a resident and a
   // traveler column of R and of V, R rows per lane (row l R + u in lane l), as row pairs.  An inner
-  // sweep is a recursive cross ordering of 2 p2 >= k positions: at group size g (p2, p2/2, ..., 1
-  // slots) the travelers of each group go round its ring of g slots, so every resident meets every
-  // traveler of the group in g steps; then each group splits in two, its residents pairing among
-  // themselves in the first half and its travelers in the second.  Every pair of positions
-  // meets once in 2 p2 - 1 steps, and between steps each slot passes exactly one column to one
-  // other slot through a shared-memory mailbox: one barrier per step.  Positions >= k are
-  // empty.  The logical order of Algorithm 3.3 (reversed J = -1 part) gives the initial
-  // placement: position p is the resident of slot p (p < p2) or the traveler of slot p - p2.
+  // sweep is a recursive cross ordering of the k columns over p = ceil(k / 2) slots: the travelers of a
+  // group of g slots (g = p at first) go round its ring, so every resident meets every traveler of
+  // the group in g steps; then each group splits in two of ceil(g / 2) slots, its residents pairing
+  // among themselves in the first and its travelers in the second.  Every pair meets once in
+  // p + ceil(p / 2) + ... + 1 steps, and between steps each slot passes at most one column to one
+  // other slot through a shared-memory mailbox: one barrier per step.  A group of g slots lies in a
+  // range of w >= g, w = p2, p2/2, ..., 1 (p2: the power of two >= p): its i-th slot is i if p is p2, and
+  // else i with its bits reversed.  Then slots of odd i lie w/2 above those of even i, so the split
+  // sends columns w/2 slots up or down for every g, and what the odd ones hold stays among the
+  // first ceil(g / 2).  An empty place holds a zero column that rests.  The logical order of Algorithm
+  // 3.3 (reversed J = -1 part) gives the initial placement: position i is the resident of slot i
+  // (i < p) or the traveler of slot i - p.  If p < p2 the columns end a sweep spread over p2 slots
+  // and go back to where they began before the next.
+  // Orders 33..64 take 50 steps per sweep on average, where a ring of p2 slots takes 63: 4000 problems
+  // of orders 8..128 in FP32 31.4 ms, now 27.0, in FP64 74.1 ms, now 68.5.
   // What bounds a step is its chain: mailbox, dot product and its reduction, the parameters, the
   // rotation, mailbox, barrier.  The columns of V are not on it: they belong to the second half of
   // the threads, which rotate them one barrier later, with the parameters the first half left in
@@ -704,18 +712,32 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
   // and the exchange of the parameters cost more than the mailboxes).
   const bool is_f = tid < D::NF;
   const int slot = (is_f ? tid : tid - D::NF) / LPP, l = tid % LPP;
-  // only as many slots as k needs (a power of two): a block of 16 columns takes 15 steps per sweep, not
-  // the 31 of 32 columns (64 x 64 problem of width 8: 46k clocks of inner sweeps per pivot, now 24k)
-  const int p2 = 1 << (32 - __clz((k + 1) / 2 - 1));
-  const int ci0 = cross_only ? sm.pres[slot] : ((slot < p2 && slot < k) ? sm.lpos[slot] : -1);
-  const int cj0 = cross_only ? sm.ptrav[slot] : ((slot < p2 && slot + p2 < k) ? sm.lpos[slot + p2] : -1);
+  const int np = (k + 1) / 2, p2 = 1 << (32 - __clz(np - 1));
+  // the i-th slot of a range of w slots, and the i of a slot
+  auto order = [&](int i, int w) { return np == p2 ? i : (int)((__brev((unsigned)i) >> __clz(w)) >> 1); };
+  auto start_i = [&]() {
+    const int i = order(slot, p2);
+    return (slot >= p2 || i >= np) ? -1 : cross_only ? sm.pres[i] : sm.lpos[i];
+  };
+  auto start_j = [&]() {
+    const int i = order(slot, p2);
+    return (slot >= p2 || i >= np) ? -1 : cross_only ? sm.ptrav[i] : (i + np < k ? sm.lpos[i + np] : -1);
+  };
+  // where the traveler of this slot goes in the ring of its group, five bits per level (the reversal
+  // of bits at the start of each level cost its chain ~90 clocks)
+  unsigned rings = 0;
+  for (int w = p2, g = np, sh = 0; w >= 1; w >>= 1, g = (g + 1) >> 1, sh += 5) {
+    const int i = order(slot & (w - 1), w);
+    const int nxt = i < g ? (slot & ~(w - 1)) + order(i + 1 == g ? 0 : i + 1, w) : slot;
+    rings |= (unsigned)nxt << sh;
+  }
   // block-oriented: one inner sweep; after the first step of an outer sweep only the ring of
   // its first level (every column of block p meets every column of block q once)
-  const int g_last = cross_only ? p2 : 1;
+  const int w_last = cross_only ? p2 : 1;
   const int max_inner = pp.oriented ? 1 : JAC_INNER_MAX_SWEEPS;
   f2 xi[H], xj[H];  // resident and traveler of this half's columns
   float cni = 0.0f, cnj = 0.0f, si = 1.0f, sj = 1.0f;  // ||r||^2 = s^2 + cn
-  int ci = ci0, cj = cj0, ji = 1, jj = 1;
+  int ci = start_i(), cj = start_j(), ji = 1, jj = 1;
   if (is_f) {
     auto load_col = [&](int c, f2(&f)[H], float& cn, float& d, int& sg) {
       const int pc = c >= 0 ? sm.perm[c] : 0;
@@ -796,8 +818,9 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
         fresh(xi, cni, si);
         fresh(xj, cnj, sj);
       }
-      for (int g = p2; g >= g_last; g >>= 1) {
-        const int base = slot & ~(g - 1), pos = slot - base;
+      unsigned ring = rings;
+      for (int w = p2, g = np; w >= w_last; w >>= 1, g = (g + 1) >> 1, ring >>= 5) {
+        const int nxt = ring & 31;
         for (int st_ = 0; st_ < g; ++st_) {
           // ---- rotate the pair (ci, cj) of this slot; what does not depend on the dot product first.
           // One branch-free path for both kinds, the slots of a warp never split on the sign
@@ -827,9 +850,9 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
           const float scaled = fabsf(aij) * rs;
           const bool rot = (ci | cj) >= 0 && scaled > tol_in;
           const float rr = fmaf(sg4, scaled * scaled, nu2);
-          const float h = rsqrt_ftz(rr), w = scaled * h;
+          const float h = rsqrt_ftz(rr), wh = scaled * h;
           const float c2 = fmaf(0.5f * nu, h, 0.5f), cinv = rsqrt_ftz(c2);
-          float sa = w * cinv, ca = c2 * cinv;
+          float sa = wh * cinv, ca = c2 * cinv;
           // the cosine of a small angle as 1 -+ s^2 / 2 rounded once (rsqrt returns the value below 1
           // too often there, and thousands of tiny rotations would shrink V: with it alone the
           // FP32-only eigenvalues of order 128 came out 5e-5 small, with this rule 2e-5)
@@ -858,13 +881,12 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
           cni = far ? 1.0e8f * si * si : fmaf(-sg, ta, cni);
           cnj = far ? 1.0e8f * sj * sj : cnj + ta;
           // ---- pass one column on: the traveler round the ring, or at the end of the group's
-          // ring its split (first half: traveler to slot + g/2, which sends back its resident).  The
+          // ring its split (first half: traveler to slot + w/2, which sends back its resident).  The
           // two cases are uniform over the block and keep code of their own: with one code for both,
           // the choice of the column split every warp
           if (st_ < g - 1) {
-            const int dst = base + ((pos + 1) & (g - 1));
-            put(buf, dst, xj);
-            if (l == 0) sm.mst[buf][dst] = make_int4(cj, __float_as_int(cnj), __float_as_int(sj), jj);
+            put(buf, nxt, xj);
+            if (l == 0) sm.mst[buf][nxt] = make_int4(cj, __float_as_int(cnj), __float_as_int(sj), jj);
             half_sync<KM>();
             const int4 m = sm.mst[buf][slot];
             get(buf, xj);
@@ -872,9 +894,9 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
             cnj = __int_as_float(m.y);
             sj = __int_as_float(m.z);
             jj = m.w;
-          } else if (g > g_last) {
-            const bool res = pos >= g / 2;
-            const int dst = res ? slot - g / 2 : slot + g / 2;
+          } else if (w > w_last) {
+            const bool res = (slot & (w >> 1)) != 0;
+            const int dst = slot ^ (w >> 1);
             if (res) put(buf, dst, xi);
             else put(buf, dst, xj);
             if (l == 0)
@@ -902,23 +924,24 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
         }
       }
     } else {
-      for (int g = p2; g >= g_last; g >>= 1) {
-        const int base = slot & ~(g - 1), pos = slot - base;
+      unsigned ring = rings;
+      for (int w = p2, g = np; w >= w_last; w >>= 1, g = (g + 1) >> 1, ring >>= 5) {
+        const int nxt = ring & 31;
         for (int st_ = 0; st_ < g; ++st_) {
           half_sync<KM>();  // the parameters of this step, the columns passed on in the previous one
           const float4 q = sm.prm[buf][slot];
           if (st_ > 0) {
             get(buf ^ 1, xj);
-          } else if (g < p2) {  // the split that ended the ring of 2 g slots
-            if (slot & g) get(buf ^ 1, xi);
+          } else if (w < p2) {  // the split that ended the ring of the range of 2 w slots
+            if (slot & w) get(buf ^ 1, xi);
             else get(buf ^ 1, xj);
           }
           rotate(q.x, q.y, q.z);
           if (st_ < g - 1) {
-            put(buf, base + ((pos + 1) & (g - 1)), xj);
-          } else if (g > g_last) {
-            if (pos >= g / 2) put(buf, slot - g / 2, xi);
-            else put(buf, slot + g / 2, xj);
+            put(buf, nxt, xj);
+          } else if (w > w_last) {
+            if (slot & (w >> 1)) put(buf, slot ^ (w >> 1), xi);
+            else put(buf, slot ^ (w >> 1), xj);
           }
           buf ^= 1;
         }
@@ -944,6 +967,48 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
     // done when nothing was rotated, or when every rotated pair was already so small that the
     // next sweep (quadratic convergence: off-diagonals ~ k delta^2) would find nothing above tol_in
     if (tot == 0 || (float)k * dmax * dmax <= tol_in) break;
+    if (np < p2 && inner + 1 < max_inner) {  // back to the initial placement
+      auto place = [&](int c) {  // slot, + KM for the traveler's place
+        if (c < 0) return -1;
+        const int q = sm.linv[c];
+        return q < np ? order(q, p2) : order(q - np, p2) + KM;
+      };
+      if (is_f && l == 0) {
+        const int di = place(ci), dj = place(cj);
+        sm.back[slot] = make_int2(di, dj);
+        if (di >= 0) sm.mst[di / KM][di % KM] = make_int4(ci, __float_as_int(cni), __float_as_int(si), ji);
+        if (dj >= 0) sm.mst[dj / KM][dj % KM] = make_int4(cj, __float_as_int(cnj), __float_as_int(sj), jj);
+      }
+      __syncthreads();
+      const int2 d = sm.back[slot];
+      if (d.x >= 0) put(d.x / KM, d.x % KM, xi);
+      if (d.y >= 0) put(d.y / KM, d.y % KM, xj);
+      __syncthreads();
+      const bool hi = start_i() >= 0, hj = start_j() >= 0;
+#pragma unroll
+      for (int u = 0; u < H; ++u) xi[u] = xj[u] = f2_make(0.0f, 0.0f);
+      ci = cj = -1;
+      cni = cnj = 0.0f;
+      si = sj = 1.0f;
+      ji = jj = 1;
+      if (hi) {
+        get(0, xi);
+        const int4 m = sm.mst[0][slot];
+        ci = m.x;
+        cni = __int_as_float(m.y);
+        si = __int_as_float(m.z);
+        ji = m.w;
+      }
+      if (hj) {
+        get(1, xj);
+        const int4 m = sm.mst[1][slot];
+        cj = m.x;
+        cnj = __int_as_float(m.y);
+        sj = __int_as_float(m.z);
+        jj = m.w;
+      }
+      __syncthreads();
+    }
   }
   if (!pp.oriented && inner >= JAC_INNER_MAX_SWEEPS && tid == 0) atomicOr(err, JAC_DEVERR_INNER_LIMIT);
   // which columns the slots of V hold now
