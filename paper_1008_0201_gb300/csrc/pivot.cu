@@ -1391,10 +1391,14 @@ __device__ __forceinline__ bool in_step(const JacProb& a, int s, int pair) {
 // k_pivot_orth: the core needs less than half the shared memory of phase 4, so three pivots run on an
 // SM while phase 4 takes the SM for a short time only (many pivots per step).  4000 problems of
 // orders 8..128, all pivots of a sweep step: 1.4 ms, against 4.1 ms with one 212 KB CTA per SM.
+// MINB: blocks per SM that the registers must allow.  The 80 registers of three (KM = 32: six) cost the
+// core 5 of its 73 thousand clocks for a 64-column block in a block-oriented step (order 512, mixed
+// precision: 14.8 ms; with 142 registers 14.4), so steps with no more pivots than SMs take all they need.
 enum { PV_FULL = 0, PV_CORE = 1, PV_SPLIT = 2 };
+constexpr int many_blocks(int km) { return km == 32 ? 6 : 3; }
 
-template <int KM, int MODE>
-__global__ void __launch_bounds__(4 * KM, MODE == PV_FULL ? (KM == 32 ? 4 : 1) : (KM == 32 ? 6 : 3))
+template <int KM, int MODE, int MINB>
+__global__ void __launch_bounds__(4 * KM, MINB)
     k_pivot(const JacProb* __restrict__ probs, int s, PivotParams pp) {
   extern __shared__ __align__(16) unsigned char pv_raw[];
   PivotSmem<KM>& sm = *reinterpret_cast<PivotSmem<KM>*>(pv_raw);
@@ -1685,9 +1689,10 @@ static bool set_attributes() {
   auto set = [](auto kern, size_t bytes) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
   };
-  bool ok = set(k_pivot<KM, PV_FULL>, sizeof(PivotSmem<KM>));
-  ok &= set(k_pivot<KM, PV_CORE>, core_smem_bytes<KM>());
-  ok &= set(k_pivot<KM, PV_SPLIT>, core_smem_bytes<KM>());
+  bool ok = set(k_pivot<KM, PV_FULL, 1>, sizeof(PivotSmem<KM>));
+  ok &= set(k_pivot<KM, PV_CORE, 1>, core_smem_bytes<KM>());
+  ok &= set(k_pivot<KM, PV_CORE, many_blocks(KM)>, core_smem_bytes<KM>());
+  ok &= set(k_pivot<KM, PV_SPLIT, many_blocks(KM)>, core_smem_bytes<KM>());
   ok &= set(k_pivot_orth<KM>, sizeof(OrthSmem<KM>));
   ok &= set(k_step_fused<KM>, FusedLayout<KM>::bytes(FusedLayout<KM>::MF));
   return ok;
@@ -1701,15 +1706,17 @@ constexpr int kSplitPivots = 152;
 template <int KM>
 static int launch_pivot(int max_half, int nprob, cudaStream_t st, const JacProb* probs, int s, const PivotParams& pp) {
   const dim3 grid(max_half, nprob);
+  const bool few = (long long)max_half * nprob <= kSplitPivots;
   if (!pp.ns_mode) {
-    k_pivot<KM, PV_CORE><<<grid, 4 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
+    if (few) k_pivot<KM, PV_CORE, 1><<<grid, 4 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
+    else k_pivot<KM, PV_CORE, many_blocks(KM)><<<grid, 4 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
     return 1;
   }
-  if ((long long)max_half * nprob <= kSplitPivots) {
-    k_pivot<KM, PV_FULL><<<grid, 4 * KM, sizeof(PivotSmem<KM>), st>>>(probs, s, pp);
+  if (few) {
+    k_pivot<KM, PV_FULL, 1><<<grid, 4 * KM, sizeof(PivotSmem<KM>), st>>>(probs, s, pp);
     return 1;
   }
-  k_pivot<KM, PV_SPLIT><<<grid, 4 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
+  k_pivot<KM, PV_SPLIT, many_blocks(KM)><<<grid, 4 * KM, core_smem_bytes<KM>(), st>>>(probs, s, pp);
   k_pivot_orth<KM><<<grid, 4 * KM, sizeof(OrthSmem<KM>), st>>>(probs, s, pp);
   return 2;
 }
