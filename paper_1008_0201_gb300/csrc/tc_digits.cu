@@ -8,8 +8,8 @@
 //     becomes 8 balanced 7-bit digits (ozaki.cuh), each an FP16 integer;
 //   - the digits are written as K-major operands with the 128-byte swizzle (X~: 8 planes of
 //     128 rows x 64 K; V~: 8 planes of 64 columns x 64 K) and one thread issues
-//     tcgen05.mma kind::f16 (M = 128, N = 64, K = 16) for every digit pair (t, u), t + u <= 8;
-//     products are exact and the level sums acc_L = sum_{t+u=L} d_t d_u stay below 2^23 (64-term
+//     tcgen05.mma kind::f16 (M = 128, K = 16, N = 64 per plane of V~, up to four planes at once)
+//     for the digit pairs (t, u), t + u <= 8; products are exact and the level sums acc_L = sum_{t+u=L} d_t d_u stay below 2^23 (64-term
 //     contraction), where the FP32 accumulation in tensor memory is exact;
 //   - levels 0..7 fill the 512 tensor-memory columns (one 64-column block per level); level 8
 //     reuses block 0 once level 0 has been read;
@@ -105,10 +105,9 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     const int r0 = (isg ? t : t - gtiles) << 7;
     const int rows = min(128, (isg ? a.mp : a.np) - r0);
     // What lies past the tile's rows or the pair's columns is not formed: a warp whose 32 rows or 16
-    // columns lie past them rests, the contraction takes ceil(k / 16) steps of 16 and the product
-    // N = 16 ceil(k / 16) columns.  (Operand rows left unwritten reach only their own, unread, rows or
-    // columns of the product.)  One pair of 64 rows and 16 columns 25.6 -> 17.9 us, 4000 problems of
-    // orders 8..128 819 -> 756 us.
+    // columns lie past them rests, and the contraction takes ceil(k / 16) steps of 16.  (Operand rows
+    // left unwritten reach only their own, unread, rows or columns of the product.)  One pair of 64 rows
+    // and 16 columns 25.6 -> 17.9 us, 4000 problems of orders 8..128 819 -> 756 us.
     const int k16 = (k + 15) >> 4;
     const bool works = 32 * (warp & 3) < rows && cq < k16;  // uniform per warp: its part of X~ and of Y
     const bool vworks = vc < 16 * k16 && vk0 < 16 * k16;    // its part of V~
@@ -126,11 +125,13 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     __syncthreads();
     // ---- column bounds c_k of the tile (a warp holds 32 rows of 16 columns)
     if (works) {
+      int e = 0;  // lane j: of column j
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)oz_bexp(x[j]));
-        if (lane == 0 && e > 0) atomicMax(&cexp[16 * cq + j], e);
+        const int ej = (int)__reduce_max_sync(0xffffffffu, (unsigned)oz_bexp(x[j]));
+        if (lane == j) e = ej;
       }
+      if (lane < 16 && e > 0) atomicMax(&cexp[16 * cq + lane], e);
     }
     __syncthreads();
     // ---- row groups of X~ and column groups of V~
@@ -198,18 +199,24 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     }
     tc::fence_proxy_async_smem();
     __syncthreads();
-    // ---- levels 0..7: block L (TMEM columns 64 L ..) accumulates sum_{t+u=L} X_t V_u
-    const uint32_t idesc = tc::idesc_f32acc(tc::FMT_F16, 128, 16 * k16, 0, 0);
+    // ---- levels 0..7: block L (TMEM columns 64 L ..) accumulates sum_{t+u=L} X_t V_u.  The planes of
+    // V~ lie one after the other, so one MMA of N = 64 nb takes X_t against planes u .. u + nb - 1 into
+    // blocks t + u .. t + u + nb - 1: 12 MMAs per 16 K in place of 36, each plane of X~ read once or
+    // twice and no descriptor formed in the loop: 15.3 -> 5.3 thousand clocks of a full tile's 60.
+    const uint64_t dx = tc::desc_sw128(xs, 16, 1024), dv = tc::desc_sw128(vs, 16, 1024);
     if (tid == 0) {
       tc::fence_after_sync();
 #pragma unroll 1
       for (int kk = 0; kk < k16; ++kk)
-#pragma unroll 1
-        for (int L = 0; L < OZ_T; ++L)
-          for (int tt = 0; tt <= L; ++tt)
-            tc::mma_f16(tb + 64 * L, tc::desc_sw128(xs + tt * TD_XPLANE + kk * 32, 16, 1024),
-                        tc::desc_sw128(vs + (L - tt) * TD_VPLANE + kk * 32, 16, 1024), idesc,
+#pragma unroll
+        for (int tt = 0; tt < OZ_T; ++tt)
+#pragma unroll
+          for (int u = 0; u < OZ_T - tt; u += 4) {
+            const int nb = (OZ_T - tt - u < 4) ? OZ_T - tt - u : 4;
+            tc::mma_f16(tb + 64 * (tt + u), dx + ((tt * TD_XPLANE + kk * 32) >> 4),
+                        dv + ((u * TD_VPLANE + kk * 32) >> 4), tc::idesc_f32acc(tc::FMT_F16, 128, 64 * nb, 0, 0),
                         (kk > 0 || tt > 0) ? 1u : 0u);
+          }
       tc::mma_commit(&bar[0]);
     }
     if (__syncthreads_or(!tc::mbar_wait(&bar[0], it & 1))) {
@@ -228,10 +235,10 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
       tc::fence_after_sync();
 #pragma unroll 1
       for (int kk = 0; kk < k16; ++kk)
+#pragma unroll
         for (int tt = 1; tt < OZ_T; ++tt)
-          tc::mma_f16(tb, tc::desc_sw128(xs + tt * TD_XPLANE + kk * 32, 16, 1024),
-                      tc::desc_sw128(vs + (8 - tt) * TD_VPLANE + kk * 32, 16, 1024), idesc,
-                      (kk > 0 || tt > 1) ? 1u : 0u);
+          tc::mma_f16(tb, dx + ((tt * TD_XPLANE + kk * 32) >> 4), dv + (((8 - tt) * TD_VPLANE + kk * 32) >> 4),
+                      tc::idesc_f32acc(tc::FMT_F16, 128, 64, 0, 0), (kk > 0 || tt > 1) ? 1u : 0u);
       tc::mma_commit(&bar[1]);
     }
     // eight output columns at a time (sixteen at once need all the registers and spill): levels 1..7,
