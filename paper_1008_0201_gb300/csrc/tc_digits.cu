@@ -91,19 +91,46 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
   const uint32_t lrow = tb + ((uint32_t)(32 * (warp & 3)) << 16) + 16 * cq;
   bool bad = false;
   int it = 0;
-  for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
-    const int pair = item / ntiles, t = item - pair * ntiles;
-    if (a.skip[pair]) continue;  // uniform over the CTA
+  // The tile after the current one is loaded while the tensor cores work on the current one: the
+  // lookups of a tile and its loads are one chain of dependent reads, 12 of the 49 thousand clocks of
+  // a tile; with the loads ahead 4 (4000 problems of orders 8..128 64.1 -> 62.6 ms).
+  struct Tile {
+    int item, pair, op, oq, wp, k, ld, rows;
+    double* col0;  // row r of the tile in column 0
+  } nx;
+  double x[16];
+  auto fetch = [&](int item) {  // the first item from here on whose pair rotated
+    int pair = 0;
+    for (; item < nitems; item += gridDim.x) {
+      pair = item / ntiles;
+      if (!a.skip[pair]) break;
+    }
+    nx.item = item;
+    if (item >= nitems) return;
+    const int t = item - pair * ntiles;
     const int* sp = a.pairs + (size_t)s * a.half * 2;
     const int p = sp[2 * pair], q = sp[2 * pair + 1];
-    const int op = a.boff[p], wp = a.boff[p + 1] - op, oq = a.boff[q], wq = a.boff[q + 1] - oq;
-    const int k = wp + wq;
-    const double* Vp = a.vp + (size_t)pair * a.apld * a.apld;
+    nx.pair = pair;
+    nx.op = a.boff[p];
+    nx.wp = a.boff[p + 1] - nx.op;
+    nx.oq = a.boff[q];
+    nx.k = nx.wp + a.boff[q + 1] - nx.oq;
     const bool isg = t < gtiles;
-    double* base = isg ? a.Gw : a.Vw;
-    const int ld = isg ? a.mp : a.np;
+    nx.ld = isg ? a.mp : a.np;
     const int r0 = (isg ? t : t - gtiles) << 7;
-    const int rows = min(128, (isg ? a.mp : a.np) - r0);
+    nx.rows = min(128, nx.ld - r0);
+    nx.col0 = (isg ? a.Gw : a.Vw) + r0 + r;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int c = 16 * cq + j;
+      x[j] = (c < nx.k && r < nx.rows) ? nx.col0[(size_t)(c < nx.wp ? nx.op + c : nx.oq + c - nx.wp) * nx.ld] : 0.0;
+    }
+  };
+  fetch(blockIdx.x);
+  while (nx.item < nitems) {
+    const Tile cur = nx;
+    const int k = cur.k, rows = cur.rows, wp = cur.wp, op = cur.op, oq = cur.oq;
+    const double* Vp = a.vp + (size_t)cur.pair * a.apld * a.apld;
     // What lies past the tile's rows or the pair's columns is not formed: a warp whose 32 rows or 16
     // columns lie past them rests, and the contraction takes ceil(k / 16) steps of 16.  (Operand rows
     // left unwritten reach only their own, unread, rows or columns of the product.)  One pair of 64 rows
@@ -111,13 +138,7 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     const int k16 = (k + 15) >> 4;
     const bool works = 32 * (warp & 3) < rows && cq < k16;  // uniform per warp: its part of X~ and of Y
     const bool vworks = vc < 16 * k16 && vk0 < 16 * k16;    // its part of V~
-    // ---- loads (all issued before use)
-    double x[16], v[8];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int c = 16 * cq + j;
-      x[j] = (c < k && r < rows) ? base[(size_t)(c < wp ? op + c : oq + c - wp) * ld + r0 + r] : 0.0;
-    }
+    double v[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = (vc < k && vk0 + j < k) ? __ldg(Vp + (size_t)vc * a.apld + vk0 + j) : 0.0;
     if (tid < 64) cexp[tid] = 0;
@@ -219,15 +240,21 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
           }
       tc::mma_commit(&bar[0]);
     }
+    fetch(cur.item + gridDim.x);
     if (__syncthreads_or(!tc::mbar_wait(&bar[0], it & 1))) {
       bad = true;
       break;
     }
     tc::fence_after_sync();
-    uint32_t l0[16];
+    int q01[16];
     if (works) {
-      tc::tmem_ld16(lrow, l0);
+      uint32_t la[16], lb[16];
+      tc::tmem_ld16(lrow, la);
+      tc::tmem_ld16(lrow + 64, lb);
       tc::tmem_wait_ld();
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        q01[j] = f32_small_int(__uint_as_float(la[j])) * 128 + f32_small_int(__uint_as_float(lb[j]));
     }
     tc::fence_before_sync();
     __syncthreads();  // level 0 read everywhere: block 0 is free for level 8
@@ -241,35 +268,23 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
                       tc::idesc_f32acc(tc::FMT_F16, 128, 64, 0, 0), (kk > 0 || tt > 1) ? 1u : 0u);
       tc::mma_commit(&bar[1]);
     }
-    // eight output columns at a time (sixteen at once need all the registers and spill): levels 1..7,
-    // two levels joined in 32 bits, then level 8
+    // four output columns at a time (more need all the registers and spill): levels 2..7, two levels
+    // joined in 32 bits, then level 8
     const int ea = rexp[r];
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      int q01[8], q23[8], q45[8], q67[8];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      int q23[4], q45[4], q67[4];
       if (works) {
-        uint32_t la[8], lb[8], lc[8];
-        tc::tmem_ld8(lrow + 64 + 8 * h, la);
-        tc::tmem_ld8(lrow + 128 + 8 * h, lb);
-        tc::tmem_ld8(lrow + 192 + 8 * h, lc);
+        uint32_t l[6][4];
+#pragma unroll
+        for (int u = 0; u < 6; ++u) tc::tmem_ld4(lrow + 64 * (u + 2) + 4 * h, l[u]);
         tc::tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          q01[j] = f32_small_int(__uint_as_float(h ? l0[8 + j] : l0[j])) * 128 + f32_small_int(__uint_as_float(la[j]));
-          q23[j] = f32_small_int(__uint_as_float(lb[j])) * 128 + f32_small_int(__uint_as_float(lc[j]));
+        for (int j = 0; j < 4; ++j) {
+          q23[j] = f32_small_int(__uint_as_float(l[0][j])) * 128 + f32_small_int(__uint_as_float(l[1][j]));
+          q45[j] = f32_small_int(__uint_as_float(l[2][j])) * 128 + f32_small_int(__uint_as_float(l[3][j]));
+          q67[j] = f32_small_int(__uint_as_float(l[4][j])) * 128 + f32_small_int(__uint_as_float(l[5][j]));
         }
-        tc::tmem_ld8(lrow + 256 + 8 * h, la);
-        tc::tmem_ld8(lrow + 320 + 8 * h, lb);
-        tc::tmem_wait_ld();
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          q45[j] = f32_small_int(__uint_as_float(la[j])) * 128 + f32_small_int(__uint_as_float(lb[j]));
-        tc::tmem_ld8(lrow + 384 + 8 * h, la);
-        tc::tmem_ld8(lrow + 448 + 8 * h, lb);
-        tc::tmem_wait_ld();
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          q67[j] = f32_small_int(__uint_as_float(la[j])) * 128 + f32_small_int(__uint_as_float(lb[j]));
       }
       if (h == 0) {
         if (__syncthreads_or(!tc::mbar_wait(&bar[1], it & 1))) {
@@ -279,17 +294,17 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
         tc::fence_after_sync();
       }
       if (works) {
-        uint32_t l8[8];
-        tc::tmem_ld8(lrow + 8 * h, l8);
+        uint32_t l8[4];
+        tc::tmem_ld4(lrow + 4 * h, l8);
         tc::tmem_wait_ld();
         if (r < rows) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int c = 16 * cq + 8 * h + j;
+          for (int j = 0; j < 4; ++j) {
+            const int c = 16 * cq + 4 * h + j;
             if (c < k) {
-              const long long hi = (long long)q01[j] * 16384 + q23[j];
+              const long long hi = (long long)q01[4 * h + j] * 16384 + q23[j];
               const long long lo = ((long long)q45[j] * 16384 + q67[j]) * 128 + f32_small_int(__uint_as_float(l8[j]));
-              base[(size_t)(c < wp ? op + c : oq + c - wp) * ld + r0 + r] =
+              cur.col0[(size_t)(c < wp ? op + c : oq + c - wp) * cur.ld] =
                   oz_assemble_small(hi, lo, 35, ea + vexp[c] - 2056 - 56);
             }
           }
