@@ -70,7 +70,7 @@ __global__ void k_gram32_tc(const JacProb* probs, int s, int CS, const __grid_co
 __global__ void k_update32_tc(const JacProb* probs, int s, int gtiles, int tpc, const __grid_constant__ CUtensorMap tmG,
                               const __grid_constant__ CUtensorMap tmV);
 __global__ void k_update_oz_tc(const JacProb* probs, int s);
-__global__ void k_gram_oz_tc(const JacProb* probs, int s, int CS);
+__global__ void k_gram_oz_tc(const JacProb* probs, int s, int CS, int VR);
 size_t tc_update_oz_smem_bytes();
 size_t tc_gram_oz_smem_bytes();
 size_t tc_gram32_smem_bytes();
@@ -527,9 +527,16 @@ int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, in
                        (const JacProb*)dprobs, s, CS32, maps->g32);
   else if (lowp)
     r = launch_cluster(k_gram32, dim3(max_half * CS32, count), CS32, 128, 0, st, (const JacProb*)dprobs, s, CS32);
-  else if (pp.oz == 2)
-    r = launch_cluster(k_gram_oz_tc, dim3(max_half * CS, count), CS, 512, tc_gram_oz_smem_bytes(), st,
-                       (const JacProb*)dprobs, s, CS);
+  else if (pp.oz == 2 || (pp.oz && km == 64 && 64 * gslabs > 128 * CS)) {
+    // Two kernels with the same bits.  The tensor-memory one carries its results through more hands
+    // before the first row counts and takes less per stage of 128 rows: with 64 rows per share (512
+    // columns) k_gram_oz 20.7 us, k_gram_oz_tc 22.5; with 288 (32 pairs, 2304 rows) 94 and 67.
+    // Two shares of the rows per CTA where one each takes a second wave of CTAs (one per SM): 32 pairs
+    // in 8 shares each 86 -> 67 us.
+    const int VR = (CS > 1 && (long long)max_half * count * CS > 152) ? 2 : 1;
+    r = launch_cluster(k_gram_oz_tc, dim3(max_half * CS / VR, count), CS / VR, 512, tc_gram_oz_smem_bytes(), st,
+                       (const JacProb*)dprobs, s, CS, VR);
+  }
   else if (pp.oz)
     r = launch_cluster(k_gram_oz, dim3(max_half * CS, count), CS, 256, oz_gram_smem_bytes(), st,
                        (const JacProb*)dprobs, s, CS);

@@ -27,8 +27,8 @@ __device__ __forceinline__ int oz_pair_col(int c, int wp, int op, int oq) { retu
 // k x k block (20 at k = 64) go to the warps (at most 3 each) and are summed in FP64 across stages.
 // Columns, rows and tiles past k and past the rows are not formed, a level sum is rounded without an
 // FP64 instruction, and the cluster's sum adds only what is there: one block of 64 rows and 16
-// columns 21.5 -> 10.4 us, 4000 problems of orders 8..128 572 -> 265 us, 32 pairs of 2304 rows
-// 112 -> 94 us (mma.sync is then ~half of a stage).
+// columns 21.5 -> 10.4 us, 4000 problems of orders 8..128 572 -> 265 us (mma.sync is then ~half of a
+// stage; blocks of many stages go to k_gram_oz_tc).
 #define OZG_ROWS 128
 #define OZG_NL 8  // levels kept: the Gram's groups are its own columns, bounds within ~4x of the terms
 #define OZG_P (OZG_ROWS + 8)  // 272-byte digit rows: 16-byte aligned, ldmatrix conflict-free

@@ -35,11 +35,6 @@ namespace {
 __device__ __forceinline__ unsigned char* align1k_d(unsigned char* p) {
   return reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~(uintptr_t)1023);
 }
-__device__ __forceinline__ int warp_max_int(int v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 }  // namespace
 
 #define TD_XPLANE 16384                       // 128 rows x 128 B
@@ -51,12 +46,6 @@ __device__ __forceinline__ int warp_max_int(int v) {
 #define TD_NO_EXP (-100000)
 
 size_t tc_update_oz_smem_bytes() { return TD_SMEM; }
-
-// the integer rounding of k_gram_oz_tc, called rather than inlined: keeping it out of line keeps the
-// unrolled kernel within the instruction cache
-__device__ __noinline__ double oz_assemble_call(long long hi, long long lo, int sh, int e) {
-  return oz_assemble(hi, lo, sh, e);
-}
 
 __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restrict__ probs, int s) {
   extern __shared__ unsigned char td_raw[];
@@ -327,42 +316,43 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
 }
 
 // ------------------------------------------------------------------------------------ Gram
-// FP64-accurate Gram block A_P = X^T X (Eq. (3.4)) from exact FP16 digit products, as k_gram_oz:
-// grid (half * CS, nprob), cluster (CS, 1, 1), the CTAs of a cluster splitting the rows; per
-// group of 128 rows every column is a scale group (bound exponent E_c), its values become 8
-// digits, levels 0..7 are kept (36 digit products per multiply-add), and the level sums of a
-// group are rounded to FP64 with the group's exponents and added up in FP64 across groups.
+// FP64-accurate Gram block A_P = X^T X (Eq. (3.4)) from exact FP16 digit products: grid
+// (half * CS / VR, nprob), cluster (CS / VR, 1, 1), 512 threads: the rows of a pair fall into CS shares as
+// in k_gram_oz, VR consecutive shares (1 or 2) to a CTA, with the same stages of 128 rows, scale groups (every column, bound exponent E_c), 8
+// digits, levels 0..7 and order of the FP64 additions: the two kernels give the same bits.
 //
-// tcgen05 layout.  The operand is X^T: 64 rows (the pair's columns) by 128 K (the group's rows),
-// as two 64-K chunks; inside a chunk the 8 digit planes follow each other (plane t at t * 8 KB),
-// so that one M = 128 operand covers planes a and a + 1.  An MMA with A = [D_a; D_{a+1}] and
-// B = D_v (N = 64) puts D_a D_v^T (level a + v) in TMEM lanes 0..63 and D_{a+1} D_v^T (level
-// a + v + 1) in lanes 64..127 of the 64-column block L = a + v.  Tiling every column v of the
-// (t, v) product table with such pairs of rows (a, a + 1), a = 0, 2, 4, .., covers each product
-// with t + v <= 7 exactly once in 20 MMAs per 16 K (instead of 36); the pairs that reach
-// t + v = 8 land in the lower half of block 7, which is not read.  Level L is then the upper half
-// of block L plus the lower half of block L - 1: the lower lanes gather their share in int64 and
-// pass it to the upper lanes through shared memory, which round each entry once (oz_assemble).
+// tcgen05 layout.  The operand is X^T: 64 rows (the pair's columns) by 128 K (the stage's rows), as two
+// 64-K chunks; inside a chunk the 8 digit planes follow each other (plane t at t * 8 KB).  So one
+// M = 128 operand covers planes a and a + 1, and one N = 64 nb operand planes v .. v + nb - 1: an MMA puts
+// D_a D_u^T (level a + u) in TMEM lanes 0..63 and D_{a+1} D_u^T (level a + u + 1) in lanes 64..127 of the
+// 64-column block a + u, u = v .. v + nb - 1.  With a = 0, 2, 4, 6 and u <= 7 - a every product with
+// t + u <= 7 is there once, in 6 MMAs per 16 K (20 with N = 64; 36 products); what reaches level 8
+// lands in the lower lanes of block 7 and is not read.  Level L is the upper lanes of block L plus the
+// lower lanes of block L - 1: each half gathers its share of a 16-column strip in integers, finishes 8
+// of the columns and passes its share of the other 8 to the other half through shared memory.
 // A_P is exactly symmetric (the level sums of (i, j) and (j, i) are the same integers), so only
 // entries j >= i are formed.
+// The MMAs take 4 thousand clocks of the 19 of a stage, where mma.sync (k_gram_oz) takes about half of
+// 34; the digits take 5, the integer sums and their rounding 8.  32 pairs of 2304 rows: 94 us with
+// k_gram_oz, 86 with one share per CTA, 67 with two.
 #define TGD_CHUNK 65536                        // 8 planes x 64 rows x 128 B
-#define TGD_TOT (2 * TGD_CHUNK)                // FP64 partial [64][65] after the digits
-#define TGD_MISC (TGD_TOT + 64 * 65 * 8)
+#define TGD_TOT (2 * TGD_CHUNK)                // FP64 partials [VR][64][65] after the digits
+#define TGD_MISC (TGD_TOT + 2 * 64 * 65 * 8)
 #define TGD_SMEM (1024 + TGD_MISC + 512 + 128)
 
 size_t tc_gram_oz_smem_bytes() { return TGD_SMEM; }
 
-__global__ void __launch_bounds__(512, 1) k_gram_oz_tc(const JacProb* __restrict__ probs, int s, int CS) {
+__global__ void __launch_bounds__(512, 1) k_gram_oz_tc(const JacProb* __restrict__ probs, int s, int CS, int VR) {
   extern __shared__ unsigned char tgd_raw[];
   unsigned char* sm = align1k_d(tgd_raw);
-  double* tot = reinterpret_cast<double*>(sm + TGD_TOT);  // [64][65], entries j >= i
-  int* E = reinterpret_cast<int*>(sm + TGD_MISC);         // [64]
+  double* C = reinterpret_cast<double*>(sm + TGD_TOT);  // [VR][64][65], entries j >= i
+  int* E = reinterpret_cast<int*>(sm + TGD_MISC);       // [64]
   uint64_t* bar = reinterpret_cast<uint64_t*>(E + 64);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 1);
-  long long* xch = reinterpret_cast<long long*>(sm);      // [64][64][2], over the digits
+  longlong2* xch = reinterpret_cast<longlong2*>(sm);    // [column][row], over the digits
   cg::cluster_group cluster = cg::this_cluster();
   const JacProb& a = probs[blockIdx.y];
-  const int pair = blockIdx.x / CS;
+  const int nc = CS / VR, pair = blockIdx.x / nc;
   const int crank = (int)cluster.block_rank();
   if (!a.active || s >= a.nsteps || pair >= a.counts[s]) return;
   const int* sp = a.pairs + (size_t)s * a.half * 2;
@@ -372,29 +362,10 @@ __global__ void __launch_bounds__(512, 1) k_gram_oz_tc(const JacProb* __restrict
   const int k = wp + wq;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rpc = ((a.mp / CS + 15) & ~15);
-  const int r_begin = min(a.mp, crank * rpc), r_end = min(a.mp, r_begin + rpc);
-  for (int e = tid; e < 64 * 65; e += 512) tot[e] = 0.0;
-  if (tid == 0) {
-    tc::mbar_init(&bar[0], 1);
-    tc::fence_barrier_init();
-  }
-  if (warp == 0) tc::tmem_alloc(tslot, 512);
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tb = *tslot;
-  constexpr uint32_t idesc = tc::idesc_f32acc(tc::FMT_F16, 128, 64, 0, 0);
-  const uint32_t ds = tc::smem_u32(sm);
-  // epilogue: warp w reads TMEM lanes 32 (w & 3) .. + 31 (operand rows), columns 16 (w >> 2) .. + 15
-  const int lrow = 32 * (warp & 3) + lane, cg16 = warp >> 2;
-  const bool upper = (warp & 3) < 2;
-  const uint32_t laddr = tb + ((uint32_t)(32 * (warp & 3)) << 16) + 16 * cg16;
-  bool bad = false;
-  int it = 0;
-  for (int g0 = r_begin; g0 < r_end; g0 += 128, ++it) {
-    const int rs = min(128, r_end - g0);
-    // warp w: columns 4 w .. 4 w + 3; lane l: group rows 4 l .. 4 l + 3 (K-adjacent digits)
-    double x[4][4];
+  auto begin_of = [&](int vr) { return min(a.mp, (crank * VR + vr) * rpc); };
+  // warp w: columns 4 w .. 4 w + 3; lane l: stage rows 4 l .. 4 l + 3 (K-adjacent digits)
+  double x[4][4];
+  auto fetch = [&](int g0, int rs) {
 #pragma unroll
     for (int cc = 0; cc < 4; ++cc) {
       const int c = 4 * warp + cc;
@@ -407,120 +378,177 @@ __global__ void __launch_bounds__(512, 1) k_gram_oz_tc(const JacProb* __restrict
         x[cc][i + 1] = v.y;
       }
     }
-    int ec[4];
+  };
+  fetch(begin_of(0), begin_of(1) - begin_of(0));
+  if (tid == 0) {
+    tc::mbar_init(&bar[0], 1);
+    tc::fence_barrier_init();
+  }
+  if (warp == 0) tc::tmem_alloc(tslot, 512);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tb = *tslot;
+  const uint64_t dd = tc::desc_sw128(tc::smem_u32(sm), 16, 1024);
+  // epilogue: warp w reads TMEM lanes 32 (w & 3) .. + 31 (operand rows) and the strip of columns
+  // c0 = 16 (w >> 2) .. + 15; it finishes columns c0 .. + 7 (upper lanes) or c0 + 8 .. + 15
+  const bool upper = (warp & 3) < 2;
+  const int i = (32 * (warp & 3) + lane) & 63, c0 = 16 * (warp >> 2);
+  const bool works = c0 + 15 >= (i & 32) && c0 < k && (i & 32) < k;  // uniform: some entry j >= i of the block
+  const uint32_t laddr = tb + ((uint32_t)(32 * (warp & 3)) << 16) + c0;
+  const int cf = c0 + (upper ? 0 : 8), cs = c0 + (upper ? 8 : 0);
+  // this lane's share of eight columns from c (c0 or c0 + 8)
+  auto gather = [&](int c, long long(&hi)[8], long long(&lo)[8]) {
+    uint32_t lv[4][8];
+    int qa[8], qb[8];
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc)
-      ec[cc] = warp_max_int(max(max(oz_bexp(x[cc][0]), oz_bexp(x[cc][1])), max(oz_bexp(x[cc][2]), oz_bexp(x[cc][3]))));
-    if (lane == 0)
+    for (int h = 0; h < 2; ++h) {
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) E[4 * warp + cc] = ec[cc];
-    // digits: operand row c (pair column), K = group rows 4 lane .. + 3 (chunk lane >> 4)
-    {
-      unsigned char* base = sm + (lane >> 4) * TGD_CHUNK;
+      for (int u = 0; u < 4; ++u) {
+        const int L = 4 * h + u, B = L - (upper ? 0 : 1);  // uniform
+        if (B >= 0) {
+          tc::tmem_ld8(laddr + (c - c0) + 64 * B, lv[u]);
+        } else {
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        unsigned long long b[4];
-        unsigned w0[OZ_T], w1[OZ_T];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) b[i] = oz_biased(x[cc][i], oz_bexp(x[cc][i]) - ec[cc]);
-        oz_split2(b[0], b[1], w0);
-        oz_split2(b[2], b[3], w1);
-        const uint32_t off = tc::sw128_offset(4 * warp + cc, (4 * lane) & 63, 2);
-#pragma unroll
-        for (int tt = 0; tt < OZ_T; ++tt)
-          *reinterpret_cast<uint2*>(base + tt * 8192 + off) = make_uint2(w0[tt], w1[tt]);
+          for (int j = 0; j < 8; ++j) lv[u][j] = 0;
+        }
       }
-    }
-    tc::fence_proxy_async_smem();
-    __syncthreads();
-    if (tid == 0) {
-      tc::fence_after_sync();
-      unsigned started = 0;
-#pragma unroll 1
-      for (int kc = 0; kc < 2; ++kc)
-#pragma unroll 1
-        for (int ks = 0; ks < 4; ++ks)
-#pragma unroll 1
-          for (int v = 0; v < OZ_T; ++v)
-            for (int a0 = 0; a0 + v <= OZ_T - 1; a0 += 2) {
-              const int L = a0 + v;
-              const uint32_t co = kc * TGD_CHUNK + ks * 32;
-              tc::mma_f16(tb + 64 * L, tc::desc_sw128(ds + co + a0 * 8192, 16, 1024),
-                          tc::desc_sw128(ds + co + v * 8192, 16, 1024), idesc, (started >> L) & 1u);
-              started |= 1u << L;
-            }
-      tc::mma_commit(&bar[0]);
-    }
-    if (__syncthreads_or(!tc::mbar_wait(&bar[0], it & 1))) {
-      bad = true;
-      break;
-    }
-    tc::fence_after_sync();
-    // gather: upper lanes (lrow < 64) hold levels 0..7 of row i = lrow in blocks 0..7, lower
-    // lanes levels 1..7 of row i = lrow - 64 in blocks 0..6
-    long long hi[16], lo[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) hi[j] = lo[j] = 0;
-#pragma unroll
-    for (int B = 0; B < OZ_T; ++B) {
-      const int L = upper ? B : B + 1;  // level held by this lane in block B (warp-uniform)
-      if (L >= OZ_T) break;
-      uint32_t lv[16];
-      tc::tmem_ld16(laddr + 64 * B, lv);
       tc::tmem_wait_ld();
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const long long iv = f32_small_int(__uint_as_float(lv[j]));
-        if (L < 4) hi[j] += iv * (1ll << (7 * (3 - L)));
-        else lo[j] += iv * (1ll << (7 * (7 - L)));
+      for (int j = 0; j < 8; ++j) {
+        qa[j] = f32_small_int(__uint_as_float(lv[0][j])) * 128 + f32_small_int(__uint_as_float(lv[1][j]));
+        qb[j] = f32_small_int(__uint_as_float(lv[2][j])) * 128 + f32_small_int(__uint_as_float(lv[3][j]));
+        (h ? lo[j] : hi[j]) = (long long)qa[j] * 16384 + qb[j];
       }
     }
-    if (!upper) {
-      const int i = lrow - 64;
+  };
+  double* out = a.Ap + (size_t)pair * a.apld * a.apld;
+  bool bad = false;
+  int it = 0;
+  for (int vr = 0; vr < VR && !bad; ++vr) {
+    const int r_begin = begin_of(vr), r_end = begin_of(vr + 1);
+    double tot[8];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        xch[(i * 64 + 16 * cg16 + j) * 2] = hi[j];
-        xch[(i * 64 + 16 * cg16 + j) * 2 + 1] = lo[j];
+    for (int j = 0; j < 8; ++j) tot[j] = 0.0;
+    for (int g0 = r_begin; g0 < r_end; g0 += 128, ++it) {
+      const int steps = (min(128, r_end - g0) + 15) >> 4;  // of 16 K
+      int ec[4];
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc)
+        ec[cc] = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(max(oz_bexp(x[cc][0]), oz_bexp(x[cc][1])),
+                                                                   max(oz_bexp(x[cc][2]), oz_bexp(x[cc][3]))));
+      if (lane == 0) *reinterpret_cast<int4*>(&E[4 * warp]) = make_int4(ec[0], ec[1], ec[2], ec[3]);
+      // digits: operand row c (pair column), K = stage rows 4 lane .. + 3 (chunk lane >> 4)
+      if (16 * steps > 4 * lane) {
+        unsigned char* base = sm + (lane >> 4) * TGD_CHUNK;
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) {
+          unsigned long long b[4];
+          unsigned w0[OZ_T], w1[OZ_T];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) b[u] = oz_biased(x[cc][u], oz_bexp(x[cc][u]) - ec[cc]);
+          oz_split2(b[0], b[1], w0);
+          oz_split2(b[2], b[3], w1);
+          const uint32_t off = tc::sw128_offset(4 * warp + cc, (4 * lane) & 63, 2);
+#pragma unroll
+          for (int tt = 0; tt < OZ_T; ++tt)
+            *reinterpret_cast<uint2*>(base + tt * 8192 + off) = make_uint2(w0[tt], w1[tt]);
+        }
       }
-    }
-    __syncthreads();
-    if (upper && lrow < k) {
-      const int i = lrow;
+      tc::fence_proxy_async_smem();
+      __syncthreads();
+      if (tid == 0) {
+        tc::fence_after_sync();
+#pragma unroll 1
+        for (int kk = 0; kk < steps; ++kk) {
+          const uint64_t dk = dd + (((kk >> 2) * TGD_CHUNK + (kk & 3) * 32) >> 4);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int c = 16 * cg16 + j;
-        if (c >= i && c < k) {
-          const long long H = hi[j] + xch[(i * 64 + c) * 2], Lo = lo[j] + xch[(i * 64 + c) * 2 + 1];
-          tot[i * 65 + c] += oz_assemble_call(H, Lo, 28, E[i] + E[c] - 2056 - 49);
+          for (int a0 = 0; a0 < OZ_T; a0 += 2)
+#pragma unroll
+            for (int v = 0; v < OZ_T - a0; v += 4) {
+              const int nb = (OZ_T - a0 - v < 4) ? OZ_T - a0 - v : 4;
+              tc::mma_f16(tb + 64 * (a0 + v), dk + ((a0 * 8192) >> 4), dk + ((v * 8192) >> 4),
+                          tc::idesc_f32acc(tc::FMT_F16, 128, 64 * nb, 0, 0), (kk > 0 || a0 > 0) ? 1u : 0u);
+            }
+        }
+        tc::mma_commit(&bar[0]);
+      }
+      if (g0 + 128 < r_end) fetch(g0 + 128, r_end - g0 - 128);
+      else if (vr + 1 < VR) fetch(r_end, begin_of(vr + 2) - r_end);
+      if (__syncthreads_or(!tc::mbar_wait(&bar[0], it & 1))) {
+        bad = true;
+        break;
+      }
+      tc::fence_after_sync();
+      long long hi[8], lo[8];
+      if (works) {
+        gather(cs, hi, lo);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) xch[(cs + j) * 64 + i] = make_longlong2(hi[j], lo[j]);
+        gather(cf, hi, lo);
+      }
+      __syncthreads();
+      if (works) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int c = cf + j;
+          if (c >= i && c < k) {
+            const longlong2 o = xch[c * 64 + i];
+            const double y = oz_assemble_small(hi[j] + o.x, lo[j] + o.y, 28, E[i] + E[c] - 2056 - 49);
+            tot[j] = (g0 == r_begin) ? y : tot[j] + y;
+          }
+        }
+      }
+      tc::fence_before_sync();
+      __syncthreads();  // TMEM, the exchange and E read before the next stage overwrites them
+    }
+    if (works) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int c = cf + j;
+        if (c < i || c >= k) continue;
+        if (CS > 1) {
+          C[vr * 64 * 65 + i * 65 + c] = tot[j];
+        } else {  // nothing to add up
+          out[c * a.apld + i] = tot[j];
+          out[i * a.apld + c] = tot[j];
         }
       }
     }
-    tc::fence_before_sync();
-    __syncthreads();  // TMEM, the exchange and E read before the next group overwrites them
   }
   if (bad && tid == 0) {
     atomicOr(a.pflags, JAC_DEVERR_TIMEOUT);
     tc::mbar_wait(&bar[0], it & 1);
   }
   tc::fence_before_sync();
-  cluster.sync();
-  const int totn = k * k, per = (totn + CS - 1) / CS;
-  const int e0 = crank * per, e1 = min(totn, e0 + per);
-  double* out = a.Ap + (size_t)pair * a.apld * a.apld;
-  for (int e = e0 + tid; e < e1; e += 512) {
-    const int i = e % k, j = e / k;
-    const int lo_ = min(i, j), hi_ = max(i, j);
-    double part[16];  // all remote loads issued before the fixed-order sum
-#pragma unroll
-    for (int rk = 0; rk < 16; ++rk) part[rk] = (rk < CS) ? cluster.map_shared_rank(tot, rk)[lo_ * 65 + hi_] : 0.0;
-    double sum = 0.0;
-#pragma unroll
-    for (int rk = 0; rk < 16; ++rk) sum += part[rk];
-    out[j * a.apld + i] = sum;
-  }
-  cluster.sync();  // keep every partial alive until all remote reads are done
+  __syncthreads();
   tc::fence_after_sync();
   if (warp == 0) tc::tmem_dealloc(tb, 512);
+  if (CS == 1) return;
+  cluster.sync();
+  // the upper triangle, rows n and k - 1 - n together as one row of k + 1 entries (as k_gram_oz)
+  const int totn = ((k + 1) >> 1) * (k + 1), per = (totn + nc - 1) / nc;
+  const int e0 = crank * per, e1 = min(totn, e0 + per);
+  for (int e = e0 + tid; e < e1; e += 512) {
+    const int n = e / (k + 1), o = e - n * (k + 1);
+    int ri = n, rj = n + o;
+    if (rj >= k) {
+      ri = k - 1 - n;
+      rj = ri + (o - (k - n));
+      if (ri == n) continue;  // the middle row of an odd block
+    }
+    double part[16];  // all remote loads issued before the fixed-order sum
+#pragma unroll
+    for (int rk = 0; rk < 16; ++rk)
+      part[rk] = (rk < CS) ? cluster.map_shared_rank(C, rk / VR)[rk % VR * 64 * 65 + ri * 65 + rj] : 0.0;
+    double sum = part[0];
+#pragma unroll
+    for (int rk = 1; rk < 16; ++rk)
+      if (rk < CS) sum += part[rk];
+    out[rj * a.apld + ri] = sum;
+    out[ri * a.apld + rj] = sum;
+  }
+  cluster.sync();  // keep every partial alive until all remote reads are done
 }
 
 }  // namespace jac
