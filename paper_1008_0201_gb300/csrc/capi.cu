@@ -791,7 +791,7 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   HostSlot slot;
   static_assert(sizeof(SweepRecord) + sizeof(int) <= kSlotBytes, "a sweep's record fits a slot");
   int* in_flags = reinterpret_cast<int*>(slot.p + sizeof(SweepRecord));
-  bool judged = false;
+  bool settled = false;
   auto fetch_verdict = [&]() {
     ck(cudaMemcpyAsync(in_flags, &L.io->flags, sizeof(int), cudaMemcpyDeviceToHost, st));
   };
@@ -835,16 +835,16 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   double prev_max = 1e300;
   SweepRecord hrec = {};
   bool bad_sign = false;
-  auto judge = [&]() {  // after a synchronization behind fetch_verdict
-    if (judged || status != JAC_OK) return;
-    judged = true;
+  auto settle = [&]() {  // after a synchronization behind fetch_verdict
+    if (settled || status != JAC_OK) return;
+    settled = true;
     bad_sign = (*in_flags & 2) != 0;
     if (bad_sign || (*in_flags & 1)) status = JAC_ENONFINITE;
   };
   if (n == 1 || weights) {  // no sweep; no plan from an invalid input
     fetch_verdict();
     ck(cudaStreamSynchronize(st));
-    judge();
+    settle();
   }
   int last_steps = 0;
   ProfRun prof;
@@ -918,11 +918,11 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
       status = r;
     }
     ck(cudaMemcpyAsync(slot.p, L.rec, sizeof(SweepRecord), cudaMemcpyDeviceToHost, st));
-    if (!judged) fetch_verdict();
+    if (!settled) fetch_verdict();
     ck(cudaStreamSynchronize(st));
     std::memcpy(&hrec, slot.p, sizeof(SweepRecord));
     if (replayed) replayed->prof.accumulate();
-    judge();
+    settle();
     if (status != JAC_OK) break;
     if (info && sweeps < 64) info->sweep_max_scaled[sweeps] = hrec.max_scaled;
     ++sweeps;
