@@ -563,7 +563,8 @@ int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, in
     // tensor-core digit update: one CTA per SM walks (pair, 128-row tile) items of its problem
     // (tslabs counts 64-row slabs, gslabs those of G).  nx CTAs per problem: the count whose last
     // wave leaves the fewest SMs idle, the larger number of items per CTA on ties (256 x 256 problems,
-    // 96 at once: 8 items each, 166 us with 2 CTAs per problem, 129 us with this rule).
+    // 96 at once: 8 items each, 166 us with 2 CTAs per problem, 129 us with this rule, 99 with the
+    // kernel as it is now).
     const int items = max_half * ((gslabs + 1) / 2 + (tslabs - gslabs + 1) / 2);
     int nx = 1;
     long long best = -1;

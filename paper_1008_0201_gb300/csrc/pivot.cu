@@ -1390,7 +1390,7 @@ __device__ __forceinline__ bool in_step(const JacProb& a, int s, int pair) {
 // V_P in FP64 storage from the FP32 transform (FP32 sweeps).  PV_SPLIT: phases 1-3, W handed to
 // k_pivot_orth: the core needs less than half the shared memory of phase 4, so three pivots run on an
 // SM while phase 4 takes the SM for a short time only (many pivots per step).  4000 problems of
-// orders 8..128, all pivots of a sweep step: 1.4 ms, against 4.1 ms with one 212 KB CTA per SM.
+// orders 8..128, all pivots of a sweep step: 1.24 ms, against 4.1 ms with one 212 KB CTA per SM.
 // MINB: blocks per SM that the registers must allow.  The 80 registers of three (KM = 32: six) cost the
 // core 5 of its 73 thousand clocks for a 64-column block in a block-oriented step (order 512, mixed
 // precision: 14.8 ms; with 142 registers 14.4), so steps with no more pivots than SMs take all they need.

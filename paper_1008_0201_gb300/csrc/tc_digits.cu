@@ -9,8 +9,9 @@
 //   - the digits are written as K-major operands with the 128-byte swizzle (X~: 8 planes of
 //     128 rows x 64 K; V~: 8 planes of 64 columns x 64 K) and one thread issues
 //     tcgen05.mma kind::f16 (M = 128, K = 16, N = 64 per plane of V~, up to four planes at once)
-//     for the digit pairs (t, u), t + u <= 8; products are exact and the level sums acc_L = sum_{t+u=L} d_t d_u stay below 2^23 (64-term
-//     contraction), where the FP32 accumulation in tensor memory is exact;
+//     for the digit pairs (t, u), t + u <= 8; products are exact and the level sums
+//     acc_L = sum_{t+u=L} d_t d_u stay below 2^23 (64-term contraction), where the FP32 accumulation in
+//     tensor memory is exact;
 //   - levels 0..7 fill the 512 tensor-memory columns (one 64-column block per level); level 8
 //     reuses block 0 once level 0 has been read;
 //   - each thread reads its row's level sums for 16 output columns, gathers them exactly in two
@@ -123,7 +124,8 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     // What lies past the tile's rows or the pair's columns is not formed: a warp whose 32 rows or 16
     // columns lie past them rests, and the contraction takes ceil(k / 16) steps of 16.  (Operand rows
     // left unwritten reach only their own, unread, rows or columns of the product.)  One pair of 64 rows
-    // and 16 columns 25.6 -> 17.9 us, 4000 problems of orders 8..128 819 -> 756 us.
+    // and 16 columns 25.6 -> 17.9 us, 4000 problems of orders 8..128 819 -> 756 us (549 with the MMAs and loads
+    // below).
     const int k16 = (k + 15) >> 4;
     const bool works = 32 * (warp & 3) < rows && cq < k16;  // uniform per warp: its part of X~ and of Y
     const bool vworks = vc < 16 * k16 && vk0 < 16 * k16;    // its part of V~
@@ -318,8 +320,9 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
 // ------------------------------------------------------------------------------------ Gram
 // FP64-accurate Gram block A_P = X^T X (Eq. (3.4)) from exact FP16 digit products: grid
 // (half * CS / VR, nprob), cluster (CS / VR, 1, 1), 512 threads: the rows of a pair fall into CS shares as
-// in k_gram_oz, VR consecutive shares (1 or 2) to a CTA, with the same stages of 128 rows, scale groups (every column, bound exponent E_c), 8
-// digits, levels 0..7 and order of the FP64 additions: the two kernels give the same bits.
+// in k_gram_oz, VR consecutive shares (1 or 2) to a CTA, with the same stages of 128 rows, scale groups
+// (every column, bound exponent E_c), 8 digits, levels 0..7 and order of the FP64 additions: the two
+// kernels give the same bits.
 //
 // tcgen05 layout.  The operand is X^T: 64 rows (the pair's columns) by 128 K (the stage's rows), as two
 // 64-K chunks; inside a chunk the 8 digit planes follow each other (plane t at t * 8 KB).  So one
