@@ -39,6 +39,7 @@
 #include "jacobi_common.cuh"
 #include "pair_cache.cuh"
 #include "ozaki.cuh"
+#include "rotation.h"
 
 namespace jac {
 
@@ -823,21 +824,13 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
         const int nxt = ring & 31;
         for (int st_ = 0; st_ < g; ++st_) {
           // ---- rotate the pair (ci, cj) of this slot; what does not depend on the dot product first.
-          // One branch-free path for both kinds, the slots of a warp never split on the sign
-          // pattern.  With x = a_jj - a_ii (trigonometric, Eq. (2.1): cot(2 phi) = x / (2 |a_ij|)) or
-          // x = a_ii + a_jj (hyperbolic: coth(2 phi) = -x / (2 |a_ij|)), everything scaled by
-          // rs = 1 / sqrt(a_ii a_jj) (nu = |x| rs, scaled = |a_ij| rs):
-          //   h = 1 / sqrt(nu^2 +- 4 scaled^2),  cos(h)^2 phi = 1/2 + nu h / 2,
-          //   |sin(h) phi| = scaled h / cos(h) phi.
-          // The roots need FP32 accuracy only: the rotation is orthogonal (J-orthogonal) to their
-          // rounding whatever the angle.  Two MUFU operations deep, ~90 clocks; by way of the
-          // tangent, with x and a_ij scaled by powers of two, it took 330.
+          // One branch-free path for both kinds (rotation.h): the slots of a warp never split on the
+          // sign pattern.
           const bool trig = ji == jj;
           const float sg = trig ? 1.0f : -1.0f, sg4 = 4.0f * sg;
           const float aii = fmaf(si, si, cni), ajj = fmaf(sj, sj, cnj);
-          const float rs = rsqrtf(aii) * rsqrtf(ajj);
           const float x = trig ? (sj - si) * (sj + si) + (cnj - cni) : aii + ajj;
-          const float nu = fminf(fabsf(x) * rs, 1.0e18f), nu2 = nu * nu;
+          const RotUnit ru = rot_unit(aii, ajj, x);
           // sign of the tangent: that of x (trigonometric), negative (hyperbolic)
           const unsigned tsign = trig ? __float_as_uint(x) & 0x80000000u : 0x80000000u;
           f2 d0 = f2_mul(xi[0], xj[0]), d1 = f2_mul(xi[1], xj[1]);
@@ -847,37 +840,22 @@ __device__ __forceinline__ int pivot_core(PivotState<KM>& sm, PivotWork<KM>& wk,
             d1 = f2_fma(xi[u + 1], xj[u + 1], d1);
           }
           const float aij = group_sum<LPP>((f2_lo(d0) + f2_lo(d1)) + (f2_hi(d0) + f2_hi(d1)));
-          const float scaled = fabsf(aij) * rs;
+          const float scaled = fabsf(aij) * ru.rs;
           const bool rot = (ci | cj) >= 0 && scaled > tol_in;
-          const float rr = fmaf(sg4, scaled * scaled, nu2);
-          const float h = rsqrt_ftz(rr), wh = scaled * h;
-          const float c2 = fmaf(0.5f * nu, h, 0.5f), cinv = rsqrt_ftz(c2);
-          float sa = wh * cinv, ca = c2 * cinv;
-          // the cosine of a small angle as 1 -+ s^2 / 2 rounded once (rsqrt returns the value below 1
-          // too often there, and thousands of tiny rotations would shrink V: with it alone the
-          // FP32-only eigenvalues of order 128 came out 5e-5 small, with this rule 2e-5)
-          const float y = sa * sa;
-          if (y < 3.8146973e-6f) ca = fmaf(-0.5f * sg, y, 1.0f);
-          // no hyperbolic angle annihilates a_ij (2 |a_ij| >= a_ii + a_jj by rounding): tanh = 0.9, the
-          // guard of Sec. 3.2
-          const bool guard = !(rr > 0.0f);
-          if (guard) {
-            ca = 2.2941573f;
-            sa = 2.0647416f;
-          }
-          const float c = rot ? ca : 1.0f;
-          const float es = rot ? __uint_as_float(__float_as_uint(sa) ^ ((__float_as_uint(aij) & 0x80000000u) ^ tsign)) : 0.0f;
+          const RotAngle ra = rot_angle(ru, sg, sg4, fabsf(aij));
+          const float c = rot ? ra.c : 1.0f;
+          const float es = rot ? __uint_as_float(__float_as_uint(ra.s) ^ ((__float_as_uint(aij) & 0x80000000u) ^ tsign)) : 0.0f;
           const float q21 = -sg * es;
           if (l == 0) sm.prm[buf][slot] = make_float4(c, es, q21, 0.0f);
           rotate(c, es, q21);
           my_rot += rot ? 1 : 0;
           my_max = fmaxf(my_max, rot ? scaled : 0.0f);
           // a_ii' = a_ii - t |a_ij|, a_jj' = a_jj + t |a_ij| (trigonometric); both move by
-          // t |a_ij| (hyperbolic: the J-trace is invariant); t = s / c, 1 / c = cinv.  Where the
+          // t |a_ij| (hyperbolic: the J-trace is invariant); t = s / c.  Where the
           // guard acted a_ij is not annihilated: both norms are put out of range, so that the columns
           // rest until the next inner sweep takes them afresh
-          const float ta = rot ? __uint_as_float(__float_as_uint(sa * cinv * fabsf(aij)) ^ tsign) : 0.0f;
-          const bool far = rot && guard;
+          const float ta = rot ? __uint_as_float(__float_as_uint(ra.s * ra.cinv * fabsf(aij)) ^ tsign) : 0.0f;
+          const bool far = rot && ra.guard;
           cni = far ? 1.0e8f * si * si : fmaf(-sg, ta, cni);
           cnj = far ? 1.0e8f * sj * sj : cnj + ta;
           // ---- pass one column on: the traveler round the ring, or at the end of the group's
