@@ -39,6 +39,7 @@
 #include "jacobi_common.cuh"
 #include "pair_cache.cuh"
 #include "ozaki.cuh"
+#include "residual_sum.h"
 #include "rotation.h"
 
 namespace jac {
@@ -1066,29 +1067,6 @@ __device__ __forceinline__ float block_max_f(float v, PivotOrth<KM>& so, int slo
   return r;
 }
 
-// (float)(2^E (hi 2^28 + lo) + x + y) by integer operations, for digit products of at most 64 terms
-// (|hi| < 2^40, |lo| < 2^43): the terms are aligned to a common unit of 2^-53 of the largest possible
-// digit product or 2^-58 of x and y, so the result is as accurate as an FP64 sum of them.  (GB300
-// issues ~1.6 FP64 operations per clock per SM; the FP64 form took 7 per entry, ~9k clocks per
-// residual of a 64-column block.)
-__device__ __forceinline__ long long align_bits(double x, int ub) {  // x in units of 2^(ub - 1075), truncated
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int e = (int)((u >> 52) & 0x7ff);
-  unsigned long long m = ((u & ((1ull << 52) - 1)) | (e ? 1ull << 52 : 0ull)) << 6;
-  m >>= min((unsigned)(ub + 6 - max(e, 1)), 63u);
-  return (u >> 63) ? -(long long)m : (long long)m;
-}
-__device__ __forceinline__ float residual_sum(long long hi, long long lo, int E, double x, double y) {
-  const int ex = max(oz_bexp(x), 1), ey = max(oz_bexp(y), 1);
-  // units of 2^(ub - 1075): hi 2^28 + lo = (hi 2^20 + (lo >> 8)) 2^8, so its unit is 2^(E + 8)
-  const int ub = max(max(ex, ey) - 6, E + 8 + 1075);
-  const long long q = ((hi << 20) + (lo >> 8)) >> min((unsigned)(ub - (E + 8 + 1075)), 63u);
-  const long long s = q + align_bits(x, ub) + align_bits(y, ub);
-  const int sh = ub - 1075;  // s 2^sh, in two exact steps (FP32 range)
-  const int h = max(min(sh / 2, 120), -120), h2 = max(min(sh - h, 120), -120);
-  return ((float)s * __int_as_float((h + 127) << 23)) * __int_as_float((h2 + 127) << 23);
-}
-
 // J-orthogonality residual M = V^T J V - J = W^T J + J W + W^T J W from digit products (ozaki.cuh).
 // The linear terms are exact; W^T J W, of size |W|^2, runs on the digit path with the columns of W
 // (over the k rows) as scale groups and J_r applied to the A digits by their sign bit.  So M is
@@ -1167,8 +1145,8 @@ __device__ float oz_residual(PivotOrth<KM>& so, const int* jphys, int k, int KP)
         const long long hi = (long long)(q[0] * 128 + q[1]) * 16384 + (q[2] * 128 + q[3]);
         const long long lo = (long long)(q[4] * 128 + q[5]) * 16384 + (q[6] * 128 + q[7]);
         // M_xj = (W^T J W)_xj + j_j W[j][x] + j_x W[x][j]
-        const float f = residual_sum(hi, lo, so.dexp[x] + so.dexp[j] - 2056 - 49, oz_neg_if(so.V[x * LDV + j], nj),
-                                     oz_neg_if(so.V[j * LDV + x], nx));
+        const float f = oz_residual_entry(hi, lo, so.dexp[x] + so.dexp[j] - 2056 - 49, oz_neg_if(so.V[x * LDV + j], nj),
+                                          oz_neg_if(so.V[j * LDV + x], nx));
         mloc = fmaxf(mloc, fabsf(f));
         sxj = nx ? -f : f;  // (J M)[x][j]
         sjx = nj ? -f : f;  // (J M)[j][x]
