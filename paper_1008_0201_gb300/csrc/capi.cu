@@ -1519,7 +1519,12 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
 namespace jac {
 // bytes of stream-ordered scratch, freed with cudaFreeAsync
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
-  if (!program_chose_pool()) {
+  // In a capture (the backward may be captured) the allocation becomes a node of the program's graph,
+  // which owns the memory; asking for the device's pools would end the capture.
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const bool plain = cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  if (plain && !program_chose_pool()) {
     if (cudaMemPool_t pool = own_pool(true)) {
       if (cudaMallocFromPoolAsync(p, bytes, pool, st) == cudaSuccess) return cudaSuccess;
       cudaGetLastError();
