@@ -261,6 +261,10 @@ struct HostSlot {
 // more than the launches it saves over the sweeps of a solve.  One step (24 columns): 799 us with a
 // graph, 755 direct; eight steps (64 columns): 3.20 ms with a graph, 3.62 direct.
 constexpr int kGraphSteps = 2;
+// Up to this many steps the verdict on the input waits for the first sweep's record (its own round trip
+// of ~15 us is 0.5% of a 64-column solve of eight steps).  Beyond, the graph of a sweep costs an
+// invalid input more than the round trip costs a valid one: 69 steps 1.23 ms instead of 0.38.
+constexpr int kVerdictSteps = 8;
 
 std::mutex g_attr_mutex;
 bool g_attr_done[64] = {};
@@ -787,8 +791,9 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
   k_check_finite<<<dim3(std::min(1024, (int)(((size_t)m * n + 255) / 256)), 1), 256, 0, st>>>(L.probs, L.io);
   launches += 2;
   // The verdict on the input is read with the record of the first sweep (its own round trip costs a
-  // small solve ~15 us): an invalid input is inactive by then, so the sweep's kernels skip it.  A
-  // schedule by weights is planned from the entries, so there the verdict comes first.
+  // small solve ~15 us): an invalid input is inactive by then, so the sweep's kernels skip it.  It
+  // comes first where a sweep has more than kVerdictSteps steps, and with a schedule by weights, which
+  // is planned from the entries.
   HostSlot slot;
   static_assert(sizeof(SweepRecord) + sizeof(int) <= kSlotBytes, "a sweep's record fits a slot");
   int* in_flags = reinterpret_cast<int*>(slot.p + sizeof(SweepRecord));
@@ -842,7 +847,7 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
     bad_sign = (*in_flags & 2) != 0;
     if (bad_sign || (*in_flags & 1)) status = JAC_ENONFINITE;
   };
-  if (n == 1 || weights) {  // no sweep; no plan from an invalid input
+  if (n == 1 || weights || P.nsteps > kVerdictSteps) {  // no sweep, no plan or no long graph for an invalid input
     fetch_verdict();
     ck(cudaStreamSynchronize(st));
     settle();
