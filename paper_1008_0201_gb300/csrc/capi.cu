@@ -268,6 +268,17 @@ constexpr int kVerdictSteps = 8;
 
 std::mutex g_attr_mutex;
 bool g_attr_done[64] = {};
+// Clusters of 2^i CTAs of k_gram_oz_tc that run at once (one CTA per SM, a cluster inside one GPC, so not
+// 152 >> i: on a GB300 7 clusters of 16, 15 of 8, 36 of 4).
+int g_gram_tc_clusters[64][5] = {};
+
+// 0 if the cluster size cannot be launched
+int gram_tc_clusters(int size) {
+  int dev = 0, i = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  while ((1 << i) < size) ++i;
+  return g_gram_tc_clusters[dev][i];
+}
 
 int setup_attributes(int dev) {
   std::lock_guard<std::mutex> lk(g_attr_mutex);
@@ -291,6 +302,24 @@ int setup_attributes(int dev) {
   ok &= cudaFuncSetAttribute(k_gram_oz_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)tc_gram_oz_smem_bytes()) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gram_oz_tc, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  for (int i = 0; i < 5 && ok; ++i) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1u << i;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(1u << i);
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = tc_gram_oz_smem_bytes();
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int c = 0;
+    if (cudaOccupancyMaxActiveClusters(&c, k_gram_oz_tc, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      c = 0;
+    }
+    g_gram_tc_clusters[dev][i] = c;
+  }
   ok &= pivot_set_attributes() == 0;
   ok &= pivot_shifted_set_attributes() == 0;
   ok &= pivot64_set_attributes() == 0;
@@ -504,8 +533,25 @@ struct TcSplit {
   int gtiles = 0, ysplit = 1, tpc = 1;
 };
 
-int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, int tslabs, int CS, int CS32, int s,
-                bool lowp, bool fallback, const PivotParams& pp, cudaStream_t st, ProfRun& prof,
+// Which digit Gram (they give the same bits): 0 for k_gram_oz, else k_gram_oz_tc with that many of the CS
+// row shares of a pair per CTA.  The tensor-memory kernel takes a whole SM per CTA and less per stage of
+// 128 rows, whatever the columns; k_gram_oz runs twice per SM, and its work falls with the columns and
+// with the rows of the last stage.  Two shares per CTA where one each needs a second wave.
+// Time of k_gram_oz_tc over that of k_gram_oz (pairs of 64 columns, rows per share 144 / 192 / 256):
+//   4 pairs in 16 shares, one per CTA                  1.05 / 1.01 / 0.91
+//   12 pairs in 16 shares, two per CTA                 0.95 / 0.90 / 0.83 (56.0, 61.5, 69.8 us with k_gram_oz)
+//   16 pairs in 16 shares: only 15 of 16 clusters of 8 run at once  1.21 / 1.17 / 1.07
+//   300 problems, one share: 64 columns                1.02 / 0.97 / 0.90; 56 columns 1.15 / 1.13 / 1.04
+int gram_tc_shares(int oz, int km, long long pairs, int CS, int mean_k, int mean_rows) {
+  const int VR = (CS > 1 && pairs > gram_tc_clusters(CS)) ? 2 : 1;
+  if (oz == 2) return VR;
+  if (!oz || km != 64 || mean_k <= 60 || (CS > 1 && pairs > gram_tc_clusters(CS / VR))) return 0;
+  return mean_rows > (VR == 2 ? 128 : 192) * CS ? VR : 0;
+}
+
+// mean_k, mean_rows: columns of a pair and rows, over the problems of the launch.
+int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, int tslabs, int CS, int CS32, int mean_k,
+                int mean_rows, int s, bool lowp, bool fallback, const PivotParams& pp, cudaStream_t st, ProfRun& prof,
                 long long& launches, const TcMaps* maps = nullptr, const TcSplit* tsp = nullptr,
                 int fused_rows = 0) {
   int r = 0;
@@ -531,16 +577,9 @@ int launch_step(JacProb* dprobs, int count, int km, int max_half, int gslabs, in
                        (const JacProb*)dprobs, s, CS32, maps->g32);
   else if (lowp)
     r = launch_cluster(k_gram32, dim3(max_half * CS32, count), CS32, 128, 0, st, (const JacProb*)dprobs, s, CS32);
-  else if (pp.oz == 2 || (pp.oz && km == 64 && 64 * gslabs > 128 * CS)) {
-    // Two kernels with the same bits.  The tensor-memory one carries its results through more hands
-    // before the first row counts and takes less per stage of 128 rows: with 64 rows per share (512
-    // columns) k_gram_oz 20.7 us, k_gram_oz_tc 22.5; with 288 (32 pairs, 2304 rows) 94 and 67.
-    // Two shares of the rows per CTA where one each takes a second wave of CTAs (one per SM): 32 pairs
-    // in 8 shares each 86 -> 67 us.
-    const int VR = (CS > 1 && (long long)max_half * count * CS > 152) ? 2 : 1;
+  else if (int VR = gram_tc_shares(pp.oz, km, count * max_half, CS, mean_k, mean_rows))
     r = launch_cluster(k_gram_oz_tc, dim3(max_half * CS / VR, count), CS / VR, 512, tc_gram_oz_smem_bytes(), st,
                        (const JacProb*)dprobs, s, CS, VR);
-  }
   else if (pp.oz)
     r = launch_cluster(k_gram_oz, dim3(max_half * CS, count), CS, 256, oz_gram_smem_bytes(), st,
                        (const JacProb*)dprobs, s, CS);
@@ -899,8 +938,8 @@ int solve_real(int m, int n, int dtype, void* Gv, int ldg, const int8_t* Jdev, c
     }
     auto record = [&](cudaStream_t ss, long long& nl, ProfRun& pr) -> int {
       for (int s = 0; s < nsteps; ++s)
-        if (int r = launch_step(L.probs, 1, P.km, P.half, gslabs, tslabs, CS, CS32, s, low, phase != 1, pp, ss, pr,
-                                nl, use_tc ? &tmaps : nullptr, use_tc ? &tsplit : nullptr, fused))
+        if (int r = launch_step(L.probs, 1, P.km, P.half, gslabs, tslabs, CS, CS32, 2 * P.boff[1], P.mp, s, low, phase != 1,
+                                pp, ss, pr, nl, use_tc ? &tmaps : nullptr, use_tc ? &tsplit : nullptr, fused))
           return r;
       k_sweep_reduce<<<1, 256, 0, ss>>>(L.probs, L.io, L.rec, 0, nullptr);
       nl += 1;
@@ -1404,14 +1443,17 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
     JacIO* io;
     SweepRecord* rec;
     int count, km, max_half, max_steps, gslabs, tslabs, max_mp;
+    long long sum_k, sum_mp;
   };
   std::vector<Cls> cls;
   auto add_cls = [&](int first, int count, int km) {
     if (count <= 0) return;
-    Cls c{d_probs + first, d_io + first, d_rec + first, count, km, 0, 0, 0, 0, 0};
+    Cls c{d_probs + first, d_io + first, d_rec + first, count, km, 0, 0, 0, 0, 0, 0, 0};
     for (int i = first; i < first + count; ++i) {
       const Plan& P = plans[order[i]];
       c.max_mp = std::max(c.max_mp, P.mp);
+      c.sum_k += 2 * P.boff[1];
+      c.sum_mp += P.mp;
       c.max_half = std::max(c.max_half, P.half);
       c.max_steps = std::max(c.max_steps, P.nsteps);
       c.gslabs = std::max(c.gslabs, (P.mp + 63) / 64);
@@ -1444,8 +1486,8 @@ int solve_batched(int batch, const int* m, const int* n, int dtype, void* const*
       if (cudaMemsetAsync(d_remaining, 0, sizeof(int), ss) != cudaSuccess) return JAC_ECUDA;
       for (auto& c : cls) {
         for (int s = 0; s < c.max_steps; ++s)
-          if (int r = launch_step(c.probs, c.count, c.km, c.max_half, c.gslabs, c.tslabs, 1, 1, s, fp32_only, true, pp,
-                                  ss, pr, nl, nullptr, nullptr,
+          if (int r = launch_step(c.probs, c.count, c.km, c.max_half, c.gslabs, c.tslabs, 1, 1, (int)(c.sum_k / c.count),
+                                  (int)(c.sum_mp / c.count), s, fp32_only, true, pp, ss, pr, nl, nullptr, nullptr,
                                   (o.fused_step == 1 && c.max_mp <= fused_step_max_rows(c.km)) ? c.max_mp : 0))
             return r;
         k_sweep_reduce<<<c.count, 256, 0, ss>>>(c.probs, c.io, c.rec, 1, d_remaining);
