@@ -40,12 +40,11 @@ WORKLOAD = ("graded complex Hermitian PD n=4096: G = B D, B complex Gaussian, D 
             "w = 32 real (16 complex) columns, block-oriented (HB), round-robin, FP32 tensor-core sweeps + "
             "FP64 polish, V accumulated")
 SAMPLE_N = 768  # order of the oracle's bounded sample of the headline workload
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per evaluated pivot pair and launch,
-# from ncu captures of one launch on the same workload at n = 1024 (realified m = 2048, 32 pairs
-# per step, every pair evaluated), scaled to the headline by rows (each pair's columns are read
-# once: the traffic grows with m).  Only kernels unchanged since their capture are listed.
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per evaluated pivot pair and launch, from an
+# ncu capture of k_gram_oz_tc (31 pairs of 16384 rows, 64 columns each: profiles/rebuilt_kernels_ncu.md),
+# scaled to the headline's 8192 rows (each pair's columns are read once).
 TRAFFIC_PER_PAIR = {
-    "gram": 33643008 / 32 * (8192 / 2048),  # k_gram_oz: profiles/digit_kernels_graded_complex_1024_ncu.md
+    "gram": (261806592 + 5471488) / 31 * (8192 / 16384),
 }
 
 

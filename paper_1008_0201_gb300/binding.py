@@ -106,6 +106,8 @@ def load_library(path=LIB_PATH):
     lib.jacobi_profile_read.restype = I
     lib.jacobi_profile_end.argtypes = []
     lib.jacobi_profile_end.restype = I
+    lib.jacobi_release_scratch.argtypes = []
+    lib.jacobi_release_scratch.restype = I
     _lib = lib
     return lib
 
@@ -127,6 +129,13 @@ def default_opts(**kw):
             val = F64_PRODUCTS[val]
         setattr(o, key, val)
     return o
+
+
+def jacobi_release_scratch():
+    """Gives the scratch memory the library keeps mapped on the current device (at most 64 MB) back."""
+    rc = load_library().jacobi_release_scratch()
+    if rc != JAC_OK:
+        raise JacobiError(rc, status_string(rc))
 
 
 def status_string(code):

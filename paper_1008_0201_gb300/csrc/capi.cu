@@ -1181,9 +1181,9 @@ int solve_complex(int m, int n, void* Gv, int ldg, const int8_t* Jdev, const jac
   const int eb = (int)std::min<size_t>(4096, ((size_t)m * n + 255) / 256);
   k_realify<<<eb, 256, 0, st>>>(m, n, static_cast<const double2*>(Gv), ldg, Jdev, Gr, Jr);
   if (cudaGetLastError() != cudaSuccess) status = JAC_ECUDA;
-  // large orders keep the pivot in shifted representation: the pairing below carries the rounding
-  // of pass 1 into the eigenvectors (pivot_shifted.cu); at 2 m >= 512 rows the FP32 sweeps never
-  // take the fused step
+  // large orders keep the pivot in shifted representation: the pairing below lets any rounding of pass 1
+  // move the eigenvectors' entries, by 1e-9 and more from this order on (both pivots measured:
+  // pivot_shifted.cu); at 2 m >= 512 rows the FP32 sweeps never take the fused step
   const bool shifted = n >= 256;
   // pass 1: the sweep as requested
   if (status == JAC_OK)

@@ -156,7 +156,7 @@ struct PairStat {
   int inner_sweeps;
   int ns_steps;
   int active;         // 1 iff some |a_ij| > tol sqrt(a_ii a_jj): the FP64 convergence test
-  int evaluated;      // 1: the pivot ran for this pair in this sweep; 0: cached (pair_cache.cu)
+  int evaluated;      // 1: the pivot ran for this pair in this sweep; 0: cached (pair_cache.cuh)
   long long cyc[4];   // SM clocks of the pivot phases: stats, Cholesky, inner sweeps, J-orth.
 };
 

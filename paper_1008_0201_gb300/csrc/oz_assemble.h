@@ -47,7 +47,8 @@ OZ_HD double oz_ldexp(double x, int e) {
 #endif
 }
 
-// 0 < sh < 64; |hi| 2^sh + |lo| < 2^126
+// The plain form, for any 0 < sh < 64 and |hi| 2^sh + |lo| < 2^126: what oz_assemble_small, which the
+// kernels call, is held to (tests).
 OZ_HD double oz_assemble(long long hi, long long lo, int sh, int e) {
   // S = hi 2^sh + lo in 128-bit two's complement (H:L)
   unsigned long long L = (unsigned long long)hi << sh;

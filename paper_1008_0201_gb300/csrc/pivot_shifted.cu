@@ -9,11 +9,15 @@
 //
 // Why it stays for complex problems of order 256 and more (solve_complex, capi.cu): a complex
 // problem is solved as the real one of twice the order, whose columns are made exact pairs between
-// two passes, and what the first pass leaves in V there (|V^*V - I| ~ 1e-11 at order 1024) reaches
-// the eigenvectors through the eigenvalue gaps.  When any rounding of the first pass changes, their
-// entries move by up to 2e-7 of the largest at order 1024 (graded, positive definite), by 1e-9 to
-// 1e-4 at order 400 (Gaussian), but by 1e-9 only at order 200.  With this kernel the large ones keep the
-// digits they have always had; the pivots are 7% to 30% of such a solve.
+// two passes, and what the first pass leaves in V there (|V^*V - I| ~ 1e-11 at order 256, 5e-11 at 512)
+// reaches the eigenvectors through the eigenvalue gaps.  It is the pairing that sets their error, not
+// the pivot: over 54 problems of orders 96..512 (Gaussian, hyperbolic, graded; FP64 and mixed) |V^*V - J|
+// and the distance to a 64-bit solution were of the same size with either pivot (order 256, FP64: 3.6e-10
+// here, 6.7e-10 with pivot.cu; order 400 9.0e-9 and 8.0e-9).  But the entries move by that much when
+// any rounding of the first pass changes: 1e-11 at order 96, 1e-9 at 256, 2e-8 at 512, and programs that
+// compare large solves keep the digits they have had.  Below 256 pivot.cu runs; the line is where
+// entries start to move by 1e-9.  Its price (FP64, full block): 42.9 ms for 26.9 at order 256, 135 for 90 at
+// 512.
 #include "jacobi_common.cuh"
 #include "pair_cache.cuh"
 #include "ozaki.cuh"

@@ -82,8 +82,8 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
   bool bad = false;
   int it = 0;
   // The tile after the current one is loaded while the tensor cores work on the current one: the
-  // lookups of a tile and its loads are one chain of dependent reads, 12 of the 49 thousand clocks of
-  // a tile; with the loads ahead 4 (4000 problems of orders 8..128 64.1 -> 62.6 ms).
+  // lookups of a tile and its loads are one chain of dependent reads, 12 of 49 thousand clocks of a
+  // tile; with the loads ahead 4 of 43 (4000 problems of orders 8..128 64.1 -> 62.6 ms).
   struct Tile {
     int item, pair, op, oq, wp, k, ld, rows;
     double* col0;  // row r of the tile in column 0
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
     // ---- levels 0..7: block L (TMEM columns 64 L ..) accumulates sum_{t+u=L} X_t V_u.  The planes of
     // V~ lie one after the other, so one MMA of N = 64 nb takes X_t against planes u .. u + nb - 1 into
     // blocks t + u .. t + u + nb - 1: 12 MMAs per 16 K in place of 36, each plane of X~ read once or
-    // twice and no descriptor formed in the loop: 15.3 -> 5.3 thousand clocks of a full tile's 60.
+    // twice and no descriptor formed in the loop: 15.3 -> 5.3 thousand clocks of a full tile, which takes 43.
     const uint64_t dx = tc::desc_sw128(xs, 16, 1024), dv = tc::desc_sw128(vs, 16, 1024);
     if (tid == 0) {
       tc::fence_after_sync();
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(512, 1) k_update_oz_tc(const JacProb* __restri
 // entries j >= i are formed.
 // The MMAs take 4 thousand clocks of the 19 of a stage, where mma.sync (k_gram_oz) takes about half of
 // 34; the digits take 5, the integer sums and their rounding 8.  32 pairs of 2304 rows: 94 us with
-// k_gram_oz, 86 with one share per CTA, 67 with two.
+// k_gram_oz, 86 with one share per CTA, 67 with two; where it is the slower one: gram_tc_shares (capi.cu).
 #define TGD_CHUNK 65536                        // 8 planes x 64 rows x 128 B
 #define TGD_TOT (2 * TGD_CHUNK)                // FP64 partials [VR][64][65] after the digits
 #define TGD_MISC (TGD_TOT + 2 * 64 * 65 * 8)
