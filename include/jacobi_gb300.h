@@ -25,6 +25,8 @@
  *     (jacobi_release_scratch), and returned to it before the call returns.  A program that
  *     gave the device a memory pool, or its default pool a release threshold, gets the
  *     scratch from there instead (cudaMallocAsync).
+ *   - Column norms of G lie within 4e-23 .. 1.8e19 (their squares within FP32's range, in any ratio to
+ *     each other); scale a factor that does not.
  *   - Errors are reported by the return value and never by abort or trap.  A negative value
  *     -k means argument k (1-based) is invalid; nothing has been written then.  Positive
  *     values are the jac_status codes below; outputs are then unspecified except for info.
@@ -274,7 +276,7 @@ int jacobi_eig_batched(int batch, const int* m, const int* n, int dtype, void* c
  * 22 G_bar, 23 ldgb, 24 s_gb    output dL/dG, or NULL (then G may be NULL)
  * 25 stream
  * Returns 0, a negative argument position, JAC_ENOMEM or JAC_ECUDA.  Asynchronous on stream
- * (its n x n x batch scratch is stream-ordered on that stream).
+ * (its n x n x batch scratch is stream-ordered on that stream).  May be captured in a CUDA graph.
  */
 int jacobi_eig_backward(int batch, int n, const double* lambda, long long s_lam, const double* U,
                         int ldu, long long s_u, const double* lambda_bar, long long s_lbar,
